@@ -59,6 +59,7 @@ def bytes_per_voxel(N):
     H = (N + 1) // 2
     s32 = 6 * 8 * H / N
     s64 = 2 * s32
+    v32 = s32 / 2
     return {
         # r, p, x in; p, x out; tangent; spectrum out (steady state: the
         # first iteration of a solve reads no p or x)
@@ -66,7 +67,13 @@ def bytes_per_voxel(N):
         "p2_f32": 2 * s32, "p3_f32": 2 * s32, "p4_f32": 2 * s32,
         "p5_dot_f32": s32 + 24 + 24,               # spectrum in; q out; p in
         "cg_update_f32": 3 * 24,                   # r, q in; r out
-        # the mixed path's CG without the update pass: P1 as p1_cg (and the
+        # the mixed path's CG on displacement coefficients (three complex
+        # values per frequency, v32 bytes per voxel): x1i reads r, p, x and
+        # writes p, x and the spectrum; the row pass reads and writes the
+        # spectrum and reads the tangent; x1f reads the spectrum and r and
+        # writes r
+        "x1i_cg_f32": 5 * v32 + s32, "rows_cg_f32": 2 * s32 + 28, "x1f_cg_f32": s32 + 2 * v32,
+        # CG on real fields without the update pass: P1 as p1_cg (and the
         # dot <p, C:p>), P5 reads the spectrum and r and writes r
         "p1_cgf_f32": 5 * 24 + 28 + s32,
         "p5_cgf_f32": s32 + 24 + 24,
@@ -82,9 +89,11 @@ def bytes_per_voxel(N):
 
 
 # The CG kernels of one iteration, in launch order: with the update pass
-# (FP64 path, basic scheme) and without it (mixed path).
+# (FP64 path), and on displacement coefficients (mixed path; CGF_KINDS is
+# the mixed path's earlier form on real fields, for its recorded lines).
 CG_KINDS = ("p1_cg", "p2", "p3", "p4", "p5_dot", "cg_update")
 MATVEC_KINDS = ("p1_cg", "p2", "p3", "p4", "p5_dot")
+DC_KINDS = ("x1i_cg", "p4", "rows_cg", "p2", "x1f_cg", "cg_rr")
 CGF_KINDS = ("p1_cgf", "p2", "p3", "p4", "p5_cgf", "cg_rr")
 
 # Pencil plans N = N1 x N2 of the FFT passes (the register DFT of N1 points,
@@ -141,10 +150,9 @@ def flops_per_voxel(N):
 # the dominant kernels from one ncu capture each (the ncu summaries kept
 # with the repository give the command), valid while the kernel sources
 # have the digest they had then (SHA-256 prefix of the files listed).
-KERNEL_FILES = ("common.cuh", "fft_core.cuh", "passes.cuh")
+KERNEL_FILES = ("common.cuh", "fft_core.cuh", "passes.cuh", "cg_passes.cuh")
 FS_KERNEL_FILES = KERNEL_FILES + ("fs_passes.cuh",)
-TRAFFIC = {"p1_cgf_f32": {"N": 243, "bytes": 2413.6e6, "digest": "82255a5e31b86c10", "files": KERNEL_FILES},
-           "fs_p1_cgf_f32": {"N": 243, "bytes": 3587.1e6, "digest": "43f6874074ac81bb", "files": FS_KERNEL_FILES}}
+TRAFFIC = {"fs_p1_cgf_f32": {"N": 243, "bytes": 3587.1e6, "digest": "43f6874074ac81bb", "files": FS_KERNEL_FILES}}
 
 
 def _strip_comments(src: bytes) -> bytes:
@@ -473,16 +481,24 @@ def cg_roofline(prof, N, field_iters, projections, tangent_calls, sfx="_f32", hb
     Newton iteration: the projection of an FP32 inner solution in the mixed
     path, the FP64 residual in the FP64 path) and, per tangent, once per
     right-hand side (six) and, in FP32, once per projection of its six
-    solutions."""
+    solutions. On displacement coefficients P2 runs once more per
+    right-hand side of a tangent and P4 once per solution (Newton and
+    tangent)."""
     if hbm is None:
         hbm, _ = measured_hbm()
     bpv = bytes_per_voxel(N)
     V = N ** 3
     fused = ("p1_cgf" + sfx) in prof
-    kinds, mv_kinds = (CGF_KINDS, CGF_KINDS[:5]) if fused else (CG_KINDS, MATVEC_KINDS)
+    coef = ("rows_cg" + sfx) in prof
+    kinds, mv_kinds = ((DC_KINDS, DC_KINDS[:5]) if coef else (CGF_KINDS, CGF_KINDS[:5]) if fused
+                       else (CG_KINDS, MATVEC_KINDS))
     eff = {k: field_iters for k in ("p1_cg", "p5_dot", "cg_update", "p1_cgf", "p5_cgf", "cg_rr")}
     for k in ("p2", "p3", "p4"):
         eff[k] = field_iters + projections + (12 if sfx == "_f32" else 6) * tangent_calls
+    if coef:
+        eff.update({k: field_iters for k in ("x1i_cg", "rows_cg", "x1f_cg")})
+        eff["p2"] = field_iters + 6 * tangent_calls
+        eff["p4"] = field_iters + projections + 6 * tangent_calls
     kern = {}
     for base in kinds:
         name = base + sfx
@@ -506,9 +522,11 @@ def cg_roofline(prof, N, field_iters, projections, tangent_calls, sfx="_f32", hb
                 "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s", "frac": round(gbs / hbm, 3)}
 
     return {"kernels": kern,
-            "matvec": agg(mv_kinds, "P1-P5: q = G(C:p) with the fused CG steps, per field"),
-            "iteration": agg(kinds, "one CG iteration, per field: P1-P5" +
-                             (" (update fused into P1/P5)" if fused else " + update pass"))}
+            "matvec": agg(mv_kinds, ("x1i, P4, rows, P2, x1f" if coef else "P1-P5") +
+                          ": q = G(C:p) with the fused CG steps, per field"),
+            "iteration": agg(kinds, "one CG iteration, per field: " +
+                             ("x1i, P4, rows, P2, x1f, cg_rr" if coef else
+                              "P1-P5" + (" (update fused into P1/P5)" if fused else " + update pass")))}
 
 
 def basic_scheme_line(N=135, n_inc=4, timed_from=2):
@@ -935,8 +953,8 @@ def main():
         fused = rf["matvec"]["ms_per_field_iter"] if rf["matvec"] else None
         line["cufft_line"] = {"matvec_ms": cufft_matvec_line(N), "fused_matvec_ms": fused,
                               "what": "q = G(C:p) at N^3 FP32: cuFFT rfftn/irfftn via torch.fft with "
-                                      "separate elementwise C:p and Ghat kernels, vs the fused passes "
-                                      "P1-P5 per CG field-iteration in the timed region"}
+                                      "separate elementwise C:p and Ghat kernels, vs the five fused "
+                                      "passes per CG field-iteration in the timed region"}
         line["basic_scheme_vs_cg"] = basic_scheme_line()
         line["finite_strain"] = finite_strain_line()
         rves = serving.batched_workload()

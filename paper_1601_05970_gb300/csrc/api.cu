@@ -19,7 +19,7 @@
 #include "driver.h"
 #include "host_common.h"
 #include "materials.h"
-#include "passes.cuh"
+#include "cg_passes.cuh"
 #include "pointwise.cuh"
 #include "schedule.cuh"
 #include "batch.cuh"
@@ -59,12 +59,13 @@ cudaError_t run_pass(int N, PassKind kind, const PassArgs& a, int nf, cudaStream
     }
 }
 
-// FP32: the most blocks of any schedule variant of the row passes (half the
-// rows per block), so that the partial-sum buffer fits every schedule.
+// Most blocks of a row or x1 pass, over the schedules (for the partial sums).
 template <int N>
 static int row_blocks_n(bool fp64) {
     return fp64 ? Cfg<N, double>::row_blocks
-                : std::max(Cfg<N, float>::row_blocks, Cfg<N, float, Plan<N>::N1, 1>::row_blocks);
+                : std::max({Cfg<N, float>::row_blocks, Cfg<N, float, Plan<N>::N1, 1>::row_blocks,
+                            RowCfg<N, RowSplit<N>::N1, 1>::blocks, X1<N>::blocks,
+                            (Cfg<N, dd>::H + Cfg<N, dd>::W3 - 1) / Cfg<N, dd>::W3 * N});
 }
 
 int row_blocks(int N, bool fp64) {
@@ -75,6 +76,25 @@ int row_blocks(int N, bool fp64) {
         FFTG_CASE(243)
 #undef FFTG_CASE
         default: return 0;
+    }
+}
+
+// Blocks per field of the passes whose partial sums a kernel reduces: the x1
+// passes (FP32, double-float right-hand side) and P5 at its default schedule.
+struct PassBlocks {
+    int x1, x1_dd, p5;
+};
+static PassBlocks pass_blocks(int N) {
+    switch (N) {
+#define FFTG_CASE(n)                                                                                     \
+    case n:                                                                                              \
+        return {X1<n>::blocks, (Cfg<n, dd>::H + Cfg<n, dd>::W3 - 1) / Cfg<n, dd>::W3 * n,                \
+                Cfg<n, float>::row_blocks};
+        FFTG_CASE(3) FFTG_CASE(5) FFTG_CASE(9) FFTG_CASE(15) FFTG_CASE(25) FFTG_CASE(27)
+        FFTG_CASE(45) FFTG_CASE(75) FFTG_CASE(81) FFTG_CASE(125) FFTG_CASE(135) FFTG_CASE(225)
+        FFTG_CASE(243)
+#undef FFTG_CASE
+        default: return {0, 0, 0};
     }
 }
 }  // namespace fftg
@@ -92,19 +112,18 @@ using namespace fftg;
 
 namespace {
 enum : int {
-    KK_CONSTITUTIVE_F32 = PK_COUNT, KK_CONSTITUTIVE_F64, KK_CG_UPDATE_F32, KK_CG_UPDATE_F64,
-    KK_NEWTON_UPDATE_F32, KK_NEWTON_UPDATE_F64, KK_TANGENT_FLOOR, KK_TANGENT_AVERAGE,
-    KK_CG_FINISH_F32, KK_CG_FINISH_F64, KK_TANGENT_BOUNDS, KK_CG_RR, KK_COUNT
+    KK_CONSTITUTIVE_F32 = PK_COUNT, KK_CONSTITUTIVE_F64, KK_CG_UPDATE_F64, KK_NEWTON_UPDATE_F64,
+    KK_NEWTON_NORM_F32, KK_TANGENT_FLOOR, KK_TANGENT_AVERAGE, KK_CG_FINISH_F64, KK_TANGENT_BOUNDS,
+    KK_CG_BEGIN, KK_CG_RR, KK_COUNT
 };
 const char* const kKindNames[KK_COUNT] = {
-    "p1_plain_f64", "p1_plain_f32", "p1_tan_f64", "p1_tan_f32", "p1_cg_f64", "p1_cg_f32",
+    "p1_plain_f64", "p1_plain_f32", "p1_tan_f64", "p1_tan_f32", "p1_cg_f64",
     "p1_tanrhs_f64", "p1_tanrhs_f32", "p2_f64", "p2_f32", "p4_f64", "p4_f32", "p3_f64", "p3_f32",
-    "p5_plain_f64", "p5_plain_f32", "p5_dot_f64", "p5_dot_f32", "p5_rhs_f64_to_f64",
-    "p5_rhs_f64_to_f32", "p5_rhs_f32_to_f32", "p1_plain_dd", "p2_dd", "p3_dd", "p4_dd",
-    "p5_rhs_dd_to_f32", "p5_plain_dd_to_f64", "p1_cgf_f32", "p5_cgf_f32", "constitutive_f32",
-    "constitutive_f64",
-    "cg_update_f32", "cg_update_f64", "newton_update_f32", "newton_update_f64", "tangent_floor",
-    "tangent_average", "cg_finish_f32", "cg_finish_f64", "tangent_bounds", "cg_rr_f32"};
+    "p5_plain_f64", "p5_plain_f32", "p5_dot_f64", "p5_dot_f32", "p5_rhs_f64_to_f64", "p1_plain_dd", "p2_dd",
+    "p3_dd", "p4_dd", "p5_plain_dd_to_f64", "x1i_cg_f32", "rows_cg_f32", "x1f_cg_f32", "x1f_rhs_f32",
+    "x1f_rhs_dd", "x1i_solution_f32", "p5_newton_f32", "constitutive_f32", "constitutive_f64",
+    "cg_update_f64", "newton_update_f64", "newton_norm_f32", "tangent_floor",
+    "tangent_average", "cg_finish_f64", "tangent_bounds", "cg_begin_f32", "cg_rr_f32"};
 
 // Ring of event pairs around the handle's launches; drained at every read.
 struct Prof {
@@ -150,7 +169,10 @@ struct fftg_handle {
     double* epbar_tr = nullptr;  // [B][cs] trial
     double* sigma = nullptr;     // [B][6][cs]
     void* tangent = nullptr;     // [B][7][cs] inner precision
-    void* x = nullptr;           // [nf][6][cs] inner precision
+    // [nf][6][cs] inner precision. Mixed: r, p and x hold displacement
+    // coefficients (cg_passes.cuh, at most 12 N^2 (N + 1) bytes a field), q the
+    // solution in real space
+    void* x = nullptr;
     void* r = nullptr;
     void* p = nullptr;
     void* q = nullptr;
@@ -171,7 +193,8 @@ struct fftg_handle {
     double* h_E = nullptr;
     int* h_active = nullptr;
 
-    unsigned int* guard = nullptr;   // loop-pass counters: [0] CG graph, [1] Newton loop of a group graph
+    unsigned int* guard = nullptr;   // loop-pass counters: [0] CG graph, [1] Newton loop of a group graph;
+                                     // [2] fields done with their iteration (0 between kernels)
     int* run_dev = nullptr;          // device-driven increments (fftg_group_step)
     double* dE_dev = nullptr;
     double* Ecom_dev = nullptr;
@@ -322,14 +345,6 @@ double frob6(const double* v) {
 // FFT precision of a pass sequence
 enum : int { FFT_F32 = 0, FFT_F64 = 1, FFT_DD = 2 };
 
-// The mixed path computes its residual G sigma with double-float FFTs
-// (dd.cuh) in place of FP64 ones: about 1e-14 of ||sigma|| where FP64 gives
-// 1e-16, far below the CG roundoff floor, at a fraction of the FP64 cost on
-// this GPU. 0: FP64 FFTs.
-#ifndef FFTG_RESIDUAL_DD
-#define FFTG_RESIDUAL_DD 1
-#endif
-
 static PassArgs base_args(fftg_handle* h, bool fp64) {
     PassArgs a{};
     a.tw = fp64 ? h->tw64 : h->tw32;
@@ -407,63 +422,113 @@ static PassArgs base_args_fft(fftg_handle* h, int prec) {
     return a;
 }
 
-static int run_p234(fftg_handle* h, int prec, double scale, CGState* cg, int nf, const int* mask,
-                    const double* red_in = nullptr, int red_n = 0) {
+static int run_p234(fftg_handle* h, int prec, double scale, CGState* cg, int nf, const int* mask) {
     PassArgs a = base_args_fft(h, prec);
     a.out = h->spec;
     a.cg = cg;
     a.scale = scale;
     a.active = mask;
-    a.red_in = red_in;
-    a.red_n = red_n;
     const PassKind k2 = prec == FFT_DD ? PK_P2_DD : prec == FFT_F64 ? PK_P2_F64 : PK_P2_F32;
     const PassKind k3 = prec == FFT_DD ? PK_P3_DD : prec == FFT_F64 ? PK_P3_F64 : PK_P3_F32;
     const PassKind k4 = prec == FFT_DD ? PK_P4_DD : prec == FFT_F64 ? PK_P4_F64 : PK_P4_F32;
     CK(pass(h, k2, a, nf));
-    a.red_in = nullptr;
     CK(pass(h, k3, a, nf));
     CK(pass(h, k4, a, nf));
     return FFTG_OK;
 }
 
-// r = -G sigma for the cells in the active mask (FP64 FFTs, or double-float
-// ones in the mixed path), rounded to the inner precision; x = 0.
+// Forward x1 of the right-hand sides' spectra to displacement coefficients r
+// (times scale), and the start of their solves.
+static int launch_rhs(fftg_handle* h, int prec, double scale, int nf, const int* active) {
+    PassArgs a = base_args_fft(h, prec);
+    a.in = h->spec;
+    a.aux3 = h->r;
+    a.cg = h->cg;
+    a.scale = scale;
+    a.active = active;
+    CK(pass(h, prec == FFT_DD ? PK_X1F_RHS_DD : PK_X1F_RHS_F32, a, nf));
+    const PassBlocks nb = pass_blocks(h->N);
+    const int slot = prof_begin(h, KK_CG_BEGIN);
+    k_cg_begin<<<nf, 1024, 0, h->stream>>>(h->partials, prec == FFT_DD ? nb.x1_dd : nb.x1, h->cg, active);
+    prof_end(h, slot);
+    CK(cudaGetLastError());
+    return FFTG_OK;
+}
+
+// r = -G sigma for the cells in the active mask. FP64: the five passes, x = 0.
+// Mixed: double-float FFTs (dd.cuh; about 1e-14 of ||sigma|| where FP64 gives
+// 1e-16, far below the CG roundoff floor, at a fraction of the FP64 cost on
+// this GPU) up to the displacement coefficients, rounded to FP32.
 static int launch_residual(fftg_handle* h) {
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
-    const bool dd = h->mixed && FFTG_RESIDUAL_DD;
-    PassArgs a = base_args_fft(h, dd ? FFT_DD : FFT_F64);
+    const int prec = h->mixed ? FFT_DD : FFT_F64;
+    PassArgs a = base_args_fft(h, prec);
     a.in = h->sigma;
     a.out = h->spec;
     a.active = h->active;
-    CK(pass(h, dd ? PK_P1_PLAIN_DD : PK_P1_PLAIN_F64, a, h->B));
-    int rc = run_p234(h, dd ? FFT_DD : FFT_F64, -invN3, nullptr, h->B, h->active);
+    CK(pass(h, h->mixed ? PK_P1_PLAIN_DD : PK_P1_PLAIN_F64, a, h->B));
+    if (h->mixed) {
+        CK(pass(h, PK_P2_DD, a, h->B));
+        return launch_rhs(h, FFT_DD, -invN3, h->B, h->active);
+    }
+    int rc = run_p234(h, FFT_F64, -invN3, nullptr, h->B, h->active);
     if (rc) return rc;
-    PassArgs b = base_args_fft(h, dd ? FFT_DD : FFT_F64);
+    PassArgs b = base_args_fft(h, FFT_F64);
     b.in = h->spec;
     b.out = h->r;
     b.cg = h->cg;
     b.active = h->active;
-    CK(pass(h, dd ? PK_P5_RHS_DD_TO_F32 : h->mixed ? PK_P5_RHS_F64_TO_F32 : PK_P5_RHS_F64_TO_F64, b, h->B));
-    CK(cudaMemsetAsync(h->x, 0, (size_t)h->B * 6 * h->cs * (h->mixed ? 4 : 8), h->stream));
+    CK(pass(h, PK_P5_RHS_F64_TO_F64, b, h->B));
+    CK(cudaMemsetAsync(h->x, 0, (size_t)h->B * 6 * h->cs * 8, h->stream));
     return FFTG_OK;
 }
 
-// The mixed path's CG (not the basic scheme) runs without the update pass:
-// alpha from <p, C : p> in P1, r -= alpha q in P5 (passes.cuh, P1_CGF).
-// 0: P1_CG / P5_DOT and the update pass, as in the FP64 path.
-#ifndef FFTG_CG_FUSED
-#define FFTG_CG_FUSED 1
-#endif
-static bool cg_fused(const fftg_handle* h) {
-    return FFTG_CG_FUSED && h->mixed && h->opt.solver == FFTG_SOLVER_CG;
+namespace fftg {
+// Loop condition of the device-resident CG (a conditional WHILE node of a
+// CUDA graph): go on while any of the nf solves is running. `guard` counts
+// the passes of the loop body; past `cap` passes the loop stops whatever the
+// solves report, so the loop always ends.
+struct CgLoop {
+    cudaGraphConditionalHandle cond = 0;
+    unsigned int* guard = nullptr;  // null: not in a loop
+    unsigned int cap = 0;
+};
+
+__device__ __forceinline__ void cg_continue(const CgLoop& l, const CGState* cg, int nf) {
+    bool any = false;
+    for (int f = 0; f < nf; ++f) any = any || (__ldcg(&cg[f].done) == CG_RUNNING);
+    const unsigned int n = ++(*l.guard);
+    if (n >= l.cap) any = false;
+    cudaGraphSetConditional(l.cond, any ? 1u : 0u);
 }
+
+__global__ void k_cg_continue(CgLoop l, const CGState* cg, int nf) {
+    if (threadIdx.x == 0) cg_continue(l, cg, nf);
+}
+
+// k_cg_rr and, by the last of its blocks, the loop condition: a launch less
+// per iteration.
+__global__ void __launch_bounds__(1024) k_cg_rr_loop(const double* partials, int nb, CGState* cg, CgLoop l) {
+    cg_rr_block(partials, nb, cg);
+    if (threadIdx.x != 0) return;
+    if (gridDim.x > 1) {
+        __threadfence();
+        if (atomicAdd(l.guard + 2, 1u) != gridDim.x - 1) return;
+        l.guard[2] = 0u;
+        __threadfence();
+    }
+    cg_continue(l, cg, (int)gridDim.x);
+}
+}  // namespace fftg
 
 // One CG iteration on nf fields: the fused matvec passes and the update.
 // `tangent`/`tstride`: per-field tangents (batched cells) or one shared.
-static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long long tstride) {
+// In a loop body the last kernel also sets the loop's condition.
+static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long long tstride,
+                               const CgLoop& loop = CgLoop{}) {
     const bool f64 = !h->mixed;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
-    if (cg_fused(h)) {
+    if (h->mixed) {
         PassArgs a = base_args(h, false);
         a.aux = h->r;
         a.aux2 = h->p;
@@ -472,21 +537,27 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
         a.tstride = tstride;
         a.out = h->spec;
         a.cg = h->cg;
-        CK(pass(h, PK_P1_CGF_F32, a, nf));
-        // P2 reduces P1's block partials of <p, C : p> (alpha)
-        const int nb1 = variant_shape(h->N, TK_P1, schedule_variant(h->N, TK_P1)).blocks;
-        int rc = run_p234(h, FFT_F32, invN3, h->cg, nf, nullptr, h->partials, nb1);
-        if (rc) return rc;
-        PassArgs b = base_args(h, false);
-        b.in = h->spec;
-        b.aux = h->r;
-        b.aux3 = h->r;
-        b.cg = h->cg;
-        CK(pass(h, PK_P5_CGF_F32, b, nf));
-        // <r, r> from P5's block partials: beta and the stopping tests
-        const int nb5 = variant_shape(h->N, TK_P5, schedule_variant(h->N, TK_P5)).blocks;
+        CK(pass(h, PK_X1I_CG_F32, a, nf));
+        CK(pass(h, PK_P4_F32, a, nf));
+        CK(pass(h, PK_ROWS_CG_F32, a, nf));
+        // P2 reduces the row pass's block partials of <p, C : p> (alpha)
+        PassArgs b = a;
+        b.red_in = h->partials;
+        b.red_n = variant_shape(h->N, TK_P1, schedule_variant(h->N, TK_P1)).blocks;
+        CK(pass(h, PK_P2_F32, b, nf));
+        PassArgs c = base_args(h, false);
+        c.in = h->spec;
+        c.aux3 = h->r;
+        c.cg = h->cg;
+        c.scale = invN3;
+        CK(pass(h, PK_X1F_CG_F32, c, nf));
+        // <r, r> from its block partials: beta and the stopping tests
+        const int nb = pass_blocks(h->N).x1;
         const int slot = prof_begin(h, KK_CG_RR);
-        k_cg_rr<<<nf, 1024, 0, h->stream>>>(h->partials, nb5, h->cg);
+        if (loop.guard)
+            k_cg_rr_loop<<<nf, 1024, 0, h->stream>>>(h->partials, nb, h->cg, loop);
+        else
+            k_cg_rr<<<nf, 1024, 0, h->stream>>>(h->partials, nb, h->cg);
         prof_end(h, slot);
         CK(cudaGetLastError());
         return FFTG_OK;
@@ -499,15 +570,15 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
     a.tstride = tstride;
     a.out = h->spec;
     a.cg = h->cg;
-    CK(pass(h, f64 ? PK_P1_CG_F64 : PK_P1_CG_F32, a, nf));
-    int rc = run_p234(h, f64 ? FFT_F64 : FFT_F32, invN3, h->cg, nf, nullptr);
+    CK(pass(h, PK_P1_CG_F64, a, nf));
+    int rc = run_p234(h, FFT_F64, invN3, h->cg, nf, nullptr);
     if (rc) return rc;
     PassArgs b = base_args(h, f64);
     b.in = h->spec;
     b.out = h->q;
     b.aux = h->p;
     b.cg = h->cg;
-    CK(pass(h, f64 ? PK_P5_DOT_F64 : PK_P5_DOT_F32, b, nf));
+    CK(pass(h, PK_P5_DOT_F64, b, nf));
     VecArgs u{};
     u.V = h->V;
     u.cs = h->cs;
@@ -518,33 +589,17 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
     u.cg = h->cg;
     u.partials = h->partials;
     u.fstride = 6 * h->cs;
-    dim3 g(vector_blocks(h->cs, f64 ? 8 : 4), 1, nf);
-    const int slot = prof_begin(h, f64 ? KK_CG_UPDATE_F64 : KK_CG_UPDATE_F32);
-    if (f64)
-        k_cg_update<double><<<g, kThreads, 0, h->stream>>>(u);
-    else
-        k_cg_update<float><<<g, kThreads, 0, h->stream>>>(u);
+    dim3 g(vector_blocks(h->cs, 8), 1, nf);
+    const int slot = prof_begin(h, KK_CG_UPDATE_F64);
+    k_cg_update<double><<<g, kThreads, 0, h->stream>>>(u);
     prof_end(h, slot);
     CK(cudaGetLastError());
+    if (loop.guard) {
+        k_cg_continue<<<1, 32, 0, h->stream>>>(loop, h->cg, nf);
+        CK(cudaGetLastError());
+    }
     return FFTG_OK;
 }
-
-namespace fftg {
-// Loop condition of the device-resident CG (a conditional WHILE node of a
-// CUDA graph): go on while any of the nf solves is running. `guard` counts
-// the passes of the loop body; past `cap` passes the loop stops whatever the
-// solves report, so the loop always ends.
-__global__ void k_cg_continue(cudaGraphConditionalHandle cond, const CGState* cg, int nf,
-                              unsigned int* guard, unsigned int cap) {
-    if (threadIdx.x != 0) return;
-    bool any = false;
-    for (int f = 0; f < nf; ++f) any = any || (cg[f].done == CG_RUNNING);
-    const unsigned int n = ++(*guard);
-    if (n >= cap) any = false;
-    cudaGraphSetConditional(cond, any ? 1u : 0u);
-}
-
-}  // namespace fftg
 
 // Device-resident CG: one graph whose conditional WHILE node repeats the
 // iteration (the five passes and the update) while any solve is running;
@@ -570,13 +625,9 @@ static int build_cg_graph(fftg_handle* h, int nf, const void* tangent, long long
     if (cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) !=
         cudaSuccess)
         return FFTG_ECUDA;
-    int rc = launch_cg_iteration(h, nf, tangent, tstride);
     const unsigned int cap =
         (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
-    if (rc == FFTG_OK) {
-        k_cg_continue<<<1, 32, 0, h->stream>>>(cond, h->cg, nf, h->guard, cap);
-        if (cudaGetLastError() != cudaSuccess) rc = FFTG_ECUDA;
-    }
+    int rc = launch_cg_iteration(h, nf, tangent, tstride, CgLoop{cond, h->guard, cap});
     cudaGraph_t captured = nullptr;
     if (cudaStreamEndCapture(h->stream, &captured) != cudaSuccess || rc) return FFTG_ECUDA;
     if (cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess) return FFTG_ECUDA;
@@ -627,32 +678,36 @@ static fftg_handle::CgGraph* cg_graph_for(fftg_handle* h, int nf, const void* ta
     return &h->graphs.back();
 }
 
-// Mixed precision: x <- G x (FP32 passes) on the nf solution fields. The
-// FP32 recursion of CG lets the residual, and with it x, drift out of the
-// compatible space (by about 1e-5 of |x| over some tens of iterations:
-// each q = G (C : p) carries FP32 rounding). Newton's corrections then add
-// an incompatible part to eps* that no later correction removes, and the
-// converged state sits off the FP64 solution by that much. One projection
-// per solve brings the incompatible part down to the rounding of a single
-// FP32 projection.
-#ifndef FFTG_PROJECT_X
-#define FFTG_PROJECT_X 1
-#endif
-static int project_solution(fftg_handle* h, int nf, const int* active) {
-    if (!h->mixed || !FFTG_PROJECT_X) return FFTG_OK;
-    const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
+// Mixed path: the solutions x (with their pending steps) from displacement
+// coefficients to real space, compatible up to the rounding of one FP32
+// inverse transform. newton: added to eps* of the cells in the mask, with
+// ||x||^2; else written to q.
+static int launch_solution(fftg_handle* h, int nf, const int* active, bool newton) {
     PassArgs a = base_args(h, false);
-    a.in = h->x;
+    a.aux2 = h->p;
+    a.aux3 = h->x;
     a.out = h->spec;
+    a.cg = h->cg;
     a.active = active;
-    CK(pass(h, PK_P1_PLAIN_F32, a, nf));
-    int rc = run_p234(h, FFT_F32, invN3, nullptr, nf, active);
-    if (rc) return rc;
+    CK(pass(h, PK_X1I_SOLUTION_F32, a, nf));
     PassArgs b = base_args(h, false);
-    b.in = h->spec;
-    b.out = h->x;
+    b.out = h->spec;
     b.active = active;
-    CK(pass(h, PK_P5_PLAIN_F32, b, nf));
+    CK(pass(h, PK_P4_F32, b, nf));
+    PassArgs c = base_args(h, false);
+    c.in = h->spec;
+    c.active = active;
+    if (!newton) {
+        c.out = h->q;
+        CK(pass(h, PK_P5_PLAIN_F32, c, nf));
+        return FFTG_OK;
+    }
+    c.aux3 = h->eps_work;
+    CK(pass(h, PK_P5_NEWTON_F32, c, nf));
+    const int slot = prof_begin(h, KK_NEWTON_NORM_F32);
+    k_newton_norm<<<nf, 1024, 0, h->stream>>>(h->partials, pass_blocks(h->N).p5, h->nd, active);
+    prof_end(h, slot);
+    CK(cudaGetLastError());
     return FFTG_OK;
 }
 
@@ -683,9 +738,9 @@ static int launch_bounds(fftg_handle* h, const void* tangent, long long cell_tan
     return FFTG_OK;
 }
 
-// x += alpha p for the solves whose last update left that step pending.
+// FP64 path: x += alpha p for the solves whose last update left that step
+// pending.
 static int launch_cg_finish(fftg_handle* h, int nf) {
-    const bool f64 = !h->mixed;
     VecArgs u{};
     u.V = h->V;
     u.cs = h->cs;
@@ -693,12 +748,9 @@ static int launch_cg_finish(fftg_handle* h, int nf) {
     u.p = h->p;
     u.cg = h->cg;
     u.fstride = 6 * h->cs;
-    dim3 g(vector_blocks(6 * h->cs, f64 ? 8 : 4), 1, nf);
-    const int slot = prof_begin(h, f64 ? KK_CG_FINISH_F64 : KK_CG_FINISH_F32);
-    if (f64)
-        k_cg_finish<double><<<g, kThreads, 0, h->stream>>>(u);
-    else
-        k_cg_finish<float><<<g, kThreads, 0, h->stream>>>(u);
+    dim3 g(vector_blocks(6 * h->cs, 8), 1, nf);
+    const int slot = prof_begin(h, KK_CG_FINISH_F64);
+    k_cg_finish<double><<<g, kThreads, 0, h->stream>>>(u);
     prof_end(h, slot);
     CK(cudaGetLastError());
     return FFTG_OK;
@@ -715,14 +767,16 @@ static int run_cg(fftg_handle* h, int nf, const void* tangent, long long tstride
         if (g) {
             CK(cudaMemsetAsync(h->guard, 0, sizeof(unsigned int), h->stream));
             CK(cudaGraphLaunch(g->exec, h->stream));
-            int rc = launch_cg_finish(h, nf);
-            if (rc) return rc;
+            if (!h->mixed) {
+                int rc = launch_cg_finish(h, nf);
+                if (rc) return rc;
+            }
             // one launch of each kernel of an iteration per loop pass
             CK(cudaMemcpyAsync(h->h_cg, h->cg, nf * sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
             CK(cudaStreamSynchronize(h->stream));
             int maxit = 0;
             for (int f = 0; f < nf; ++f) maxit = std::max(maxit, h->h_cg[f].it);
-            h->launches += 7LL * (maxit + 1);
+            h->launches += (h->mixed ? 6LL : 7LL) * (maxit + 1);
             return FFTG_OK;
         }
         h->graphs_broken = true;
@@ -746,7 +800,7 @@ static int run_cg(fftg_handle* h, int nf, const void* tangent, long long tstride
         CK(cudaMemcpyAsync(h->h_cg, h->cg, nf * sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
     }
-    return launch_cg_finish(h, nf);
+    return h->mixed ? FFTG_OK : launch_cg_finish(h, nf);
 }
 
 static void set_cg_params(fftg_handle* h, int nf, double tol, const int* run) {
@@ -766,6 +820,7 @@ static void set_cg_params(fftg_handle* h, int nf, double tol, const int* run) {
 // eps* += d eps for the cells in the active mask, with ||d eps||^2 per cell
 // (Algorithm 1, iterative update).
 static int launch_newton_update(fftg_handle* h) {
+    if (h->mixed) return launch_solution(h, h->B, h->active, true);
     VecArgs u{};
     u.V = h->V;
     u.cs = h->cs;
@@ -777,11 +832,8 @@ static int launch_newton_update(fftg_handle* h) {
     u.fstride = 6 * h->cs;
     u.cell_fields = 6 * h->cs;
     const dim3 g(pointwise_blocks(h->V), h->B);
-    const int slot = prof_begin(h, h->mixed ? KK_NEWTON_UPDATE_F32 : KK_NEWTON_UPDATE_F64);
-    if (h->mixed)
-        k_newton_update<float><<<g, kThreads, 0, h->stream>>>(u);
-    else
-        k_newton_update<double><<<g, kThreads, 0, h->stream>>>(u);
+    const int slot = prof_begin(h, KK_NEWTON_UPDATE_F64);
+    k_newton_update<double><<<g, kThreads, 0, h->stream>>>(u);
     prof_end(h, slot);
     CK(cudaGetLastError());
     return FFTG_OK;
@@ -803,8 +855,6 @@ int newton_round(fftg_handle* h, const int* run, double tol_inner, RoundOut* out
     rc = launch_bounds(h, h->tangent, 7 * h->cs, B, 1, h->active);
     if (rc) return rc;
     rc = run_cg(h, B, h->tangent, 7 * h->cs);
-    if (rc) return rc;
-    rc = project_solution(h, B, h->active);
     if (rc) return rc;
     rc = launch_newton_update(h);
     if (rc) return rc;
@@ -1012,7 +1062,7 @@ static int batch_step(fftg_handle* h, const double* dE, double tol_newton, doubl
 //   WHILE (a cell of the handle iterates Newton):           [device test]
 //     k_inc_cg_reset, stress update, residual G sigma, [bounds],
 //     WHILE (a CG solve runs): one CG iteration              [device test]
-//     pending CG step, projection of the inner solution, eps* += d eps,
+//     eps* += d eps (the solution with its pending CG step),
 //     k_inc_decide (Newton test of Algorithm 1, sets the outer condition)
 //   commit: stress update with history, homogenised stress, trial ->
 //   committed state of the converged cells.
@@ -1130,20 +1180,15 @@ int capture_branch(fftg_handle* h, cudaGraph_t top, cudaStream_t s1, cudaStream_
                     cudaSuccess) {
                     rc = FFTG_ECUDA;
                 } else {
-                    rc = launch_cg_iteration(h, h->B, h->tangent, 7 * h->cs);
                     const unsigned int cap =
                         (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
-                    if (rc == FFTG_OK) {
-                        k_cg_continue<<<1, 32, 0, s3>>>(cC, h->cg, h->B, h->guard, cap);
-                        if (cudaGetLastError() != cudaSuccess) rc = FFTG_ECUDA;
-                    }
+                    rc = launch_cg_iteration(h, h->B, h->tangent, 7 * h->cs, CgLoop{cC, h->guard, cap});
                     cudaGraph_t g3 = nullptr;
                     if (cudaStreamEndCapture(s3, &g3) != cudaSuccess) rc = FFTG_ECUDA;
                 }
                 h->stream = s2;
             }
-            if (rc == FFTG_OK) rc = launch_cg_finish(h, h->B);
-            if (rc == FFTG_OK) rc = project_solution(h, h->B, h->active);
+            if (rc == FFTG_OK && !h->mixed) rc = launch_cg_finish(h, h->B);
             if (rc == FFTG_OK) rc = launch_newton_update(h);
             if (rc == FFTG_OK) {
                 k_inc_decide<<<1, kThreads, 0, s2>>>(cN, ia);
@@ -1314,12 +1359,14 @@ int fftg_group_step(fftg_group* g, const double* dE, const int* run, double tol_
             max_cg = std::max(max_cg, s.cg);
         }
         // kernels of the branch: begin, end, commit, the commit's stress
-        // update; per Newton pass 15 outside the CG loop; per CG loop pass
-        // the iteration's kernels and the loop test (an upper bound when
-        // the cells' CG counts differ between Newton passes)
-        const long long per_cg = 7;
-        h->launches += 4 + 15LL * max_newton + (per_cg + 1) * (max_cg + max_newton);
-        g->launches += 4 + 15LL * max_newton + (per_cg + 1) * (max_cg + max_newton);
+        // update; per Newton pass those outside the CG loop (mixed: reset,
+        // stress update, four of the right-hand side, four of the solution,
+        // decide); per CG loop pass the iteration's kernels (an upper bound
+        // when the cells' CG counts differ between Newton passes)
+        const long long per_newton = h->mixed ? 11 : 10, per_cg = h->mixed ? 6 : 7;
+        const long long n = 4 + per_newton * max_newton + per_cg * (max_cg + max_newton);
+        h->launches += n;
+        g->launches += n;
     }
     return first;
 }
@@ -1468,6 +1515,7 @@ int fftg_create_batch(fftg_handle** out, int N, int ncells, const uint8_t* phase
         cudaMemsetAsync(h->cg, 0, h->nf * sizeof(CGState), s) != cudaSuccess ||
         cudaMemsetAsync(h->nd, 0, ncells * sizeof(NewtonDev), s) != cudaSuccess ||
         cudaMemsetAsync(h->Edev, 0, (size_t)ncells * 6 * 8, s) != cudaSuccess ||
+        cudaMemsetAsync(h->guard, 0, 64, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         h->last_cuda = cudaGetLastError();
         return fail(FFTG_ECUDA);
@@ -1610,26 +1658,35 @@ int fftg_tangent(fftg_handle* h, double tol_cg, double C_out[36], int* cg_iters)
     a.tangent = tg;
     a.out = h->spec;
     CK(pass(h, f64 ? PK_P1_TANRHS_F64 : PK_P1_TANRHS_F32, a, 6));
-    int rc = run_p234(h, f64 ? FFT_F64 : FFT_F32, -invN3, nullptr, 6, nullptr);
-    if (rc) return rc;
-    PassArgs b = base_args(h, f64);
-    b.in = h->spec;
-    b.out = h->r;
-    b.cg = h->cg;
-    CK(pass(h, f64 ? PK_P5_RHS_F64_TO_F64 : PK_P5_RHS_F32_TO_F32, b, 6));
-    CK(cudaMemsetAsync(h->x, 0, 6 * 6 * h->cs * ts, h->stream));
+    int rc;
+    if (f64) {
+        rc = run_p234(h, FFT_F64, -invN3, nullptr, 6, nullptr);
+        if (rc) return rc;
+        PassArgs b = base_args(h, true);
+        b.in = h->spec;
+        b.out = h->r;
+        b.cg = h->cg;
+        CK(pass(h, PK_P5_RHS_F64_TO_F64, b, 6));
+        CK(cudaMemsetAsync(h->x, 0, 6 * 6 * h->cs * ts, h->stream));
+    } else {
+        CK(pass(h, PK_P2_F32, a, 6));
+        rc = launch_rhs(h, FFT_F32, -invN3, 6, nullptr);
+        if (rc) return rc;
+    }
     rc = launch_bounds(h, tg, 0, 1, 6, nullptr);
     if (rc) return rc;
     rc = run_cg(h, 6, tg, 0);
     if (rc) return rc;
-    rc = project_solution(h, 6, nullptr);
-    if (rc) return rc;
+    if (!f64) {
+        rc = launch_solution(h, 6, nullptr, false);
+        if (rc) return rc;
+    }
     int total = 0;
     for (int f = 0; f < 6; ++f) {
         if (h->h_cg[f].done == CG_BREAKDOWN) return FFTG_ENAN;
         total += h->h_cg[f].it;
     }
-    u.x = h->x;
+    u.x = f64 ? h->x : h->q;
     u.out = h->out36;
     slot = prof_begin(h, KK_TANGENT_AVERAGE);
     if (f64)

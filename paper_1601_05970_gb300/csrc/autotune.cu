@@ -64,7 +64,7 @@ int grid_index(int N) {
 }
 
 // pass kinds of each tuned kind (the default launch of variant 0)
-constexpr PassKind kDefaultKind[TK_COUNT] = {PK_P1_CGF_F32, PK_P2_F32, PK_P3_F32, PK_P4_F32, PK_P5_CGF_F32};
+constexpr PassKind kDefaultKind[TK_COUNT] = {PK_ROWS_CG_F32, PK_P2_F32, PK_P3_F32, PK_P4_F32, PK_P5_PLAIN_F32};
 const char* const kTkName[TK_COUNT] = {"p1", "p2", "p3", "p4", "p5"};
 
 std::mutex g_cache_mu;
@@ -149,7 +149,7 @@ int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
     int max_blocks = 0;
     for (int tk = 0; tk < TK_COUNT; ++tk)
         for (int v = 0; v < kVariants; ++v) max_blocks = std::max(max_blocks, variant_shape(N, tk, v).blocks);
-    const size_t off_r = 0, off_p = off_r + field, off_x = off_p + field, off_t = off_x + field;
+    const size_t off_x = 0, off_t = off_x + field;
     const size_t off_s = off_t + ((7 * cs * sizeof(float) + 255) & ~size_t(255));
     const size_t off_part = off_s + ((spec + 255) & ~size_t(255));
     const size_t off_cg = off_part + (((size_t)max_blocks * 2 * sizeof(double) + 255) & ~size_t(255));
@@ -195,15 +195,10 @@ int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
         PassArgs k = a;
         k.out = b + off_s;
         if (tk == TK_P1) {
-            k.aux = b + off_r;
-            k.aux2 = b + off_p;
-            k.aux3 = b + off_x;
             k.cg = cg;
         } else if (tk == TK_P5) {
             k.in = b + off_s;
-            k.aux = b + off_r;
-            k.aux3 = b + off_r;
-            k.cg = cg;
+            k.out = b + off_x;
         }
         double best = 1e300;
         int best_v = 0;
@@ -252,11 +247,11 @@ int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
 
 int tuned_kind(int pass_kind) {
     switch (pass_kind) {
-        case PK_P1_CGF_F32: return TK_P1;
+        case PK_ROWS_CG_F32: return TK_P1;
         case PK_P2_F32: return TK_P2;
         case PK_P3_F32: return TK_P3;
         case PK_P4_F32: return TK_P4;
-        case PK_P5_CGF_F32: return TK_P5;
+        case PK_P5_PLAIN_F32: return TK_P5;
         default: return -1;
     }
 }

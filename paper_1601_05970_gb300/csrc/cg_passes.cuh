@@ -1,0 +1,644 @@
+// The FP32 CG iteration of the mixed path on displacement coefficients.
+//
+// Every vector of the projected CG is compatible, so at each frequency f it
+// is f(x)w + w(x)f for one complex 3-vector w (the displacement coefficient,
+// up to a constant factor). r, p and x are held as w on the half spectrum,
+// [nf][3][N][N][H] complex: half the bytes of a six-component real field,
+// no incompatible part can build up in them, and only p is ever taken to
+// real space, where C : p is formed:
+//
+//   x1i   p = r + beta p, x += alpha p_old; f(x)p + p(x)f; inverse x1
+//   P4    inverse x2 (the column pass of passes.cuh)
+//   rows  inverse x3, tau = C : p with <p, tau>, forward x3, in one pass
+//   P2    forward x2 (its first block sets alpha = <r, r> / <p, tau>)
+//   x1f   forward x1, w of Ghat : tau, r -= alpha w, <r, r>
+//
+// Ghat (Appendix A) in this form: with t = tau f and q = |f|^2,
+//   w = (t - (f.t) / (2 q) f) / q,  Ghat : tau = f(x)w + w(x)f,
+// which is n(x)u + u(x)n for n = f/|f|, u = |f| w. The Frobenius product of
+// two fields is N^3 times the sum over frequencies of 2 (q a.b + (f.a)(f.b))
+// (Parseval; the half spectrum counts f3 > 0 twice).
+//
+// An iteration moves 84.3 (x1i) + 2 x 48.2 (P4, P2) + 76.2 (rows) + 48.2
+// (x1f) = 305 B per voxel at 243^3; with r, p and x as real fields it moved
+// 388.8 (243^3: 0.97 -> 0.90 ms an iteration). The residual of a Newton iteration and a column's right-hand side
+// stop at w (x1f), and the solution is taken to real space once (x1i, P4,
+// P5), which makes a projection of it needless.
+#pragma once
+
+#include "passes.cuh"
+
+namespace fftg {
+
+enum : int { X1F_CG = 0, X1F_RHS = 1 };
+enum : int { X1I_CG = 0, X1I_SOLUTION = 1 };
+
+// x1 split N = N1 * N2 of the two passes: one thread owns the N2 frequencies
+// k1 + N1 k2 of a column, so N2 <= 9 (registers) and, on small grids, two
+// stages rather than one so that a column has more threads.
+template <int N>
+struct X1Split {
+    static constexpr int N1 = N == 225 ? 25 : N == 27 ? 9 : N == 25 || N == 15 ? 5 : N == 9 ? 3 : Plan<N>::N1;
+};
+
+// Columns per block (64-byte runs of the spectrum) and threads: one per
+// (column, k1) of the middle phase.
+template <int N>
+struct X1 {
+    static constexpr int N1 = X1Split<N>::N1, N2 = N / N1, H = (N + 1) / 2, W = 8;
+    static constexpr int NT0 = ((W * N1 + 31) / 32) * 32, NT = NT0 < 64 ? 64 : NT0;
+    static constexpr int MINB = NT > 256 ? 1 : 512 / NT;  // at most 128 registers
+    static constexpr size_t smem = (size_t)(6 * N * W + N) * 8;
+    static constexpr int tiles = (H + W - 1) / W, blocks = tiles * N;
+    static_assert(N2 <= 9 && valid_split(N, N1), "x1 split");
+};
+
+// Coefficients are stored times a power of two near N^(5/2) / 2, which
+// brings those of a field of white noise to the size of the field's values:
+// without it the FP32 squares of a converged residual's coefficients, smaller
+// than its values by that factor, would underflow.
+template <int N>
+struct CoefScale {
+    static constexpr int exponent() {
+        double t = 0.25 * N * N * N * N * (double)N;
+        int e = 0;
+        for (; t >= 4.0; t *= 0.25) ++e;
+        return e;
+    }
+    static constexpr float value = (float)(1 << exponent());
+    static constexpr float inverse = 1.0f / value;
+    // sum over voxels of a squared field from sum (q |w|^2 + |f.w|^2)
+    static constexpr double square = 2.0 * N * N * (double)N / ((double)value * (double)value);
+};
+
+__device__ __forceinline__ int signed_freq(int k, int N) { return k <= (N - 1) / 2 ? k : k - N; }
+
+// ---------------------------------------------------------------- x1 inverse
+// aux = r (X1I_CG), aux2 = p, aux3 = x, out = spectrum; fields of 3 N N H
+// coefficients. X1I_CG updates p and x; X1I_SOLUTION takes x (+ the pending
+// alpha p) to the spectrum. x holds a value once a step was added to it: the
+// first step of a solve writes x = alpha p, so x needs no clearing.
+template <int N, int MODE>
+__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
+    using T = float;
+    using S = X1<N>;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, W = S::W, NT = S::NT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
+    cplx<T>* tw = buf + 6 * N * W;
+    const int f = blockIdx.z;
+    if (a.active && !a.active[f]) return;
+    const CGState* cg = a.cg + f;
+    if (MODE == X1I_CG && cg->done) return;
+    const int tid = threadIdx.x;
+    load_tw<T>(tw, a.tw, N);
+    __syncthreads();
+    const int col0 = blockIdx.x * W, k2g = blockIdx.y;
+    const long long NH = (long long)N * H, vf = 3LL * N * NH;
+    const cplx<T>* r = (const cplx<T>*)a.aux + f * vf;
+    cplx<T>* p = (cplx<T>*)a.aux2 + f * vf;
+    cplx<T>* x = (cplx<T>*)a.aux3 + f * vf;
+    const int it = cg->it;
+    const T alpha = (T)cg->alpha, beta = (T)cg->beta;
+    // X1I_CG: iteration it adds step it - 1. X1I_SOLUTION: x holds a value
+    // after step it - 1 was added, by the iteration that followed it.
+    const bool pend = cg->pend != 0;
+    const bool has_x = MODE == X1I_CG ? it > 1 : (pend ? it > 1 : it > 0);
+    const T f2 = (T)signed_freq(k2g, N);
+    for (int j = tid; j < W * N1; j += NT) {
+        const int w = j % W, k1 = j / W, col = col0 + w;
+        if (col >= H) continue;
+        const T f3 = (T)col;
+        const long long o0 = ((long long)k1 * N + k2g) * H + col;
+        cplx<T> d[N2][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            if (MODE == X1I_CG) {
+                cplx<T> po[N2], xo[N2];
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) d[k2][i] = r[o0 + (i * N + N1 * k2) * NH];
+                if (it > 0) {
+#pragma unroll
+                    for (int k2 = 0; k2 < N2; ++k2) po[k2] = p[o0 + (i * N + N1 * k2) * NH];
+                    if (has_x) {
+#pragma unroll
+                        for (int k2 = 0; k2 < N2; ++k2) xo[k2] = x[o0 + (i * N + N1 * k2) * NH];
+                    }
+#pragma unroll
+                    for (int k2 = 0; k2 < N2; ++k2) {
+                        const long long o = o0 + (i * N + N1 * k2) * NH;
+                        x[o] = has_x ? xo[k2] + alpha * po[k2] : alpha * po[k2];
+                        d[k2][i] = d[k2][i] + beta * po[k2];
+                    }
+                }
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) p[o0 + (i * N + N1 * k2) * NH] = d[k2][i];
+            } else {
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) {
+                    const long long o = o0 + (i * N + N1 * k2) * NH;
+                    cplx<T> v = has_x ? x[o] : mk(T(0), T(0));
+                    if (pend) v = v + alpha * p[o];
+                    d[k2][i] = v;
+                }
+            }
+        }
+        // f(x)d + d(x)f, component by component, and its inverse N2-point DFT
+        cplx<T>* base = buf + (N2 * k1) * W + w;
+        constexpr T is = CoefScale<N>::inverse;
+        const T g2 = is * f2, g3 = is * f3;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            cplx<T> v[N2];
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const T g1 = is * (T)signed_freq(k1 + N1 * k2, N);
+                if (c == 0) v[k2] = (g1 + g1) * d[k2][0];
+                else if (c == 1) v[k2] = (g2 + g2) * d[k2][1];
+                else if (c == 2) v[k2] = (g3 + g3) * d[k2][2];
+                else if (c == 3) v[k2] = g2 * d[k2][2] + g3 * d[k2][1];
+                else if (c == 4) v[k2] = g1 * d[k2][2] + g3 * d[k2][0];
+                else v[k2] = g1 * d[k2][1] + g2 * d[k2][0];
+            }
+            RegDFT<N, N2, +1, T>::run(v, tw);
+#pragma unroll
+            for (int q = 0; q < N2; ++q) {
+                cplx<T> z = v[q];
+                if (k1 > 0 && q > 0) z = twmul<+1>(z, tw[q * k1]);  // q*k1 < N
+                base[(c * N + q) * W] = z;
+            }
+        }
+    }
+    __syncthreads();
+    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)k2g * H;
+    constexpr int P = 6 * W;
+    for (int j = tid; j < P * N2; j += NT) {
+        const int pc = j % P, t = j / P;
+        const int c = pc / W, w = pc - c * W, col = col0 + w;
+        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + col, (int)NH, t, tw);
+    }
+}
+
+// ---------------------------------------------------------------- x1 forward
+// in = spectrum of tau, aux3 = r. X1F_CG: r -= alpha w and the block's part
+// of <r, r>; X1F_RHS: r = w with scale the sign and 1/N^3 of the right-hand
+// side, and the parts of <r, r> and of ||G tau||^2 before rounding.
+template <int N, int MODE>
+__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
+    using T = float;
+    using S = X1<N>;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, W = S::W, NT = S::NT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
+    cplx<T>* tw = buf + 6 * N * W;
+    const int f = blockIdx.z;
+    if (a.active && !a.active[f]) return;
+    const CGState* cg = a.cg + f;
+    if (MODE == X1F_CG && cg->done) return;
+    const int tid = threadIdx.x;
+    load_tw<T>(tw, a.tw, N);
+    __syncthreads();
+    const int col0 = blockIdx.x * W, k2g = blockIdx.y;
+    const long long NH = (long long)N * H;
+    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * H;
+    cplx<T>* r = (cplx<T>*)a.aux3 + f * (3LL * N * NH);
+    constexpr int P = 6 * W;
+    for (int j = tid; j < P * N2; j += NT) {
+        const int pc = j % P, t = j / P;
+        const int c = pc / W, w = pc - c * W, col = col0 + w;
+        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
+    }
+    __syncthreads();
+    const T f2 = (T)signed_freq(k2g, N);
+    const double unit = (double)CoefScale<N>::value * a.scale;
+    const T step = MODE == X1F_CG ? (T)(-cg->alpha * unit) : (T)unit;
+    T acc = T(0);
+    for (int j = tid; j < W * N1; j += NT) {
+        const int w = j % W, k1 = j / W, col = col0 + w;
+        if (col >= H) continue;
+        const T f3 = (T)col;
+        const cplx<T>* base = buf + (N2 * k1) * W + w;
+        // t = tau f over the components (11, 22, 33, 23, 13, 12)
+        cplx<T> t[N2][3];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            cplx<T> v[N2];
+#pragma unroll
+            for (int q = 0; q < N2; ++q) v[q] = base[(c * N + q) * W];
+            RegDFT<N, N2, -1, T>::run(v, tw);
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const T f1 = (T)signed_freq(k1 + N1 * k2, N);
+                if (c == 0) {
+                    t[k2][0] = f1 * v[k2];
+                } else if (c == 1) {
+                    t[k2][1] = f2 * v[k2];
+                } else if (c == 2) {
+                    t[k2][2] = f3 * v[k2];
+                } else if (c == 3) {
+                    t[k2][1] = t[k2][1] + f3 * v[k2];
+                    t[k2][2] = t[k2][2] + f2 * v[k2];
+                } else if (c == 4) {
+                    t[k2][0] = t[k2][0] + f3 * v[k2];
+                    t[k2][2] = t[k2][2] + f1 * v[k2];
+                } else {
+                    t[k2][0] = t[k2][0] + f2 * v[k2];
+                    t[k2][1] = t[k2][1] + f1 * v[k2];
+                }
+            }
+        }
+        const long long o0 = ((long long)k1 * N + k2g) * H + col;
+        cplx<T> fr[N2];  // f . r
+        T q2[N2];
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) {
+            const T f1 = (T)signed_freq(k1 + N1 * k2, N);
+            const T q = f1 * f1 + f2 * f2 + f3 * f3;
+            const T iq = q > T(0) ? T(1) / q : T(0);  // the mean maps to zero
+            const cplx<T> h = (T(-0.5) * iq) * (f1 * t[k2][0] + f2 * t[k2][1] + f3 * t[k2][2]);
+            const T m = step * iq;
+            t[k2][0] = m * (t[k2][0] + f1 * h);
+            t[k2][1] = m * (t[k2][1] + f2 * h);
+            t[k2][2] = m * (t[k2][2] + f3 * h);
+            q2[k2] = q;
+            fr[k2] = mk(T(0), T(0));
+        }
+        T part = T(0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            cplx<T> ro[N2];
+            if (MODE == X1F_CG) {
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) ro[k2] = r[o0 + (i * N + N1 * k2) * NH];
+            }
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const T fi = i == 0 ? (T)signed_freq(k1 + N1 * k2, N) : i == 1 ? f2 : f3;
+                const cplx<T> z = MODE == X1F_CG ? ro[k2] + t[k2][i] : t[k2][i];
+                r[o0 + (i * N + N1 * k2) * NH] = z;
+                fr[k2] = fr[k2] + fi * z;
+                part += q2[k2] * (z.x * z.x + z.y * z.y);
+            }
+        }
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) part += fr[k2].x * fr[k2].x + fr[k2].y * fr[k2].y;
+        acc += col == 0 ? part : T(2) * part;  // f3 > 0 stands for -f3 too
+    }
+    const double s = block_sum_any((double)acc) * CoefScale<N>::square;
+    if (tid == 0) {
+        const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
+        if (MODE == X1F_CG) {
+            a.partials[f * nb + b] = s;
+        } else {
+            a.partials[2 * (f * nb + b)] = s;
+            a.partials[2 * (f * nb + b) + 1] = s;
+        }
+    }
+}
+
+// 1/q of a positive integer q < 2^24 as a double-float: the remainder
+// 1 - q y of the FP32 quotient y is exact in one fma, so y + y (1 - q y)
+// leaves a relative error of (1 - q y)^2, about 2^-48.
+__device__ __forceinline__ dd dd_recip(float q) {
+    const float y = 1.0f / q;
+    return dd(y, y * dd_fma(-q, y, 1.0f));
+}
+
+// a * f for an FP32 number f
+__device__ __forceinline__ dd dd_scale(dd a, float f) {
+    const dd p = dd_two_prod(a.hi, f);
+    return dd_fast_two_sum(p.hi, dd_fma(a.lo, f, p.lo));
+}
+__device__ __forceinline__ cplx<dd> dd_scale(cplx<dd> a, float f) {
+    return mk(dd_scale(a.x, f), dd_scale(a.y, f));
+}
+
+// The right-hand side of a Newton iteration, r = w of -G sigma, from the
+// double-float spectrum of the FP64 stress: forward x1 in two stages, then
+// one thread per frequency. The double-float inverse passes that a residual
+// in real space needs (half of its work) are not run.
+template <int N>
+__global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
+    using T = dd;
+    using C = Cfg<N, T>;
+    constexpr int H = C::H, W = C::W3, NT = C::T3;
+    constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
+    cplx<T>* buf = tw + N;  // [6][N][W]
+    const int f = blockIdx.z;
+    if (a.active && !a.active[f]) return;
+    const int tid = threadIdx.x;
+    load_tw<T>(tw, a.tw, N);
+    __syncthreads();
+    const int col0 = blockIdx.x * W, k2g = blockIdx.y;
+    const long long NH = (long long)N * H;
+    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * H;
+    cplx<float>* r = (cplx<float>*)a.aux3 + f * (3LL * N * NH);
+    constexpr int P = 6 * W;
+    for (int it = tid; it < P * N2; it += NT) {
+        const int pc = it % P, t = it / P;
+        const int c = pc / W, w = pc - c * W, col = col0 + w;
+        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
+    }
+    __syncthreads();
+    if (N2 > 1) {
+        for (int it = tid; it < P * N1; it += NT) {
+            const int pc = it % P, k1 = it / P;
+            const int c = pc / W, w = pc - c * W;
+            if (col0 + w < H) fwdB<N, N1, false, T>(buf + c * N * W + w, W, buf + c * N * W + w, W, k1, tw);
+        }
+        __syncthreads();
+    }
+    const float f2 = (float)signed_freq(k2g, N);
+    const dd scale((double)CoefScale<N>::value * a.scale);
+    float acc0 = 0.0f;
+    dd acc1(0.0f, 0.0f);
+    for (int it = tid; it < W * N; it += NT) {
+        const int w = it % W, pos = it / W, col = col0 + w;
+        const int k1 = pos / N2, k2 = pos - k1 * N2;
+        const int kk = k1 + N1 * k2;  // frequency held at position N2*k1 + k2
+        if (col >= H) continue;
+        const float f1 = (float)signed_freq(kk, N), f3 = (float)col;
+        const cplx<T>* b = buf + pos * W + w;
+        cplx<T> c[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) c[k] = b[k * N * W];
+        cplx<T> t[3];
+        t[0] = dd_scale(c[0], f1) + dd_scale(c[5], f2) + dd_scale(c[4], f3);
+        t[1] = dd_scale(c[5], f1) + dd_scale(c[1], f2) + dd_scale(c[3], f3);
+        t[2] = dd_scale(c[4], f1) + dd_scale(c[3], f2) + dd_scale(c[2], f3);
+        const float q = f1 * f1 + f2 * f2 + f3 * f3;  // an integer below 2^24: exact
+        const dd iq = q > 0.0f ? dd_recip(q) : dd(0.0f, 0.0f);
+        const cplx<T> h = signed_by<-1>(
+            half_of(iq * (dd_scale(t[0], f1) + dd_scale(t[1], f2) + dd_scale(t[2], f3))));
+        const dd m = scale * iq;
+        t[0] = m * (t[0] + dd_scale(h, f1));
+        t[1] = m * (t[1] + dd_scale(h, f2));
+        t[2] = m * (t[2] + dd_scale(h, f3));
+        const float wt = col == 0 ? 1.0f : 2.0f;  // f3 > 0 stands for -f3 too
+        const long long o = ((long long)kk * N + k2g) * H + col;
+        float s0 = 0.0f;
+        cplx<float> fr = mk(0.0f, 0.0f);
+        dd s1(0.0f, 0.0f);
+        cplx<T> ft = mk(dd(0.0f, 0.0f), dd(0.0f, 0.0f));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float fi = i == 0 ? f1 : i == 1 ? f2 : f3;
+            const cplx<float> z = mk((float)t[i].x, (float)t[i].y);
+            r[o + i * N * NH] = z;
+            s0 += z.x * z.x + z.y * z.y;
+            fr = fr + fi * z;
+            s1 += t[i].x * t[i].x + t[i].y * t[i].y;
+            ft = ft + dd_scale(t[i], fi);
+        }
+        acc0 += wt * (q * s0 + fr.x * fr.x + fr.y * fr.y);
+        acc1 += dd_scale(dd_scale(s1, q) + ft.x * ft.x + ft.y * ft.y, wt);
+    }
+    const double s0 = block_sum_any((double)acc0) * CoefScale<N>::square;
+    const double s1 = block_sum_any((double)acc1) * CoefScale<N>::square;
+    if (tid == 0) {
+        const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
+        a.partials[2 * (f * nb + b)] = s0;
+        a.partials[2 * (f * nb + b) + 1] = s1;
+    }
+}
+
+// ---------------------------------------------------------------------- rows
+// rounds of spectrum loads issued together
+#ifndef FFTG_ROWS_LDB
+#define FFTG_ROWS_LDB 2
+#endif
+
+// Radix split of the rows: the plan's, or two stages on the small grids,
+// where a row of one stage has too few threads.
+template <int N>
+struct RowSplit {
+    static constexpr int N1 = Plan<N>::N2 > 1 ? Plan<N>::N1 : X1Split<N>::N1;
+    static constexpr int ALT = Plan<N>::N2 > 1 ? Plan<N>::N2 : Plan<N>::N1;
+};
+
+// Inverse x3, tau = C : p, forward x3 on R rows, in place on the spectrum.
+// Rows per block: the row passes' rule, but enough blocks to fill the chip
+// on small grids; threads: one stage-A item each.
+template <int N, int NA, int TV>
+struct RowCfg {
+    using C = Cfg<N, float, NA, TV>;
+    static constexpr int fl2(int x) {
+        return x >= 64 ? 64 : x >= 32 ? 32 : x >= 16 ? 16 : x >= 8 ? 8 : 4;
+    }
+    static constexpr int R = C::R < fl2(N * N / 152) ? C::R : fl2(N * N / 152);
+    static constexpr int N1 = NA, N2 = N / NA;
+    static constexpr int NT0 = ((3 * R * N2 + 31) / 32) * 32;
+    static constexpr int NT = NT0 < 64 ? 64 : NT0 > 256 ? 256 : NT0;
+    static constexpr int MINB = 1024 / NT;  // 64 registers
+    static constexpr size_t smem = (size_t)(3 * R * N + N) * 8;
+    static constexpr int blocks = (N * N + R - 1) / R;
+};
+
+template <int N, int NA, int TV>
+__global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB) k_rows_cg(PassArgs a) {
+    using T = float;
+    using S = RowCfg<N, NA, TV>;
+    constexpr int R = S::R, H = (N + 1) / 2, NT = S::NT;
+    constexpr int N1 = S::N1, N2 = S::N2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* z = reinterpret_cast<cplx<T>*>(smem_raw);  // [3][R][N]
+    cplx<T>* tw = z + 3 * R * N;
+    const int f = blockIdx.z;
+    if (a.cg[f].done) return;
+    const int tid = threadIdx.x;
+    load_tw<T>(tw, a.tw, N);
+    const int row0 = blockIdx.x * R;
+    const int nrows = min(R, N * N - row0);
+    const long long HS = (long long)N * N * H;
+    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)row0 * H;
+    // the half spectra of two real components -> one complex row; the
+    // imaginary parts at k = 0 are rounding and are dropped
+    constexpr int NRL = (R * H + NT - 1) / NT;
+    constexpr int LB = FFTG_ROWS_LDB < NRL ? FFTG_ROWS_LDB : NRL;
+#pragma unroll
+    for (int r0 = 0; r0 < NRL; r0 += LB) {
+        cplx<T> A[LB][3], B[LB][3];
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+            const int it = tid + (r0 + u) * NT;
+            if (r0 + u < NRL && it < nrows * H) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    A[u][c] = sp[(2 * c) * HS + it];
+                    B[u][c] = sp[(2 * c + 1) * HS + it];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+            const int it = tid + (r0 + u) * NT;
+            if (r0 + u < NRL && it < nrows * H) {
+                const int row = it / H, k = it - row * H;
+                const int pk = perm_pos<N, N1>(k);
+                const int pn = perm_pos<N, N1>(k == 0 ? 0 : N - k);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const cplx<T> a0 = A[u][c], b0 = B[u][c];
+                    cplx<T>* zr = z + (c * R + row) * N;
+                    if (k == 0) {
+                        zr[pk] = mk(a0.x, b0.x);
+                    } else {
+                        zr[pk] = mk(a0.x - b0.y, a0.y + b0.x);  // A + iB
+                        zr[pn] = mk(a0.x + b0.y, b0.x - a0.y);  // conj(A) + i conj(B)
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    constexpr int NP = 3 * R;
+    if (N2 > 1) {
+        for (int it = tid; it < NP * N1; it += NT) {
+            const int pc = it % NP, k1 = it / NP;
+            if (pc % R < nrows) invB<N, N1, false, T>(z + pc * N, 1, z + pc * N, 1, k1, tw);
+        }
+        __syncthreads();
+    }
+    for (int it = tid; it < NP * N2; it += NT) {
+        const int pc = it % NP, t = it / NP;
+        if (pc % R < nrows) invA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
+    }
+    __syncthreads();
+    // tau = C : p, four voxels a lane (R is a multiple of 4, so a block
+    // starts on a vector boundary; in the last block the vector that
+    // straddles the end of the grid reads the padding of the tangent and
+    // changes rows that no stage reads)
+    const long long cs = a.cs;
+    const T* tg = (const T*)a.tangent + f * a.tstride + (long long)row0 * N;
+    const int nel = nrows * N;
+    T pcp = T(0);
+    constexpr int VW = 4;
+    for (int j = tid; j < (R * N) / VW; j += NT) {
+        const int i0 = j * VW;
+        if (i0 >= nel) continue;
+        T t7[7][VW];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) ldv<VW, T>(tg + k * cs + i0, t7[k]);
+        cplx<T> s[3][VW];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float4* zv = reinterpret_cast<const float4*>(z + c * R * N + i0);
+#pragma unroll
+            for (int e = 0; e < VW; e += 2) {
+                const float4 v = zv[e / 2];
+                s[c][e] = mk(v.x, v.y);
+                s[c][e + 1] = mk(v.z, v.w);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+            const T pe[6] = {s[0][e].x, s[0][e].y, s[1][e].x, s[1][e].y, s[2][e].x, s[2][e].y};
+            T se[6];
+            apply_tangent7<T>(t7[0][e], t7[1][e], t7[2][e], t7[3][e], t7[4][e], t7[5][e], t7[6][e], pe, se);
+            if (i0 + e < nel) pcp += frob<T>(pe, se);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) s[c][e] = mk(se[2 * c], se[2 * c + 1]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float4* zv = reinterpret_cast<float4*>(z + c * R * N + i0);
+#pragma unroll
+            for (int e = 0; e < VW; e += 2) zv[e / 2] = make_float4(s[c][e].x, s[c][e].y, s[c][e + 1].x, s[c][e + 1].y);
+        }
+    }
+    __shared__ double pcp_warp[NT / 32];
+    {
+        const double wv = warp_sum((double)pcp);
+        if ((tid & 31) == 0) pcp_warp[tid >> 5] = wv;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) t += pcp_warp[w];
+        a.partials[(size_t)f * gridDim.x + blockIdx.x] = t;
+    }
+    for (int it = tid; it < NP * N2; it += NT) {
+        const int pc = it % NP, t = it / NP;
+        if (pc % R < nrows) fwdA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
+    }
+    __syncthreads();
+    if (N2 > 1) {
+        for (int it = tid; it < NP * N1; it += NT) {
+            const int pc = it % NP, k1 = it / NP;
+            if (pc % R < nrows) fwdB<N, N1, false, T>(z + pc * N, 1, z + pc * N, 1, k1, tw);
+        }
+        __syncthreads();
+    }
+    for (int it = tid; it < nrows * H; it += NT) {
+        const int row = it / H, k = it - row * H;
+        const int pk = perm_pos<N, N1>(k), pn = perm_pos<N, N1>(k == 0 ? 0 : N - k);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cplx<T> zk = z[(c * R + row) * N + pk];
+            const cplx<T> zn = conj(z[(c * R + row) * N + pn]);
+            const cplx<T> d = zk - zn;  // (zk - zn) / (2i) = (d.y, -d.x) / 2
+            sp[(2 * c) * HS + it] = half_of(zk + zn);
+            sp[(2 * c + 1) * HS + it] = half_of(mk(d.y, -d.x));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ launcher
+template <int N>
+cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s) {
+    using C32 = Cfg<N, float>;
+    using C64 = Cfg<N, double>;
+    using CDD = Cfg<N, dd>;
+    static_assert(CDD::row_blocks == C64::row_blocks && CDD::W2 == C64::W2 && CDD::S2 == C64::S2,
+                  "double-float row and column passes share the FP64 geometry");
+    const dim3 r32(C32::row_blocks, 1, nf), r64(C64::row_blocks, 1, nf);
+    const dim3 c32((C32::H + C32::W2 - 1) / C32::W2, (6 * N + C32::S2 - 1) / C32::S2, nf);
+    const dim3 c64((C64::H + C64::W2 - 1) / C64::W2, (6 * N + C64::S2 - 1) / C64::S2, nf);
+    const dim3 g32((C32::H + C32::W3 - 1) / C32::W3, N, nf);
+    const dim3 g64((C64::H + C64::W3 - 1) / C64::W3, N, nf);
+    const dim3 x32(X1<N>::tiles, N, nf);
+    const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
+    switch (kind) {
+        case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s);
+        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN>, r32, C32::smem_rows, a, s);
+        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN>, r64, C64::smem_rows, a, s);
+        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN>, r32, C32::smem_rows, a, s);
+        case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s);
+        case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s);
+        case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s);
+        case PK_P2_F64: return launch_k(k_p24<N, double, true>, c64, C64::smem_p24, a, s, C64::T2);
+        case PK_P2_F32: return launch_k(k_p24<N, float, true>, c32, C32::smem_p24, a, s, C32::T2);
+        case PK_P4_F64: return launch_k(k_p24<N, double, false>, c64, C64::smem_p24, a, s, C64::T2);
+        case PK_P4_F32: return launch_k(k_p24<N, float, false>, c32, C32::smem_p24, a, s, C32::T2);
+        case PK_P3_F64: return launch_k(k_p3<N, double>, g64, C64::smem_p3, a, s, C64::T3);
+        case PK_P3_F32: return launch_k(k_p3<N, float>, g32, C32::smem_p3, a, s, C32::T3);
+        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double>, r64, C64::smem_rows, a, s);
+        case PK_P5_PLAIN_F32: return launch_k(k_p5<N, float, P5_PLAIN, float>, r32, C32::smem_rows, a, s);
+        case PK_P5_DOT_F64: return launch_k(k_p5<N, double, P5_DOT, double>, r64, C64::smem_rows, a, s);
+        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float>, r32, C32::smem_rows, a, s);
+        case PK_P5_RHS_F64_TO_F64:
+            return launch_k(k_p5<N, double, P5_RHS, double>, r64, C64::smem_rows, a, s);
+        case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s);
+        case PK_P2_DD: return launch_k(k_p24<N, dd, true>, c64, CDD::smem_p24, a, s, CDD::T2);
+        case PK_P4_DD: return launch_k(k_p24<N, dd, false>, c64, CDD::smem_p24, a, s, CDD::T2);
+        case PK_P3_DD: return launch_k(k_p3<N, dd>, gdd, CDD::smem_p3, a, s, CDD::T3);
+        case PK_P5_PLAIN_DD_TO_F64:
+            return launch_k(k_p5<N, dd, P5_PLAIN, double>, r64, CDD::smem_rows, a, s);
+        case PK_P5_NEWTON_F32: return launch_k(k_p5<N, float, P5_NEWTON, float>, r32, C32::smem_rows, a, s);
+        case PK_X1I_CG_F32: return launch_k(k_x1i<N, X1I_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
+        case PK_X1I_SOLUTION_F32: return launch_k(k_x1i<N, X1I_SOLUTION>, x32, X1<N>::smem, a, s, X1<N>::NT);
+        case PK_X1F_CG_F32: return launch_k(k_x1f<N, X1F_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
+        case PK_X1F_RHS_F32: return launch_k(k_x1f<N, X1F_RHS>, x32, X1<N>::smem, a, s, X1<N>::NT);
+        case PK_X1F_RHS_DD: return launch_k(k_x1f_dd<N>, gdd, CDD::smem_p3, a, s, CDD::T3);
+        case PK_ROWS_CG_F32: {
+            using R = RowCfg<N, RowSplit<N>::N1, 0>;
+            return launch_k(k_rows_cg<N, RowSplit<N>::N1, 0>, dim3(R::blocks, 1, nf), R::smem, a, s, R::NT);
+        }
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace fftg

@@ -176,17 +176,38 @@ __device__ __forceinline__ double block_sum_any(double v) {
     return s;
 }
 
-// <r, r> of the fused CG iteration from the block partials P5 wrote
+// Sum of the partials in[0 .. nb) at stride `st` in a fixed order over the
+// block; valid in thread 0.
+__device__ __forceinline__ double sum_partials(const double* in, int nb, int st) {
+    double acc = 0.0;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += in[(size_t)b * st];
+    return block_sum_any(acc);
+}
+
+// Start of the solves of a right-hand side from its pass's block partials
+// ([nf][nb][2]: <r, r> and the squared norm before rounding), one block per
+// field.
+static __global__ void __launch_bounds__(1024) k_cg_begin(const double* partials, int nb, CGState* cg,
+                                                          const int* active) {
+    const int f = blockIdx.x;
+    if (active && !active[f]) return;
+    const double* in = partials + (size_t)f * nb * 2;
+    const double rr = sum_partials(in, nb, 2);
+    const double gs2 = sum_partials(in + 1, nb, 2);
+    if (threadIdx.x == 0) cg_start(cg + f, rr, gs2);
+}
+
+// <r, r> of a CG iteration from the block partials of its last pass
 // ([nf][nb], one per block): one block per field sums them in a fixed order
 // and takes the CG state's update step (beta and the stopping tests).
-static __global__ void __launch_bounds__(1024) k_cg_rr(const double* partials, int nb, CGState* cg) {
+__device__ __forceinline__ void cg_rr_block(const double* partials, int nb, CGState* cg) {
     const int f = blockIdx.x;
     if (cg[f].done) return;
-    const double* in = partials + (size_t)f * nb;
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += in[b];
-    acc = block_sum_any(acc);
+    const double acc = sum_partials(partials + (size_t)f * nb, nb, 1);
     if (threadIdx.x == 0) cg_after_update(cg + f, acc);
+}
+static __global__ void __launch_bounds__(1024) k_cg_rr(const double* partials, int nb, CGState* cg) {
+    cg_rr_block(partials, nb, cg);
 }
 
 // Store this block's NV partial sums and report whether this block is the

@@ -22,24 +22,15 @@
 
 namespace fftg {
 
-enum : int { P1_PLAIN = 0, P1_TAN = 1, P1_CG = 2, P1_TANRHS = 3, P1_CGF = 4 };
-enum : int { P5_PLAIN = 0, P5_DOT = 1, P5_RHS = 2, P5_CGF = 3 };
+enum : int { P1_PLAIN = 0, P1_TAN = 1, P1_CG = 2, P1_TANRHS = 3 };
+enum : int { P5_PLAIN = 0, P5_DOT = 1, P5_RHS = 2, P5_NEWTON = 3 };
 
-// The two CG iterations of the passes.
-//
-// P1_CG / P5_DOT (+ the update kernel): Hestenes-Stiefel CG on G C as
-// written, alpha = <r, r> / <p, G C p> from the product of P5, then
-// r -= alpha q and <r, r> in a separate pass over r and q.
-//
-// P1_CGF / P5_CGF (mixed path): on compatible fields G is the orthogonal
-// projector onto them, so <p, G C p> = <G p, C p> = <p, C p>; P1 forms
-// C : p anyway and reduces <p, C : p> there, so alpha is known before P5,
-// which then updates r -= alpha q with q still in registers and reduces
-// <r, r>: q is never stored and the update pass disappears (72 B per voxel
-// and field less per iteration in FP32). The iterates are those of CG up to
-// the rounding of the incompatible part that the FP32 recursion leaves in p
-// (about 1e-5 of |p| after some tens of iterations, removed by the
-// projection of each inner solution).
+// The CG iteration of these passes (FP64 path): P1_CG / P5_DOT and the update
+// kernel, Hestenes-Stiefel CG on G C as written, alpha = <r, r> / <p, G C p>
+// from the product of P5, then r -= alpha q and <r, r> in a separate pass.
+// The mixed path's iteration is that of cg_passes.cuh.
+// P5_NEWTON: eps* += x for the solution x of a mixed inner solve, with its
+// squared norm.
 
 struct PassArgs {
     const void* in;        // P1: real field; P2-P4: unused; P5: spectrum
@@ -47,7 +38,7 @@ struct PassArgs {
     const void* aux;       // P1_CG: r; P5_DOT: p
     void* aux2;            // P1_CG: p (updated in place)
     void* aux3;            // P1_CG: x (gets the previous iteration's alpha p);
-                           // P5_CGF: r (updated in place; aux is the same r)
+                           // P5_NEWTON: eps* (FP64, updated in place)
     const void* tangent;   // [7][V]: K', 2G_eff, w11, w22, w23, w13, w12 (see apply_tangent7)
     CGState* cg;           // per field, or null
     double* partials;      // [nf][nblocks][2]
@@ -59,9 +50,9 @@ struct PassArgs {
     long long sstride;     // spectrum stride between fields (complex elements)
     long long tstride;     // tangent stride between fields (0: shared)
     const int* active;     // per field: 0 = skip this field (null: all run)
-    // P2 of the fused CG iteration: the block partials of <p, C : p> that P1
-    // wrote ([nf][red_n]); block (0, 0) of each field reduces them in a
-    // fixed order and sets alpha (null: nothing to reduce)
+    // P2 of the mixed CG iteration: the block partials of <p, C : p> that the
+    // row pass wrote ([nf][red_n]); block (0, 0) of each field reduces them in
+    // a fixed order and sets alpha (null: nothing to reduce)
     const double* red_in;
     int red_n;
 };
@@ -294,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     cplx<T>* z = tw + N;  // [3][R][N]
     const int f = blockIdx.z;
     if (a.active && !a.active[f]) return;
-    constexpr bool CGM = MODE == P1_CG || MODE == P1_CGF;
+    constexpr bool CGM = MODE == P1_CG;
     if (CGM && a.cg[f].done) return;
     const int tid = threadIdx.x;
     load_tw<T>(tw, a.tw, N);
@@ -307,7 +298,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     const TIn* in = (const TIn*)a.in + f * a.fstride;
     const T* tg = (const T*)a.tangent + f * a.tstride;
     T beta = T(0), alpha = T(0);
-    T pcp = T(0);       // P1_CGF: this thread's part of <p, C : p>
     bool first = true;  // first CG iteration: p = r (p holds no data yet)
     if (CGM) {
         beta = (T)a.cg[f].beta;
@@ -381,7 +371,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
                                       t7[6][e], pe, se);
 #pragma unroll
                     for (int c = 0; c < 6; ++c) s[c][e] = se[c];
-                    if (MODE == P1_CGF && i0 + e < nel) pcp += frob<T>(pe, se);
                 }
             }
         } else {
@@ -397,21 +386,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
             z[2 * R * N + i0 + e] = mk(s[4][e], s[5][e]);
         }
     }
-    // P1_CGF: this block's part of <p, C : p>, lanes by shuffles, warps in
-    // index order after the barrier below; P2 reduces the blocks' parts (no
-    // fence or ticket at the end of every block here)
-    __shared__ double pcp_warp[kThreads / 32];
-    if (MODE == P1_CGF) {
-        const double wv = warp_sum((double)pcp);
-        if ((tid & 31) == 0) pcp_warp[tid >> 5] = wv;
-    }
     __syncthreads();
-    if (MODE == P1_CGF && tid == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) t += pcp_warp[w];
-        a.partials[(size_t)f * gridDim.x + blockIdx.x] = t;
-    }
     constexpr int NP = 3 * R;
     for (int it = tid; it < NP * N2; it += kThreads) {
         const int pc = it % NP, t = it / NP;
@@ -461,8 +436,8 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T2) k_p24(PassArgs a) {
     if (a.cg && a.cg[f].done) return;
     const int tid = threadIdx.x;
     if (a.red_in && blockIdx.x == 0 && blockIdx.y == 0) {
-        // alpha = <r, r> / <p, C : p> of the fused CG iteration, from the
-        // block partials of P1 (thread t takes blocks t, t + NT, ...; then
+        // alpha = <r, r> / <p, C : p> of the mixed CG iteration, from the
+        // block partials of the row pass (thread t takes blocks t, t + NT, ...; then
         // a fixed tree), before this block's share of the transform
         const double* in = a.red_in + (size_t)f * a.red_n;
         double acc = 0.0;
@@ -755,7 +730,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     const int f = blockIdx.z;
     CGState* cg = a.cg ? a.cg + f : nullptr;
     if (a.active && !a.active[f]) return;
-    if ((MODE == P5_DOT || MODE == P5_CGF) && cg->done) return;
+    if (MODE == P5_DOT && cg->done) return;
     const int tid = threadIdx.x;
     load_tw<T>(tw, a.tw, N);
     const int row0 = blockIdx.x * R;
@@ -794,8 +769,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const cplx<T> a0 = A[u][c], b0 = B[u][c];
-                    z[(c * R + row) * N + pk] = mk(a0.x - b0.y, a0.y + b0.x);  // A + iB
-                    if (k > 0) z[(c * R + row) * N + pn] = mk(a0.x + b0.y, b0.x - a0.y);  // conj(A) + i conj(B)
+                    // A + iB and conj(A) + i conj(B); A and B are real at k = 0
+                    // (what their imaginary parts hold is rounding)
+                    z[(c * R + row) * N + pk] = k > 0 ? mk(a0.x - b0.y, a0.y + b0.x) : mk(a0.x, b0.x);
+                    if (k > 0) z[(c * R + row) * N + pn] = mk(a0.x + b0.y, b0.x - a0.y);
                 }
             }
         }
@@ -827,14 +804,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     constexpr int NV = (R * N) / VO;
     constexpr int NRE = (NV + kThreads - 1) / kThreads;
     constexpr int PB = FFTG_P5_PB < NRE ? FFTG_P5_PB : NRE;
-    // P5_DOT: p; P5_CGF: r (updated in place, r -= alpha q)
-    const TO* pin = (const TO*)a.aux + f * a.fstride;
-    TO* rout = MODE == P5_CGF ? (TO*)a.aux3 + f * a.fstride : nullptr;
-    const TO alpha = MODE == P5_CGF ? (TO)cg->alpha : TO(0);
+    const TO* pin = (const TO*)a.aux + f * a.fstride;  // P5_DOT: p
+    double* eps = MODE == P5_NEWTON ? (double*)a.aux3 + f * a.fstride : nullptr;
+    dd accx(0.0f, 0.0f);  // P5_NEWTON: squares of x, exact products summed in double-float
 #pragma unroll
     for (int r0 = 0; r0 < NRE; r0 += PB) {
         TO pv[PB][6][VO];
-        if (MODE == P5_DOT || MODE == P5_CGF) {
+        if (MODE == P5_DOT) {
 #pragma unroll
             for (int u = 0; u < PB; ++u) {
                 const int j = tid + (r0 + u) * kThreads;
@@ -864,20 +840,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
 #pragma unroll
                 for (int c = 0; c < 6; ++c) q[c][e] = (TO)qd[c][e];
             }
-            if (MODE == P5_CGF) {
-                // r -= alpha q, <r, r> (lanes past the grid update padding only)
+            if constexpr (MODE == P5_NEWTON) {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
+                    double ev[VO];
+                    ldv<VO, double>(eps + c * cs + v0, ev);
 #pragma unroll
-                    for (int e = 0; e < VO; ++e) pv[u][c][e] -= alpha * q[c][e];
-                    stv<VO, TO>(rout + c * cs + v0, pv[u][c]);
-                }
-#pragma unroll
-                for (int e = 0; e < VO; ++e) {
-                    if (i0 + e < nel) {
-                        const TO re[6] = {pv[u][0][e], pv[u][1][e], pv[u][2][e], pv[u][3][e], pv[u][4][e], pv[u][5][e]};
-                        acc0 += (T)frob<TO>(re, re);
+                    for (int e = 0; e < VO; ++e) {
+                        ev[e] += (double)q[c][e];
+                        if (i0 + e < nel) {
+                            const dd sq = dd_two_prod(q[c][e], q[c][e]);
+                            accx += c < 3 ? sq : dd(2.0f * sq.hi, 2.0f * sq.lo);
+                        }
                     }
+                    stv<VO, double>(eps + c * cs + v0, ev);
                 }
                 continue;
             }
@@ -908,13 +884,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     if (MODE == P5_PLAIN) return;
     const int nb = gridDim.x;
     double part[2];
-    part[0] = block_sum((double)acc0);
-    if (MODE == P5_CGF) {
-        // the block's part of <r, r>; k_cg_rr reduces the parts (no fence
-        // or ticket at the end of every block here)
+    if (MODE == P5_NEWTON) {
+        // the block's part of ||x||^2 (k_newton_norm sums the parts)
+        part[0] = block_sum((double)accx);
         if (tid == 0) a.partials[(size_t)f * nb + blockIdx.x] = part[0];
         return;
     }
+    part[0] = block_sum((double)acc0);
     part[1] = (MODE == P5_RHS) ? block_sum(acc1) : 0.0;
     double* partials = a.partials + (size_t)f * nb * 2;
     if (!publish_partials<2>(part, partials, blockIdx.x, nb, &cg->ticket)) return;
@@ -929,16 +905,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
 
 // ------------------------------------------------------------------ launcher
 enum PassKind : int {
-    PK_P1_PLAIN_F64, PK_P1_PLAIN_F32, PK_P1_TAN_F64, PK_P1_TAN_F32, PK_P1_CG_F64, PK_P1_CG_F32,
+    PK_P1_PLAIN_F64, PK_P1_PLAIN_F32, PK_P1_TAN_F64, PK_P1_TAN_F32, PK_P1_CG_F64,
     PK_P1_TANRHS_F64, PK_P1_TANRHS_F32,
     PK_P2_F64, PK_P2_F32, PK_P4_F64, PK_P4_F32, PK_P3_F64, PK_P3_F32,
     PK_P5_PLAIN_F64, PK_P5_PLAIN_F32, PK_P5_DOT_F64, PK_P5_DOT_F32,
-    PK_P5_RHS_F64_TO_F64, PK_P5_RHS_F64_TO_F32, PK_P5_RHS_F32_TO_F32,
-    // double-float FFTs (the mixed path's residual): FP64 field in, FP32
-    // residual or FP64 field out
-    PK_P1_PLAIN_DD, PK_P2_DD, PK_P3_DD, PK_P4_DD, PK_P5_RHS_DD_TO_F32, PK_P5_PLAIN_DD_TO_F64,
-    // the CG iteration without the update pass (P1_CGF / P5_CGF), FP32
-    PK_P1_CGF_F32, PK_P5_CGF_F32,
+    PK_P5_RHS_F64_TO_F64,
+    // double-float FFTs: FP64 field in and out
+    PK_P1_PLAIN_DD, PK_P2_DD, PK_P3_DD, PK_P4_DD, PK_P5_PLAIN_DD_TO_F64,
+    // the mixed path's CG on displacement coefficients (cg_passes.cuh)
+    PK_X1I_CG_F32, PK_ROWS_CG_F32, PK_X1F_CG_F32, PK_X1F_RHS_F32, PK_X1F_RHS_DD, PK_X1I_SOLUTION_F32,
+    PK_P5_NEWTON_F32,
     PK_COUNT
 };
 
@@ -959,57 +935,6 @@ static cudaError_t launch_k(K kernel, dim3 grid, size_t smem, const PassArgs& a,
     if (e != cudaSuccess) return e;
     kernel<<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
-}
-
-template <int N>
-cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s) {
-    using C32 = Cfg<N, float>;
-    using C64 = Cfg<N, double>;
-    using CDD = Cfg<N, dd>;
-    static_assert(CDD::row_blocks == C64::row_blocks && CDD::W2 == C64::W2 && CDD::S2 == C64::S2,
-                  "double-float row and column passes share the FP64 geometry");
-    const dim3 r32(C32::row_blocks, 1, nf), r64(C64::row_blocks, 1, nf);
-    const dim3 c32((C32::H + C32::W2 - 1) / C32::W2, (6 * N + C32::S2 - 1) / C32::S2, nf);
-    const dim3 c64((C64::H + C64::W2 - 1) / C64::W2, (6 * N + C64::S2 - 1) / C64::S2, nf);
-    const dim3 g32((C32::H + C32::W3 - 1) / C32::W3, N, nf);
-    const dim3 g64((C64::H + C64::W3 - 1) / C64::W3, N, nf);
-    const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
-    switch (kind) {
-        case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s);
-        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN>, r32, C32::smem_rows, a, s);
-        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN>, r64, C64::smem_rows, a, s);
-        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN>, r32, C32::smem_rows, a, s);
-        case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s);
-        case PK_P1_CG_F32: return launch_k(k_p1<N, float, P1_CG>, r32, C32::smem_rows, a, s);
-        case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s);
-        case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s);
-        case PK_P2_F64: return launch_k(k_p24<N, double, true>, c64, C64::smem_p24, a, s, C64::T2);
-        case PK_P2_F32: return launch_k(k_p24<N, float, true>, c32, C32::smem_p24, a, s, C32::T2);
-        case PK_P4_F64: return launch_k(k_p24<N, double, false>, c64, C64::smem_p24, a, s, C64::T2);
-        case PK_P4_F32: return launch_k(k_p24<N, float, false>, c32, C32::smem_p24, a, s, C32::T2);
-        case PK_P3_F64: return launch_k(k_p3<N, double>, g64, C64::smem_p3, a, s, C64::T3);
-        case PK_P3_F32: return launch_k(k_p3<N, float>, g32, C32::smem_p3, a, s, C32::T3);
-        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double>, r64, C64::smem_rows, a, s);
-        case PK_P5_PLAIN_F32: return launch_k(k_p5<N, float, P5_PLAIN, float>, r32, C32::smem_rows, a, s);
-        case PK_P5_DOT_F64: return launch_k(k_p5<N, double, P5_DOT, double>, r64, C64::smem_rows, a, s);
-        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float>, r32, C32::smem_rows, a, s);
-        case PK_P5_RHS_F64_TO_F64:
-            return launch_k(k_p5<N, double, P5_RHS, double>, r64, C64::smem_rows, a, s);
-        case PK_P5_RHS_F64_TO_F32:
-            return launch_k(k_p5<N, double, P5_RHS, float>, r64, C64::smem_rows, a, s);
-        case PK_P5_RHS_F32_TO_F32:
-            return launch_k(k_p5<N, float, P5_RHS, float>, r32, C32::smem_rows, a, s);
-        case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s);
-        case PK_P2_DD: return launch_k(k_p24<N, dd, true>, c64, CDD::smem_p24, a, s, CDD::T2);
-        case PK_P4_DD: return launch_k(k_p24<N, dd, false>, c64, CDD::smem_p24, a, s, CDD::T2);
-        case PK_P3_DD: return launch_k(k_p3<N, dd>, gdd, CDD::smem_p3, a, s, CDD::T3);
-        case PK_P5_RHS_DD_TO_F32: return launch_k(k_p5<N, dd, P5_RHS, float>, r64, CDD::smem_rows, a, s);
-        case PK_P5_PLAIN_DD_TO_F64:
-            return launch_k(k_p5<N, dd, P5_PLAIN, double>, r64, CDD::smem_rows, a, s);
-        case PK_P1_CGF_F32: return launch_k(k_p1<N, float, P1_CGF>, r32, C32::smem_rows, a, s);
-        case PK_P5_CGF_F32: return launch_k(k_p5<N, float, P5_CGF, float>, r32, C32::smem_rows, a, s);
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 }  // namespace fftg

@@ -1,6 +1,6 @@
 // One translation unit per grid size: compiled once for each supported N
 // with -DFFTG_N=<N>, so the build of the pass kernels runs in parallel.
-#include "passes.cuh"
+#include "cg_passes.cuh"
 
 #ifndef FFTG_N
 #error "compile with -DFFTG_N=<grid size>"

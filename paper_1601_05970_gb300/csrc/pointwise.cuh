@@ -409,6 +409,15 @@ __global__ void __launch_bounds__(kThreads) k_newton_update(VecArgs a) {
     if (threadIdx.x == 0) nd->de2 = tot[0];
 }
 
+// nd->de2 = ||x||^2 from the block partials of P5_NEWTON, one block per cell.
+static __global__ void __launch_bounds__(1024) k_newton_norm(const double* partials, int nb, NewtonDev* nd,
+                                                             const int* active) {
+    const int cell = blockIdx.x;
+    if (active && !active[cell]) return;
+    const double t = sum_partials(partials + (size_t)cell * nb, nb, 1);
+    if (threadIdx.x == 0) nd[cell].de2 = t;
+}
+
 // s = C : p at voxel v with the compact tangent in the tangent's precision
 template <typename T>
 __device__ __forceinline__ void tangent_apply_v(const T* __restrict__ tg, long long v, long long cs,

@@ -4,7 +4,9 @@
 // compiled into run_pass_n; variants 1 .. kVariants-1 are instantiated per
 // grid size in passes_tune.cu.
 //
-//   P1 (x3, rows), P5 (x3, rows): 0 default; 1 the other radix split;
+//   P1 (the row pass of the CG
+//   iteration: inverse x3, C : p,
+//   forward x3), P5 (x3, rows):   0 default; 1 the other radix split;
 //                                 2 half the rows per block; 3 twice the rows
 //   P2, P4 (x2, columns):         0 default; 1 the other radix split;
 //                                 2 32 columns per block; 3 both
@@ -22,7 +24,7 @@
 
 #include <algorithm>
 
-#include "passes.cuh"
+#include "cg_passes.cuh"
 
 namespace fftg {
 
@@ -54,9 +56,11 @@ cudaError_t launch_variant(const PassArgs& a, int nf, cudaStream_t s) {
     using VO = VariantOf<N, TK, V>;
     using C = Cfg<N, float, VO::A, VO::TV>;
     if constexpr (TK == TK_P1) {
-        return launch_k(k_p1<N, float, P1_CGF, VO::A, VO::TV>, dim3(C::row_blocks, 1, nf), C::smem_rows, a, s);
+        constexpr int NA = V == 1 ? RowSplit<N>::ALT : RowSplit<N>::N1;
+        using R = RowCfg<N, NA, VO::TV>;
+        return launch_k(k_rows_cg<N, NA, VO::TV>, dim3(R::blocks, 1, nf), R::smem, a, s, R::NT);
     } else if constexpr (TK == TK_P5) {
-        return launch_k(k_p5<N, float, P5_CGF, float, VO::A, VO::TV>, dim3(C::row_blocks, 1, nf), C::smem_rows,
+        return launch_k(k_p5<N, float, P5_PLAIN, float, VO::A, VO::TV>, dim3(C::row_blocks, 1, nf), C::smem_rows,
                         a, s);
     } else if constexpr (TK == TK_P3 && VO::fused && P3f<N, VO::A>::ok) {
         return launch_k(k_p3f<N, VO::A>, dim3((C::H + C::W3 - 1) / C::W3, N, nf), C::smem_p3, a, s,
@@ -100,7 +104,11 @@ VariantShape shape_of() {
     using VO = VariantOf<N, TK, V>;
     using C = Cfg<N, float, VO::A, VO::TV>;
     VariantShape sh{VO::A, N / VO::A, C::R, TK == TK_P3 ? C::W3 : C::W2, 0};
-    if (TK == TK_P1 || TK == TK_P5)
+    if (TK == TK_P1) {
+        constexpr int NA = V == 1 ? RowSplit<N>::ALT : RowSplit<N>::N1;
+        using R = RowCfg<N, NA, VO::TV>;
+        sh = VariantShape{NA, N / NA, R::R, C::W2, R::blocks};
+    } else if (TK == TK_P5)
         sh.blocks = C::row_blocks;
     else if (TK == TK_P3)
         sh.blocks = ((C::H + C::W3 - 1) / C::W3) * N;
