@@ -145,7 +145,7 @@ struct fftg_handle {
     int N = 0;
     long long V = 0;
     long long cs = 0;            // component stride of the fields (padded)
-    int H = 0;
+    int HP = 0;                  // row pitch of the spectra
     int mixed = 1;
     int nrhs = 6;
     int B = 1;                   // cells
@@ -170,8 +170,7 @@ struct fftg_handle {
     double* sigma = nullptr;     // [B][6][cs]
     void* tangent = nullptr;     // [B][7][cs] inner precision
     // [nf][6][cs] inner precision. Mixed: r, p and x hold displacement
-    // coefficients (cg_passes.cuh, at most 12 N^2 (N + 1) bytes a field), q the
-    // solution in real space
+    // coefficients (cg_passes.cuh), q the solution in real space
     void* x = nullptr;
     void* r = nullptr;
     void* p = nullptr;
@@ -274,10 +273,10 @@ struct Layout {
 
 Layout make_layout(int N, int mixed, int nrhs, int B) {
     const size_t cs = (size_t)comp_stride(N);
-    const size_t H = (size_t)(N + 1) / 2;
+    const size_t HP = (size_t)spec_pitch(N);
     const size_t ts = mixed ? 4 : 8;
     const size_t nf = (size_t)std::max(B, std::max(1, nrhs));
-    const size_t spec1 = 6 * (size_t)N * N * H;  // complex elements per field
+    const size_t spec1 = 6 * (size_t)N * N * HP;  // complex elements per field
     const size_t spec = std::max((size_t)B * spec1 * 16, nf * spec1 * 2 * ts);
     const size_t rb = (size_t)std::max(fftg::row_blocks(N, true), fftg::row_blocks(N, false));
     const size_t npart = std::max({(size_t)kMaxPointwiseBlocks * 36, rb * 2 * nf,
@@ -300,9 +299,11 @@ Layout make_layout(int N, int mixed, int nrhs, int B) {
     L.off_epbar_tr = take(Bs * cs * 8);
     L.off_sigma = take(Bs * 6 * cs * 8);
     L.off_tangent = take(Bs * 7 * cs * ts);
-    L.off_x = take(nf * 6 * cs * ts);
-    L.off_r = take(nf * 6 * cs * ts);
-    L.off_p = take(nf * 6 * cs * ts);
+    // mixed: fields of displacement coefficients; p also stages FP32 fields
+    const size_t vec = nf * std::max(6 * cs * ts, mixed ? (size_t)coef_elements(N) * 8 : 0);
+    L.off_x = take(vec);
+    L.off_r = take(vec);
+    L.off_p = take(vec);
     L.off_q = take(nf * 6 * cs * ts);
     L.off_spec = take(spec);
     L.off_tw32 = take((size_t)N * 8);
@@ -351,7 +352,7 @@ static PassArgs base_args(fftg_handle* h, bool fp64) {
     a.partials = h->partials;
     a.cs = h->cs;
     a.fstride = 6 * h->cs;
-    a.sstride = 6LL * h->N * h->N * h->H;
+    a.sstride = 6LL * h->N * h->N * h->HP;
     a.tstride = 0;
     return a;
 }
@@ -1423,7 +1424,7 @@ int fftg_create_batch(fftg_handle** out, int N, int ncells, const uint8_t* phase
     h->N = N;
     h->V = (long long)V;
     h->cs = comp_stride(N);
-    h->H = (N + 1) / 2;
+    h->HP = spec_pitch(N);
     h->mixed = o.precision == FFTG_MIXED;
     h->nrhs = o.nrhs_tangent;
     h->B = ncells;

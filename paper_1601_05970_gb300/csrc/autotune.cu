@@ -143,9 +143,9 @@ struct DeviceBuffer {
 // keeps the fastest (median of `reps` launches, each bracketed by events).
 int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
     const size_t cs = (size_t)comp_stride(N);
-    const size_t H = (size_t)(N + 1) / 2;
+    const size_t HP = (size_t)spec_pitch(N);
     const size_t field = 6 * cs * sizeof(float);
-    const size_t spec = 6 * (size_t)N * N * H * 2 * sizeof(float);
+    const size_t spec = 6 * (size_t)N * N * HP * 2 * sizeof(float);
     int max_blocks = 0;
     for (int tk = 0; tk < TK_COUNT; ++tk)
         for (int v = 0; v < kVariants; ++v) max_blocks = std::max(max_blocks, variant_shape(N, tk, v).blocks);
@@ -181,7 +181,7 @@ int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
     a.partials = (double*)(b + off_part);
     a.cs = (long long)cs;
     a.fstride = 6 * (long long)cs;
-    a.sstride = 6LL * N * N * (long long)H;
+    a.sstride = 6LL * N * N * (long long)HP;
     a.tangent = b + off_t;
     a.scale = 1.0 / ((double)N * N * N);
     cudaEvent_t e0, e1;

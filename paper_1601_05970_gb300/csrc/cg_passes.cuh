@@ -3,7 +3,7 @@
 // Every vector of the projected CG is compatible, so at each frequency f it
 // is f(x)w + w(x)f for one complex 3-vector w (the displacement coefficient,
 // up to a constant factor). r, p and x are held as w on the half spectrum,
-// [nf][3][N][N][H] complex: half the bytes of a six-component real field,
+// [nf][3][N][N][HP] complex: half the bytes of a six-component real field,
 // no incompatible part can build up in them, and only p is ever taken to
 // real space, where C : p is formed:
 //
@@ -21,7 +21,7 @@
 //
 // An iteration moves 84.3 (x1i) + 2 x 48.2 (P4, P2) + 76.2 (rows) + 48.2
 // (x1f) = 305 B per voxel at 243^3; with r, p and x as real fields it moved
-// 388.8 (243^3: 0.97 -> 0.90 ms an iteration). The residual of a Newton iteration and a column's right-hand side
+// 388.8 (243^3: 1.12 -> 0.95 ms an iteration). The residual of a Newton iteration and a column's right-hand side
 // stop at w (x1f), and the solution is taken to real space once (x1i, P4,
 // P5), which makes a projection of it needless.
 #pragma once
@@ -33,25 +33,51 @@ namespace fftg {
 enum : int { X1F_CG = 0, X1F_RHS = 1 };
 enum : int { X1I_CG = 0, X1I_SOLUTION = 1 };
 
-// x1 split N = N1 * N2 of the two passes: one thread owns the N2 frequencies
-// k1 + N1 k2 of a column, so N2 <= 9 (registers) and, on small grids, two
-// stages rather than one so that a column has more threads.
+// x1 split N = N1 * N2 of the two passes: on small grids two stages rather
+// than one, so that a column has more threads.
 template <int N>
 struct X1Split {
     static constexpr int N1 = N == 225 ? 25 : N == 27 ? 9 : N == 25 || N == 15 ? 5 : N == 9 ? 3 : Plan<N>::N1;
 };
 
-// Columns per block (64-byte runs of the spectrum) and threads: one per
-// (column, k1) of the middle phase.
+// Blocks of the x1 passes: W columns (64-byte runs of the spectrum), as many
+// blocks per SM as shared memory allows up to four, about 1000 threads an SM
+// among them and at most one stage-A item a thread. Stage B and the
+// frequency points are phases of their own (28 warps an SM at 243^3): with a
+// column's N2 frequencies in one thread's registers (14 warps) x1i and x1f
+// took 282 and 210 us there, in this form 283 and 203 us, and with the
+// vectors stored tile by tile (below) 234 and 179 us, 5.2 and 3.9 TB/s. Tiles
+// of three components and twice the blocks: 303 and 228 us.
 template <int N>
 struct X1 {
-    static constexpr int N1 = X1Split<N>::N1, N2 = N / N1, H = (N + 1) / 2, W = 8;
-    static constexpr int NT0 = ((W * N1 + 31) / 32) * 32, NT = NT0 < 64 ? 64 : NT0;
-    static constexpr int MINB = NT > 256 ? 1 : 512 / NT;  // at most 128 registers
+    static constexpr int N1 = X1Split<N>::N1, N2 = N / N1, H = (N + 1) / 2, HP = spec_pitch(N), W = 8;
     static constexpr size_t smem = (size_t)(6 * N * W + N) * 8;
+    static constexpr int NB0 = (int)(220 * 1024 / smem), NB = NB0 > 4 ? 4 : NB0;
+    static constexpr int items = ((6 * W * N2 + 31) / 32) * 32, most = 1024 / NB;
+    static constexpr int NT = items < most ? items : most;
+    static constexpr int MINB = N1 > 15 && NB == 4 ? 3 : 1024 / NT;  // 64 registers; 25-point DFTs 85
     static constexpr int tiles = (H + W - 1) / W, blocks = tiles * N;
-    static_assert(N2 <= 9 && valid_split(N, N1), "x1 split");
+    static_assert(valid_split(N, N1) && W == kCoefTile, "x1 tiles of column pairs");
 };
+
+// Only the x1 passes touch the vectors, so these are laid out as their
+// blocks take them: [nf][N (x2)][tiles][3][N (x1)][W], a block's part one run
+// of 24 N W bytes (the columns past H in the last tile are never read back).
+template <int N>
+__device__ __forceinline__ long long coef_field() { return 3LL * N * N * X1<N>::tiles * X1<N>::W; }
+template <int N>
+__device__ __forceinline__ long long coef_tile(int tile, int k2) {
+    return ((long long)k2 * X1<N>::tiles + tile) * (3 * N * X1<N>::W);
+}
+
+__device__ __forceinline__ void ld_pair(const cplx<float>* p, cplx<float> (&v)[2]) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = mk(t.x, t.y);
+    v[1] = mk(t.z, t.w);
+}
+__device__ __forceinline__ void st_pair(cplx<float>* p, const cplx<float> (&v)[2]) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+}
 
 // Coefficients are stored times a power of two near N^(5/2) / 2, which
 // brings those of a field of white noise to the size of the field's values:
@@ -73,16 +99,29 @@ struct CoefScale {
 
 __device__ __forceinline__ int signed_freq(int k, int N) { return k <= (N - 1) / 2 ? k : k - N; }
 
+// Rounds of spectrum loads of the row pass issued together: with 4 it takes
+// 248 us at 243^3, with 2 261 us. Fetching the tangent to L2 ahead of its use
+// (a bulk prefetch at the block's start) made it 16 us slower; C : p in the
+// registers of the N1-point stage (9 points of all three packed rows, a
+// shared-memory pass less, 80 registers) 290 us.
+#ifndef FFTG_ROWS_LDB
+#define FFTG_ROWS_LDB 4
+#endif
+
 // ---------------------------------------------------------------- x1 inverse
-// aux = r (X1I_CG), aux2 = p, aux3 = x, out = spectrum; fields of 3 N N H
+// aux = r (X1I_CG), aux2 = p, aux3 = x, out = spectrum; fields of 3 N N HP
 // coefficients. X1I_CG updates p and x; X1I_SOLUTION takes x (+ the pending
 // alpha p) to the spectrum. x holds a value once a step was added to it: the
 // first step of a solve writes x = alpha p, so x needs no clearing.
+//
+// A thread takes column pairs (16-byte loads; the pair past an odd H is
+// padding of the row pitch), then stage B and stage A of the inverse run on
+// the tile in shared memory.
 template <int N, int MODE>
 __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
     using T = float;
     using S = X1<N>;
-    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, W = S::W, NT = S::NT;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W, NT = S::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
     cplx<T>* tw = buf + 6 * N * W;
@@ -92,86 +131,89 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
     if (MODE == X1I_CG && cg->done) return;
     const int tid = threadIdx.x;
     load_tw<T>(tw, a.tw, N);
-    __syncthreads();
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
-    const long long NH = (long long)N * H, vf = 3LL * N * NH;
-    const cplx<T>* r = (const cplx<T>*)a.aux + f * vf;
-    cplx<T>* p = (cplx<T>*)a.aux2 + f * vf;
-    cplx<T>* x = (cplx<T>*)a.aux3 + f * vf;
+    const long long NH = (long long)N * HP, vo = f * coef_field<N>() + coef_tile<N>(blockIdx.x, k2g);
+    const cplx<T>* r = (const cplx<T>*)a.aux + vo;
+    cplx<T>* p = (cplx<T>*)a.aux2 + vo;
+    cplx<T>* x = (cplx<T>*)a.aux3 + vo;
     const int it = cg->it;
     const T alpha = (T)cg->alpha, beta = (T)cg->beta;
     // X1I_CG: iteration it adds step it - 1. X1I_SOLUTION: x holds a value
     // after step it - 1 was added, by the iteration that followed it.
     const bool pend = cg->pend != 0;
     const bool has_x = MODE == X1I_CG ? it > 1 : (pend ? it > 1 : it > 0);
-    const T f2 = (T)signed_freq(k2g, N);
-    for (int j = tid; j < W * N1; j += NT) {
-        const int w = j % W, k1 = j / W, col = col0 + w;
+    constexpr T is = CoefScale<N>::inverse;
+    const T g2 = is * (T)signed_freq(k2g, N);
+    for (int j = tid; j < (W / 2) * N; j += NT) {
+        const int w = 2 * (j % (W / 2)), kk = j / (W / 2), col = col0 + w;
         if (col >= H) continue;
-        const T f3 = (T)col;
-        const long long o0 = ((long long)k1 * N + k2g) * H + col;
-        cplx<T> d[N2][3];
+        const int o = kk * W + w;
+        cplx<T> d[3][2], po[3][2], xo[3][2];
+        if (MODE == X1I_CG) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            if (MODE == X1I_CG) {
-                cplx<T> po[N2], xo[N2];
+            for (int i = 0; i < 3; ++i) ld_pair(r + o + i * N * W, d[i]);
+            if (it > 0) {
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) d[k2][i] = r[o0 + (i * N + N1 * k2) * NH];
-                if (it > 0) {
+                for (int i = 0; i < 3; ++i) ld_pair(p + o + i * N * W, po[i]);
+                if (has_x) {
 #pragma unroll
-                    for (int k2 = 0; k2 < N2; ++k2) po[k2] = p[o0 + (i * N + N1 * k2) * NH];
-                    if (has_x) {
-#pragma unroll
-                        for (int k2 = 0; k2 < N2; ++k2) xo[k2] = x[o0 + (i * N + N1 * k2) * NH];
-                    }
-#pragma unroll
-                    for (int k2 = 0; k2 < N2; ++k2) {
-                        const long long o = o0 + (i * N + N1 * k2) * NH;
-                        x[o] = has_x ? xo[k2] + alpha * po[k2] : alpha * po[k2];
-                        d[k2][i] = d[k2][i] + beta * po[k2];
-                    }
+                    for (int i = 0; i < 3; ++i) ld_pair(x + o + i * N * W, xo[i]);
                 }
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) p[o0 + (i * N + N1 * k2) * NH] = d[k2][i];
-            } else {
+                for (int i = 0; i < 3; ++i) {
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) {
-                    const long long o = o0 + (i * N + N1 * k2) * NH;
-                    cplx<T> v = has_x ? x[o] : mk(T(0), T(0));
-                    if (pend) v = v + alpha * p[o];
-                    d[k2][i] = v;
+                    for (int e = 0; e < 2; ++e) {
+                        xo[i][e] = has_x ? xo[i][e] + alpha * po[i][e] : alpha * po[i][e];
+                        d[i][e] = d[i][e] + beta * po[i][e];
+                    }
+                    st_pair(x + o + i * N * W, xo[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) st_pair(p + o + i * N * W, d[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if (has_x) {
+                    ld_pair(x + o + i * N * W, d[i]);
+                } else {
+                    d[i][0] = d[i][1] = mk(T(0), T(0));
+                }
+                if (pend) {
+                    ld_pair(p + o + i * N * W, po[i]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) d[i][e] = d[i][e] + alpha * po[i][e];
                 }
             }
         }
-        // f(x)d + d(x)f, component by component, and its inverse N2-point DFT
-        cplx<T>* base = buf + (N2 * k1) * W + w;
-        constexpr T is = CoefScale<N>::inverse;
-        const T g2 = is * f2, g3 = is * f3;
+        // f(x)d + d(x)f at the frequency's place in permuted order
+        const T g1 = is * (T)signed_freq(kk, N);
+        cplx<T>* b = buf + perm_pos<N, N1>(kk) * W + w;
+        cplx<T> v[6][2];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            cplx<T> v[N2];
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                const T g1 = is * (T)signed_freq(k1 + N1 * k2, N);
-                if (c == 0) v[k2] = (g1 + g1) * d[k2][0];
-                else if (c == 1) v[k2] = (g2 + g2) * d[k2][1];
-                else if (c == 2) v[k2] = (g3 + g3) * d[k2][2];
-                else if (c == 3) v[k2] = g2 * d[k2][2] + g3 * d[k2][1];
-                else if (c == 4) v[k2] = g1 * d[k2][2] + g3 * d[k2][0];
-                else v[k2] = g1 * d[k2][1] + g2 * d[k2][0];
-            }
-            RegDFT<N, N2, +1, T>::run(v, tw);
-#pragma unroll
-            for (int q = 0; q < N2; ++q) {
-                cplx<T> z = v[q];
-                if (k1 > 0 && q > 0) z = twmul<+1>(z, tw[q * k1]);  // q*k1 < N
-                base[(c * N + q) * W] = z;
-            }
+        for (int e = 0; e < 2; ++e) {
+            const T g3 = is * (T)(col + e);
+            v[0][e] = (g1 + g1) * d[0][e];
+            v[1][e] = (g2 + g2) * d[1][e];
+            v[2][e] = (g3 + g3) * d[2][e];
+            v[3][e] = g2 * d[2][e] + g3 * d[1][e];
+            v[4][e] = g1 * d[2][e] + g3 * d[0][e];
+            v[5][e] = g1 * d[1][e] + g2 * d[0][e];
         }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) st_pair(b + c * N * W, v[c]);
     }
     __syncthreads();
-    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)k2g * H;
     constexpr int P = 6 * W;
+    if (N2 > 1) {
+        for (int j = tid; j < P * N1; j += NT) {
+            const int pc = j % P, k1 = j / P;
+            const int c = pc / W, w = pc - c * W;
+            if (col0 + w < H) invB<N, N1, false, T>(buf + c * N * W + w, W, buf + c * N * W + w, W, k1, tw);
+        }
+        __syncthreads();
+    }
+    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)k2g * HP;
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
@@ -187,7 +229,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
     using T = float;
     using S = X1<N>;
-    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, W = S::W, NT = S::NT;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W, NT = S::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
     cplx<T>* tw = buf + 6 * N * W;
@@ -199,9 +241,9 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
     load_tw<T>(tw, a.tw, N);
     __syncthreads();
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
-    const long long NH = (long long)N * H;
-    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * H;
-    cplx<T>* r = (cplx<T>*)a.aux3 + f * (3LL * N * NH);
+    const long long NH = (long long)N * HP;
+    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * HP;
+    cplx<T>* r = (cplx<T>*)a.aux3 + f * coef_field<N>() + coef_tile<N>(blockIdx.x, k2g);
     constexpr int P = 6 * W;
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
@@ -209,80 +251,57 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
         if (col < H) fwdA<N, N1, T>(sp + c * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
+    if (N2 > 1) {
+        for (int j = tid; j < P * N1; j += NT) {
+            const int pc = j % P, k1 = j / P;
+            const int c = pc / W, w = pc - c * W;
+            if (col0 + w < H) fwdB<N, N1, false, T>(buf + c * N * W + w, W, buf + c * N * W + w, W, k1, tw);
+        }
+        __syncthreads();
+    }
     const T f2 = (T)signed_freq(k2g, N);
     const double unit = (double)CoefScale<N>::value * a.scale;
     const T step = MODE == X1F_CG ? (T)(-cg->alpha * unit) : (T)unit;
     T acc = T(0);
-    for (int j = tid; j < W * N1; j += NT) {
-        const int w = j % W, k1 = j / W, col = col0 + w;
+    for (int j = tid; j < (W / 2) * N; j += NT) {
+        const int w = 2 * (j % (W / 2)), kk = j / (W / 2), col = col0 + w;
         if (col >= H) continue;
-        const T f3 = (T)col;
-        const cplx<T>* base = buf + (N2 * k1) * W + w;
-        // t = tau f over the components (11, 22, 33, 23, 13, 12)
-        cplx<T> t[N2][3];
+        const int o = kk * W + w;
+        cplx<T> z[3][2];
+        if (MODE == X1F_CG) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            cplx<T> v[N2];
-#pragma unroll
-            for (int q = 0; q < N2; ++q) v[q] = base[(c * N + q) * W];
-            RegDFT<N, N2, -1, T>::run(v, tw);
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                const T f1 = (T)signed_freq(k1 + N1 * k2, N);
-                if (c == 0) {
-                    t[k2][0] = f1 * v[k2];
-                } else if (c == 1) {
-                    t[k2][1] = f2 * v[k2];
-                } else if (c == 2) {
-                    t[k2][2] = f3 * v[k2];
-                } else if (c == 3) {
-                    t[k2][1] = t[k2][1] + f3 * v[k2];
-                    t[k2][2] = t[k2][2] + f2 * v[k2];
-                } else if (c == 4) {
-                    t[k2][0] = t[k2][0] + f3 * v[k2];
-                    t[k2][2] = t[k2][2] + f1 * v[k2];
-                } else {
-                    t[k2][0] = t[k2][0] + f2 * v[k2];
-                    t[k2][1] = t[k2][1] + f1 * v[k2];
-                }
-            }
+            for (int i = 0; i < 3; ++i) ld_pair(r + o + i * N * W, z[i]);
         }
-        const long long o0 = ((long long)k1 * N + k2g) * H + col;
-        cplx<T> fr[N2];  // f . r
-        T q2[N2];
+        const cplx<T>* b = buf + perm_pos<N, N1>(kk) * W + w;
+        cplx<T> c[6][2];
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-            const T f1 = (T)signed_freq(k1 + N1 * k2, N);
+        for (int k = 0; k < 6; ++k) ld_pair(b + k * N * W, c[k]);
+        const T f1 = (T)signed_freq(kk, N);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const T f3 = (T)(col + e);
+            cplx<T> t0 = f1 * c[0][e] + f2 * c[5][e] + f3 * c[4][e];
+            cplx<T> t1 = f1 * c[5][e] + f2 * c[1][e] + f3 * c[3][e];
+            cplx<T> t2 = f1 * c[4][e] + f2 * c[3][e] + f3 * c[2][e];
             const T q = f1 * f1 + f2 * f2 + f3 * f3;
-            const T iq = q > T(0) ? T(1) / q : T(0);  // the mean maps to zero
-            const cplx<T> h = (T(-0.5) * iq) * (f1 * t[k2][0] + f2 * t[k2][1] + f3 * t[k2][2]);
+            const T iq = q > T(0) ? __frcp_rn(q) : T(0);  // the mean maps to zero
+            const cplx<T> h = (T(-0.5) * iq) * (f1 * t0 + f2 * t1 + f3 * t2);
             const T m = step * iq;
-            t[k2][0] = m * (t[k2][0] + f1 * h);
-            t[k2][1] = m * (t[k2][1] + f2 * h);
-            t[k2][2] = m * (t[k2][2] + f3 * h);
-            q2[k2] = q;
-            fr[k2] = mk(T(0), T(0));
-        }
-        T part = T(0);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            cplx<T> ro[N2];
-            if (MODE == X1F_CG) {
-#pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) ro[k2] = r[o0 + (i * N + N1 * k2) * NH];
-            }
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                const T fi = i == 0 ? (T)signed_freq(k1 + N1 * k2, N) : i == 1 ? f2 : f3;
-                const cplx<T> z = MODE == X1F_CG ? ro[k2] + t[k2][i] : t[k2][i];
-                r[o0 + (i * N + N1 * k2) * NH] = z;
-                fr[k2] = fr[k2] + fi * z;
-                part += q2[k2] * (z.x * z.x + z.y * z.y);
-            }
+            t0 = m * (t0 + f1 * h);
+            t1 = m * (t1 + f2 * h);
+            t2 = m * (t2 + f3 * h);
+            z[0][e] = MODE == X1F_CG ? z[0][e] + t0 : t0;
+            z[1][e] = MODE == X1F_CG ? z[1][e] + t1 : t1;
+            z[2][e] = MODE == X1F_CG ? z[2][e] + t2 : t2;
+            const cplx<T> fr = f1 * z[0][e] + f2 * z[1][e] + f3 * z[2][e];
+            const T s = z[0][e].x * z[0][e].x + z[0][e].y * z[0][e].y + z[1][e].x * z[1][e].x +
+                        z[1][e].y * z[1][e].y + z[2][e].x * z[2][e].x + z[2][e].y * z[2][e].y;
+            // f3 > 0 stands for -f3 too; the column past an odd H is padding
+            const T part = q * s + fr.x * fr.x + fr.y * fr.y;
+            if (col + e < H) acc += col + e == 0 ? part : T(2) * part;
         }
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) part += fr[k2].x * fr[k2].x + fr[k2].y * fr[k2].y;
-        acc += col == 0 ? part : T(2) * part;  // f3 > 0 stands for -f3 too
+        for (int i = 0; i < 3; ++i) st_pair(r + o + i * N * W, z[i]);
     }
     const double s = block_sum_any((double)acc) * CoefScale<N>::square;
     if (tid == 0) {
@@ -321,7 +340,7 @@ template <int N>
 __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
     using T = dd;
     using C = Cfg<N, T>;
-    constexpr int H = C::H, W = C::W3, NT = C::T3;
+    constexpr int H = C::H, HP = C::HP, W = C::W3, NT = C::T3;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -332,9 +351,9 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
     load_tw<T>(tw, a.tw, N);
     __syncthreads();
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
-    const long long NH = (long long)N * H;
-    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * H;
-    cplx<float>* r = (cplx<float>*)a.aux3 + f * (3LL * N * NH);
+    const long long NH = (long long)N * HP;
+    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * HP;
+    cplx<float>* r = (cplx<float>*)a.aux3 + f * coef_field<N>();
     constexpr int P = 6 * W;
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
@@ -377,7 +396,8 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
         t[1] = m * (t[1] + dd_scale(h, f2));
         t[2] = m * (t[2] + dd_scale(h, f3));
         const float wt = col == 0 ? 1.0f : 2.0f;  // f3 > 0 stands for -f3 too
-        const long long o = ((long long)kk * N + k2g) * H + col;
+        constexpr int WX = X1<N>::W;
+        const long long o = coef_tile<N>(col / WX, k2g) + kk * WX + col % WX;
         float s0 = 0.0f;
         cplx<float> fr = mk(0.0f, 0.0f);
         dd s1(0.0f, 0.0f);
@@ -386,7 +406,7 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
         for (int i = 0; i < 3; ++i) {
             const float fi = i == 0 ? f1 : i == 1 ? f2 : f3;
             const cplx<float> z = mk((float)t[i].x, (float)t[i].y);
-            r[o + i * N * NH] = z;
+            r[o + i * N * WX] = z;
             s0 += z.x * z.x + z.y * z.y;
             fr = fr + fi * z;
             s1 += t[i].x * t[i].x + t[i].y * t[i].y;
@@ -405,11 +425,6 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
 }
 
 // ---------------------------------------------------------------------- rows
-// rounds of spectrum loads issued together
-#ifndef FFTG_ROWS_LDB
-#define FFTG_ROWS_LDB 2
-#endif
-
 // Radix split of the rows: the plan's, or two stages on the small grids,
 // where a row of one stage has too few threads.
 template <int N>
@@ -430,7 +445,7 @@ struct RowCfg {
     static constexpr int R = C::R < fl2(N * N / 152) ? C::R : fl2(N * N / 152);
     static constexpr int N1 = NA, N2 = N / NA;
     static constexpr int NT0 = ((3 * R * N2 + 31) / 32) * 32;
-    static constexpr int NT = NT0 < 64 ? 64 : NT0 > 256 ? 256 : NT0;
+    static constexpr int NT = NT0 < 64 ? 64 : NT0 > 448 ? 448 : NT0;
     static constexpr int MINB = 1024 / NT;  // 64 registers
     static constexpr size_t smem = (size_t)(3 * R * N + N) * 8;
     static constexpr int blocks = (N * N + R - 1) / R;
@@ -440,7 +455,7 @@ template <int N, int NA, int TV>
 __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB) k_rows_cg(PassArgs a) {
     using T = float;
     using S = RowCfg<N, NA, TV>;
-    constexpr int R = S::R, H = (N + 1) / 2, NT = S::NT;
+    constexpr int R = S::R, H = (N + 1) / 2, HP = spec_pitch(N), NT = S::NT;
     constexpr int N1 = S::N1, N2 = S::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* z = reinterpret_cast<cplx<T>*>(smem_raw);  // [3][R][N]
@@ -451,8 +466,10 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
     load_tw<T>(tw, a.tw, N);
     const int row0 = blockIdx.x * R;
     const int nrows = min(R, N * N - row0);
-    const long long HS = (long long)N * N * H;
-    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)row0 * H;
+    const long long HS = (long long)N * N * HP;
+    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)row0 * HP;
+    const long long cs = a.cs;
+    const T* tg = (const T*)a.tangent + f * a.tstride + (long long)row0 * N;
     // the half spectra of two real components -> one complex row; the
     // imaginary parts at k = 0 are rounding and are dropped
     constexpr int NRL = (R * H + NT - 1) / NT;
@@ -464,10 +481,11 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
         for (int u = 0; u < LB; ++u) {
             const int it = tid + (r0 + u) * NT;
             if (r0 + u < NRL && it < nrows * H) {
+                const int row = it / H, o = it + row * (HP - H);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    A[u][c] = sp[(2 * c) * HS + it];
-                    B[u][c] = sp[(2 * c + 1) * HS + it];
+                    A[u][c] = sp[(2 * c) * HS + o];
+                    B[u][c] = sp[(2 * c + 1) * HS + o];
                 }
             }
         }
@@ -506,15 +524,13 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
         if (pc % R < nrows) invA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
     }
     __syncthreads();
-    // tau = C : p, four voxels a lane (R is a multiple of 4, so a block
+    // tau = C : p, two voxels a lane (R is a multiple of 4, so a block
     // starts on a vector boundary; in the last block the vector that
     // straddles the end of the grid reads the padding of the tangent and
     // changes rows that no stage reads)
-    const long long cs = a.cs;
-    const T* tg = (const T*)a.tangent + f * a.tstride + (long long)row0 * N;
     const int nel = nrows * N;
     T pcp = T(0);
-    constexpr int VW = 4;
+    constexpr int VW = 2;
     for (int j = tid; j < (R * N) / VW; j += NT) {
         const int i0 = j * VW;
         if (i0 >= nel) continue;
@@ -573,15 +589,15 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
         __syncthreads();
     }
     for (int it = tid; it < nrows * H; it += NT) {
-        const int row = it / H, k = it - row * H;
+        const int row = it / H, k = it - row * H, o = row * HP + k;
         const int pk = perm_pos<N, N1>(k), pn = perm_pos<N, N1>(k == 0 ? 0 : N - k);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const cplx<T> zk = z[(c * R + row) * N + pk];
             const cplx<T> zn = conj(z[(c * R + row) * N + pn]);
             const cplx<T> d = zk - zn;  // (zk - zn) / (2i) = (d.y, -d.x) / 2
-            sp[(2 * c) * HS + it] = half_of(zk + zn);
-            sp[(2 * c + 1) * HS + it] = half_of(mk(d.y, -d.x));
+            sp[(2 * c) * HS + o] = half_of(zk + zn);
+            sp[(2 * c + 1) * HS + o] = half_of(mk(d.y, -d.x));
         }
     }
 }

@@ -350,7 +350,7 @@ struct FsLayout {
 };
 
 FsLayout fs_layout(int N, bool mixed) {
-    const size_t cs = (size_t)comp_stride(N), H = (size_t)(N + 1) / 2;
+    const size_t cs = (size_t)comp_stride(N), HP = (size_t)spec_pitch(N);
     const size_t ts = mixed ? 4 : 8;
     const size_t rb = (size_t)std::max(fs_row_blocks(N, true), fs_row_blocks(N, false));
     const size_t npart = std::max((size_t)kFsPointBlocks * 10, rb * 2);
@@ -371,7 +371,7 @@ FsLayout fs_layout(int N, bool mixed) {
     L.off_r = take(9 * cs * ts);
     L.off_p = take(9 * cs * ts);
     L.off_q = take(9 * cs * ts);
-    L.off_spec = take(9 * (size_t)N * N * H * 16);  // FP64 complex: the residual's size
+    L.off_spec = take(9 * (size_t)N * N * HP * 16);  // FP64 complex: the residual's size
     L.off_tw32 = take((size_t)N * 8);
     L.off_tw64 = take((size_t)N * 16);
     L.off_twdd = take((size_t)N * 16);
@@ -393,7 +393,7 @@ bool fs_options_valid(const fftg_options& o) {
 }  // namespace
 
 struct fftg_fs_handle {
-    int N = 0, H = 0;
+    int N = 0;
     long long V = 0, cs = 0;
     int mixed = 1;
     fftg_options opt{};
@@ -829,7 +829,6 @@ int fftg_fs_create(fftg_fs_handle** out, int N, const uint8_t* phase, int nphase
     fftg_fs_handle* h = new (std::nothrow) fftg_fs_handle();
     if (!h) return FFTG_ENOMEM;
     h->N = N;
-    h->H = (N + 1) / 2;
     h->V = (long long)V;
     h->cs = comp_stride(N);
     h->mixed = o.precision == FFTG_MIXED;

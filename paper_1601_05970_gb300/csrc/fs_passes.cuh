@@ -2,7 +2,7 @@
 // as the next step of the method): the projected matvec q = G (K : p) and
 // the residual G P on real fields of nine components, the deformation-
 // gradient-like tensor A_ij at component 3i + j, [9][cs], and a half
-// spectrum [9][N][N][H].
+// spectrum [9][N][N][HP] (row pitch spec_pitch).
 //
 // The five passes are those of the small-strain path with three changes:
 //  * nine real components share five complex FFTs per row (pairs (0,1),
@@ -88,7 +88,7 @@ struct FsArgs {
 
 template <int N, typename T>
 struct FsCfg {
-    static constexpr int H = (N + 1) / 2;
+    static constexpr int H = (N + 1) / 2, HP = spec_pitch(N);
     static constexpr int CS = (int)sizeof(cplx<T>);
     static constexpr int fl2(int x) {
         return x >= 32 ? 32 : x >= 16 ? 16 : x >= 8 ? 8 : x >= 4 ? 4 : x >= 2 ? 2 : 1;
@@ -161,7 +161,7 @@ __device__ __forceinline__ void svk_tangent_apply(const T (&h)[9], T lam, T mu, 
 template <int N, typename T, int MODE>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1) k_fs_p1(FsArgs a) {
     using C = FsCfg<N, T>;
-    constexpr int R = C::R, H = C::H, VW = C::VW;
+    constexpr int R = C::R, H = C::H, HP = C::HP, VW = C::VW;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -316,11 +316,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
     // Split each packed transform Z = FFT(a + i b) into the half spectra
     // A_k = (Z_k + conj Z_{N-k})/2 and B_k = (Z_k - conj Z_{N-k})/(2i).
     cplx<T>* out = (cplx<T>*)a.out;
-    const long long HS = (long long)N * N * H;
+    const long long HS = (long long)N * N * HP;
     for (int it = tid; it < nrows * H; it += kThreads) {
         const int row = it / H, k = it - row * H;
         const int pk = perm_pos<N>(k), pn = perm_pos<N>(k == 0 ? 0 : N - k);
-        const long long o = (long long)(row0 + row) * H + k;
+        const long long o = (long long)(row0 + row) * HP + k;
 #pragma unroll
         for (int c = 0; c < kFsPairs; ++c) {
             const cplx<T> zk = z[(c * R + row) * N + pk];
@@ -359,7 +359,7 @@ __device__ __forceinline__ void ghat_fs_point(cplx<T>* b, int cs, int f1, int f2
 template <int N, typename T>
 __global__ void __launch_bounds__(FsCfg<N, T>::T3) k_fs_p3(FsArgs a) {
     using C = FsCfg<N, T>;
-    constexpr int H = C::H, W = C::W3, NT = C::T3;
+    constexpr int H = C::H, HP = C::HP, W = C::W3, NT = C::T3;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -371,11 +371,11 @@ __global__ void __launch_bounds__(FsCfg<N, T>::T3) k_fs_p3(FsArgs a) {
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
     cplx<T>* sp = (cplx<T>*)a.out;
     constexpr int P = kFsComp * W;
-    const long long NH = (long long)N * H;
+    const long long NH = (long long)N * HP;
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) fwdA<N, T>(sp + c * N * NH + k2g * H + col, (int)NH, buf + c * N * W + w, W, t, tw);
+        if (col < H) fwdA<N, T>(sp + c * N * NH + k2g * HP + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
     const T scale = (T)a.scale;
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(FsCfg<N, T>::T3) k_fs_p3(FsArgs a) {
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) invA<N, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * H + col, (int)NH, t, tw);
+        if (col < H) invA<N, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * HP + col, (int)NH, t, tw);
     }
 }
 
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(FsCfg<N, T>::T3) k_fs_p3(FsArgs a) {
 template <int N, typename T, int MODE, typename TO>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1) k_fs_p5(FsArgs a) {
     using C = FsCfg<N, T>;
-    constexpr int R = C::R, H = C::H;
+    constexpr int R = C::R, H = C::H, HP = C::HP;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     const long long base = (long long)row0 * N;
     const int nel = nrows * N;
     const cplx<T>* in = (const cplx<T>*)a.in;
-    const long long HS = (long long)N * N * H;
+    const long long HS = (long long)N * N * HP;
     // Spectrum rows -> tile, the loads of FFTG_FS_P5_LDB rounds issued
     // before their stores.
     constexpr int NRL = (R * H + kThreads - 1) / kThreads;
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
             const int it = tid + (r0 + u) * kThreads;
             if (r0 + u < NRL && it < nrows * H) {
                 const int row = it / H, k = it - row * H;
-                const long long o = (long long)(row0 + row) * H + k;
+                const long long o = (long long)(row0 + row) * HP + k;
 #pragma unroll
                 for (int c = 0; c < kFsPairs; ++c) {
                     A[u][c] = in[(2 * c) * HS + o];

@@ -24,6 +24,23 @@ inline long long comp_stride(int N) {
     return ((V + 4 + 31) / 32) * 32;
 }
 
+// Row pitch of the half spectra, in complex elements: (N + 1) / 2 rounded up
+// to a multiple of 4, so that every row starts on a 32-byte sector and the
+// runs of 8 and 16 columns that the x1 and x2 passes take touch no sector
+// twice; on the grids whose spectrum is far larger than L2, of 16 (128-byte
+// lines: an in-place copy in the x2 pattern 128 -> 120 us at 243^3).
+constexpr int spec_pitch(int N) {
+    const int H = (N + 1) / 2, u = N > 200 ? 16 : 4;
+    return (H + u - 1) / u * u;
+}
+
+// The x1 passes of the mixed CG (cg_passes.cuh) take kCoefTile columns a
+// block, and its vectors are stored tile by tile: complex elements a field.
+constexpr int kCoefTile = 8;
+constexpr long long coef_elements(int N) {
+    return 3LL * N * N * (((N + 1) / 2 + kCoefTile - 1) / kCoefTile * kCoefTile);
+}
+
 // w_N^j = exp(-2 pi i j / N), evaluated in long double on the host: FP64,
 // FP32 and (when twdd is not null) double-float (hi, lo) pairs, 4 floats
 // per twiddle (re.hi, re.lo, im.hi, im.lo).

@@ -1,6 +1,7 @@
 // The five grid passes of the projected matvec q = G (C : p) and of the
 // residual G sigma, on a real field [nf][6][N][N][N] and a half spectrum
-// [nf][6][N][N][H], H = (N+1)/2 (odd N: no Nyquist mode, Section 2.3).
+// [nf][6][N][N][HP], H = (N+1)/2 columns (odd N: no Nyquist mode, Section
+// 2.3) at the padded row pitch HP = spec_pitch(N).
 //
 //   P1 (rows, x3)  [p = r + beta p]; tau = C : p (Section 4.2 tangent) or
 //                  tau = input; real-to-complex FFT along x3: two real
@@ -19,6 +20,7 @@
 #include "common.cuh"
 #include "dd.cuh"
 #include "fft_core.cuh"
+#include "host_common.h"
 
 namespace fftg {
 
@@ -168,7 +170,7 @@ __device__ __forceinline__ void stv(T* p, const T (&v)[W]) {
 template <int N, typename T, int NA = Plan<N>::N1, int TV = 0>
 struct Cfg {
     static constexpr int PN1 = NA, PN2 = N / NA;
-    static constexpr int H = (N + 1) / 2;
+    static constexpr int H = (N + 1) / 2, HP = spec_pitch(N);
     static constexpr int CS = (int)sizeof(cplx<T>);
     static constexpr int BUDGET = 100 * 1024;
     static constexpr int ROW_BUDGET = 50 * 1024;
@@ -278,7 +280,7 @@ template <int N, typename T, int MODE, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
     k_p1(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
-    constexpr int R = C::R, H = C::H;
+    constexpr int R = C::R, H = C::H, HP = C::HP;
     constexpr int N1 = NA, N2 = N / NA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -401,11 +403,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
         __syncthreads();
     }
     cplx<T>* out = (cplx<T>*)a.out + f * a.sstride;
-    const long long HS = (long long)N * N * H;
+    const long long HS = (long long)N * N * HP;
     for (int it = tid; it < nrows * H; it += kThreads) {
         const int row = it / H, k = it - row * H;
         const int pk = perm_pos<N, N1>(k), pn = perm_pos<N, N1>(k == 0 ? 0 : N - k);
-        const long long o = (long long)(row0 + row) * H + k;
+        const long long o = (long long)(row0 + row) * HP + k;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const cplx<T> zk = z[(c * R + row) * N + pk];
@@ -426,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
 template <int N, typename T, bool FWD, int NC = 6, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T2) k_p24(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
-    constexpr int H = C::H, W = C::W2, S = C::S2, NT = C::T2;
+    constexpr int H = C::H, HP = C::HP, W = C::W2, S = C::S2, NT = C::T2;
     constexpr int N1 = NA, N2 = N / NA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -455,28 +457,28 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T2) k_p24(PassArgs a) {
             const int pc = it % P, t = it / P;
             const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
             if (col < H && slab < NC * N)
-                fwdA<N, N1, T>(sp + (long long)slab * N * H + col, H, buf + s * N * W + w, W, t, tw);
+                fwdA<N, N1, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, t, tw);
         }
         __syncthreads();
         for (int it = tid; it < P * N1; it += NT) {
             const int pc = it % P, k1 = it / P;
             const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
             if (col < H && slab < NC * N)
-                fwdB<N, N1, true, T>(buf + s * N * W + w, W, sp + (long long)slab * N * H + col, H, k1, tw);
+                fwdB<N, N1, true, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, k1, tw);
         }
     } else {
         for (int it = tid; it < P * N1; it += NT) {
             const int pc = it % P, k1 = it / P;
             const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
             if (col < H && slab < NC * N)
-                invB<N, N1, true, T>(sp + (long long)slab * N * H + col, H, buf + s * N * W + w, W, k1, tw);
+                invB<N, N1, true, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, k1, tw);
         }
         __syncthreads();
         for (int it = tid; it < P * N2; it += NT) {
             const int pc = it % P, t = it / P;
             const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
             if (col < H && slab < NC * N)
-                invA<N, N1, T>(buf + s * N * W + w, W, sp + (long long)slab * N * H + col, H, t, tw);
+                invA<N, N1, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, t, tw);
         }
     }
 }
@@ -559,7 +561,7 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T3, (sizeof(T) == 4 && Cfg<
                                                       ? (Cfg<N, T, NA, TV>::T3 <= 256 ? 4 : 2)
                                                       : is_dd_v<T> ? FFTG_DD_P3_MINB : 1) k_p3(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
-    constexpr int H = C::H, W = C::W3, NT = C::T3;
+    constexpr int H = C::H, HP = C::HP, W = C::W3, NT = C::T3;
     constexpr int N1 = NA, N2 = N / NA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -573,11 +575,11 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T3, (sizeof(T) == 4 && Cfg<
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
     cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride;
     constexpr int P = 6 * W;
-    const long long NH = (long long)N * H;
+    const long long NH = (long long)N * HP;
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + k2g * H + col, (int)NH, buf + c * N * W + w, W, t, tw);
+        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + k2g * HP + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
     p3_tile_middle<N, N1, W, NT, T>(buf, tw, col0, k2g, (T)a.scale, tid);
@@ -585,7 +587,7 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T3, (sizeof(T) == 4 && Cfg<
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * H + col, (int)NH, t, tw);
+        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * HP + col, (int)NH, t, tw);
     }
 }
 
@@ -619,7 +621,7 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
     using T = float;
     using S = P3f<N, NA>;
     static_assert(S::ok, "fused P3 needs a two-stage split with N2 <= 9");
-    constexpr int H = (N + 1) / 2, W = S::W, N1 = NA, N2 = N / NA, NT = S::NT;
+    constexpr int H = (N + 1) / 2, HP = spec_pitch(N), W = S::W, N1 = NA, N2 = N / NA, NT = S::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* buf = tw + N;  // [6][N][W]
@@ -632,11 +634,11 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
     const int col0 = blockIdx.x * W, k2g = blockIdx.y;
     cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride;
     constexpr int P = 6 * W;
-    const long long NH = (long long)N * H;
+    const long long NH = (long long)N * HP;
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + k2g * H + col, (int)NH, buf + c * N * W + w, W, t, tw);
+        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + k2g * HP + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
     const T scale = (T)a.scale;
@@ -711,7 +713,7 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * H + col, (int)NH, t, tw);
+        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + k2g * HP + col, (int)NH, t, tw);
     }
 }
 
@@ -722,7 +724,7 @@ template <int N, typename T, int MODE, typename TO, int NA = Plan<N>::N1, int TV
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
     k_p5(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
-    constexpr int R = C::R, H = C::H;
+    constexpr int R = C::R, H = C::H, HP = C::HP;
     constexpr int N1 = NA, N2 = N / NA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -738,7 +740,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     const long long base = (long long)row0 * N;
     const int nel = nrows * N;
     const cplx<T>* in = (const cplx<T>*)a.in + f * a.sstride;
-    const long long HS = (long long)N * N * H;
+    const long long HS = (long long)N * N * HP;
     // Spectrum rows -> tile: the loads of FFTG_P5_LDB rounds are issued
     // before their stores, so that more of them are in flight.
     constexpr int NRL = (R * H + kThreads - 1) / kThreads;
@@ -751,7 +753,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
             const int it = tid + (r0 + u) * kThreads;
             if (r0 + u < NRL && it < nrows * H) {
                 const int row = it / H, k = it - row * H;
-                const long long o = (long long)(row0 + row) * H + k;
+                const long long o = (long long)(row0 + row) * HP + k;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     A[u][c] = in[(2 * c) * HS + o];
