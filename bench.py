@@ -151,8 +151,8 @@ def flops_per_voxel(N):
 # with the repository give the command), valid while the kernel sources
 # have the digest they had then (SHA-256 prefix of the files listed).
 KERNEL_FILES = ("common.cuh", "fft_core.cuh", "passes.cuh", "cg_passes.cuh")
-FS_KERNEL_FILES = KERNEL_FILES + ("fs_passes.cuh",)
-TRAFFIC = {"fs_p1_cgf_f32": {"N": 243, "bytes": 3587.1e6, "digest": "43f6874074ac81bb", "files": FS_KERNEL_FILES}}
+FS_KERNEL_FILES = KERNEL_FILES + ("fs_passes.cuh", "fs_cg_passes.cuh")
+TRAFFIC = {}
 
 
 def _strip_comments(src: bytes) -> bytes:
@@ -567,9 +567,15 @@ def fs_bytes_per_voxel(N):
     the tangent data is H = F - I, 36 B, and the phase byte)."""
     H = (N + 1) // 2
     s32 = 9 * 8 * H / N
+    v32 = s32 / 3
     return {"fs_p1_cg_f32": 5 * 36 + 36 + 1 + s32,
             "fs_p2_f32": 2 * s32, "fs_p3_f32": 2 * s32, "fs_p4_f32": 2 * s32,
             "fs_p5_dot_f32": s32 + 36 + 36, "fs_cg_update_f32": 3 * 36,
+            # on coefficients (v32 bytes a vector): six of the nine
+            # components pass x1; the row pass reads H and the phase
+            "fs_x1i_cg_f32": 5 * v32 + 2 * v32, "fs_p4_grad_f32": 2 * v32 + s32,
+            "fs_rows_cg_f32": 2 * s32 + 36 + 1, "fs_p2_grad_f32": s32 + 2 * v32,
+            "fs_x1f_cg_f32": 2 * v32 + 2 * v32,
             # without the update pass: P1 as above (and <p, K:p>); P5 reads
             # the spectrum and r and writes r
             "fs_p1_cgf_f32": 5 * 36 + 36 + 1 + s32, "fs_p5_cgf_f32": s32 + 36 + 36,
@@ -654,13 +660,18 @@ def finite_strain_line(N=243, warm=1, timed=2):
     eff = {"fs_p1_cg_f32": it, "fs_p5_dot_f32": it, "fs_cg_update_f32": it,
            "fs_p1_cgf_f32": it, "fs_p5_cgf_f32": it, "fs_cg_rr_f32": it,
            "fs_p2_f32": it + solves + 9 * timed, "fs_p3_f32": it + solves + 9 * timed,
-           "fs_p4_f32": it + solves + 9 * timed}
+           "fs_p4_f32": it + solves + 9 * timed,
+           "fs_x1i_cg_f32": it, "fs_rows_cg_f32": it, "fs_x1f_cg_f32": it,
+           "fs_p4_grad_f32": it + solves, "fs_p2_grad_f32": it + 9 * timed}
     kind, (kms, kn) = max(((k, v) for k, v in prof.items() if k in bpv), key=lambda kv: kv[1][0])
     hbm, peak_kind = measured_hbm()
     alg = eff[kind] * V * bpv[kind]
     achieved = alg / (kms * 1e-3) / 1e9
-    fused = "fs_p1_cgf_f32" in prof
-    it_kinds = (("fs_p1_cgf_f32", "fs_p2_f32", "fs_p3_f32", "fs_p4_f32", "fs_p5_cgf_f32", "fs_cg_rr_f32")
+    coef = "fs_rows_cg_f32" in prof
+    fused = coef or "fs_p1_cgf_f32" in prof
+    it_kinds = (("fs_x1i_cg_f32", "fs_p4_grad_f32", "fs_rows_cg_f32", "fs_p2_grad_f32", "fs_x1f_cg_f32",
+                 "fs_cg_rr_f32") if coef else
+                ("fs_p1_cgf_f32", "fs_p2_f32", "fs_p3_f32", "fs_p4_f32", "fs_p5_cgf_f32", "fs_cg_rr_f32")
                 if fused else
                 ("fs_p1_cg_f32", "fs_p2_f32", "fs_p3_f32", "fs_p4_f32", "fs_p5_dot_f32", "fs_cg_update_f32"))
     iteration = None
@@ -668,7 +679,8 @@ def finite_strain_line(N=243, warm=1, timed=2):
         ims = sum(prof[k][0] / eff[k] for k in it_kinds)
         ib = sum(bpv[k] for k in it_kinds)
         ig = ib * V / (ims * 1e-3) / 1e9
-        iteration = {"what": "one CG iteration, per field" + (" (update fused into P1/P5)" if fused else ""),
+        iteration = {"what": "one CG iteration, per field" + (" (on coefficients)" if coef else
+                                                             " (update fused into P1/P5)" if fused else ""),
                      "ms_per_field_iter": round(ims, 4), "bytes_per_voxel": round(ib, 1),
                      "achieved": round(ig, 1), "peak": hbm, "unit": "GB/s", "frac": round(ig / hbm, 3)}
     return {

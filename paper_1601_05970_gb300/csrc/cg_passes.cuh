@@ -93,9 +93,15 @@ struct CoefScale {
     }
     static constexpr float value = (float)(1 << exponent());
     static constexpr float inverse = 1.0f / value;
-    // sum over voxels of a squared field from sum (q |w|^2 + |f.w|^2)
+    // sum over voxels of a squared field from sum (q |w|^2 + |f.w|^2); half
+    // of it from sum q |a|^2 of a gradient field
     static constexpr double square = 2.0 * N * N * (double)N / ((double)value * (double)value);
 };
+
+// Component of the nine of a finite-strain spectrum that holds field c of the
+// six the x1 passes take: (i, 1) for the fields that f1 multiplies, (i, 3) for
+// the others.
+__device__ __forceinline__ int fs_slot(int c) { return c < 3 ? 3 * c : 3 * (c - 3) + 2; }
 
 __device__ __forceinline__ int signed_freq(int k, int N) { return k <= (N - 1) / 2 ? k : k - N; }
 
@@ -117,7 +123,10 @@ __device__ __forceinline__ int signed_freq(int k, int N) { return k <= (N - 1) /
 // A thread takes column pairs (16-byte loads; the pair past an odd H is
 // padding of the row pitch), then stage B and stage A of the inverse run on
 // the tile in shared memory.
-template <int N, int MODE>
+//
+// FS (finite strain): the vectors are a_i of gradient fields a(x)f, and six
+// fields go on: f1 a_i and a_i (the x2 pass applies f2 and f3 to the latter).
+template <int N, int MODE, bool FS = false>
 __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
     using T = float;
     using S = X1<N>;
@@ -192,6 +201,14 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
         cplx<T> v[6][2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
+            if (FS) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    v[i][e] = g1 * d[i][e];
+                    v[3 + i][e] = is * d[i][e];
+                }
+                continue;
+            }
             const T g3 = is * (T)(col + e);
             v[0][e] = (g1 + g1) * d[0][e];
             v[1][e] = (g2 + g2) * d[1][e];
@@ -217,7 +234,8 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + c * N * NH + col, (int)NH, t, tw);
+        const int comp = FS ? fs_slot(c) : c;
+        if (col < H) invA<N, N1, T>(buf + c * N * W + w, W, sp + comp * N * NH + col, (int)NH, t, tw);
     }
 }
 
@@ -225,7 +243,8 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
 // in = spectrum of tau, aux3 = r. X1F_CG: r -= alpha w and the block's part
 // of <r, r>; X1F_RHS: r = w with scale the sign and 1/N^3 of the right-hand
 // side, and the parts of <r, r> and of ||G tau||^2 before rounding.
-template <int N, int MODE>
+// FS: t_i = f1 A_i1 + B_i of the six fields that the x2 pass leaves, w = t / q.
+template <int N, int MODE, bool FS = false>
 __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
     using T = float;
     using S = X1<N>;
@@ -248,7 +267,8 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
+        const int comp = FS ? fs_slot(c) : c;
+        if (col < H) fwdA<N, N1, T>(sp + comp * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
     if (N2 > 1) {
@@ -280,20 +300,27 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const T f3 = (T)(col + e);
-            cplx<T> t0 = f1 * c[0][e] + f2 * c[5][e] + f3 * c[4][e];
-            cplx<T> t1 = f1 * c[5][e] + f2 * c[1][e] + f3 * c[3][e];
-            cplx<T> t2 = f1 * c[4][e] + f2 * c[3][e] + f3 * c[2][e];
             const T q = f1 * f1 + f2 * f2 + f3 * f3;
             const T iq = q > T(0) ? __frcp_rn(q) : T(0);  // the mean maps to zero
-            const cplx<T> h = (T(-0.5) * iq) * (f1 * t0 + f2 * t1 + f3 * t2);
             const T m = step * iq;
-            t0 = m * (t0 + f1 * h);
-            t1 = m * (t1 + f2 * h);
-            t2 = m * (t2 + f3 * h);
+            cplx<T> t0, t1, t2;
+            if (FS) {
+                t0 = m * (f1 * c[0][e] + c[3][e]);
+                t1 = m * (f1 * c[1][e] + c[4][e]);
+                t2 = m * (f1 * c[2][e] + c[5][e]);
+            } else {
+                t0 = f1 * c[0][e] + f2 * c[5][e] + f3 * c[4][e];
+                t1 = f1 * c[5][e] + f2 * c[1][e] + f3 * c[3][e];
+                t2 = f1 * c[4][e] + f2 * c[3][e] + f3 * c[2][e];
+                const cplx<T> h = (T(-0.5) * iq) * (f1 * t0 + f2 * t1 + f3 * t2);
+                t0 = m * (t0 + f1 * h);
+                t1 = m * (t1 + f2 * h);
+                t2 = m * (t2 + f3 * h);
+            }
             z[0][e] = MODE == X1F_CG ? z[0][e] + t0 : t0;
             z[1][e] = MODE == X1F_CG ? z[1][e] + t1 : t1;
             z[2][e] = MODE == X1F_CG ? z[2][e] + t2 : t2;
-            const cplx<T> fr = f1 * z[0][e] + f2 * z[1][e] + f3 * z[2][e];
+            const cplx<T> fr = FS ? mk(T(0), T(0)) : f1 * z[0][e] + f2 * z[1][e] + f3 * z[2][e];
             const T s = z[0][e].x * z[0][e].x + z[0][e].y * z[0][e].y + z[1][e].x * z[1][e].x +
                         z[1][e].y * z[1][e].y + z[2][e].x * z[2][e].x + z[2][e].y * z[2][e].y;
             // f3 > 0 stands for -f3 too; the column past an odd H is padding
@@ -303,7 +330,7 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
 #pragma unroll
         for (int i = 0; i < 3; ++i) st_pair(r + o + i * N * W, z[i]);
     }
-    const double s = block_sum_any((double)acc) * CoefScale<N>::square;
+    const double s = block_sum_any((double)acc) * (FS ? 0.5 : 1.0) * CoefScale<N>::square;
     if (tid == 0) {
         const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
         if (MODE == X1F_CG) {
@@ -336,7 +363,7 @@ __device__ __forceinline__ cplx<dd> dd_scale(cplx<dd> a, float f) {
 // double-float spectrum of the FP64 stress: forward x1 in two stages, then
 // one thread per frequency. The double-float inverse passes that a residual
 // in real space needs (half of its work) are not run.
-template <int N>
+template <int N, bool FS = false>
 __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
     using T = dd;
     using C = Cfg<N, T>;
@@ -358,7 +385,8 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
     for (int it = tid; it < P * N2; it += NT) {
         const int pc = it % P, t = it / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
-        if (col < H) fwdA<N, N1, T>(sp + c * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
+        const int comp = FS ? fs_slot(c) : c;
+        if (col < H) fwdA<N, N1, T>(sp + comp * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
     __syncthreads();
     if (N2 > 1) {
@@ -384,17 +412,22 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) c[k] = b[k * N * W];
         cplx<T> t[3];
-        t[0] = dd_scale(c[0], f1) + dd_scale(c[5], f2) + dd_scale(c[4], f3);
-        t[1] = dd_scale(c[5], f1) + dd_scale(c[1], f2) + dd_scale(c[3], f3);
-        t[2] = dd_scale(c[4], f1) + dd_scale(c[3], f2) + dd_scale(c[2], f3);
         const float q = f1 * f1 + f2 * f2 + f3 * f3;  // an integer below 2^24: exact
         const dd iq = q > 0.0f ? dd_recip(q) : dd(0.0f, 0.0f);
-        const cplx<T> h = signed_by<-1>(
-            half_of(iq * (dd_scale(t[0], f1) + dd_scale(t[1], f2) + dd_scale(t[2], f3))));
         const dd m = scale * iq;
-        t[0] = m * (t[0] + dd_scale(h, f1));
-        t[1] = m * (t[1] + dd_scale(h, f2));
-        t[2] = m * (t[2] + dd_scale(h, f3));
+        if (FS) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) t[i] = m * (dd_scale(c[i], f1) + c[3 + i]);
+        } else {
+            t[0] = dd_scale(c[0], f1) + dd_scale(c[5], f2) + dd_scale(c[4], f3);
+            t[1] = dd_scale(c[5], f1) + dd_scale(c[1], f2) + dd_scale(c[3], f3);
+            t[2] = dd_scale(c[4], f1) + dd_scale(c[3], f2) + dd_scale(c[2], f3);
+            const cplx<T> h = signed_by<-1>(
+                half_of(iq * (dd_scale(t[0], f1) + dd_scale(t[1], f2) + dd_scale(t[2], f3))));
+            t[0] = m * (t[0] + dd_scale(h, f1));
+            t[1] = m * (t[1] + dd_scale(h, f2));
+            t[2] = m * (t[2] + dd_scale(h, f3));
+        }
         const float wt = col == 0 ? 1.0f : 2.0f;  // f3 > 0 stands for -f3 too
         constexpr int WX = X1<N>::W;
         const long long o = coef_tile<N>(col / WX, k2g) + kk * WX + col % WX;
@@ -412,11 +445,17 @@ __global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
             s1 += t[i].x * t[i].x + t[i].y * t[i].y;
             ft = ft + dd_scale(t[i], fi);
         }
-        acc0 += wt * (q * s0 + fr.x * fr.x + fr.y * fr.y);
-        acc1 += dd_scale(dd_scale(s1, q) + ft.x * ft.x + ft.y * ft.y, wt);
+        if (FS) {
+            acc0 += wt * q * s0;
+            acc1 += dd_scale(dd_scale(s1, q), wt);
+        } else {
+            acc0 += wt * (q * s0 + fr.x * fr.x + fr.y * fr.y);
+            acc1 += dd_scale(dd_scale(s1, q) + ft.x * ft.x + ft.y * ft.y, wt);
+        }
     }
-    const double s0 = block_sum_any((double)acc0) * CoefScale<N>::square;
-    const double s1 = block_sum_any((double)acc1) * CoefScale<N>::square;
+    const double square = (FS ? 0.5 : 1.0) * CoefScale<N>::square;
+    const double s0 = block_sum_any((double)acc0) * square;
+    const double s1 = block_sum_any((double)acc1) * square;
     if (tid == 0) {
         const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
         a.partials[2 * (f * nb + b)] = s0;

@@ -15,7 +15,7 @@
 #include <vector>
 
 #include "../../include/fftg_fs.h"
-#include "fs_passes.cuh"
+#include "fs_cg_passes.cuh"
 #include "host_common.h"
 
 namespace fftg {
@@ -52,6 +52,20 @@ int fs_row_blocks(int N, bool fp64) {
         FFTG_FS_GRIDS(FFTG_CASE)
 #undef FFTG_CASE
         default: return 0;
+    }
+}
+
+// Blocks of the coefficient passes whose partial sums a kernel reduces.
+struct FsBlocks {
+    int rows, x1, x1_dd;
+};
+static FsBlocks fs_blocks(int N) {
+    switch (N) {
+#define FFTG_CASE(n) \
+    case n: return {FsRowCfg<n>::blocks, X1<n>::blocks, (Cfg<n, dd>::H + Cfg<n, dd>::W3 - 1) / Cfg<n, dd>::W3 * n};
+        FFTG_FS_GRIDS(FFTG_CASE)
+#undef FFTG_CASE
+        default: return {0, 0, 0};
     }
 }
 
@@ -245,6 +259,12 @@ __global__ void __launch_bounds__(kThreads) k_fs_newton_update(FsPointArgs a) {
     if (threadIdx.x == 0) a.dev->de2 = tot[0];
 }
 
+// dev->de2 = ||x||^2 from the block partials of FS_P5_NEWTON.
+static __global__ void __launch_bounds__(1024) k_fs_newton_norm(const double* partials, int nb, FsDev* dev) {
+    const double t = sum_partials(partials, nb, 1);
+    if (threadIdx.x == 0) dev->de2 = t;
+}
+
 // Macroscopic tangent, column `unit`: ||K : E_unit||^2 summed over voxels
 // gives the CG roundoff floor of the right-hand side -G (K : E_unit).
 template <typename T>
@@ -307,13 +327,22 @@ __global__ void __launch_bounds__(kThreads) k_fs_tangent_average(FsPointArgs a) 
 }
 
 // Loop condition of the device-resident CG graph; stops after `cap` passes
-// whatever the solve reports.
-__global__ void k_fs_cg_continue(cudaGraphConditionalHandle cond, const CGState* cg, unsigned int* guard,
-                                 unsigned int cap) {
-    if (threadIdx.x != 0) return;
+// whatever the solve reports. The mixed path's last kernel sets it itself.
+__device__ __forceinline__ void fs_cg_continue(cudaGraphConditionalHandle cond, const CGState* cg,
+                                               unsigned int* guard, unsigned int cap) {
     bool run = cg->done == CG_RUNNING;
     if (++(*guard) >= cap) run = false;
     cudaGraphSetConditional(cond, run ? 1u : 0u);
+}
+__global__ void k_fs_cg_continue(cudaGraphConditionalHandle cond, const CGState* cg, unsigned int* guard,
+                                 unsigned int cap) {
+    if (threadIdx.x == 0) fs_cg_continue(cond, cg, guard, cap);
+}
+__global__ void __launch_bounds__(1024) k_fs_cg_rr_loop(const double* partials, int nb, CGState* cg,
+                                                        cudaGraphConditionalHandle cond, unsigned int* guard,
+                                                        unsigned int cap) {
+    cg_rr_block(partials, nb, cg);
+    if (threadIdx.x == 0) fs_cg_continue(cond, cg, guard, cap);
 }
 
 }  // namespace fftg
@@ -323,20 +352,21 @@ using namespace fftg;
 namespace {
 
 enum : int {
-    FSK_CONSTITUTIVE_F32 = FK_COUNT, FSK_CONSTITUTIVE_F64, FSK_CG_UPDATE_F32, FSK_CG_UPDATE_F64,
-    FSK_CG_FINISH_F32, FSK_CG_FINISH_F64, FSK_NEWTON_UPDATE_F32, FSK_NEWTON_UPDATE_F64, FSK_TANGENT_FLOOR,
-    FSK_TANGENT_AVERAGE, FSK_CG_RR, FSK_COUNT
+    FSK_CONSTITUTIVE_F32 = FK_COUNT, FSK_CONSTITUTIVE_F64, FSK_CG_UPDATE_F64, FSK_CG_FINISH_F64,
+    FSK_NEWTON_UPDATE_F64, FSK_NEWTON_NORM_F32, FSK_TANGENT_FLOOR, FSK_TANGENT_AVERAGE, FSK_CG_BEGIN, FSK_CG_RR,
+    FSK_COUNT
 };
 const char* const kFsKindNames[FSK_COUNT] = {
-    "fs_p1_plain_f64", "fs_p1_plain_f32", "fs_p1_tan_f64", "fs_p1_tan_f32", "fs_p1_cg_f64", "fs_p1_cg_f32",
+    "fs_p1_plain_f64", "fs_p1_plain_f32", "fs_p1_tan_f64", "fs_p1_tan_f32", "fs_p1_cg_f64",
     "fs_p2_f64", "fs_p2_f32", "fs_p3_f64", "fs_p3_f32", "fs_p4_f64", "fs_p4_f32",
     "fs_p5_plain_f64", "fs_p5_plain_f32", "fs_p5_dot_f64", "fs_p5_dot_f32",
-    "fs_p5_rhs_f64_to_f64", "fs_p5_rhs_f64_to_f32", "fs_p1_plain_dd", "fs_p2_dd", "fs_p3_dd", "fs_p4_dd",
-    "fs_p5_rhs_dd_to_f32", "fs_p5_plain_dd_to_f64", "fs_p1_tanrhs_f64", "fs_p1_tanrhs_f32",
-    "fs_p5_rhs_f32_to_f32", "fs_p1_cgf_f32", "fs_p5_cgf_f32",
-    "fs_constitutive_f32", "fs_constitutive_f64", "fs_cg_update_f32", "fs_cg_update_f64",
-    "fs_cg_finish_f32", "fs_cg_finish_f64", "fs_newton_update_f32", "fs_newton_update_f64",
-    "fs_tangent_floor", "fs_tangent_average", "fs_cg_rr_f32"};
+    "fs_p5_rhs_f64_to_f64", "fs_p1_plain_dd", "fs_p2_dd", "fs_p3_dd", "fs_p4_dd",
+    "fs_p5_plain_dd_to_f64", "fs_p1_tanrhs_f64", "fs_p1_tanrhs_f32",
+    "fs_x1i_cg_f32", "fs_p4_grad_f32", "fs_rows_cg_f32", "fs_p2_grad_f32", "fs_x1f_cg_f32", "fs_p2_grad_dd",
+    "fs_x1f_rhs_f32", "fs_x1f_rhs_dd", "fs_x1i_solution_f32", "fs_p5_newton_f32",
+    "fs_constitutive_f32", "fs_constitutive_f64", "fs_cg_update_f64", "fs_cg_finish_f64",
+    "fs_newton_update_f64", "fs_newton_norm_f32", "fs_tangent_floor", "fs_tangent_average", "fs_cg_begin_f32",
+    "fs_cg_rr_f32"};
 
 // Iterations without a new minimum of <r, r> after which an FP32 inner
 // solve counts as stagnated (as in the small-strain driver).
@@ -352,7 +382,8 @@ struct FsLayout {
 FsLayout fs_layout(int N, bool mixed) {
     const size_t cs = (size_t)comp_stride(N), HP = (size_t)spec_pitch(N);
     const size_t ts = mixed ? 4 : 8;
-    const size_t rb = (size_t)std::max(fs_row_blocks(N, true), fs_row_blocks(N, false));
+    const FsBlocks fb = fs_blocks(N);
+    const size_t rb = (size_t)std::max({fs_row_blocks(N, true), fs_row_blocks(N, false), fb.rows, fb.x1, fb.x1_dd});
     const size_t npart = std::max((size_t)kFsPointBlocks * 10, rb * 2);
     FsLayout L{};
     size_t o = 0;
@@ -367,9 +398,11 @@ FsLayout fs_layout(int N, bool mixed) {
     L.off_Fwork = take(9 * cs * 8);
     L.off_P = take(9 * cs * 8);
     L.off_hgrad = take(9 * cs * ts);
-    L.off_x = take(9 * cs * ts);
-    L.off_r = take(9 * cs * ts);
-    L.off_p = take(9 * cs * ts);
+    // mixed: fields of coefficients; x also stages FP32 fields
+    const size_t vec = std::max(9 * cs * ts, mixed ? (size_t)coef_elements(N) * 8 : 0);
+    L.off_x = take(vec);
+    L.off_r = take(vec);
+    L.off_p = take(vec);
     L.off_q = take(9 * cs * ts);
     L.off_spec = take(9 * (size_t)N * N * HP * 16);  // FP64 complex: the residual's size
     L.off_tw32 = take((size_t)N * 8);
@@ -491,12 +524,6 @@ cudaError_t fs_pass(fftg_fs_handle* h, FsPassKind kind, const FsArgs& a) {
 // FFT precision of a pass sequence
 enum : int { FFT_F32 = 0, FFT_F64 = 1, FFT_DD = 2 };
 
-// The mixed path's residual G P uses double-float FFTs of the FP64 stress
-// (as the small-strain driver does); 0: FP64 FFTs.
-#ifndef FFTG_RESIDUAL_DD
-#define FFTG_RESIDUAL_DD 1
-#endif
-
 FsArgs fs_args(fftg_fs_handle* h, int prec) {
     FsArgs a{};
     a.tw = prec == FFT_DD ? h->twdd : prec == FFT_F64 ? h->tw64 : h->tw32;
@@ -531,15 +558,11 @@ FsPointArgs point_args(fftg_fs_handle* h) {
 }
 
 // Spectrum passes P2, P3 (scale on Ghat), P4.
-int fs_p234(fftg_fs_handle* h, int prec, double scale, CGState* cg, const double* red_in = nullptr,
-            int red_n = 0) {
+int fs_p234(fftg_fs_handle* h, int prec, double scale, CGState* cg) {
     FsArgs a = fs_args(h, prec);
     a.cg = cg;
     a.scale = scale;
-    a.red_in = red_in;
-    a.red_n = red_n;
     CK(fs_pass(h, prec == FFT_DD ? FK_P2_DD : prec == FFT_F64 ? FK_P2_F64 : FK_P2_F32, a));
-    a.red_in = nullptr;
     CK(fs_pass(h, prec == FFT_DD ? FK_P3_DD : prec == FFT_F64 ? FK_P3_F64 : FK_P3_F32, a));
     CK(fs_pass(h, prec == FFT_DD ? FK_P4_DD : prec == FFT_F64 ? FK_P4_F64 : FK_P4_F32, a));
     return FFTG_OK;
@@ -562,59 +585,85 @@ int fs_constitutive(fftg_fs_handle* h, const double* F, bool write_h, CGState* c
     return FFTG_OK;
 }
 
-// r = -G P (FP64 FFTs, or double-float ones in the mixed path) rounded to
-// the inner precision, CG start; x = 0.
-int fs_residual(fftg_fs_handle* h) {
-    const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
-    const int prec = (h->mixed && FFTG_RESIDUAL_DD) ? FFT_DD : FFT_F64;
+// Forward x2 and x1 of the right-hand side's spectrum to coefficients r (times
+// scale), and the start of the solve.
+int fs_rhs(fftg_fs_handle* h, int prec, double scale) {
     FsArgs a = fs_args(h, prec);
-    a.in = h->P;
-    CK(fs_pass(h, prec == FFT_DD ? FK_P1_PLAIN_DD : FK_P1_PLAIN_F64, a));
-    int rc = fs_p234(h, prec, -invN3, nullptr);
-    if (rc) return rc;
-    FsArgs b = fs_args(h, prec);
-    b.in = h->spec;
-    b.out = h->r;
-    b.cg = h->cg;
-    CK(fs_pass(h, prec == FFT_DD ? FK_P5_RHS_DD_TO_F32 : h->mixed ? FK_P5_RHS_F64_TO_F32 : FK_P5_RHS_F64_TO_F64, b));
-    CK(cudaMemsetAsync(h->x, 0, 9 * h->cs * (h->mixed ? 4 : 8), h->stream));
+    CK(fs_pass(h, prec == FFT_DD ? FK_P2_GRAD_DD : FK_P2_GRAD_F32, a));
+    a.in = h->spec;
+    a.aux3 = h->r;
+    a.cg = h->cg;
+    a.scale = scale;
+    CK(fs_pass(h, prec == FFT_DD ? FK_X1F_RHS_DD : FK_X1F_RHS_F32, a));
+    const FsBlocks nb = fs_blocks(h->N);
+    const int slot = fs_prof_begin(h, FSK_CG_BEGIN);
+    k_cg_begin<<<1, 1024, 0, h->stream>>>(h->partials, prec == FFT_DD ? nb.x1_dd : nb.x1, h->cg, nullptr);
+    fs_prof_end(h, slot);
+    CK(cudaGetLastError());
     return FFTG_OK;
 }
 
-// The mixed path's CG runs without the update pass: alpha from <p, K : p>
-// in P1, r -= alpha q in P5 (fs_passes.cuh, FS_P1_CGF). 0: P1 / P5 with
-// <p, q> and the update pass, as in the FP64 path.
-#ifndef FFTG_FS_CG_FUSED
-#define FFTG_FS_CG_FUSED 1
-#endif
-bool fs_cg_fused(const fftg_fs_handle* h) { return FFTG_FS_CG_FUSED && h->mixed; }
+// r = -G P and the CG start. FP64: the five passes, x = 0. Mixed: double-float
+// FFTs of the FP64 stress up to the coefficients, rounded to FP32.
+int fs_residual(fftg_fs_handle* h) {
+    const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
+    const int prec = h->mixed ? FFT_DD : FFT_F64;
+    FsArgs a = fs_args(h, prec);
+    a.in = h->P;
+    CK(fs_pass(h, prec == FFT_DD ? FK_P1_PLAIN_DD : FK_P1_PLAIN_F64, a));
+    if (h->mixed) return fs_rhs(h, FFT_DD, -invN3);
+    int rc = fs_p234(h, FFT_F64, -invN3, nullptr);
+    if (rc) return rc;
+    FsArgs b = fs_args(h, FFT_F64);
+    b.in = h->spec;
+    b.out = h->r;
+    b.cg = h->cg;
+    CK(fs_pass(h, FK_P5_RHS_F64_TO_F64, b));
+    CK(cudaMemsetAsync(h->x, 0, 9 * h->cs * 8, h->stream));
+    return FFTG_OK;
+}
 
-// One CG iteration: P1 (x, p updates and K : p), P2-P4, P5 (q, <p, q>),
-// then r -= alpha q; in the mixed path P1 (with <p, K : p>), P2-P4 and P5
-// (r -= alpha q, <r, r>).
-int fs_cg_iteration(fftg_fs_handle* h) {
+// The loop that an iteration is captured into (cond set: the iteration's last
+// kernel sets the loop's condition).
+struct FsLoop {
+    cudaGraphConditionalHandle cond = 0;
+    bool on = false;
+    unsigned int cap = 0;
+};
+
+// One CG iteration. Mixed: on coefficients (fs_cg_passes.cuh). FP64: P1 (x, p
+// updates and K : p), P2-P4, P5 (q, <p, q>), then r -= alpha q.
+int fs_cg_iteration(fftg_fs_handle* h, const FsLoop& loop = FsLoop{}) {
     const bool f64 = !h->mixed;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     const int prec = f64 ? FFT_F64 : FFT_F32;
-    if (fs_cg_fused(h)) {
+    if (h->mixed) {
+        const FsBlocks nb = fs_blocks(h->N);
         FsArgs a = fs_args(h, FFT_F32);
         a.aux = h->r;
         a.aux2 = h->p;
         a.aux3 = h->x;
         a.cg = h->cg;
-        CK(fs_pass(h, FK_P1_CGF_F32, a));
-        // P2 reduces P1's block partials of <p, K : p> (alpha)
-        int rc = fs_p234(h, FFT_F32, invN3, h->cg, h->partials, fs_row_blocks(h->N, false));
-        if (rc) return rc;
-        FsArgs b = fs_args(h, FFT_F32);
-        b.in = h->spec;
-        b.aux = h->r;
-        b.aux3 = h->r;
-        b.cg = h->cg;
-        CK(fs_pass(h, FK_P5_CGF_F32, b));
-        // <r, r> from P5's block partials: beta and the stopping tests
+        CK(fs_pass(h, FK_X1I_CG_F32, a));
+        CK(fs_pass(h, FK_P4_GRAD_F32, a));
+        CK(fs_pass(h, FK_ROWS_CG_F32, a));
+        // P2 reduces the row pass's block partials of <p, K : p> (alpha)
+        FsArgs b = a;
+        b.red_in = h->partials;
+        b.red_n = nb.rows;
+        CK(fs_pass(h, FK_P2_GRAD_F32, b));
+        FsArgs c = fs_args(h, FFT_F32);
+        c.in = h->spec;
+        c.aux3 = h->r;
+        c.cg = h->cg;
+        c.scale = invN3;
+        CK(fs_pass(h, FK_X1F_CG_F32, c));
+        // <r, r> from its block partials: beta and the stopping tests
         const int slot = fs_prof_begin(h, FSK_CG_RR);
-        k_cg_rr<<<1, 1024, 0, h->stream>>>(h->partials, fs_row_blocks(h->N, false), h->cg);
+        if (loop.on)
+            k_fs_cg_rr_loop<<<1, 1024, 0, h->stream>>>(h->partials, nb.x1, h->cg, loop.cond, h->guard, loop.cap);
+        else
+            k_cg_rr<<<1, 1024, 0, h->stream>>>(h->partials, nb.x1, h->cg);
         fs_prof_end(h, slot);
         CK(cudaGetLastError());
         return FFTG_OK;
@@ -624,7 +673,7 @@ int fs_cg_iteration(fftg_fs_handle* h) {
     a.aux2 = h->p;
     a.aux3 = h->x;
     a.cg = h->cg;
-    CK(fs_pass(h, f64 ? FK_P1_CG_F64 : FK_P1_CG_F32, a));
+    CK(fs_pass(h, FK_P1_CG_F64, a));
     int rc = fs_p234(h, prec, invN3, h->cg);
     if (rc) return rc;
     FsArgs b = fs_args(h, prec);
@@ -632,25 +681,25 @@ int fs_cg_iteration(fftg_fs_handle* h) {
     b.out = h->q;
     b.aux = h->p;
     b.cg = h->cg;
-    CK(fs_pass(h, f64 ? FK_P5_DOT_F64 : FK_P5_DOT_F32, b));
+    CK(fs_pass(h, FK_P5_DOT_F64, b));
     FsPointArgs u = point_args(h);
-    const int slot = fs_prof_begin(h, f64 ? FSK_CG_UPDATE_F64 : FSK_CG_UPDATE_F32);
-    if (f64)
-        k_fs_cg_update<double><<<fs_vector_blocks(h->cs, 8), kThreads, 0, h->stream>>>(u);
-    else
-        k_fs_cg_update<float><<<fs_vector_blocks(h->cs, 4), kThreads, 0, h->stream>>>(u);
+    const int slot = fs_prof_begin(h, FSK_CG_UPDATE_F64);
+    k_fs_cg_update<double><<<fs_vector_blocks(h->cs, 8), kThreads, 0, h->stream>>>(u);
     fs_prof_end(h, slot);
     CK(cudaGetLastError());
+    if (loop.on) {
+        k_fs_cg_continue<<<1, 32, 0, h->stream>>>(loop.cond, h->cg, h->guard, loop.cap);
+        CK(cudaGetLastError());
+    }
     return FFTG_OK;
 }
 
+// FP64 path: x += alpha p where the last update left the step pending.
 int fs_cg_finish(fftg_fs_handle* h) {
+    if (h->mixed) return FFTG_OK;
     FsPointArgs u = point_args(h);
-    const int slot = fs_prof_begin(h, h->mixed ? FSK_CG_FINISH_F32 : FSK_CG_FINISH_F64);
-    if (h->mixed)
-        k_fs_cg_finish<float><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
-    else
-        k_fs_cg_finish<double><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
+    const int slot = fs_prof_begin(h, FSK_CG_FINISH_F64);
+    k_fs_cg_finish<double><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
     fs_prof_end(h, slot);
     CK(cudaGetLastError());
     return FFTG_OK;
@@ -683,12 +732,8 @@ int fs_build_graph(fftg_fs_handle* h) {
         cudaSuccess)
         return FFTG_ECUDA;
     const long long before = h->launches;
-    int rc = fs_cg_iteration(h);
     const unsigned int cap = (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
-    if (rc == FFTG_OK) {
-        k_fs_cg_continue<<<1, 32, 0, h->stream>>>(cond, h->cg, h->guard, cap);
-        if (cudaGetLastError() != cudaSuccess) rc = FFTG_ECUDA;
-    }
+    const int rc = fs_cg_iteration(h, FsLoop{cond, true, cap});
     h->launches = before;  // capture enqueues nothing
     cudaGraph_t captured = nullptr;
     if (cudaStreamEndCapture(h->stream, &captured) != cudaSuccess || rc) return FFTG_ECUDA;
@@ -718,7 +763,7 @@ int fs_run_cg(fftg_fs_handle* h) {
             if (rc) return rc;
             CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
             CK(cudaStreamSynchronize(h->stream));
-            h->launches += 7LL * (h->h_cg->it + 1);  // one of each per loop pass
+            h->launches += (h->mixed ? 6LL : 7LL) * (h->h_cg->it + 1);  // one of each per loop pass
             return FFTG_OK;
         }
     }
@@ -740,20 +785,42 @@ int fs_run_cg(fftg_fs_handle* h) {
     return fs_cg_finish(h);
 }
 
-// Mixed precision: x <- G x in FP32 after each solve (the FP32 recursion
-// lets x drift out of the compatible space; see the small-strain driver).
-int fs_project_solution(fftg_fs_handle* h) {
-    if (!h->mixed) return FFTG_OK;
-    const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
+// Mixed path: the solution x (with its pending step) from coefficients to real
+// space, a gradient field up to the rounding of one FP32 inverse transform.
+// newton: added to F* during the increment, with ||x||^2; else written to q.
+int fs_solution(fftg_fs_handle* h, bool newton) {
     FsArgs a = fs_args(h, FFT_F32);
-    a.in = h->x;
-    CK(fs_pass(h, FK_P1_PLAIN_F32, a));
-    int rc = fs_p234(h, FFT_F32, invN3, nullptr);
-    if (rc) return rc;
+    a.aux2 = h->p;
+    a.aux3 = h->x;
+    a.cg = h->cg;
+    CK(fs_pass(h, FK_X1I_SOLUTION_F32, a));
     FsArgs b = fs_args(h, FFT_F32);
-    b.in = h->spec;
-    b.out = h->x;
-    CK(fs_pass(h, FK_P5_PLAIN_F32, b));
+    CK(fs_pass(h, FK_P4_GRAD_F32, b));
+    FsArgs c = fs_args(h, FFT_F32);
+    c.in = h->spec;
+    c.out = h->q;
+    if (!newton) {
+        CK(fs_pass(h, FK_P5_PLAIN_F32, c));
+        return FFTG_OK;
+    }
+    c.aux3 = h->Fwork;
+    CK(fs_pass(h, FK_P5_NEWTON_F32, c));
+    const int slot = fs_prof_begin(h, FSK_NEWTON_NORM_F32);
+    k_fs_newton_norm<<<1, 1024, 0, h->stream>>>(h->partials, fs_row_blocks(h->N, false), h->dev);
+    fs_prof_end(h, slot);
+    CK(cudaGetLastError());
+    return FFTG_OK;
+}
+
+// F* += x (Algorithm 1's update) with ||x||^2.
+int fs_newton_update(fftg_fs_handle* h) {
+    if (h->mixed) return fs_solution(h, true);
+    FsPointArgs u = point_args(h);
+    u.Fw = h->Fwork;
+    const int slot = fs_prof_begin(h, FSK_NEWTON_UPDATE_F64);
+    k_fs_newton_update<double><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
+    fs_prof_end(h, slot);
+    CK(cudaGetLastError());
     return FFTG_OK;
 }
 
@@ -920,17 +987,8 @@ int fftg_fs_step(fftg_fs_handle* h, const double dF[9], double tol_newton, doubl
         fs_set_cg(h, tol_inner);
         CK(cudaMemcpyAsync(h->cg, h->h_cg, sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
         if ((rc = fs_constitutive(h, h->Fwork, true, h->cg)) || (rc = fs_residual(h)) || (rc = fs_run_cg(h)) ||
-            (rc = fs_project_solution(h)))
+            (rc = fs_newton_update(h)))
             break;
-        FsPointArgs u = point_args(h);
-        u.Fw = h->Fwork;
-        const int slot = fs_prof_begin(h, h->mixed ? FSK_NEWTON_UPDATE_F32 : FSK_NEWTON_UPDATE_F64);
-        if (h->mixed)
-            k_fs_newton_update<float><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
-        else
-            k_fs_newton_update<double><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
-        fs_prof_end(h, slot);
-        CK(cudaGetLastError());
         CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaMemcpyAsync(h->h_dev, h->dev, sizeof(FsDev), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
@@ -1007,18 +1065,23 @@ int fftg_fs_tangent(fftg_fs_handle* h, double tol_cg, double C_out[81], int* cg_
             k_fs_tangent_floor<float><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);
         fs_prof_end(h, slot);
         CK(cudaGetLastError());
-        // r = -G (K : E_unit) in the inner precision; CG start; x = 0
+        // r = -G (K : E_unit) in the inner precision; CG start
         FsArgs a = fs_args(h, prec);
         a.unit = unit;
         CK(fs_pass(h, f64 ? FK_P1_TANRHS_F64 : FK_P1_TANRHS_F32, a));
-        if ((rc = fs_p234(h, prec, -invN3, nullptr))) return rc;
-        FsArgs b = fs_args(h, prec);
-        b.in = h->spec;
-        b.out = h->r;
-        b.cg = h->cg;
-        CK(fs_pass(h, f64 ? FK_P5_RHS_F64_TO_F64 : FK_P5_RHS_F32_TO_F32, b));
-        CK(cudaMemsetAsync(h->x, 0, 9 * h->cs * (f64 ? 8 : 4), h->stream));
-        if ((rc = fs_run_cg(h)) || (rc = fs_project_solution(h))) return rc;
+        if (f64) {
+            if ((rc = fs_p234(h, prec, -invN3, nullptr))) return rc;
+            FsArgs b = fs_args(h, prec);
+            b.in = h->spec;
+            b.out = h->r;
+            b.cg = h->cg;
+            CK(fs_pass(h, FK_P5_RHS_F64_TO_F64, b));
+            CK(cudaMemsetAsync(h->x, 0, 9 * h->cs * 8, h->stream));
+        } else if ((rc = fs_rhs(h, FFT_F32, -invN3))) {
+            return rc;
+        }
+        if ((rc = fs_run_cg(h)) || (!f64 && (rc = fs_solution(h, false)))) return rc;
+        if (!f64) u.x = h->q;
         if (h->h_cg->done == CG_BREAKDOWN) return FFTG_ENAN;
         total += h->h_cg->it;
         slot = fs_prof_begin(h, FSK_TANGENT_AVERAGE);

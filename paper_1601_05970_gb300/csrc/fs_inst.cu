@@ -1,6 +1,6 @@
 // Finite-strain pass kernels of one grid size, compiled once for each
 // supported N with -DFFTG_N=<N> (in parallel with the other units).
-#include "fs_passes.cuh"
+#include "fs_cg_passes.cuh"
 
 #ifndef FFTG_N
 #error "compile with -DFFTG_N=<grid size>"

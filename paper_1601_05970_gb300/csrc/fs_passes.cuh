@@ -28,19 +28,18 @@ namespace fftg {
 constexpr int kFsComp = 9;
 constexpr int kFsPairs = 5;
 
-enum : int { FS_P1_PLAIN = 0, FS_P1_TAN = 1, FS_P1_CG = 2, FS_P1_TANRHS = 3, FS_P1_CGF = 4 };
-enum : int { FS_P5_PLAIN = 0, FS_P5_DOT = 1, FS_P5_RHS = 2, FS_P5_CGF = 3 };
-// FS_P1_CGF / FS_P5_CGF: the CG iteration without the update pass, as in
-// the small-strain passes (P1_CGF): G projects orthogonally onto gradient
-// fields, so <p, G K p> = <p, K p> for a gradient field p; P1 reduces
-// <p, K : p> (alpha), P5 updates r -= alpha q and reduces <r, r>.
+enum : int { FS_P1_PLAIN = 0, FS_P1_TAN = 1, FS_P1_CG = 2, FS_P1_TANRHS = 3 };
+enum : int { FS_P5_PLAIN = 0, FS_P5_DOT = 1, FS_P5_RHS = 2, FS_P5_NEWTON = 3 };
+// FS_P5_NEWTON: F* += x for the solution x of a mixed inner solve, with its
+// squared norm. The mixed path's CG iteration is that of fs_cg_passes.cuh.
 
 struct FsArgs {
     const void* in;        // P1: real field; P5: spectrum
     void* out;             // P1: spectrum; P2-P4: spectrum (in place); P5: real field
     const void* aux;       // P1_CG: r; P5_DOT: p
     void* aux2;            // P1_CG: p (updated in place)
-    void* aux3;            // P1_CG: x (gets the previous iteration's alpha p)
+    void* aux3;            // P1_CG: x (gets the previous iteration's alpha p);
+                           // P5_NEWTON: F* (FP64, updated in place)
     const void* hgrad;     // P1_TAN, P1_CG: H = F - I, [9][cs] in the FFT precision
     const uint8_t* phase;  // [cs]
     const double* lame;    // [nphase][2]: lambda, mu
@@ -50,7 +49,7 @@ struct FsArgs {
     double scale;          // P3: factor on Ghat (+-1/N^3)
     long long cs;          // component stride of the real fields (elements)
     int unit;              // P1_TANRHS: tau = K : E_unit, E_unit the unit tensor at component unit
-    const double* red_in;  // P2 of the fused CG iteration: P1's block partials of <p, K : p>
+    const double* red_in;  // P2 of the mixed CG iteration: the row pass's block partials of <p, K : p>
     int red_n;             // (reduced by P2's first block, which sets alpha)
 };
 
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* z = tw + N;  // [5][R][N]
-    constexpr bool CGM = MODE == FS_P1_CG || MODE == FS_P1_CGF;
+    constexpr bool CGM = MODE == FS_P1_CG;
     if (CGM && a.cg->done) return;
     const int tid = threadIdx.x;
     load_tw<T>(tw, a.tw, N);
@@ -176,7 +175,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
     const int nel = nrows * N;
     const long long cs = a.cs;
     T beta = T(0), alpha = T(0);
-    T pkp = T(0);  // FS_P1_CGF: this thread's part of <p, K : p>
     bool first = true;
     if (CGM) {
         beta = (T)a.cg->beta;
@@ -268,10 +266,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
                     svk_tangent_apply<T>(he, (T)m[0], (T)m[1], pe, se);
 #pragma unroll
                     for (int c = 0; c < 9; ++c) s[c][e] = se[c];
-                    if (MODE == FS_P1_CGF && i0 + e < nel) {
-#pragma unroll
-                        for (int c = 0; c < 9; ++c) pkp += pe[c] * se[c];
-                    }
                 }
             }
         } else {
@@ -287,19 +281,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
             z[4 * R * N + i0 + e] = mk(s[8][e], T(0));
         }
     }
-    // FS_P1_CGF: this block's part of <p, K : p> (P2 reduces the parts)
-    __shared__ double pkp_warp[kThreads / 32];
-    if (MODE == FS_P1_CGF) {
-        const double wv = warp_sum((double)pkp);
-        if ((tid & 31) == 0) pkp_warp[tid >> 5] = wv;
-    }
     __syncthreads();
-    if (MODE == FS_P1_CGF && tid == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) t += pkp_warp[w];
-        a.partials[blockIdx.x] = t;
-    }
     constexpr int NP = kFsPairs * R;
     for (int it = tid; it < NP * N2; it += kThreads) {
         const int pc = it % NP, t = it / NP;
@@ -474,7 +456,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* z = tw + N;  // [5][R][N]
     CGState* cg = a.cg;
-    if ((MODE == FS_P5_DOT || MODE == FS_P5_CGF) && cg->done) return;
+    if (MODE == FS_P5_DOT && cg->done) return;
     const int tid = threadIdx.x;
     load_tw<T>(tw, a.tw, N);
     const int row0 = blockIdx.x * R;
@@ -513,8 +495,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
 #pragma unroll
                 for (int c = 0; c < kFsPairs; ++c) {
                     const cplx<T> a0 = A[u][c], b0 = B[u][c];
-                    z[(c * R + row) * N + pk] = mk(a0.x - b0.y, a0.y + b0.x);                  // A + iB
-                    if (k > 0) z[(c * R + row) * N + pn] = mk(a0.x + b0.y, b0.x - a0.y);  // conj(A) + i conj(B)
+                    // A + iB and conj(A) + i conj(B); A and B are real at k = 0
+                    // (what their imaginary parts hold is rounding)
+                    z[(c * R + row) * N + pk] = k > 0 ? mk(a0.x - b0.y, a0.y + b0.x) : mk(a0.x, b0.x);
+                    if (k > 0) z[(c * R + row) * N + pn] = mk(a0.x + b0.y, b0.x - a0.y);
                 }
             }
         }
@@ -535,9 +519,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     __syncthreads();
     const long long cs = a.cs;
     TO* out = (TO*)a.out;
-    const TO* pin = (const TO*)a.aux;   // FS_P5_DOT: p; FS_P5_CGF: r
-    TO* rout = MODE == FS_P5_CGF ? (TO*)a.aux3 : nullptr;
-    const TO alpha = MODE == FS_P5_CGF ? (TO)cg->alpha : TO(0);
+    const TO* pin = (const TO*)a.aux;  // FS_P5_DOT: p
+    double* Fw = MODE == FS_P5_NEWTON ? (double*)a.aux3 : nullptr;
+    dd accx(0.0f, 0.0f);  // FS_P5_NEWTON: squares of x, exact products summed in double-float
     T acc0 = T(0);
     double acc1 = 0.0;
     // VO voxels per lane (at most 16 bytes of TO): p is loaded before q is
@@ -549,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
         if (i0 >= nel) continue;
         const long long v0 = base + i0;
         TO pv[9][VO];
-        if (MODE == FS_P5_DOT || MODE == FS_P5_CGF) {
+        if (MODE == FS_P5_DOT) {
 #pragma unroll
             for (int c = 0; c < 9; ++c) ldv<VO, TO>(pin + c * cs + v0, pv[c]);
         }
@@ -567,19 +551,18 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
 #pragma unroll
             for (int c = 0; c < 9; ++c) q[c][e] = (TO)qd[c][e];
         }
-        if (MODE == FS_P5_CGF) {
-            // r -= alpha q, <r, r> (lanes past the grid update padding only)
+        if constexpr (MODE == FS_P5_NEWTON) {
+            double fv[9][VO];
+#pragma unroll
+            for (int c = 0; c < 9; ++c) ldv<VO, double>(Fw + c * cs + v0, fv[c]);
 #pragma unroll
             for (int c = 0; c < 9; ++c) {
 #pragma unroll
-                for (int e = 0; e < VO; ++e) pv[c][e] -= alpha * q[c][e];
-                stv<VO, TO>(rout + c * cs + v0, pv[c]);
-            }
-#pragma unroll
-            for (int e = 0; e < VO; ++e) {
-                if (i0 + e >= nel) continue;
-#pragma unroll
-                for (int c = 0; c < 9; ++c) acc0 += (T)(pv[c][e] * pv[c][e]);
+                for (int e = 0; e < VO; ++e) {
+                    fv[c][e] += (double)q[c][e];
+                    if (i0 + e < nel) accx += dd_two_prod(q[c][e], q[c][e]);
+                }
+                stv<VO, double>(Fw + c * cs + v0, fv[c]);
             }
             continue;
         }
@@ -603,12 +586,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     if (MODE == FS_P5_PLAIN) return;
     const int nb = gridDim.x;
     double part[2];
-    part[0] = block_sum((double)acc0);
-    if (MODE == FS_P5_CGF) {
-        // the block's part of <r, r> (k_cg_rr reduces the parts)
+    if (MODE == FS_P5_NEWTON) {
+        // the block's part of ||x||^2 (k_fs_newton_norm sums the parts)
+        part[0] = block_sum((double)accx);
         if (tid == 0) a.partials[blockIdx.x] = part[0];
         return;
     }
+    part[0] = block_sum((double)acc0);
     part[1] = (MODE == FS_P5_RHS) ? block_sum(acc1) : 0.0;
     if (!publish_partials<2>(part, a.partials, blockIdx.x, nb, &cg->ticket)) return;
     double tot[2];
@@ -622,16 +606,17 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
 
 // ------------------------------------------------------------------ launcher
 enum FsPassKind : int {
-    FK_P1_PLAIN_F64, FK_P1_PLAIN_F32, FK_P1_TAN_F64, FK_P1_TAN_F32, FK_P1_CG_F64, FK_P1_CG_F32,
+    FK_P1_PLAIN_F64, FK_P1_PLAIN_F32, FK_P1_TAN_F64, FK_P1_TAN_F32, FK_P1_CG_F64,
     FK_P2_F64, FK_P2_F32, FK_P3_F64, FK_P3_F32, FK_P4_F64, FK_P4_F32,
     FK_P5_PLAIN_F64, FK_P5_PLAIN_F32, FK_P5_DOT_F64, FK_P5_DOT_F32,
-    FK_P5_RHS_F64_TO_F64, FK_P5_RHS_F64_TO_F32,
-    // double-float FFTs (the mixed path's residual)
-    FK_P1_PLAIN_DD, FK_P2_DD, FK_P3_DD, FK_P4_DD, FK_P5_RHS_DD_TO_F32, FK_P5_PLAIN_DD_TO_F64,
+    FK_P5_RHS_F64_TO_F64,
+    // double-float FFTs: FP64 field in and out
+    FK_P1_PLAIN_DD, FK_P2_DD, FK_P3_DD, FK_P4_DD, FK_P5_PLAIN_DD_TO_F64,
     // right-hand sides of the macroscopic tangent
-    FK_P1_TANRHS_F64, FK_P1_TANRHS_F32, FK_P5_RHS_F32_TO_F32,
-    // the CG iteration without the update pass (FS_P1_CGF / FS_P5_CGF), FP32
-    FK_P1_CGF_F32, FK_P5_CGF_F32,
+    FK_P1_TANRHS_F64, FK_P1_TANRHS_F32,
+    // the mixed path's CG on coefficients (fs_cg_passes.cuh)
+    FK_X1I_CG_F32, FK_P4_GRAD_F32, FK_ROWS_CG_F32, FK_P2_GRAD_F32, FK_X1F_CG_F32, FK_P2_GRAD_DD,
+    FK_X1F_RHS_F32, FK_X1F_RHS_DD, FK_X1I_SOLUTION_F32, FK_P5_NEWTON_F32,
     FK_COUNT
 };
 
@@ -667,54 +652,6 @@ static cudaError_t launch_fs_p24(const FsArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     k_p24<N, T, FWD, kFsComp><<<g, C::T2, C::smem_p24, s>>>(b);
     return cudaGetLastError();
-}
-
-template <int N>
-cudaError_t run_fs_pass_n(FsPassKind kind, const FsArgs& a, cudaStream_t s) {
-    using C32 = FsCfg<N, float>;
-    using C64 = FsCfg<N, double>;
-    using CDD = FsCfg<N, dd>;
-    static_assert(CDD::row_blocks == C64::row_blocks && CDD::W3 == C64::W3,
-                  "double-float passes share the FP64 geometry");
-    const dim3 r32(C32::row_blocks), r64(C64::row_blocks);
-    const dim3 g32((C32::H + C32::W3 - 1) / C32::W3, N), g64((C64::H + C64::W3 - 1) / C64::W3, N);
-    const size_t m32 = C32::smem_rows, m64 = C64::smem_rows;
-    switch (kind) {
-        case FK_P1_PLAIN_F64: return launch_fs(k_fs_p1<N, double, FS_P1_PLAIN>, r64, kThreads, m64, a, s);
-        case FK_P1_PLAIN_F32: return launch_fs(k_fs_p1<N, float, FS_P1_PLAIN>, r32, kThreads, m32, a, s);
-        case FK_P1_TAN_F64: return launch_fs(k_fs_p1<N, double, FS_P1_TAN>, r64, kThreads, m64, a, s);
-        case FK_P1_TAN_F32: return launch_fs(k_fs_p1<N, float, FS_P1_TAN>, r32, kThreads, m32, a, s);
-        case FK_P1_CG_F64: return launch_fs(k_fs_p1<N, double, FS_P1_CG>, r64, kThreads, m64, a, s);
-        case FK_P1_CG_F32: return launch_fs(k_fs_p1<N, float, FS_P1_CG>, r32, kThreads, m32, a, s);
-        case FK_P2_F64: return launch_fs_p24<N, double, true>(a, s);
-        case FK_P2_F32: return launch_fs_p24<N, float, true>(a, s);
-        case FK_P4_F64: return launch_fs_p24<N, double, false>(a, s);
-        case FK_P4_F32: return launch_fs_p24<N, float, false>(a, s);
-        case FK_P3_F64: return launch_fs(k_fs_p3<N, double>, g64, C64::T3, C64::smem_p3, a, s);
-        case FK_P3_F32: return launch_fs(k_fs_p3<N, float>, g32, C32::T3, C32::smem_p3, a, s);
-        case FK_P5_PLAIN_F64: return launch_fs(k_fs_p5<N, double, FS_P5_PLAIN, double>, r64, kThreads, m64, a, s);
-        case FK_P5_PLAIN_F32: return launch_fs(k_fs_p5<N, float, FS_P5_PLAIN, float>, r32, kThreads, m32, a, s);
-        case FK_P5_DOT_F64: return launch_fs(k_fs_p5<N, double, FS_P5_DOT, double>, r64, kThreads, m64, a, s);
-        case FK_P5_DOT_F32: return launch_fs(k_fs_p5<N, float, FS_P5_DOT, float>, r32, kThreads, m32, a, s);
-        case FK_P5_RHS_F64_TO_F64:
-            return launch_fs(k_fs_p5<N, double, FS_P5_RHS, double>, r64, kThreads, m64, a, s);
-        case FK_P5_RHS_F64_TO_F32:
-            return launch_fs(k_fs_p5<N, double, FS_P5_RHS, float>, r64, kThreads, m64, a, s);
-        case FK_P1_PLAIN_DD: return launch_fs(k_fs_p1<N, dd, FS_P1_PLAIN>, r64, kThreads, m64, a, s);
-        case FK_P2_DD: return launch_fs_p24<N, dd, true>(a, s);
-        case FK_P4_DD: return launch_fs_p24<N, dd, false>(a, s);
-        case FK_P3_DD: return launch_fs(k_fs_p3<N, dd>, g64, CDD::T3, CDD::smem_p3, a, s);
-        case FK_P5_RHS_DD_TO_F32: return launch_fs(k_fs_p5<N, dd, FS_P5_RHS, float>, r64, kThreads, m64, a, s);
-        case FK_P5_PLAIN_DD_TO_F64:
-            return launch_fs(k_fs_p5<N, dd, FS_P5_PLAIN, double>, r64, kThreads, m64, a, s);
-        case FK_P1_TANRHS_F64: return launch_fs(k_fs_p1<N, double, FS_P1_TANRHS>, r64, kThreads, m64, a, s);
-        case FK_P1_TANRHS_F32: return launch_fs(k_fs_p1<N, float, FS_P1_TANRHS>, r32, kThreads, m32, a, s);
-        case FK_P5_RHS_F32_TO_F32:
-            return launch_fs(k_fs_p5<N, float, FS_P5_RHS, float>, r32, kThreads, m32, a, s);
-        case FK_P1_CGF_F32: return launch_fs(k_fs_p1<N, float, FS_P1_CGF>, r32, kThreads, m32, a, s);
-        case FK_P5_CGF_F32: return launch_fs(k_fs_p5<N, float, FS_P5_CGF, float>, r32, kThreads, m32, a, s);
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 }  // namespace fftg
