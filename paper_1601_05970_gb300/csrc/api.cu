@@ -121,7 +121,8 @@ const char* const kKindNames[KK_COUNT] = {
     "p1_tanrhs_f64", "p1_tanrhs_f32", "p2_f64", "p2_f32", "p4_f64", "p4_f32", "p3_f64", "p3_f32",
     "p5_plain_f64", "p5_plain_f32", "p5_dot_f64", "p5_dot_f32", "p5_rhs_f64_to_f64", "p1_plain_dd", "p2_dd",
     "p3_dd", "p4_dd", "p5_plain_dd_to_f64", "x1i_cg_f32", "rows_cg_f32", "x1f_cg_f32", "x1f_rhs_f32",
-    "x1f_rhs_dd", "x1i_solution_f32", "p5_newton_f32", "constitutive_f32", "constitutive_f64",
+    "x1f_rhs_dd", "x1i_solution_f32", "p5_newton_f32", "p1_user_f64", "p1_user_dd", "p5_user_f32",
+    "p5_dot_user_f64", "constitutive_f32", "constitutive_f64",
     "cg_update_f64", "newton_update_f64", "newton_norm_f32", "tangent_floor",
     "tangent_average", "cg_finish_f64", "tangent_bounds", "cg_begin_f32", "cg_rr_f32"};
 
@@ -376,10 +377,13 @@ static inline double* cell_field(double* base, const fftg_handle* h, int c) {
 // null) skips cells.
 static int launch_constitutive(fftg_handle* h, const int* mask_dev, int ncells, int cell0,
                                const double* eps, double* sigma, bool write_history, CGState* cg,
-                               bool write_tangent = true, bool elastic_only = false) {
+                               bool write_tangent = true, bool elastic_only = false,
+                               const double* user_eps = nullptr, double* user_sigma = nullptr) {
     ConstArgs a{};
     a.V = h->V;
     a.cs = h->cs;
+    a.ecs = user_eps ? h->V : h->cs;
+    a.scs = user_sigma ? h->V : h->cs;
     a.Edev = h->Edev + 6 * cell0;
     a.eps = eps + (size_t)cell0 * 6 * h->cs;
     a.eps_p = h->eps_p + (size_t)cell0 * 6 * h->cs;
@@ -402,6 +406,9 @@ static int launch_constitutive(fftg_handle* h, const int* mask_dev, int ncells, 
     a.cell_fields = 6 * h->cs;
     a.cell_scalar = h->cs;
     a.cell_tangent = 7 * h->cs;
+    // a caller's fields ([6][V], one cell) in place of the handle's
+    if (user_eps) a.eps = user_eps;
+    if (user_sigma) a.sigma = user_sigma;
     const dim3 g(pointwise_blocks(h->V), ncells);
     const int slot = prof_begin(h, h->mixed ? KK_CONSTITUTIVE_F32 : KK_CONSTITUTIVE_F64);
     if (h->mixed)
@@ -1782,29 +1789,44 @@ int fftg_get_field(fftg_handle* h, int which, double* out) {
     }
 }
 
+// A caller's field as the kernels can take it: device pointers are read and
+// written in place; one that is not aligned to its elements goes through the
+// handle's scratch (`tmp`, contiguous).
+static bool element_aligned(const void* p, size_t es) { return ((uintptr_t)p & (es - 1)) == 0; }
+static bool overlap(const void* a, const void* b, size_t bytes) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + bytes && y < x + bytes;
+}
+
 int fftg_op_project(fftg_handle* h, int precision, const void* tau, void* out) {
     if (!h || !tau || !out || (precision != FFTG_FP64 && precision != FFTG_MIXED && precision != FFTG_DD))
         return FFTG_EINVAL;
     const int prec = precision == FFTG_FP64 ? FFT_F64 : precision == FFTG_DD ? FFT_DD : FFT_F32;
     const bool f64 = prec != FFT_F32;  // FP64 buffers (FFTG_FP64, FFTG_DD)
-    const size_t es = f64 ? 8 : 4;
-    // internal scratch in the padded layout: FP64 in sigma / eps_work, FP32
-    // in p / q (these hold no state between increments)
-    void* in_buf = f64 ? (void*)h->sigma : h->p;
-    void* out_buf = f64 ? (void*)h->eps_work : h->q;
-    CK(copy_field(h, in_buf, true, tau, false, es, cudaMemcpyDeviceToDevice));
+    const size_t es = f64 ? 8 : 4, bytes = 6 * (size_t)h->V * es;
+    // scratch: sigma and q hold no state between increments
+    void* tmp = f64 ? (void*)h->sigma : h->q;
+    const void* in = tau;
+    if (!element_aligned(tau, es)) {
+        CK(cudaMemcpyAsync(tmp, tau, bytes, cudaMemcpyDeviceToDevice, h->stream));
+        in = tmp;
+    }
+    void* dst = element_aligned(out, es) ? out : tmp;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
+    // P1 has read all of `in` before P5 writes, so the fields may overlap
     PassArgs a = base_args_fft(h, prec);
-    a.in = in_buf;
+    a.in = in;
     a.out = h->spec;
-    CK(pass(h, prec == FFT_DD ? PK_P1_PLAIN_DD : f64 ? PK_P1_PLAIN_F64 : PK_P1_PLAIN_F32, a, 1));
+    a.ucs = h->V;
+    CK(pass(h, prec == FFT_DD ? PK_P1_USER_DD : f64 ? PK_P1_USER_F64 : PK_P1_PLAIN_F32, a, 1));
     int rc = run_p234(h, prec, invN3, nullptr, 1, nullptr);
     if (rc) return rc;
     PassArgs b = base_args_fft(h, prec);
     b.in = h->spec;
-    b.out = out_buf;
-    CK(pass(h, prec == FFT_DD ? PK_P5_PLAIN_DD_TO_F64 : f64 ? PK_P5_PLAIN_F64 : PK_P5_PLAIN_F32, b, 1));
-    CK(copy_field(h, out, false, out_buf, true, es, cudaMemcpyDeviceToDevice));
+    b.out = dst;
+    b.ucs = h->V;
+    CK(pass(h, prec == FFT_DD ? PK_P5_PLAIN_DD_TO_F64 : f64 ? PK_P5_PLAIN_F64 : PK_P5_USER_F32, b, 1));
+    if (dst != out) CK(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToDevice, h->stream));
     return FFTG_OK;
 }
 
@@ -1813,15 +1835,21 @@ int fftg_op_constitutive(fftg_handle* h, const double dE[6], const double* eps, 
     const int cell = h->sel;
     for (int c = 0; c < 6; ++c) h->h_E[6 * cell + c] = h->E[6 * cell + c] + (dE ? dE[c] : 0.0);
     CK(cudaMemcpyAsync(h->Edev + 6 * cell, h->h_E + 6 * cell, 48, cudaMemcpyHostToDevice, h->stream));
-    const double* e = h->eps_star;
-    if (eps) {
-        CK(copy_field(h, cell_field(h->eps_work, h, cell), true, eps, false, 8, cudaMemcpyDeviceToDevice));
-        e = h->eps_work;
+    const size_t bytes = 6 * (size_t)h->V * 8;
+    // a voxel's strain is read before its stress is written, by one thread:
+    // the fields may be the same; where they overlap otherwise, or are not
+    // aligned, they go through the handle's
+    const double* ue = eps;
+    double* us = sigma;
+    const bool stage = eps && sigma && (const void*)eps != (void*)sigma && overlap(eps, sigma, bytes);
+    if (eps && (stage || !element_aligned(eps, 8))) {
+        CK(cudaMemcpyAsync(h->eps_work, eps, bytes, cudaMemcpyDeviceToDevice, h->stream));
+        ue = h->eps_work;
     }
-    int rc = launch_constitutive(h, nullptr, 1, cell, e, h->sigma, false, nullptr);
+    if (sigma && !element_aligned(sigma, 8)) us = h->sigma;
+    int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, true, false, ue, us);
     if (rc) return rc;
-    if (sigma)
-        CK(copy_field(h, sigma, false, cell_field(h->sigma, h, cell), true, 8, cudaMemcpyDeviceToDevice));
+    if (us != sigma) CK(cudaMemcpyAsync(sigma, us, bytes, cudaMemcpyDeviceToDevice, h->stream));
     h->have_tangent[cell] = 0;
     return FFTG_OK;
 }
@@ -1830,14 +1858,23 @@ int fftg_op_matvec(fftg_handle* h, int precision, const void* p, void* q, double
     if (!h || !p || !q) return FFTG_EINVAL;
     const bool f64 = precision == FFTG_FP64;
     if (f64 == (bool)h->mixed) return FFTG_EINVAL;  // must match the tangent's precision
-    const size_t es = f64 ? 8 : 4;
+    const size_t es = f64 ? 8 : 4, bytes = 6 * (size_t)h->V * es;
     set_cg_params(h, 1, 1.0, nullptr);
     h->h_cg[0].rr = 1.0;
     CK(cudaMemcpyAsync(h->cg, h->h_cg, h->nf * sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
-    CK(copy_field(h, h->p, true, p, false, es, cudaMemcpyDeviceToDevice));
+    // p is read again for <p, q> while q is written, a voxel by one thread:
+    // the fields may be the same; otherwise as in fftg_op_constitutive
+    const void* up = p;
+    void* uq = q;
+    if ((p != q && overlap(p, q, bytes)) || !element_aligned(p, es)) {
+        CK(cudaMemcpyAsync(h->p, p, bytes, cudaMemcpyDeviceToDevice, h->stream));
+        up = h->p;
+    }
+    if (!element_aligned(q, es)) uq = h->q;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     PassArgs a = base_args(h, f64);
-    a.in = h->p;
+    a.in = up;
+    a.ucs = h->V;
     a.tangent = (const char*)h->tangent + (size_t)h->sel * 7 * h->cs * es;
     a.out = h->spec;
     CK(pass(h, f64 ? PK_P1_TAN_F64 : PK_P1_TAN_F32, a, 1));
@@ -1845,11 +1882,12 @@ int fftg_op_matvec(fftg_handle* h, int precision, const void* p, void* q, double
     if (rc) return rc;
     PassArgs b = base_args(h, f64);
     b.in = h->spec;
-    b.out = h->q;
-    b.aux = h->p;
+    b.out = uq;
+    b.aux = up;
+    b.ucs = h->V;
     b.cg = h->cg;
-    CK(pass(h, f64 ? PK_P5_DOT_F64 : PK_P5_DOT_F32, b, 1));
-    CK(copy_field(h, q, false, h->q, true, es, cudaMemcpyDeviceToDevice));
+    CK(pass(h, f64 ? PK_P5_DOT_USER_F64 : PK_P5_DOT_F32, b, 1));
+    if (uq != q) CK(cudaMemcpyAsync(q, uq, bytes, cudaMemcpyDeviceToDevice, h->stream));
     if (pq) {
         CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));

@@ -64,7 +64,7 @@ int grid_index(int N) {
 }
 
 // pass kinds of each tuned kind (the default launch of variant 0)
-constexpr PassKind kDefaultKind[TK_COUNT] = {PK_ROWS_CG_F32, PK_P2_F32, PK_P3_F32, PK_P4_F32, PK_P5_PLAIN_F32};
+constexpr PassKind kDefaultKind[TK_COUNT] = {PK_ROWS_CG_F32, PK_P2_F32, PK_P3_F32, PK_P4_F32, PK_P5_USER_F32};
 const char* const kTkName[TK_COUNT] = {"p1", "p2", "p3", "p4", "p5"};
 
 std::mutex g_cache_mu;
@@ -180,6 +180,7 @@ int tune(int N, cudaStream_t s, int reps, double* ms_out, int* chosen) {
     a.tw = b + off_tw;
     a.partials = (double*)(b + off_part);
     a.cs = (long long)cs;
+    a.ucs = (long long)N * N * N;
     a.fstride = 6 * (long long)cs;
     a.sstride = 6LL * N * N * (long long)HP;
     a.tangent = b + off_t;
@@ -251,7 +252,7 @@ int tuned_kind(int pass_kind) {
         case PK_P2_F32: return TK_P2;
         case PK_P3_F32: return TK_P3;
         case PK_P4_F32: return TK_P4;
-        case PK_P5_PLAIN_F32: return TK_P5;
+        case PK_P5_USER_F32: return TK_P5;
         default: return -1;
     }
 }

@@ -658,9 +658,9 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
     switch (kind) {
         case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s);
-        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN>, r32, C32::smem_rows, a, s);
-        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN>, r64, C64::smem_rows, a, s);
-        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN>, r32, C32::smem_rows, a, s);
+        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN, 1>, r32, C32::smem_rows, a, s);
+        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN, 1>, r64, C64::smem_rows, a, s);
+        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN, 1>, r32, C32::smem_rows, a, s);
         case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s);
         case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s);
         case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s);
@@ -670,10 +670,10 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P4_F32: return launch_k(k_p24<N, float, false>, c32, C32::smem_p24, a, s, C32::T2);
         case PK_P3_F64: return launch_k(k_p3<N, double>, g64, C64::smem_p3, a, s, C64::T3);
         case PK_P3_F32: return launch_k(k_p3<N, float>, g32, C32::smem_p3, a, s, C32::T3);
-        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double>, r64, C64::smem_rows, a, s);
+        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double, 1>, r64, C64::smem_rows, a, s);
         case PK_P5_PLAIN_F32: return launch_k(k_p5<N, float, P5_PLAIN, float>, r32, C32::smem_rows, a, s);
         case PK_P5_DOT_F64: return launch_k(k_p5<N, double, P5_DOT, double>, r64, C64::smem_rows, a, s);
-        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float>, r32, C32::smem_rows, a, s);
+        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float, 1>, r32, C32::smem_rows, a, s);
         case PK_P5_RHS_F64_TO_F64:
             return launch_k(k_p5<N, double, P5_RHS, double>, r64, C64::smem_rows, a, s);
         case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s);
@@ -681,7 +681,12 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P4_DD: return launch_k(k_p24<N, dd, false>, c64, CDD::smem_p24, a, s, CDD::T2);
         case PK_P3_DD: return launch_k(k_p3<N, dd>, gdd, CDD::smem_p3, a, s, CDD::T3);
         case PK_P5_PLAIN_DD_TO_F64:
-            return launch_k(k_p5<N, dd, P5_PLAIN, double>, r64, CDD::smem_rows, a, s);
+            return launch_k(k_p5<N, dd, P5_PLAIN, double, 1>, r64, CDD::smem_rows, a, s);
+        case PK_P1_USER_F64: return launch_k(k_p1<N, double, P1_PLAIN, 1>, r64, C64::smem_rows, a, s);
+        case PK_P1_USER_DD: return launch_k(k_p1<N, dd, P1_PLAIN, 1>, r64, CDD::smem_rows, a, s);
+        case PK_P5_USER_F32: return launch_k(k_p5<N, float, P5_PLAIN, float, 1>, r32, C32::smem_rows, a, s);
+        case PK_P5_DOT_USER_F64:
+            return launch_k(k_p5<N, double, P5_DOT, double, 1>, r64, C64::smem_rows, a, s);
         case PK_P5_NEWTON_F32: return launch_k(k_p5<N, float, P5_NEWTON, float>, r32, C32::smem_rows, a, s);
         case PK_X1I_CG_F32: return launch_k(k_x1i<N, X1I_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1I_SOLUTION_F32: return launch_k(k_x1i<N, X1I_SOLUTION>, x32, X1<N>::smem, a, s, X1<N>::NT);

@@ -529,6 +529,7 @@ FsArgs fs_args(fftg_fs_handle* h, int prec) {
     a.tw = prec == FFT_DD ? h->twdd : prec == FFT_F64 ? h->tw64 : h->tw32;
     a.partials = h->partials;
     a.cs = h->cs;
+    a.ucs = h->cs;
     a.phase = h->phase;
     a.lame = h->lame;
     a.hgrad = h->hgrad;
@@ -1160,22 +1161,26 @@ int fftg_fs_op_project(fftg_fs_handle* h, int precision, const void* A_dev, void
         return FFTG_EINVAL;
     const int prec = precision == FFTG_FP64 ? FFT_F64 : precision == FFTG_DD ? FFT_DD : FFT_F32;
     const bool f64 = prec != FFT_F32;  // FP64 buffers (FFTG_FP64, FFTG_DD)
-    const size_t el = f64 ? 8 : 4;
-    // staged through the padded buffer P (FP64) or x (FP32)
-    void* buf = f64 ? (void*)h->P : h->x;
-    if (!f64 && !h->mixed) return FFTG_EINVAL;  // FP32 buffers exist only in a mixed handle
-    h->P_current = false;
-    CK(fs_copy(h, buf, true, A_dev, false, el, cudaMemcpyDeviceToDevice));
+    const size_t el = f64 ? 8 : 4, bytes = 9 * (size_t)h->V * el;
+    if (!f64 && !h->mixed) return FFTG_EINVAL;  // FP32 transforms exist only in a mixed handle
+    // device pointers are used in place (P1 has read all of A before P5 writes);
+    // one that is not aligned to its elements goes through P (FP64) or q (FP32)
+    void* tmp = f64 ? (void*)h->P : h->q;
+    const bool in_ok = ((uintptr_t)A_dev & (el - 1)) == 0, out_ok = ((uintptr_t)out_dev & (el - 1)) == 0;
+    if (f64 && !(in_ok && out_ok)) h->P_current = false;
+    if (!in_ok) CK(cudaMemcpyAsync(tmp, A_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
     FsArgs a = fs_args(h, prec);
-    a.in = buf;
+    a.in = in_ok ? A_dev : tmp;
+    a.ucs = h->V;
     CK(fs_pass(h, prec == FFT_DD ? FK_P1_PLAIN_DD : f64 ? FK_P1_PLAIN_F64 : FK_P1_PLAIN_F32, a));
     int rc = fs_p234(h, prec, 1.0 / ((double)h->N * h->N * h->N), nullptr);
     if (rc) return rc;
     FsArgs b = fs_args(h, prec);
     b.in = h->spec;
-    b.out = buf;
+    b.out = out_ok ? out_dev : tmp;
+    b.ucs = h->V;
     CK(fs_pass(h, prec == FFT_DD ? FK_P5_PLAIN_DD_TO_F64 : f64 ? FK_P5_PLAIN_F64 : FK_P5_PLAIN_F32, b));
-    CK(fs_copy(h, out_dev, false, buf, true, el, cudaMemcpyDeviceToDevice));
+    if (!out_ok) CK(cudaMemcpyAsync(out_dev, tmp, bytes, cudaMemcpyDeviceToDevice, h->stream));
     return FFTG_OK;
 }
 
@@ -1189,10 +1194,21 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     if (rc) return rc;
     if ((rc = fs_constitutive(h, h->Fstar, true, nullptr))) return rc;
     h->P_current = true;
-    CK(fs_copy(h, h->p, true, p_dev, false, el, cudaMemcpyDeviceToDevice));
+    // p is read again for <p, q> while q is written, a voxel by one thread: the
+    // fields may be the same; where they overlap otherwise, or are not aligned
+    // to their elements, they go through the handle's
+    const size_t bytes = 9 * (size_t)h->V * el;
+    const uintptr_t pa = (uintptr_t)p_dev, qa = (uintptr_t)q_dev;
+    const void* up = p_dev;
+    void* uq = (qa & (el - 1)) ? h->q : q_dev;
+    if ((pa != qa && pa < qa + bytes && qa < pa + bytes) || (pa & (el - 1))) {
+        CK(cudaMemcpyAsync(h->p, p_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
+        up = h->p;
+    }
     const int prec = f64 ? FFT_F64 : FFT_F32;
     FsArgs a = fs_args(h, prec);
-    a.in = h->p;
+    a.in = up;
+    a.ucs = h->V;
     CK(fs_pass(h, f64 ? FK_P1_TAN_F64 : FK_P1_TAN_F32, a));
     if ((rc = fs_p234(h, prec, 1.0 / ((double)h->N * h->N * h->N), nullptr))) return rc;
     // <p, q> through the DOT pass on a scratch CG state
@@ -1200,11 +1216,12 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     CK(cudaMemcpyAsync(h->cg, h->h_cg, sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
     FsArgs b = fs_args(h, prec);
     b.in = h->spec;
-    b.out = h->q;
-    b.aux = h->p;
+    b.out = uq;
+    b.aux = up;
+    b.ucs = h->V;
     b.cg = h->cg;
     CK(fs_pass(h, f64 ? FK_P5_DOT_F64 : FK_P5_DOT_F32, b));
-    CK(fs_copy(h, q_dev, false, h->q, true, el, cudaMemcpyDeviceToDevice));
+    if (uq != q_dev) CK(cudaMemcpyAsync(q_dev, uq, bytes, cudaMemcpyDeviceToDevice, h->stream));
     if (pq) {
         CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));

@@ -48,6 +48,7 @@ struct FsArgs {
     const void* tw;        // w_N^j, j < N, in the FFT precision
     double scale;          // P3: factor on Ghat (+-1/N^3)
     long long cs;          // component stride of the real fields (elements)
+    long long ucs;         // that of in and out (and the p of P5_DOT): cs, or N^3 for a caller's fields
     int unit;              // P1_TANRHS: tau = K : E_unit, E_unit the unit tensor at component unit
     const double* red_in;  // P2 of the mixed CG iteration: the row pass's block partials of <p, K : p>
     int red_n;             // (reduced by P2's first block, which sets alpha)
@@ -107,7 +108,7 @@ struct FsCfg {
     static constexpr int row_blocks = (N * N + R - 1) / R;
     static_assert(smem_rows <= 227 * 1024 && smem_p3 <= 227 * 1024, "shared memory per block");
     static_assert(T3 <= 1024 && T3 % 32 == 0, "threads per block");
-    static_assert((R * N) % VW == 0 && (VW == 1 || VW == 2 || VW == 4), "vector width");
+    static_assert(VW == 1, "a caller's components start on any element");
 };
 
 // tau = K(F) : d for St. Venant-Kirchhoff, from h = F - I.
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1
 #pragma unroll
                         for (int e = 0; e < VW; ++e) t[e] = TIn(c == a.unit ? 1 : 0);
                     } else {
-                        ldv<VW, TIn>(in + c * cs + v0, t);
+                        ldv<VW, TIn>(in + c * a.ucs + v0, t);
                     }
 #pragma unroll
                     for (int e = 0; e < VW; ++e) p[c][e] = T(t[e]);
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
         TO pv[9][VO];
         if (MODE == FS_P5_DOT) {
 #pragma unroll
-            for (int c = 0; c < 9; ++c) ldv<VO, TO>(pin + c * cs + v0, pv[c]);
+            for (int c = 0; c < 9; ++c) ldv<VO, TO>(pin + c * a.ucs + v0, pv[c]);
         }
         T qd[9][VO];
         TO q[9][VO];
@@ -567,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
             continue;
         }
 #pragma unroll
-        for (int c = 0; c < 9; ++c) stv<VO, TO>(out + c * cs + v0, q[c]);
+        for (int c = 0; c < 9; ++c) stv<VO, TO>(out + c * a.ucs + v0, q[c]);
         if (MODE == FS_P5_PLAIN) continue;
 #pragma unroll
         for (int e = 0; e < VO; ++e) {

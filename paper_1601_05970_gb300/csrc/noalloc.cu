@@ -108,7 +108,7 @@ extern "C" int fftg_constitutive_noalloc(int N, const double E[6], const double*
     if (cudaMemcpyAsync(dmats, m, sizeof(m), cudaMemcpyHostToDevice, s) != cudaSuccess) return FFTG_ECUDA;
     ConstArgs a{};
     a.V = (long long)N * N * N;
-    a.cs = a.V;  // caller fields are [6][N^3], unpadded
+    a.cs = a.ecs = a.scs = a.V;  // caller fields are [6][N^3], unpadded
     for (int c = 0; c < 6; ++c) a.E[c] = E[c];
     a.eps = eps_dev;
     a.eps_p = eps_p_dev;

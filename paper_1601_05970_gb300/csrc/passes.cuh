@@ -52,6 +52,7 @@ struct PassArgs {
     long long sstride;     // spectrum stride between fields (complex elements)
     long long tstride;     // tangent stride between fields (0: shared)
     const int* active;     // per field: 0 = skip this field (null: all run)
+    long long ucs;         // caller's fields (U = 1 of P1 and P5): component stride, any alignment
     // P2 of the mixed CG iteration: the block partials of <p, C : p> that the
     // row pass wrote ([nf][red_n]); block (0, 0) of each field reduces them in
     // a fixed order and sets alpha (null: nothing to reduce)
@@ -276,7 +277,11 @@ struct Vec16<double> {
 };
 
 // ----------------------------------------------------------------------- P1
-template <int N, typename T, int MODE, int NA = Plan<N>::N1, int TV = 0>
+// U = 1: `in` is a caller's [6][N^3] field, whose components start on any
+// element: one voxel a lane, the loads of several rounds issued together. The
+// projection of an FP32 field at 243^3 takes 741 us; with the field copied
+// to and from the padded layout (96 B per voxel) it took 1169.
+template <int N, typename T, int MODE, int U = 0, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
     k_p1(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
@@ -314,7 +319,38 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     // only the padding of the component (cs >= N^3 + 4), and its lanes past
     // the grid belong to rows that the FFT stages skip.
     constexpr int VW = C::VW;
-    for (int j = tid; j < (R * N) / VW; j += kThreads) {
+    if constexpr (U != 0) {
+        static_assert(MODE == P1_PLAIN || MODE == P1_TAN, "a caller's field is projected or multiplied");
+        constexpr int UN = sizeof(TIn) == 4 ? 4 : 2;
+        const long long us = a.ucs;
+        for (int j0 = tid; j0 < R * N; j0 += UN * kThreads) {
+            TIn t[UN][6];
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const int j = j0 + u * kThreads;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) t[u][c] = j < nel ? in[c * us + base + j] : TIn(0);
+            }
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const int j = j0 + u * kThreads;
+                if (j >= R * N) continue;
+                T s[6] = {T(t[u][0]), T(t[u][1]), T(t[u][2]), T(t[u][3]), T(t[u][4]), T(t[u][5])};
+                if constexpr (MODE == P1_TAN) {
+                    if (j < nel) {
+                        T t7[7], pe[6] = {s[0], s[1], s[2], s[3], s[4], s[5]};
+#pragma unroll
+                        for (int k = 0; k < 7; ++k) t7[k] = tg[k * cs + base + j];
+                        apply_tangent7<T>(t7[0], t7[1], t7[2], t7[3], t7[4], t7[5], t7[6], pe, s);
+                    }
+                }
+                z[j] = mk(s[0], s[1]);
+                z[R * N + j] = mk(s[2], s[3]);
+                z[2 * R * N + j] = mk(s[4], s[5]);
+            }
+        }
+    }
+    for (int j = U ? R * N : tid; j < (R * N) / VW; j += kThreads) {
         const int i0 = j * VW;
         T s[6][VW];
         if (i0 < nel) {
@@ -720,7 +756,8 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
 // ----------------------------------------------------------------------- P5
 // T: FFT precision; TO: output real type (P5_RHS writes the CG residual r
 // in the inner precision).
-template <int N, typename T, int MODE, typename TO, int NA = Plan<N>::N1, int TV = 0>
+// U = 1: `out` (and the p of P5_DOT) are a caller's fields, as in P1.
+template <int N, typename T, int MODE, typename TO, int U = 0, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
     k_p5(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
@@ -793,7 +830,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
         if (pc % R < nrows) invA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
     }
     __syncthreads();
-    const long long cs = a.cs;
+    const long long cs = U ? a.ucs : a.cs;
     TO* out = (TO*)a.out + f * a.fstride;
     T acc0 = T(0);
     double acc1 = 0.0;
@@ -801,7 +838,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     // per component for q and p. With VO = 1 the tile reads are free of bank
     // conflicts. Lanes past the grid in the last block write only component
     // padding and are left out of the sums.
-    constexpr int VO = (FFTG_P5_VW * (int)sizeof(TO) > 16) ? 16 / (int)sizeof(TO) : FFTG_P5_VW;
+    constexpr int VO = U ? 1 : (FFTG_P5_VW * (int)sizeof(TO) > 16) ? 16 / (int)sizeof(TO) : FFTG_P5_VW;
     // FFTG_P5_PB rounds at a time: the loads of p for all of them first.
     constexpr int NV = (R * N) / VO;
     constexpr int NRE = (NV + kThreads - 1) / kThreads;
@@ -917,6 +954,9 @@ enum PassKind : int {
     // the mixed path's CG on displacement coefficients (cg_passes.cuh)
     PK_X1I_CG_F32, PK_ROWS_CG_F32, PK_X1F_CG_F32, PK_X1F_RHS_F32, PK_X1F_RHS_DD, PK_X1I_SOLUTION_F32,
     PK_P5_NEWTON_F32,
+    // the operators on a caller's fields (U = 1); so are P1_PLAIN_F32, P1_TAN,
+    // P5_PLAIN_F64 and P5_PLAIN_DD_TO_F64, which nothing else runs
+    PK_P1_USER_F64, PK_P1_USER_DD, PK_P5_USER_F32, PK_P5_DOT_USER_F64,
     PK_COUNT
 };
 

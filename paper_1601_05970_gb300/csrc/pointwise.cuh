@@ -31,6 +31,7 @@ inline int vector_blocks(long long cs, int elem_bytes) {
 struct ConstArgs {
     long long V;
     long long cs;            // component stride of the fields (>= V)
+    long long ecs, scs;      // those of eps and sigma (a caller's fields: V)
     double E[6];
     const double* eps;       // [6][V] fluctuation eps*
     const double* eps_p;     // [6][V] committed plastic strain
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_constitutive(ConstArgs a) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             ep[c] = eps_p[c * cs + v];
-            e[c] = E[c] + eps[c * cs + v] - (nle ? 0.0 : ep[c]);
+            e[c] = E[c] + eps[c * a.ecs + v] - (nle ? 0.0 : ep[c]);
         }
         const double eb = epbar[v];
         const double tr = e[0] + e[1] + e[2];
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_constitutive(ConstArgs a) {
         sig[2] += kt;
         if (sigma) {
 #pragma unroll
-            for (int c = 0; c < 6; ++c) sigma[c * cs + v] = sig[c];
+            for (int c = 0; c < 6; ++c) sigma[c * a.scs + v] = sig[c];
         }
         if (eps_p_new) {
 #pragma unroll

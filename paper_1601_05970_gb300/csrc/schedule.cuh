@@ -47,7 +47,8 @@ template <int N, int TK, int V>
 struct VariantOf {
     static constexpr bool cols = TK == TK_P2 || TK == TK_P4;
     static constexpr bool fused = TK == TK_P3 && V == 3;
-    static constexpr int A = (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A : Plan<N>::N1;
+    // (the fused P3 at 225^3: 25 x 9, since 15 x 15 has no stage of at most 9)
+    static constexpr int A = fused && N == 225 ? 25 : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A : Plan<N>::N1;
     static constexpr int TV = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
 };
 
@@ -60,7 +61,7 @@ cudaError_t launch_variant(const PassArgs& a, int nf, cudaStream_t s) {
         using R = RowCfg<N, NA, VO::TV>;
         return launch_k(k_rows_cg<N, NA, VO::TV>, dim3(R::blocks, 1, nf), R::smem, a, s, R::NT);
     } else if constexpr (TK == TK_P5) {
-        return launch_k(k_p5<N, float, P5_PLAIN, float, VO::A, VO::TV>, dim3(C::row_blocks, 1, nf), C::smem_rows,
+        return launch_k(k_p5<N, float, P5_PLAIN, float, 1, VO::A, VO::TV>, dim3(C::row_blocks, 1, nf), C::smem_rows,
                         a, s);
     } else if constexpr (TK == TK_P3 && VO::fused && P3f<N, VO::A>::ok) {
         return launch_k(k_p3f<N, VO::A>, dim3((C::H + C::W3 - 1) / C::W3, N, nf), C::smem_p3, a, s,
