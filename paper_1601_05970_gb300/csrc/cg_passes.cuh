@@ -652,7 +652,6 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     const dim3 r32(C32::row_blocks, 1, nf), r64(C64::row_blocks, 1, nf);
     const dim3 c32((C32::H + C32::W2 - 1) / C32::W2, (6 * N + C32::S2 - 1) / C32::S2, nf);
     const dim3 c64((C64::H + C64::W2 - 1) / C64::W2, (6 * N + C64::S2 - 1) / C64::S2, nf);
-    const dim3 g32((C32::H + C32::W3 - 1) / C32::W3, N, nf);
     const dim3 g64((C64::H + C64::W3 - 1) / C64::W3, N, nf);
     const dim3 x32(X1<N>::tiles, N, nf);
     const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
@@ -669,7 +668,15 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P4_F64: return launch_k(k_p24<N, double, false>, c64, C64::smem_p24, a, s, C64::T2);
         case PK_P4_F32: return launch_k(k_p24<N, float, false>, c32, C32::smem_p24, a, s, C32::T2);
         case PK_P3_F64: return launch_k(k_p3<N, double>, g64, C64::smem_p3, a, s, C64::T3);
-        case PK_P3_F32: return launch_k(k_p3<N, float>, g32, C32::smem_p3, a, s, C32::T3);
+        case PK_P3_F32: {
+            using D = P3Default<N>;
+            using C = Cfg<N, float, D::A, D::TV>;
+            const dim3 g((C::H + C::W3 - 1) / C::W3, N, nf);
+            if constexpr (D::fused)
+                return launch_k(k_p3f<N, D::A>, g, C::smem_p3, a, s, P3f<N, D::A>::NT);
+            else
+                return launch_k(k_p3<N, float, D::A, D::TV>, g, C::smem_p3, a, s, C::T3);
+        }
         case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double, 1>, r64, C64::smem_rows, a, s);
         case PK_P5_PLAIN_F32: return launch_k(k_p5<N, float, P5_PLAIN, float>, r32, C32::smem_rows, a, s);
         case PK_P5_DOT_F64: return launch_k(k_p5<N, double, P5_DOT, double>, r64, C64::smem_rows, a, s);

@@ -753,6 +753,18 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
     }
 }
 
+// Default schedule of the FP32 P3, from the projection of one field (us,
+// default tile / half tile / fused): 45^3 10.3 / 8.5 / 12.3, 75^3 14.1 / 12.5 /
+// 12.5, 81^3 16.3 / 15.7 / 14.4, 125^3 37.3 / 34.6 / 30.5, 135^3 38.9 / 39.3 /
+// 37.3, 225^3 219 / 209 / 174 (fused: 25 x 9, since 15 x 15 has no stage of at
+// most 9 points), 243^3 229 / 233 / 217. Below 45^3 all take the launch's time.
+template <int N>
+struct P3Default {
+    static constexpr bool fused = N >= 75;
+    static constexpr int A = N == 225 ? 25 : Plan<N>::N1, TV = N == 45 ? 1 : 0;
+    static_assert(!fused || P3f<N, A>::ok, "fused P3");
+};
+
 // ----------------------------------------------------------------------- P5
 // T: FFT precision; TO: output real type (P5_RHS writes the CG residual r
 // in the inner precision).

@@ -10,12 +10,12 @@
 //                                 2 half the rows per block; 3 twice the rows
 //   P2, P4 (x2, columns):         0 default; 1 the other radix split;
 //                                 2 32 columns per block; 3 both
-//   P3 (x1 + Ghat, columns):      0 default; 1 the other radix split;
-//                                 2 half the columns per block;
-//                                 3 the default tile with stage B, Ghat
-//                                   and the inverse stage B in one phase
-//                                   (k_p3f; splits with 1 < N2 <= 9, else
-//                                   the default)
+//   P3 (x1 + Ghat, columns):      0 default (P3Default); 1 the other radix
+//                                 split; 2 half the columns per block;
+//                                 3 a full tile with stage B, Ghat and the
+//                                   inverse stage B in one phase (k_p3f;
+//                                   splits with 1 < N2 <= 9, else the
+//                                   default)
 //
 // A schedule changes only how the same transforms are split into register
 // DFTs and how pencils are grouped into blocks: the results agree to FP32
@@ -47,9 +47,11 @@ template <int N, int TK, int V>
 struct VariantOf {
     static constexpr bool cols = TK == TK_P2 || TK == TK_P4;
     static constexpr bool fused = TK == TK_P3 && V == 3;
-    // (the fused P3 at 225^3: 25 x 9, since 15 x 15 has no stage of at most 9)
-    static constexpr int A = fused && N == 225 ? 25 : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A : Plan<N>::N1;
-    static constexpr int TV = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
+    static constexpr bool p3d = TK == TK_P3 && V == 0;  // as P3Default has it
+    static constexpr int A = (fused || p3d) && N == 225 ? 25
+                             : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A
+                                                             : Plan<N>::N1;
+    static constexpr int TV = p3d ? P3Default<N>::TV : V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
 };
 
 template <int N, int TK, int V>
