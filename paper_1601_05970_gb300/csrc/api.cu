@@ -25,7 +25,9 @@
 #include "batch.cuh"
 
 namespace fftg {
-#define FFTG_EXTERN_N(n) extern template cudaError_t run_pass_n<n>(PassKind, const PassArgs&, int, cudaStream_t);
+#define FFTG_EXTERN_N(n)                                                                  \
+    extern template cudaError_t run_pass_n<n>(PassKind, const PassArgs&, int, cudaStream_t); \
+    extern template cudaError_t run_cluster_n<n>(const PassArgs&, int, int, int, int*, cudaStream_t);
 FFTG_EXTERN_N(3)
 FFTG_EXTERN_N(5)
 FFTG_EXTERN_N(9)
@@ -59,6 +61,17 @@ cudaError_t run_pass(int N, PassKind kind, const PassArgs& a, int nf, cudaStream
     }
 }
 
+static cudaError_t run_cluster(int N, const PassArgs& a, int nf, int cl, int cap, int* size, cudaStream_t s) {
+    switch (N) {
+#define FFTG_CASE(n) case n: return run_cluster_n<n>(a, nf, cl, cap, size, s);
+        FFTG_CASE(3) FFTG_CASE(5) FFTG_CASE(9) FFTG_CASE(15) FFTG_CASE(25) FFTG_CASE(27)
+#undef FFTG_CASE
+        default:
+            if (size) *size = 0;
+            return cl ? cudaErrorInvalidValue : cudaSuccess;
+    }
+}
+
 // Most blocks of a row or x1 pass, over the schedules (for the partial sums).
 template <int N>
 static int row_blocks_n(bool fp64) {
@@ -81,20 +94,21 @@ int row_blocks(int N, bool fp64) {
 
 // Blocks per field of the passes whose partial sums a kernel reduces: the x1
 // passes (FP32, double-float right-hand side) and P5 at its default schedule.
+// planes: those of the plane pass, 0 where P4, the row pass and P2 run.
 struct PassBlocks {
-    int x1, x1_dd, p5;
+    int x1, x1_dd, p5, planes;
 };
 static PassBlocks pass_blocks(int N) {
     switch (N) {
 #define FFTG_CASE(n)                                                                                     \
     case n:                                                                                              \
         return {X1<n>::blocks, (Cfg<n, dd>::H + Cfg<n, dd>::W3 - 1) / Cfg<n, dd>::W3 * n,                \
-                Cfg<n, float>::row_blocks};
+                Cfg<n, float>::row_blocks, PlaneCfg<n>::ok ? n : 0};
         FFTG_CASE(3) FFTG_CASE(5) FFTG_CASE(9) FFTG_CASE(15) FFTG_CASE(25) FFTG_CASE(27)
         FFTG_CASE(45) FFTG_CASE(75) FFTG_CASE(81) FFTG_CASE(125) FFTG_CASE(135) FFTG_CASE(225)
         FFTG_CASE(243)
 #undef FFTG_CASE
-        default: return {0, 0, 0};
+        default: return {0, 0, 0, 0};
     }
 }
 }  // namespace fftg
@@ -114,17 +128,17 @@ namespace {
 enum : int {
     KK_CONSTITUTIVE_F32 = PK_COUNT, KK_CONSTITUTIVE_F64, KK_CG_UPDATE_F64, KK_NEWTON_UPDATE_F64,
     KK_NEWTON_NORM_F32, KK_TANGENT_FLOOR, KK_TANGENT_AVERAGE, KK_CG_FINISH_F64, KK_TANGENT_BOUNDS,
-    KK_CG_BEGIN, KK_CG_RR, KK_COUNT
+    KK_CG_BEGIN, KK_CG_RR, KK_CG_CLUSTER, KK_COUNT
 };
 const char* const kKindNames[KK_COUNT] = {
     "p1_plain_f64", "p1_plain_f32", "p1_tan_f64", "p1_tan_f32", "p1_cg_f64",
     "p1_tanrhs_f64", "p1_tanrhs_f32", "p2_f64", "p2_f32", "p4_f64", "p4_f32", "p3_f64", "p3_f32",
     "p5_plain_f64", "p5_plain_f32", "p5_dot_f64", "p5_dot_f32", "p5_rhs_f64_to_f64", "p1_plain_dd", "p2_dd",
-    "p3_dd", "p4_dd", "p5_plain_dd_to_f64", "x1i_cg_f32", "rows_cg_f32", "x1f_cg_f32", "x1f_rhs_f32",
+    "p3_dd", "p4_dd", "p5_plain_dd_to_f64", "x1i_cg_f32", "rows_cg_f32", "plane_cg_f32", "x1f_cg_f32", "x1f_rhs_f32",
     "x1f_rhs_dd", "x1i_solution_f32", "p5_newton_f32", "p1_user_f64", "p1_user_dd", "p5_user_f32",
     "p5_dot_user_f64", "constitutive_f32", "constitutive_f64",
     "cg_update_f64", "newton_update_f64", "newton_norm_f32", "tangent_floor",
-    "tangent_average", "cg_finish_f64", "tangent_bounds", "cg_begin_f32", "cg_rr_f32"};
+    "tangent_average", "cg_finish_f64", "tangent_bounds", "cg_begin_f32", "cg_rr_f32", "cg_cluster_f32"};
 
 // Ring of event pairs around the handle's launches; drained at every read.
 struct Prof {
@@ -152,6 +166,7 @@ struct fftg_handle {
     int B = 1;                   // cells
     int nf = 6;                  // CG fields held: max(B, nrhs)
     int sel = 0;                 // cell addressed by the single-cell calls
+    int cluster = 0;             // blocks per cluster of the small grids' CG (0: the pass kernels)
     fftg_options opt{};
     cudaStream_t stream = nullptr;
     cudaError_t last_cuda = cudaSuccess;
@@ -546,26 +561,32 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
         a.out = h->spec;
         a.cg = h->cg;
         CK(pass(h, PK_X1I_CG_F32, a, nf));
-        CK(pass(h, PK_P4_F32, a, nf));
-        CK(pass(h, PK_ROWS_CG_F32, a, nf));
-        // P2 reduces the row pass's block partials of <p, C : p> (alpha)
-        PassArgs b = a;
-        b.red_in = h->partials;
-        b.red_n = variant_shape(h->N, TK_P1, schedule_variant(h->N, TK_P1)).blocks;
-        CK(pass(h, PK_P2_F32, b, nf));
         PassArgs c = base_args(h, false);
         c.in = h->spec;
         c.aux3 = h->r;
         c.cg = h->cg;
         c.scale = invN3;
+        const PassBlocks blocks = pass_blocks(h->N);
+        c.partials = h->partials + (size_t)nf * blocks.planes;
+        if (blocks.planes) {
+            CK(pass(h, PK_PLANE_CG_F32, a, nf));  // its last block sets alpha
+        } else {
+            CK(pass(h, PK_P4_F32, a, nf));
+            CK(pass(h, PK_ROWS_CG_F32, a, nf));
+            // P2 reduces the row pass's block partials (alpha)
+            PassArgs b = a;
+            b.red_in = h->partials;
+            b.red_n = variant_shape(h->N, TK_P1, schedule_variant(h->N, TK_P1)).blocks;
+            CK(pass(h, PK_P2_F32, b, nf));
+        }
         CK(pass(h, PK_X1F_CG_F32, c, nf));
         // <r, r> from its block partials: beta and the stopping tests
-        const int nb = pass_blocks(h->N).x1;
+        const int nb = blocks.x1;
         const int slot = prof_begin(h, KK_CG_RR);
         if (loop.guard)
-            k_cg_rr_loop<<<nf, 1024, 0, h->stream>>>(h->partials, nb, h->cg, loop);
+            k_cg_rr_loop<<<nf, 1024, 0, h->stream>>>(c.partials, nb, h->cg, loop);
         else
-            k_cg_rr<<<nf, 1024, 0, h->stream>>>(h->partials, nb, h->cg);
+            k_cg_rr<<<nf, 1024, 0, h->stream>>>(c.partials, nb, h->cg);
         prof_end(h, slot);
         CK(cudaGetLastError());
         return FFTG_OK;
@@ -607,6 +628,11 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
         CK(cudaGetLastError());
     }
     return FFTG_OK;
+}
+
+// Kernels of one iteration in a loop body.
+static long long iteration_launches(const fftg_handle* h) {
+    return !h->mixed ? 8 : pass_blocks(h->N).planes ? 4 : 6;
 }
 
 // Device-resident CG: one graph whose conditional WHILE node repeats the
@@ -764,11 +790,48 @@ static int launch_cg_finish(fftg_handle* h, int nf) {
     return FFTG_OK;
 }
 
+// Blocks per cluster for nf solves: the largest that keeps all of them on the
+// chip together. us an iteration with 16 / 8 / 4 blocks: one cell of 27^3
+// 26 / 44 / 76, eight 34 / 45 / 78, sixteen 58 / 59 / 79, thirty-two 89 / 61 /
+// 80, sixty-four 164 / 120 / 111; 15^3: one 13 / 17 / 23, sixteen 29 / 20 / 24,
+// sixty-four 78 / 42 / 29.
+static int cluster_blocks(int most, int nf) {
+    int c = most;
+    while (c > 4 && (long long)nf * c > (c == 16 ? 160 : 256)) c /= 2;
+    return c;
+}
+
+// Small grids, mixed path: the nf solves as one launch (k_cg_cluster).
+static int launch_cg_cluster(fftg_handle* h, int nf, const void* tangent, long long tstride) {
+    PassArgs a = base_args(h, false);
+    a.aux = h->r;
+    a.aux2 = h->p;
+    a.aux3 = h->x;
+    a.tangent = tangent;
+    a.tstride = tstride;
+    a.out = h->spec;
+    a.cg = h->cg;
+    a.scale = 1.0 / ((double)h->N * h->N * h->N);
+    const int cap = (h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4;
+    const int slot = prof_begin(h, KK_CG_CLUSTER);
+    const cudaError_t e = run_cluster(h->N, a, nf, cluster_blocks(h->cluster, nf), cap, nullptr, h->stream);
+    prof_end(h, slot);
+    CK(e);
+    return FFTG_OK;
+}
+
 // Runs CG iterations until every one of the nf solves is done: as one graph
 // launch (device-resident loop), or, with profiling on or graphs disabled,
 // in chunks enqueued from the host (kernels of a finished solve return at
 // entry, so a chunk may overrun the last iteration without effect).
 static int run_cg(fftg_handle* h, int nf, const void* tangent, long long tstride) {
+    if (h->cluster) {
+        int rc = launch_cg_cluster(h, nf, tangent, tstride);
+        if (rc) return rc;
+        CK(cudaMemcpyAsync(h->h_cg, h->cg, nf * sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaStreamSynchronize(h->stream));
+        return FFTG_OK;
+    }
     const bool profiling = h->prof && h->prof->on;
     if (h->opt.cg_graph && !profiling && !h->graphs_broken) {
         fftg_handle::CgGraph* g = cg_graph_for(h, nf, tangent, tstride);
@@ -784,7 +847,7 @@ static int run_cg(fftg_handle* h, int nf, const void* tangent, long long tstride
             CK(cudaStreamSynchronize(h->stream));
             int maxit = 0;
             for (int f = 0; f < nf; ++f) maxit = std::max(maxit, h->h_cg[f].it);
-            h->launches += (h->mixed ? 6LL : 7LL) * (maxit + 1);
+            h->launches += iteration_launches(h) * (maxit + 1);
             return FFTG_OK;
         }
         h->graphs_broken = true;
@@ -1147,7 +1210,7 @@ int capture_branch(fftg_handle* h, cudaGraph_t top, cudaStream_t s1, cudaStream_
     IncArgs ia = inc_args(h, tol_newton, tol_inner);
     cudaStream_t own = h->stream;
     int rc = FFTG_OK;
-    cudaGraphConditionalHandle cN, cC;
+    cudaGraphConditionalHandle cN = 0, cC = 0;
     cudaGraph_t bodyN = nullptr, bodyC = nullptr;
     h->stream = s1;
     if (cudaStreamBeginCaptureToGraph(s1, top, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
@@ -1171,18 +1234,20 @@ int capture_branch(fftg_handle* h, cudaGraph_t top, cudaStream_t s1, cudaStream_
             cudaSuccess) {
             rc = FFTG_ECUDA;
         } else {
-            if (cudaGraphConditionalHandleCreate(&cC, bodyN, 1, cudaGraphCondAssignDefault) != cudaSuccess) {
+            if (!h->cluster &&
+                cudaGraphConditionalHandleCreate(&cC, bodyN, 1, cudaGraphCondAssignDefault) != cudaSuccess) {
                 rc = FFTG_ECUDA;
             } else {
-                k_inc_cg_reset<<<1, kThreads, 0, s2>>>(cC, ia);
+                k_inc_cg_reset<<<1, kThreads, 0, s2>>>(cC, !h->cluster, ia);
                 if (cudaGetLastError() != cudaSuccess) rc = FFTG_ECUDA;
             }
             if (rc == FFTG_OK) rc = launch_constitutive(h, h->active, h->B, 0, h->eps_work, h->sigma, false, h->cg);
             if (rc == FFTG_OK) rc = launch_residual(h);
             if (rc == FFTG_OK) rc = launch_bounds(h, h->tangent, 7 * h->cs, h->B, 1, h->active);
-            if (rc == FFTG_OK) rc = add_while(s2, cC, &bodyC);
-            // the CG body
-            if (rc == FFTG_OK) {
+            // the CG solves: one launch on small grids, else a loop
+            if (rc == FFTG_OK && h->cluster) rc = launch_cg_cluster(h, h->B, h->tangent, 7 * h->cs);
+            if (rc == FFTG_OK && !h->cluster) rc = add_while(s2, cC, &bodyC);
+            if (rc == FFTG_OK && !h->cluster) {
                 h->stream = s3;
                 if (cudaStreamBeginCaptureToGraph(s3, bodyC, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) !=
                     cudaSuccess) {
@@ -1371,7 +1436,8 @@ int fftg_group_step(fftg_group* g, const double* dE, const int* run, double tol_
         // stress update, four of the right-hand side, four of the solution,
         // decide); per CG loop pass the iteration's kernels (an upper bound
         // when the cells' CG counts differ between Newton passes)
-        const long long per_newton = h->mixed ? 11 : 10, per_cg = h->mixed ? 6 : 7;
+        const long long per_newton = (h->mixed ? 11 : 10) + (h->cluster ? 1 : 0);
+        const long long per_cg = h->cluster ? 0 : iteration_launches(h);
         const long long n = 4 + per_newton * max_newton + per_cg * (max_cg + max_newton);
         h->launches += n;
         g->launches += n;
@@ -1527,6 +1593,10 @@ int fftg_create_batch(fftg_handle** out, int N, int ncells, const uint8_t* phase
         cudaStreamSynchronize(s) != cudaSuccess) {
         h->last_cuda = cudaGetLastError();
         return fail(FFTG_ECUDA);
+    }
+    if (h->mixed && run_cluster(N, PassArgs{}, 0, 0, 0, &h->cluster, s) != cudaSuccess) {
+        cudaGetLastError();
+        h->cluster = 0;
     }
     *out = h;
     return FFTG_OK;

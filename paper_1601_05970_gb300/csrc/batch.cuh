@@ -72,8 +72,8 @@ __global__ void k_inc_begin(cudaGraphConditionalHandle newton_cond, IncArgs a) {
 
 // Start of a Newton iteration: fresh CG states for the active cells (the
 // others are marked converged, so their CG kernels return at entry); the
-// CG loop's condition starts true.
-__global__ void k_inc_cg_reset(cudaGraphConditionalHandle cg_cond, IncArgs a) {
+// CG loop's condition starts true (has_loop: there is one).
+__global__ void k_inc_cg_reset(cudaGraphConditionalHandle cg_cond, bool has_loop, IncArgs a) {
     for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
         CGState c = a.cg_template;
         c.done = a.active[b] ? CG_RUNNING : CG_CONVERGED;
@@ -81,7 +81,7 @@ __global__ void k_inc_cg_reset(cudaGraphConditionalHandle cg_cond, IncArgs a) {
     }
     if (threadIdx.x == 0) {
         *a.cg_guard = 0u;
-        cudaGraphSetConditional(cg_cond, 1u);
+        if (has_loop) cudaGraphSetConditional(cg_cond, 1u);
     }
 }
 

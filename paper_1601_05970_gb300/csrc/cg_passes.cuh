@@ -126,30 +126,21 @@ __device__ __forceinline__ int signed_freq(int k, int N) { return k <= (N - 1) /
 //
 // FS (finite strain): the vectors are a_i of gradient fields a(x)f, and six
 // fields go on: f1 a_i and a_i (the x2 pass applies f2 and f3 to the latter).
-template <int N, int MODE, bool FS = false>
-__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
+template <int N, int MODE, bool FS, int NT, bool GROUP>
+__device__ __forceinline__ void x1i_tile(int tile, int k2g, int it, float alpha, float beta, bool pend,
+                                         const cplx<float>* r, cplx<float>* p, cplx<float>* x, cplx<float>* sp,
+                                         cplx<float>* buf, const cplx<float>* tw, int tid, int bar) {
     using T = float;
     using S = X1<N>;
-    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W, NT = S::NT;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
-    cplx<T>* tw = buf + 6 * N * W;
-    const int f = blockIdx.z;
-    if (a.active && !a.active[f]) return;
-    const CGState* cg = a.cg + f;
-    if (MODE == X1I_CG && cg->done) return;
-    const int tid = threadIdx.x;
-    load_tw<T>(tw, a.tw, N);
-    const int col0 = blockIdx.x * W, k2g = blockIdx.y;
-    const long long NH = (long long)N * HP, vo = f * coef_field<N>() + coef_tile<N>(blockIdx.x, k2g);
-    const cplx<T>* r = (const cplx<T>*)a.aux + vo;
-    cplx<T>* p = (cplx<T>*)a.aux2 + vo;
-    cplx<T>* x = (cplx<T>*)a.aux3 + vo;
-    const int it = cg->it;
-    const T alpha = (T)cg->alpha, beta = (T)cg->beta;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W;
+    const int col0 = tile * W;
+    const long long NH = (long long)N * HP, vo = coef_tile<N>(tile, k2g);
+    r += vo;
+    p += vo;
+    x += vo;
+    sp += (long long)k2g * HP;
     // X1I_CG: iteration it adds step it - 1. X1I_SOLUTION: x holds a value
     // after step it - 1 was added, by the iteration that followed it.
-    const bool pend = cg->pend != 0;
     const bool has_x = MODE == X1I_CG ? it > 1 : (pend ? it > 1 : it > 0);
     constexpr T is = CoefScale<N>::inverse;
     const T g2 = is * (T)signed_freq(k2g, N);
@@ -220,7 +211,7 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) st_pair(b + c * N * W, v[c]);
     }
-    __syncthreads();
+    tile_sync<NT, GROUP>(bar);
     constexpr int P = 6 * W;
     if (N2 > 1) {
         for (int j = tid; j < P * N1; j += NT) {
@@ -228,9 +219,8 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
             const int c = pc / W, w = pc - c * W;
             if (col0 + w < H) invB<N, N1, false, T>(buf + c * N * W + w, W, buf + c * N * W + w, W, k1, tw);
         }
-        __syncthreads();
+        tile_sync<NT, GROUP>(bar);
     }
-    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)k2g * HP;
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
         const int c = pc / W, w = pc - c * W, col = col0 + w;
@@ -239,30 +229,46 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
     }
 }
 
+template <int N, int MODE, bool FS = false>
+__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1i(PassArgs a) {
+    using T = float;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
+    cplx<T>* tw = buf + 6 * N * X1<N>::W;
+    const int f = blockIdx.z;
+    if (a.active && !a.active[f]) return;
+    const CGState* cg = a.cg + f;
+    if (MODE == X1I_CG && cg->done) return;
+    load_tw<T>(tw, a.tw, N);
+    const long long vf = f * coef_field<N>();
+    x1i_tile<N, MODE, FS, X1<N>::NT, false>(blockIdx.x, blockIdx.y, cg->it, (T)cg->alpha, (T)cg->beta, cg->pend != 0,
+                                            (const cplx<T>*)a.aux + vf, (cplx<T>*)a.aux2 + vf,
+                                            (cplx<T>*)a.aux3 + vf, (cplx<T>*)a.out + f * a.sstride, buf, tw,
+                                            threadIdx.x, 0);
+}
+
+// Sum of in[0 .. n) by one warp in a fixed order, in every lane.
+__device__ __forceinline__ double warp_total(const double* in, int n, int lane) {
+    double acc = 0.0;
+    for (int b = lane; b < n; b += 32) acc += __ldcg(in + b);
+    return warp_sum(acc);
+}
+
 // ---------------------------------------------------------------- x1 forward
 // in = spectrum of tau, aux3 = r. X1F_CG: r -= alpha w and the block's part
 // of <r, r>; X1F_RHS: r = w with scale the sign and 1/N^3 of the right-hand
 // side, and the parts of <r, r> and of ||G tau||^2 before rounding.
 // FS: t_i = f1 A_i1 + B_i of the six fields that the x2 pass leaves, w = t / q.
-template <int N, int MODE, bool FS = false>
-__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
+template <int N, int MODE, bool FS, int NT, bool GROUP>
+__device__ __forceinline__ float x1f_tile(int tile, int k2g, float step, const cplx<float>* sp, cplx<float>* r,
+                                          cplx<float>* buf, const cplx<float>* tw, int tid, int bar) {
     using T = float;
     using S = X1<N>;
-    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W, NT = S::NT;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
-    cplx<T>* tw = buf + 6 * N * W;
-    const int f = blockIdx.z;
-    if (a.active && !a.active[f]) return;
-    const CGState* cg = a.cg + f;
-    if (MODE == X1F_CG && cg->done) return;
-    const int tid = threadIdx.x;
-    load_tw<T>(tw, a.tw, N);
-    __syncthreads();
-    const int col0 = blockIdx.x * W, k2g = blockIdx.y;
+    constexpr int N1 = S::N1, N2 = S::N2, H = S::H, HP = S::HP, W = S::W;
+    const int col0 = tile * W;
     const long long NH = (long long)N * HP;
-    const cplx<T>* sp = (const cplx<T>*)a.in + f * a.sstride + (long long)k2g * HP;
-    cplx<T>* r = (cplx<T>*)a.aux3 + f * coef_field<N>() + coef_tile<N>(blockIdx.x, k2g);
+    sp += (long long)k2g * HP;
+    r += coef_tile<N>(tile, k2g);
     constexpr int P = 6 * W;
     for (int j = tid; j < P * N2; j += NT) {
         const int pc = j % P, t = j / P;
@@ -270,18 +276,16 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
         const int comp = FS ? fs_slot(c) : c;
         if (col < H) fwdA<N, N1, T>(sp + comp * N * NH + col, (int)NH, buf + c * N * W + w, W, t, tw);
     }
-    __syncthreads();
+    tile_sync<NT, GROUP>(bar);
     if (N2 > 1) {
         for (int j = tid; j < P * N1; j += NT) {
             const int pc = j % P, k1 = j / P;
             const int c = pc / W, w = pc - c * W;
             if (col0 + w < H) fwdB<N, N1, false, T>(buf + c * N * W + w, W, buf + c * N * W + w, W, k1, tw);
         }
-        __syncthreads();
+        tile_sync<NT, GROUP>(bar);
     }
     const T f2 = (T)signed_freq(k2g, N);
-    const double unit = (double)CoefScale<N>::value * a.scale;
-    const T step = MODE == X1F_CG ? (T)(-cg->alpha * unit) : (T)unit;
     T acc = T(0);
     for (int j = tid; j < (W / 2) * N; j += NT) {
         const int w = 2 * (j % (W / 2)), kk = j / (W / 2), col = col0 + w;
@@ -330,8 +334,27 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
 #pragma unroll
         for (int i = 0; i < 3; ++i) st_pair(r + o + i * N * W, z[i]);
     }
+    return acc;
+}
+
+template <int N, int MODE, bool FS = false>
+__global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
+    using T = float;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);  // [6][N][W]
+    cplx<T>* tw = buf + 6 * N * X1<N>::W;
+    const int f = blockIdx.z;
+    if (a.active && !a.active[f]) return;
+    const CGState* cg = a.cg + f;
+    if (MODE == X1F_CG && cg->done) return;
+    load_tw<T>(tw, a.tw, N);
+    __syncthreads();
+    const double unit = (double)CoefScale<N>::value * a.scale;
+    const T acc = x1f_tile<N, MODE, FS, X1<N>::NT, false>(
+        blockIdx.x, blockIdx.y, MODE == X1F_CG ? (T)(-cg->alpha * unit) : (T)unit,
+        (const cplx<T>*)a.in + f * a.sstride, (cplx<T>*)a.aux3 + f * coef_field<N>(), buf, tw, threadIdx.x, 0);
     const double s = block_sum_any((double)acc) * (FS ? 0.5 : 1.0) * CoefScale<N>::square;
-    if (tid == 0) {
+    if (threadIdx.x == 0) {
         const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
         if (MODE == X1F_CG) {
             a.partials[f * nb + b] = s;
@@ -490,25 +513,18 @@ struct RowCfg {
     static constexpr int blocks = (N * N + R - 1) / R;
 };
 
-template <int N, int NA, int TV>
-__global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB) k_rows_cg(PassArgs a) {
+// `sp` and `tg` are those of the rows row0 .. row0 + R of `rows`; the spectrum
+// has the pitch HP and component stride HS (global or shared memory), and the
+// tangent is read VW voxels a lane (VW = 2: even offsets).
+template <int N, int N1, int R, int NT, bool GROUP, int HP, int VW>
+__device__ __forceinline__ void rows_tile(int row0, int rows, cplx<float>* sp, long long HS, const float* tg,
+                                          long long cs, cplx<float>* z, const cplx<float>* tw, double* warp_part,
+                                          int tid, int bar) {
     using T = float;
-    using S = RowCfg<N, NA, TV>;
-    constexpr int R = S::R, H = (N + 1) / 2, HP = spec_pitch(N), NT = S::NT;
-    constexpr int N1 = S::N1, N2 = S::N2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<T>* z = reinterpret_cast<cplx<T>*>(smem_raw);  // [3][R][N]
-    cplx<T>* tw = z + 3 * R * N;
-    const int f = blockIdx.z;
-    if (a.cg[f].done) return;
-    const int tid = threadIdx.x;
-    load_tw<T>(tw, a.tw, N);
-    const int row0 = blockIdx.x * R;
-    const int nrows = min(R, N * N - row0);
-    const long long HS = (long long)N * N * HP;
-    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride + (long long)row0 * HP;
-    const long long cs = a.cs;
-    const T* tg = (const T*)a.tangent + f * a.tstride + (long long)row0 * N;
+    constexpr int H = (N + 1) / 2, N2 = N / N1;
+    const int nrows = min(R, rows - row0);
+    sp += (long long)row0 * HP;
+    tg += (long long)row0 * N;
     // the half spectra of two real components -> one complex row; the
     // imaginary parts at k = 0 are rounding and are dropped
     constexpr int NRL = (R * H + NT - 1) / NT;
@@ -549,27 +565,25 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
             }
         }
     }
-    __syncthreads();
+    tile_sync<NT, GROUP>(bar);
     constexpr int NP = 3 * R;
     if (N2 > 1) {
         for (int it = tid; it < NP * N1; it += NT) {
             const int pc = it % NP, k1 = it / NP;
             if (pc % R < nrows) invB<N, N1, false, T>(z + pc * N, 1, z + pc * N, 1, k1, tw);
         }
-        __syncthreads();
+        tile_sync<NT, GROUP>(bar);
     }
     for (int it = tid; it < NP * N2; it += NT) {
         const int pc = it % NP, t = it / NP;
         if (pc % R < nrows) invA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
     }
-    __syncthreads();
-    // tau = C : p, two voxels a lane (R is a multiple of 4, so a block
-    // starts on a vector boundary; in the last block the vector that
+    tile_sync<NT, GROUP>(bar);
+    // tau = C : p (VW = 2: R N is even; in the last block the vector that
     // straddles the end of the grid reads the padding of the tangent and
     // changes rows that no stage reads)
     const int nel = nrows * N;
     T pcp = T(0);
-    constexpr int VW = 2;
     for (int j = tid; j < (R * N) / VW; j += NT) {
         const int i0 = j * VW;
         if (i0 >= nel) continue;
@@ -579,13 +593,11 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
         cplx<T> s[3][VW];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float4* zv = reinterpret_cast<const float4*>(z + c * R * N + i0);
-#pragma unroll
-            for (int e = 0; e < VW; e += 2) {
-                const float4 v = zv[e / 2];
-                s[c][e] = mk(v.x, v.y);
-                s[c][e + 1] = mk(v.z, v.w);
-            }
+            const cplx<T>* zc = z + c * R * N + i0;
+            if constexpr (VW == 2)
+                ld_pair(zc, s[c]);
+            else
+                s[c][0] = zc[0];
         }
 #pragma unroll
         for (int e = 0; e < VW; ++e) {
@@ -598,34 +610,29 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            float4* zv = reinterpret_cast<float4*>(z + c * R * N + i0);
-#pragma unroll
-            for (int e = 0; e < VW; e += 2) zv[e / 2] = make_float4(s[c][e].x, s[c][e].y, s[c][e + 1].x, s[c][e + 1].y);
+            cplx<T>* zc = z + c * R * N + i0;
+            if constexpr (VW == 2)
+                st_pair(zc, s[c]);
+            else
+                zc[0] = s[c][0];
         }
     }
-    __shared__ double pcp_warp[NT / 32];
     {
         const double wv = warp_sum((double)pcp);
-        if ((tid & 31) == 0) pcp_warp[tid >> 5] = wv;
+        if ((tid & 31) == 0) warp_part[tid >> 5] = wv;
     }
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < NT / 32; ++w) t += pcp_warp[w];
-        a.partials[(size_t)f * gridDim.x + blockIdx.x] = t;
-    }
+    tile_sync<NT, GROUP>(bar);
     for (int it = tid; it < NP * N2; it += NT) {
         const int pc = it % NP, t = it / NP;
         if (pc % R < nrows) fwdA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
     }
-    __syncthreads();
+    tile_sync<NT, GROUP>(bar);
     if (N2 > 1) {
         for (int it = tid; it < NP * N1; it += NT) {
             const int pc = it % NP, k1 = it / NP;
             if (pc % R < nrows) fwdB<N, N1, false, T>(z + pc * N, 1, z + pc * N, 1, k1, tw);
         }
-        __syncthreads();
+        tile_sync<NT, GROUP>(bar);
     }
     for (int it = tid; it < nrows * H; it += NT) {
         const int row = it / H, k = it - row * H, o = row * HP + k;
@@ -639,6 +646,242 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
             sp[(2 * c + 1) * HS + o] = half_of(mk(d.y, -d.x));
         }
     }
+}
+
+template <int N, int NA, int TV>
+__global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB) k_rows_cg(PassArgs a) {
+    using T = float;
+    using S = RowCfg<N, NA, TV>;
+    constexpr int R = S::R, NT = S::NT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double pcp_warp[NT / 32];
+    cplx<T>* z = reinterpret_cast<cplx<T>*>(smem_raw);  // [3][R][N]
+    cplx<T>* tw = z + 3 * R * N;
+    const int f = blockIdx.z;
+    if (a.cg[f].done) return;
+    load_tw<T>(tw, a.tw, N);
+    constexpr int HP = spec_pitch(N);
+    rows_tile<N, NA, R, NT, false, HP, 2>(blockIdx.x * R, N * N, (cplx<T>*)a.out + f * a.sstride,
+                                          (long long)N * N * HP, (const T*)a.tangent + f * a.tstride, a.cs, z, tw,
+                                          pcp_warp, threadIdx.x, 0);
+    // the block's part of <p, C : p> (written before the last barriers)
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) t += pcp_warp[w];
+        a.partials[(size_t)f * gridDim.x + blockIdx.x] = t;
+    }
+}
+
+// -------------------------------------------------------------------- planes
+// P4, the row pass and P2 act within one x1 plane. Where a plane's six
+// components are small in shared memory one block takes it through all three:
+// 76 B per voxel from and to global memory instead of 173, and two launches
+// less an iteration. An iteration takes 39 instead of 50 us on one cell of
+// 45^3 and 122 instead of 131 on sixteen. At 75^3 a plane takes 209 KB, one
+// block of 20 warps an SM: 64 instead of 65 us on one cell but 508 instead of
+// 481 on sixteen, so the line lies below it.
+template <int N>
+struct PlaneCfg {
+    static constexpr bool ok = N <= 45;
+    static constexpr int H = (N + 1) / 2, N1 = N == 3 || N == 5 ? N : X1Split<N>::N1, N2 = N / N1;
+    // groups of GT threads share the rows, R a turn (R even)
+    static constexpr int GT = 128, G = N <= 27 ? 4 : 3, R = 8, NT = GT * G, MINB = 2;
+    static constexpr int row_tiles = (N + R - 1) / R;
+    static constexpr int elems = 6 * N * H + (6 * N * H & 1) + G * 3 * R * N;  // plane, then the groups' rows
+    static constexpr size_t smem = (size_t)(elems + N) * 8;
+    static_assert(!ok || smem <= 227 * 1024, "shared memory per block");
+};
+
+// One x1 plane by the NT threads of the block: `sp` and `tg` are the plane's.
+// The plane's <p, C : p> is left in group_part, one number a group.
+template <int N>
+__device__ __forceinline__ void plane_tile(cplx<float>* sp, const float* tg, long long cs, cplx<float>* buf,
+                                           const cplx<float>* tw, double* warp_part, double* group_part) {
+    using T = float;
+    using S = PlaneCfg<N>;
+    constexpr int H = S::H, HP = spec_pitch(N), N1 = S::N1, N2 = S::N2, NT = S::NT, GT = S::GT, P = 6 * H;
+    const long long comp = (long long)N * N * HP;
+    for (int it = threadIdx.x; it < P * N1; it += NT) {
+        const int pc = it % P, k1 = it / P;
+        const int c = pc / H, w = pc - c * H;
+        invB<N, N1, true, T>(sp + c * comp + w, HP, buf + c * N * H + w, H, k1, tw);
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < P * N2; it += NT) {
+        const int pc = it % P, t = it / P;
+        cplx<T>* b = buf + (pc / H) * N * H + pc % H;
+        invA<N, N1, T>(b, H, b, H, t, tw);
+    }
+    __syncthreads();
+    {
+        const int g = threadIdx.x / GT, tid = threadIdx.x - g * GT;
+        cplx<T>* z = buf + 6 * N * H + (6 * N * H & 1) + g * 3 * S::R * N;
+        double* wp = warp_part + g * (GT / 32);
+        double sum = 0.0;
+        for (int j = g; j < S::row_tiles; j += S::G) {
+            rows_tile<N, RowSplit<N>::N1, S::R, GT, true, H, 1>(j * S::R, N, buf, N * H, tg, cs, z, tw, wp, tid, 1 + g);
+            if (tid == 0)
+                for (int w = 0; w < GT / 32; ++w) sum += wp[w];
+            tile_sync<GT, true>(1 + g);
+        }
+        if (tid == 0) group_part[g] = sum;
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < P * N2; it += NT) {
+        const int pc = it % P, t = it / P;
+        cplx<T>* b = buf + (pc / H) * N * H + pc % H;
+        fwdA<N, N1, T>(b, H, b, H, t, tw);
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < P * N1; it += NT) {
+        const int pc = it % P, k1 = it / P;
+        const int c = pc / H, w = pc - c * H;
+        fwdB<N, N1, true, T>(buf + c * N * H + w, H, sp + c * comp + w, HP, k1, tw);
+    }
+}
+
+// The plane's part of <p, C : p>, after a barrier (thread 0).
+template <int N>
+__device__ __forceinline__ double plane_part(const double* group_part) {
+    double t = 0.0;
+#pragma unroll
+    for (int g = 0; g < PlaneCfg<N>::G; ++g) t += group_part[g];
+    return t;
+}
+
+template <int N>
+__global__ void __launch_bounds__(PlaneCfg<N>::NT, PlaneCfg<N>::MINB) k_plane_cg(PassArgs a) {
+    using T = float;
+    using S = PlaneCfg<N>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double warp_part[S::NT / 32], group_part[S::G];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
+    cplx<T>* tw = buf + S::elems;
+    const int f = blockIdx.z;
+    if (a.cg[f].done) return;
+    load_tw<T>(tw, a.tw, N);
+    __syncthreads();
+    plane_tile<N>((cplx<T>*)a.out + f * a.sstride + (long long)blockIdx.x * N * spec_pitch(N),
+                  (const T*)a.tangent + f * a.tstride + (long long)blockIdx.x * N * N, a.cs, buf, tw, warp_part,
+                  group_part);
+    // the field's last block sums the planes' parts of <p, C : p>: alpha
+    __shared__ bool last;
+    double* part = a.partials + (size_t)f * N;
+    CGState* cg = a.cg + f;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = plane_part<N>(group_part);
+        __threadfence();
+        last = atomicAdd(&cg->ticket, 1u) == N - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    const double pq = warp_total(part, N, threadIdx.x);
+    if (threadIdx.x == 0) {
+        cg->ticket = 0u;
+        cg_after_dot(cg, pq);
+    }
+}
+
+// --------------------------------------------------------------- small grids
+// The whole CG solve of a field by one thread-block cluster: below 45^3 an
+// iteration's six kernels do a few microseconds of work each, and launches
+// and the loop's condition take most of the time. The phases are those above,
+// x1 tiles over groups of GT threads and planes over the blocks, with the
+// hardware's cluster barrier (which orders global memory within the cluster)
+// between them; every block
+// keeps the solve's scalars and takes the same steps, block 0 writes them
+// back. The blocks of a cluster are resident together by construction, so no
+// wait depends on another launch. An iteration takes 11 instead of 37 us on one
+// cell of 15^3, 23 instead of 39 on one of 27^3 and 59 instead of 78 on
+// thirty-two of them.
+template <int N>
+struct ClusterCg {
+    static constexpr bool ok = N <= 27;
+    using PL = PlaneCfg<N>;
+    static constexpr int GT = PL::GT, G = PL::G, NT = PL::NT;
+    static constexpr int x1_elems = G * 6 * N * X1<N>::W;
+    static constexpr int elems = x1_elems > PL::elems ? x1_elems : PL::elems;
+    static constexpr size_t smem = (size_t)(elems + N) * 8;
+    // partial sums of a field: one of each plane, then one of each x1 tile
+    static constexpr int partials = N + X1<N>::blocks;
+};
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int N>
+__global__ void __launch_bounds__(ClusterCg<N>::NT, 2) k_cg_cluster(PassArgs a, int cl, int cap) {
+    using T = float;
+    using S = ClusterCg<N>;
+    constexpr int GT = S::GT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ CGState st;
+    __shared__ double warp_part[S::NT / 32], group_part[S::G];
+    const int f = blockIdx.x / cl, rank = blockIdx.x - f * cl;
+    if (a.cg[f].done) return;  // the same for every block of the cluster
+    const int tid = threadIdx.x % GT, g = threadIdx.x / GT, bar = 1 + g;
+    const int group = rank * S::G + g, groups = cl * S::G;
+    cplx<T>* all = reinterpret_cast<cplx<T>*>(smem_raw);
+    cplx<T>* buf = all + g * 6 * N * X1<N>::W;
+    cplx<T>* tw = all + S::elems;
+    double* wp = warp_part + g * (GT / 32);
+    load_tw<T>(tw, a.tw, N);
+    if (threadIdx.x == 0) st = a.cg[f];
+    __syncthreads();
+    const long long vf = f * coef_field<N>();
+    cplx<T>* r = (cplx<T>*)a.aux + vf;
+    cplx<T>* p = (cplx<T>*)a.aux2 + vf;
+    cplx<T>* x = (cplx<T>*)a.aux3 + vf;
+    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride;
+    const T* tg = (const T*)a.tangent + f * a.tstride;
+    double* part = a.partials + (size_t)f * S::partials;
+    double* part_x1 = part + N;
+    const double unit = (double)CoefScale<N>::value * a.scale;
+    for (int pass = 0; pass < cap && st.done == CG_RUNNING; ++pass) {
+        for (int j = group; j < X1<N>::blocks; j += groups) {
+            x1i_tile<N, X1I_CG, false, GT, true>(j % X1<N>::tiles, j / X1<N>::tiles, st.it, (T)st.alpha, (T)st.beta,
+                                                 st.pend != 0, r, p, x, sp, buf, tw, tid, bar);
+            tile_sync<GT, true>(bar);  // the tile's buffer is free again
+        }
+        cluster_sync();
+        for (int j = rank; j < N; j += cl) {
+            plane_tile<N>(sp + (long long)j * N * spec_pitch(N), tg + (long long)j * N * N, a.cs, all, tw, warp_part,
+                          group_part);
+            if (threadIdx.x == 0) part[j] = plane_part<N>(group_part);
+            __syncthreads();
+        }
+        cluster_sync();
+        if (threadIdx.x < 32) {
+            const double pq = warp_total(part, N, threadIdx.x);
+            if (threadIdx.x == 0) cg_after_dot(&st, pq);
+        }
+        __syncthreads();
+        if (st.done != CG_RUNNING) break;  // the same in every block
+        for (int j = group; j < X1<N>::blocks; j += groups) {
+            const T acc = x1f_tile<N, X1F_CG, false, GT, true>(j % X1<N>::tiles, j / X1<N>::tiles,
+                                                               (T)(-st.alpha * unit), sp, r, buf, tw, tid, bar);
+            const double wv = warp_sum((double)acc);
+            if ((tid & 31) == 0) wp[tid >> 5] = wv;
+            tile_sync<GT, true>(bar);
+            if (tid == 0) {
+                double t = 0.0;
+#pragma unroll
+                for (int w = 0; w < GT / 32; ++w) t += wp[w];
+                part_x1[j] = t * CoefScale<N>::square;
+            }
+            tile_sync<GT, true>(bar);
+        }
+        cluster_sync();
+        if (threadIdx.x < 32) {
+            const double rr = warp_total(part_x1, X1<N>::blocks, threadIdx.x);
+            if (threadIdx.x == 0) cg_after_update(&st, rr);
+        }
+        __syncthreads();
+    }
+    if (rank == 0 && threadIdx.x == 0) a.cg[f] = st;
 }
 
 // ------------------------------------------------------------------ launcher
@@ -700,11 +943,60 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_X1F_CG_F32: return launch_k(k_x1f<N, X1F_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1F_RHS_F32: return launch_k(k_x1f<N, X1F_RHS>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1F_RHS_DD: return launch_k(k_x1f_dd<N>, gdd, CDD::smem_p3, a, s, CDD::T3);
+        case PK_PLANE_CG_F32: {
+            using S = PlaneCfg<N>;
+            if constexpr (S::ok)
+                return launch_k(k_plane_cg<N>, dim3(N, 1, nf), S::smem, a, s, S::NT);
+            else
+                return cudaErrorInvalidValue;
+        }
         case PK_ROWS_CG_F32: {
             using R = RowCfg<N, RowSplit<N>::N1, 0>;
             return launch_k(k_rows_cg<N, RowSplit<N>::N1, 0>, dim3(R::blocks, 1, nf), R::smem, a, s, R::NT);
         }
         default: return cudaErrorInvalidValue;
+    }
+}
+
+// The solve of nf fields by clusters of cl blocks (cl = 0: the largest size,
+// 16 or 8, that the device takes, or 0, is written to *size and nothing runs).
+template <int N>
+cudaError_t run_cluster_n(const PassArgs& a, int nf, int cl, int cap, int* size, cudaStream_t s) {
+    if constexpr (!ClusterCg<N>::ok) {
+        if (size) *size = 0;
+        return cl ? cudaErrorInvalidValue : cudaSuccess;
+    } else {
+        using S = ClusterCg<N>;
+        cudaError_t e = cudaFuncSetAttribute(k_cg_cluster<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_cg_cluster<N>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.blockDim = dim3(S::NT);
+        cfg.dynamicSmemBytes = S::smem;
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cl) {
+            at.val.clusterDim.x = cl;
+            cfg.gridDim = dim3(nf * cl);
+            return cudaLaunchKernelEx(&cfg, k_cg_cluster<N>, a, cl, cap);
+        }
+        *size = 0;
+        for (int c : {16, 8}) {
+            int n = 0;
+            at.val.clusterDim.x = c;
+            cfg.gridDim = dim3(c);
+            if (cudaOccupancyMaxActiveClusters(&n, k_cg_cluster<N>, &cfg) == cudaSuccess && n > 0) {
+                *size = c;
+                break;
+            }
+            cudaGetLastError();
+        }
+        return cudaSuccess;
     }
 }
 

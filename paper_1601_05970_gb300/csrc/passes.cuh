@@ -457,15 +457,61 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     }
 }
 
+// Barrier of the NT threads that share a tile: the block, or (GROUP) one of
+// its groups by the hardware barrier `bar`.
+template <int NT, bool GROUP>
+__device__ __forceinline__ void tile_sync(int bar) {
+    if constexpr (GROUP)
+        asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+    else
+        __syncthreads();
+}
+
 // -------------------------------------------------------------- P2 / P4 (x2)
+// S slabs x W columns by NT threads. A slab is one (component, x1) plane of
+// the spectrum `sp` of one field; slabs of them in all (6 N here, 9 N in the
+// finite-strain passes).
+template <int N, typename T, bool FWD, int N1, int W, int S, int NT, bool GROUP>
+__device__ __forceinline__ void p24_tile(cplx<T>* sp, cplx<T>* buf, const cplx<T>* tw, int col0, int slab0, int slabs,
+                                         int tid, int bar) {
+    constexpr int H = (N + 1) / 2, HP = spec_pitch(N), N2 = N / N1, P = S * W;
+    if (FWD) {
+        for (int it = tid; it < P * N2; it += NT) {
+            const int pc = it % P, t = it / P;
+            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
+            if (col < H && slab < slabs)
+                fwdA<N, N1, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, t, tw);
+        }
+        tile_sync<NT, GROUP>(bar);
+        for (int it = tid; it < P * N1; it += NT) {
+            const int pc = it % P, k1 = it / P;
+            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
+            if (col < H && slab < slabs)
+                fwdB<N, N1, true, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, k1, tw);
+        }
+    } else {
+        for (int it = tid; it < P * N1; it += NT) {
+            const int pc = it % P, k1 = it / P;
+            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
+            if (col < H && slab < slabs)
+                invB<N, N1, true, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, k1, tw);
+        }
+        tile_sync<NT, GROUP>(bar);
+        for (int it = tid; it < P * N2; it += NT) {
+            const int pc = it % P, t = it / P;
+            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
+            if (col < H && slab < slabs)
+                invA<N, N1, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, t, tw);
+        }
+    }
+}
+
 // Blocks of T2 = (slabs x columns x N2) threads: stage A is one item per
-// thread; stage B takes N1/N2 rounds. A slab is one (component, x1) plane
-// of the spectrum; NC components (6 here, 9 in the finite-strain passes).
+// thread; stage B takes N1/N2 rounds.
 template <int N, typename T, bool FWD, int NC = 6, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T2) k_p24(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
-    constexpr int H = C::H, HP = C::HP, W = C::W2, S = C::S2, NT = C::T2;
-    constexpr int N1 = NA, N2 = N / NA;
+    constexpr int W = C::W2, S = C::S2, NT = C::T2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* buf = tw + N;  // [S][N][W]
@@ -485,38 +531,8 @@ __global__ void __launch_bounds__(Cfg<N, T, NA, TV>::T2) k_p24(PassArgs a) {
     }
     load_tw<T>(tw, a.tw, N);
     __syncthreads();
-    const int col0 = blockIdx.x * W, slab0 = blockIdx.y * S;
-    cplx<T>* sp = (cplx<T>*)a.out + f * a.sstride;
-    constexpr int P = S * W;
-    if (FWD) {
-        for (int it = tid; it < P * N2; it += NT) {
-            const int pc = it % P, t = it / P;
-            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
-            if (col < H && slab < NC * N)
-                fwdA<N, N1, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, t, tw);
-        }
-        __syncthreads();
-        for (int it = tid; it < P * N1; it += NT) {
-            const int pc = it % P, k1 = it / P;
-            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
-            if (col < H && slab < NC * N)
-                fwdB<N, N1, true, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, k1, tw);
-        }
-    } else {
-        for (int it = tid; it < P * N1; it += NT) {
-            const int pc = it % P, k1 = it / P;
-            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
-            if (col < H && slab < NC * N)
-                invB<N, N1, true, T>(sp + (long long)slab * N * HP + col, HP, buf + s * N * W + w, W, k1, tw);
-        }
-        __syncthreads();
-        for (int it = tid; it < P * N2; it += NT) {
-            const int pc = it % P, t = it / P;
-            const int s = pc / W, w = pc - s * W, col = col0 + w, slab = slab0 + s;
-            if (col < H && slab < NC * N)
-                invA<N, N1, T>(buf + s * N * W + w, W, sp + (long long)slab * N * HP + col, HP, t, tw);
-        }
-    }
+    p24_tile<N, T, FWD, NA, W, S, NT, false>((cplx<T>*)a.out + f * a.sstride, buf, tw, blockIdx.x * W, blockIdx.y * S,
+                                             NC * N, tid, 0);
 }
 
 // 1/sqrt(x): CUDA's rsqrtf (about 2 ulp, far inside the FP32 path's
@@ -964,7 +980,7 @@ enum PassKind : int {
     // double-float FFTs: FP64 field in and out
     PK_P1_PLAIN_DD, PK_P2_DD, PK_P3_DD, PK_P4_DD, PK_P5_PLAIN_DD_TO_F64,
     // the mixed path's CG on displacement coefficients (cg_passes.cuh)
-    PK_X1I_CG_F32, PK_ROWS_CG_F32, PK_X1F_CG_F32, PK_X1F_RHS_F32, PK_X1F_RHS_DD, PK_X1I_SOLUTION_F32,
+    PK_X1I_CG_F32, PK_ROWS_CG_F32, PK_PLANE_CG_F32, PK_X1F_CG_F32, PK_X1F_RHS_F32, PK_X1F_RHS_DD, PK_X1I_SOLUTION_F32,
     PK_P5_NEWTON_F32,
     // the operators on a caller's fields (U = 1); so are P1_PLAIN_F32, P1_TAN,
     // P5_PLAIN_F64 and P5_PLAIN_DD_TO_F64, which nothing else runs
