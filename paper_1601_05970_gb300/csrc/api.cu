@@ -78,7 +78,7 @@ static int row_blocks_n(bool fp64) {
     return fp64 ? Cfg<N, double>::row_blocks
                 : std::max({Cfg<N, float>::row_blocks, Cfg<N, float, Plan<N>::N1, 1>::row_blocks,
                             RowCfg<N, RowSplit<N>::N1, 1>::blocks, X1<N>::blocks,
-                            (Cfg<N, dd>::H + Cfg<N, dd>::W3 - 1) / Cfg<N, dd>::W3 * N});
+                            (X1dd<N>::H + X1dd<N>::W3 - 1) / X1dd<N>::W3 * N});
 }
 
 int row_blocks(int N, bool fp64) {
@@ -102,7 +102,7 @@ static PassBlocks pass_blocks(int N) {
     switch (N) {
 #define FFTG_CASE(n)                                                                                     \
     case n:                                                                                              \
-        return {X1<n>::blocks, (Cfg<n, dd>::H + Cfg<n, dd>::W3 - 1) / Cfg<n, dd>::W3 * n,                \
+        return {X1<n>::blocks, (X1dd<n>::H + X1dd<n>::W3 - 1) / X1dd<n>::W3 * n,                \
                 Cfg<n, float>::row_blocks, PlaneCfg<n>::ok ? n : 0};
         FFTG_CASE(3) FFTG_CASE(5) FFTG_CASE(9) FFTG_CASE(15) FFTG_CASE(25) FFTG_CASE(27)
         FFTG_CASE(45) FFTG_CASE(75) FFTG_CASE(81) FFTG_CASE(125) FFTG_CASE(135) FFTG_CASE(225)

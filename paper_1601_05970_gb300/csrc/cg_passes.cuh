@@ -386,12 +386,17 @@ __device__ __forceinline__ cplx<dd> dd_scale(cplx<dd> a, float f) {
 // double-float spectrum of the FP64 stress: forward x1 in two stages, then
 // one thread per frequency. The double-float inverse passes that a residual
 // in real space needs (half of its work) are not run.
+// Small grids take two stages (a double-float DFT of 27 points in one thread
+// needs more registers than there are).
+template <int N>
+using X1dd = Cfg<N, dd, N <= 27 ? X1Split<N>::N1 : Plan<N>::N1>;
+
 template <int N, bool FS = false>
-__global__ void __launch_bounds__(Cfg<N, dd>::T3) k_x1f_dd(PassArgs a) {
+__global__ void __launch_bounds__(X1dd<N>::T3) k_x1f_dd(PassArgs a) {
     using T = dd;
-    using C = Cfg<N, T>;
+    using C = X1dd<N>;
     constexpr int H = C::H, HP = C::HP, W = C::W3, NT = C::T3;
-    constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
+    constexpr int N1 = C::PN1, N2 = C::PN2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* buf = tw + N;  // [6][N][W]
@@ -892,7 +897,10 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     using CDD = Cfg<N, dd>;
     static_assert(CDD::row_blocks == C64::row_blocks && CDD::W2 == C64::W2 && CDD::S2 == C64::S2,
                   "double-float row and column passes share the FP64 geometry");
+    using U32 = Cfg<N, float, Plan<N>::N1, 3>;
+    using U64 = Cfg<N, double, Plan<N>::N1, 3>;
     const dim3 r32(C32::row_blocks, 1, nf), r64(C64::row_blocks, 1, nf);
+    const dim3 u32(U32::row_blocks, 1, nf), u64(U64::row_blocks, 1, nf);
     const dim3 c32((C32::H + C32::W2 - 1) / C32::W2, (6 * N + C32::S2 - 1) / C32::S2, nf);
     const dim3 c64((C64::H + C64::W2 - 1) / C64::W2, (6 * N + C64::S2 - 1) / C64::S2, nf);
     const dim3 g64((C64::H + C64::W3 - 1) / C64::W3, N, nf);
@@ -900,9 +908,9 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
     switch (kind) {
         case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s);
-        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN, 1>, r32, C32::smem_rows, a, s);
-        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN, 1>, r64, C64::smem_rows, a, s);
-        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN, 1>, r32, C32::smem_rows, a, s);
+        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
+        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
+        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
         case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s);
         case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s);
         case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s);
@@ -913,17 +921,17 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P3_F64: return launch_k(k_p3<N, double>, g64, C64::smem_p3, a, s, C64::T3);
         case PK_P3_F32: {
             using D = P3Default<N>;
-            using C = Cfg<N, float, D::A, D::TV>;
+            using C = Cfg<N, float, D::A>;
             const dim3 g((C::H + C::W3 - 1) / C::W3, N, nf);
             if constexpr (D::fused)
                 return launch_k(k_p3f<N, D::A>, g, C::smem_p3, a, s, P3f<N, D::A>::NT);
             else
-                return launch_k(k_p3<N, float, D::A, D::TV>, g, C::smem_p3, a, s, C::T3);
+                return launch_k(k_p3<N, float, D::A>, g, C::smem_p3, a, s, C::T3);
         }
-        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double, 1>, r64, C64::smem_rows, a, s);
+        case PK_P5_PLAIN_F64: return launch_k(k_p5<N, double, P5_PLAIN, double, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
         case PK_P5_PLAIN_F32: return launch_k(k_p5<N, float, P5_PLAIN, float>, r32, C32::smem_rows, a, s);
         case PK_P5_DOT_F64: return launch_k(k_p5<N, double, P5_DOT, double>, r64, C64::smem_rows, a, s);
-        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float, 1>, r32, C32::smem_rows, a, s);
+        case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
         case PK_P5_RHS_F64_TO_F64:
             return launch_k(k_p5<N, double, P5_RHS, double>, r64, C64::smem_rows, a, s);
         case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s);
@@ -931,18 +939,21 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P4_DD: return launch_k(k_p24<N, dd, false>, c64, CDD::smem_p24, a, s, CDD::T2);
         case PK_P3_DD: return launch_k(k_p3<N, dd>, gdd, CDD::smem_p3, a, s, CDD::T3);
         case PK_P5_PLAIN_DD_TO_F64:
-            return launch_k(k_p5<N, dd, P5_PLAIN, double, 1>, r64, CDD::smem_rows, a, s);
-        case PK_P1_USER_F64: return launch_k(k_p1<N, double, P1_PLAIN, 1>, r64, C64::smem_rows, a, s);
-        case PK_P1_USER_DD: return launch_k(k_p1<N, dd, P1_PLAIN, 1>, r64, CDD::smem_rows, a, s);
-        case PK_P5_USER_F32: return launch_k(k_p5<N, float, P5_PLAIN, float, 1>, r32, C32::smem_rows, a, s);
+            return launch_k(k_p5<N, dd, P5_PLAIN, double, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
+        case PK_P1_USER_F64: return launch_k(k_p1<N, double, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
+        case PK_P1_USER_DD: return launch_k(k_p1<N, dd, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
+        case PK_P5_USER_F32: return launch_k(k_p5<N, float, P5_PLAIN, float, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
         case PK_P5_DOT_USER_F64:
-            return launch_k(k_p5<N, double, P5_DOT, double, 1>, r64, C64::smem_rows, a, s);
+            return launch_k(k_p5<N, double, P5_DOT, double, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
         case PK_P5_NEWTON_F32: return launch_k(k_p5<N, float, P5_NEWTON, float>, r32, C32::smem_rows, a, s);
         case PK_X1I_CG_F32: return launch_k(k_x1i<N, X1I_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1I_SOLUTION_F32: return launch_k(k_x1i<N, X1I_SOLUTION>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1F_CG_F32: return launch_k(k_x1f<N, X1F_CG>, x32, X1<N>::smem, a, s, X1<N>::NT);
         case PK_X1F_RHS_F32: return launch_k(k_x1f<N, X1F_RHS>, x32, X1<N>::smem, a, s, X1<N>::NT);
-        case PK_X1F_RHS_DD: return launch_k(k_x1f_dd<N>, gdd, CDD::smem_p3, a, s, CDD::T3);
+        case PK_X1F_RHS_DD: {
+            using X = X1dd<N>;
+            return launch_k(k_x1f_dd<N>, dim3((X::H + X::W3 - 1) / X::W3, N, nf), X::smem_p3, a, s, X::T3);
+        }
         case PK_PLANE_CG_F32: {
             using S = PlaneCfg<N>;
             if constexpr (S::ok)

@@ -62,7 +62,7 @@ struct FsBlocks {
 static FsBlocks fs_blocks(int N) {
     switch (N) {
 #define FFTG_CASE(n) \
-    case n: return {FsRowCfg<n>::blocks, X1<n>::blocks, (Cfg<n, dd>::H + Cfg<n, dd>::W3 - 1) / Cfg<n, dd>::W3 * n};
+    case n: return {FsRowCfg<n>::blocks, X1<n>::blocks, (X1dd<n>::H + X1dd<n>::W3 - 1) / X1dd<n>::W3 * n};
         FFTG_FS_GRIDS(FFTG_CASE)
 #undef FFTG_CASE
         default: return {0, 0, 0};

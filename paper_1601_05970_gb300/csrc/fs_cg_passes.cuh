@@ -355,7 +355,7 @@ cudaError_t run_fs_pass_n(FsPassKind kind, const FsArgs& a, cudaStream_t s) {
         case FK_X1F_CG_F32: return launch_fs_x1(k_x1f<N, X1F_CG, true>, x32, X1<N>::NT, X1<N>::smem, a, s);
         case FK_X1F_RHS_F32: return launch_fs_x1(k_x1f<N, X1F_RHS, true>, x32, X1<N>::NT, X1<N>::smem, a, s);
         case FK_X1F_RHS_DD: {
-            using X = Cfg<N, dd>;
+            using X = X1dd<N>;
             return launch_fs_x1(k_x1f_dd<N, true>, dim3((X::H + X::W3 - 1) / X::W3, N), X::T3, X::smem_p3, a, s);
         }
         case FK_P4_GRAD_F32: {

@@ -165,7 +165,8 @@ __device__ __forceinline__ void stv(T* p, const T (&v)[W]) {
 
 // Block shapes of the passes for the radix split N = NA * (N / NA) and the
 // tile variant TV (the autotuner's schedules; NA = Plan<N>::N1, TV = 0 are
-// the defaults): P1/P5 rows per block R (TV 1: half, 2: double), P3
+// the defaults): P1/P5 rows per block R (TV 1: half, 2: double, 3: for one
+// field), P3
 // columns per block W3 (TV 1: half, 2: double, within the shared memory of
 // a block), P2/P4 columns per block W2 (FP32, TV 1: 32 instead of 16).
 template <int N, typename T, int NA = Plan<N>::N1, int TV = 0>
@@ -179,9 +180,20 @@ struct Cfg {
     static constexpr int fl2(int x) {
         return x >= 64 ? 64 : x >= 32 ? 32 : x >= 16 ? 16 : x >= 8 ? 8 : x >= 4 ? 4 : x >= 2 ? 2 : 1;
     }
+    // Blocks that a pass over one field should have at least: the tiles of P3
+    // and, with two-stage plans, of P2/P4 are halved until it does, and the
+    // rows of the operators on a caller's field (TV 3: always one field) are
+    // fewer. FP64, 45^3: P3 50 -> 30 us, P2/P4 29 -> 18 us (90 and 68 blocks
+    // before), a projection 181 -> 123 us, in FP32 35 -> 25 us. The row passes
+    // of the solvers keep their rows: with 4 instead of 16 P1 took 28 instead
+    // of 25 us there, and a double-float P1 of 32 cells of 27^3 208 instead of
+    // 78 us; so do P2/P4 with one-stage plans (84 instead of 52 us).
+    static constexpr int FILL = 256;
+    static constexpr int lo(int a, int b) { return a < b ? a : b; }
     // rows per block in P1/P5: a power of two >= 4, so that a block's rows
     // are a whole number of 16-byte vectors
-    static constexpr int R0 = FFTG_ROWS > 0 ? FFTG_ROWS : fl2(ROW_BUDGET / (3 * N * CS));
+    static constexpr int R0 = FFTG_ROWS > 0 ? FFTG_ROWS : TV == 3 ? lo(fl2(ROW_BUDGET / (3 * N * CS)), fl2(N * N / FILL))
+                                                           : fl2(ROW_BUDGET / (3 * N * CS));
     static constexpr int R1 = R0 < 4 ? 4 : R0;
     static constexpr int R = TV == 1 ? (R1 / 2 < 4 ? 4 : R1 / 2)
                              : TV == 2 && (size_t)(3 * 2 * R1 * N + N) * CS <= SMEM_MAX ? 2 * R1 : R1;
@@ -198,8 +210,9 @@ struct Cfg {
                                       ? fl2(512 / (6 * PN2))
                                       : fl2(512 / (2 * PN1)));
     static constexpr int WD = WDa < WDt ? WDa : WDt;
-    static constexpr int W3d = is_dd_v<T> ? (FFTG_DD_P3_W > 0 ? FFTG_DD_P3_W : (WD > W3a ? WD : W3a))
-                               : (FFTG_P3_W > 0 && FFTG_P3_W < W3a) ? FFTG_P3_W : W3a;
+    static constexpr int cols_to_fill(int w) { return w > 2 && ((H + w - 1) / w) * N < FILL ? cols_to_fill(w / 2) : w; }
+    static constexpr int W3d = cols_to_fill(is_dd_v<T> ? (FFTG_DD_P3_W > 0 ? FFTG_DD_P3_W : (WD > W3a ? WD : W3a))
+                               : (FFTG_P3_W > 0 && FFTG_P3_W < W3a) ? FFTG_P3_W : W3a);
     static constexpr int rup32(int x) { return ((x + 31) / 32) * 32; }
     static constexpr int cap(int x) { return x > 1024 ? 1024 : x; }
     static constexpr bool p3_fits(int w) {
@@ -208,16 +221,22 @@ struct Cfg {
     }
     static constexpr int W3 = TV == 1 ? (W3d / 2 < 1 ? 1 : W3d / 2)
                               : TV == 2 && W3d < 32 && p3_fits(2 * W3d) ? 2 * W3d : W3d;
-    static constexpr int W2 = (CS == 8) ? (TV == 1 ? 32 : 16) : 32;         // columns, P2/P4
-    static constexpr int S2 = fl2(BUDGET / (N * W2 * CS)) > 16 ? 16 : fl2(BUDGET / (N * W2 * CS));
+    static constexpr int W2a = (CS == 8) ? (TV == 1 ? 32 : 16) : 32;         // columns, P2/P4
+    static constexpr int W2 = TV == 0 && PN2 > 1 && N < 75 && W2a > 16 ? 16 : W2a;
+    static constexpr int S2a = fl2(BUDGET / (N * W2 * CS)) > 16 ? 16 : fl2(BUDGET / (N * W2 * CS));
+    static constexpr int slabs_to_fill(int s) {
+        return PN2 > 1 && s > 1 && ((H + W2 - 1) / W2) * (6 * N / s) < FILL ? slabs_to_fill(s / 2) : s;
+    }
+    static constexpr int S2 = slabs_to_fill(S2a);
     // threads of the column passes: one stage-A item per thread
     static constexpr int T2 = cap(rup32(S2 * W2 * PN2));
     // P3: one stage-A item per thread, and (FFTG_P3_TB) at least 2*W*N1
     // threads (448 at 243^3 rather than 432: the configuration measured)
     static constexpr int T3a = rup32(6 * W3 * PN2);
     static constexpr int T3b = FFTG_P3_TB ? rup32(2 * W3 * PN1) : 0;
-    // single-stage plans (N2 = 1) loop over the middle stages with 256 threads
-    static constexpr int T3 = PN2 == 1 ? (T3a > 256 ? cap(T3a) : 256) : cap(T3a > T3b ? T3a : T3b);
+    // single-stage plans (N2 = 1): the threads of the middle phase, one a point
+    static constexpr int T3c = W3 * N >= 256 ? 256 : rup32(W3 * N) < 64 ? 64 : rup32(W3 * N);
+    static constexpr int T3 = PN2 == 1 ? (T3a > T3c ? cap(T3a) : T3c) : cap(T3a > T3b ? T3a : T3b);
     static constexpr size_t smem_rows = (size_t)(3 * R * N + N) * CS;
     static constexpr size_t smem_p3 = (size_t)(6 * W3 * N + N) * CS;
     static constexpr size_t smem_p24 = (size_t)(S2 * W2 * N + N) * CS;
@@ -770,14 +789,13 @@ __global__ void __launch_bounds__(P3f<N, NA>::NT, 2) k_p3f(PassArgs a) {
 }
 
 // Default schedule of the FP32 P3, from the projection of one field (us,
-// default tile / half tile / fused): 45^3 10.3 / 8.5 / 12.3, 75^3 14.1 / 12.5 /
-// 12.5, 81^3 16.3 / 15.7 / 14.4, 125^3 37.3 / 34.6 / 30.5, 135^3 38.9 / 39.3 /
-// 37.3, 225^3 219 / 209 / 174 (fused: 25 x 9, since 15 x 15 has no stage of at
-// most 9 points), 243^3 229 / 233 / 217. Below 45^3 all take the launch's time.
+// full tile / fused): 45^3 10.3 / 12.3, 75^3 14.1 / 12.5, 81^3 16.3 / 14.4, 125^3
+// 37.3 / 30.5, 135^3 38.9 / 37.3, 225^3 219 / 174 (fused: 25 x 9, since 15 x 15
+// has no stage of at most 9 points), 243^3 229 / 217.
 template <int N>
 struct P3Default {
     static constexpr bool fused = N >= 75;
-    static constexpr int A = N == 225 ? 25 : Plan<N>::N1, TV = N == 45 ? 1 : 0;
+    static constexpr int A = N == 225 ? 25 : Plan<N>::N1;
     static_assert(!fused || P3f<N, A>::ok, "fused P3");
 };
 

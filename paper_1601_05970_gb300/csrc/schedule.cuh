@@ -51,7 +51,7 @@ struct VariantOf {
     static constexpr int A = (fused || p3d) && N == 225 ? 25
                              : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A
                                                              : Plan<N>::N1;
-    static constexpr int TV = p3d ? P3Default<N>::TV : V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
+    static constexpr int TV = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
 };
 
 template <int N, int TK, int V>
