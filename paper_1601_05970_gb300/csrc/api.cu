@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -277,6 +278,27 @@ static cudaError_t pass(fftg_handle* h, PassKind kind, const PassArgs& a, int nf
 }
 
 namespace {
+
+// Largest cluster of the small grids' CG that the current device takes (0: the
+// pass kernels); a property of device and grid size, asked for once a process
+// (the query takes about 2 ms).
+int most_cluster_blocks(int N, cudaStream_t s) {
+    constexpr int kDevices = 16;
+    static std::atomic<int> known[kDevices][28];  // size + 1; 0: not asked yet
+    int dev = 0;
+    if (N > 27 || cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < kDevices) {
+        const int k = known[dev][N].load(std::memory_order_relaxed);
+        if (k) return k - 1;
+    }
+    int size = 0;
+    if (fftg::run_cluster(N, PassArgs{}, 0, 0, 0, &size, s) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (dev < kDevices) known[dev][N].store(size + 1, std::memory_order_relaxed);
+    return size;
+}
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
@@ -1594,10 +1616,7 @@ int fftg_create_batch(fftg_handle** out, int N, int ncells, const uint8_t* phase
         h->last_cuda = cudaGetLastError();
         return fail(FFTG_ECUDA);
     }
-    if (h->mixed && run_cluster(N, PassArgs{}, 0, 0, 0, &h->cluster, s) != cudaSuccess) {
-        cudaGetLastError();
-        h->cluster = 0;
-    }
+    if (h->mixed) h->cluster = most_cluster_blocks(N, s);
     *out = h;
     return FFTG_OK;
 }

@@ -109,6 +109,7 @@ struct FsPointArgs {
     const void* p;
     const void* q;
     double* Fw;             // Newton update: F* += x
+    int skip_sums;          // constitutive: 1: dev->sum is not read (only the commit's call needs it)
     int unit;               // tangent kernels: the perturbed component 3k + l
 };
 
@@ -116,20 +117,25 @@ struct FsPointArgs {
 // with H = F - I, which keeps small strains free of cancellation) and
 // S = lambda tr(E) I + 2 mu E.
 __device__ __forceinline__ void svk_stress(const double (&h)[9], double lam, double mu, double (&P)[9]) {
-    double E[9];
+    // E and S are symmetric: components (i, j) with i <= j, at 3 i + j
+    double S[9];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
+        for (int j = i; j < 3; ++j) {
             double hh = 0.0;
 #pragma unroll
             for (int k = 0; k < 3; ++k) hh += h[3 * k + i] * h[3 * k + j];
-            E[3 * i + j] = 0.5 * (h[3 * i + j] + h[3 * j + i] + hh);
+            S[3 * i + j] = 0.5 * (h[3 * i + j] + h[3 * j + i] + hh);  // E
         }
-    const double le = lam * (E[0] + E[4] + E[8]);
-    double S[9];
+    const double le = lam * (S[0] + S[4] + S[8]);
 #pragma unroll
-    for (int c = 0; c < 9; ++c) S[c] = 2.0 * mu * E[c] + ((c % 4 == 0) ? le : 0.0);
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) {
+            S[3 * i + j] = 2.0 * mu * S[3 * i + j] + (i == j ? le : 0.0);
+            S[3 * j + i] = S[3 * i + j];
+        }
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -162,10 +168,28 @@ __global__ void __launch_bounds__(kThreads) k_fs_constitutive(FsPointArgs a) {
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
             if (a.P) a.P[c * cs + v] = P[c];
-            if (a.hgrad) ((TT*)a.hgrad)[c * cs + v] = (TT)h[c];
+            if (a.hgrad) {
+                if constexpr (sizeof(TT) == 4)
+                    ((TT*)a.hgrad)[c * cs + v] = f32_of(h[c]);
+                else
+                    ((TT*)a.hgrad)[c * cs + v] = h[c];
+            }
             acc[0] += P[c] * P[c];
-            acc[1 + c] += P[c];
         }
+        if (!a.skip_sums) {
+#pragma unroll
+            for (int c = 0; c < 9; ++c) acc[1 + c] += P[c];
+        }
+    }
+    if (a.skip_sums) {
+        const double one[1] = {block_sum(acc[0])};
+        if (!publish_partials<1>(one, a.partials, blockIdx.x, gridDim.x, &a.dev->ticket)) return;
+        double p2[1];
+        reduce_partials<1>(a.partials, gridDim.x, &a.dev->ticket, p2);
+        if (threadIdx.x != 0) return;
+        a.dev->p2 = p2[0];
+        if (a.cg) a.cg->floor2 = kRoundoffRel * kRoundoffRel * p2[0];
+        return;
     }
     double part[10];
 #pragma unroll
@@ -576,6 +600,7 @@ int fs_constitutive(fftg_fs_handle* h, const double* F, bool write_h, CGState* c
     u.P = h->P;
     u.hgrad = write_h ? h->hgrad : nullptr;
     u.cg = cg;
+    u.skip_sums = write_h ? 1 : 0;  // the mean stress is read after calls without H only
     const int slot = fs_prof_begin(h, h->mixed ? FSK_CONSTITUTIVE_F32 : FSK_CONSTITUTIVE_F64);
     if (h->mixed)
         k_fs_constitutive<float><<<fs_point_blocks(h->V), kThreads, 0, h->stream>>>(u);

@@ -41,6 +41,7 @@ inline void pack_phase(const fftg_phase& m, double* row) {
     row[5] = m.eps0;
     row[6] = m.t0;
     row[7] = (double)m.model;
+    row[8] = 1.0 / (3.0 * m.G + m.H);
 }
 
 }  // namespace fftg
