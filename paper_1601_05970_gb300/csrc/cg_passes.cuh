@@ -907,13 +907,13 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     const dim3 x32(X1<N>::tiles, N, nf);
     const dim3 gdd((CDD::H + CDD::W3 - 1) / CDD::W3, N, nf);
     switch (kind) {
-        case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s);
-        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
-        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
-        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
-        case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s);
-        case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s);
-        case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s);
+        case PK_P1_PLAIN_F64: return launch_k(k_p1<N, double, P1_PLAIN>, r64, C64::smem_rows, a, s, C64::TR);
+        case PK_P1_PLAIN_F32: return launch_k(k_p1<N, float, P1_PLAIN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s, U32::TR);
+        case PK_P1_TAN_F64: return launch_k(k_p1<N, double, P1_TAN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s, U64::TR);
+        case PK_P1_TAN_F32: return launch_k(k_p1<N, float, P1_TAN, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s, U32::TR);
+        case PK_P1_CG_F64: return launch_k(k_p1<N, double, P1_CG>, r64, C64::smem_rows, a, s, C64::TR);
+        case PK_P1_TANRHS_F64: return launch_k(k_p1<N, double, P1_TANRHS>, r64, C64::smem_rows, a, s, C64::TR);
+        case PK_P1_TANRHS_F32: return launch_k(k_p1<N, float, P1_TANRHS>, r32, C32::smem_rows, a, s, C32::TR);
         case PK_P2_F64: return launch_k(k_p24<N, double, true>, c64, C64::smem_p24, a, s, C64::T2);
         case PK_P2_F32: return launch_k(k_p24<N, float, true>, c32, C32::smem_p24, a, s, C32::T2);
         case PK_P4_F64: return launch_k(k_p24<N, double, false>, c64, C64::smem_p24, a, s, C64::T2);
@@ -934,14 +934,14 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
         case PK_P5_DOT_F32: return launch_k(k_p5<N, float, P5_DOT, float, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
         case PK_P5_RHS_F64_TO_F64:
             return launch_k(k_p5<N, double, P5_RHS, double>, r64, C64::smem_rows, a, s);
-        case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s);
+        case PK_P1_PLAIN_DD: return launch_k(k_p1<N, dd, P1_PLAIN>, r64, CDD::smem_rows, a, s, CDD::TR);
         case PK_P2_DD: return launch_k(k_p24<N, dd, true>, c64, CDD::smem_p24, a, s, CDD::T2);
         case PK_P4_DD: return launch_k(k_p24<N, dd, false>, c64, CDD::smem_p24, a, s, CDD::T2);
         case PK_P3_DD: return launch_k(k_p3<N, dd>, gdd, CDD::smem_p3, a, s, CDD::T3);
         case PK_P5_PLAIN_DD_TO_F64:
             return launch_k(k_p5<N, dd, P5_PLAIN, double, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
-        case PK_P1_USER_F64: return launch_k(k_p1<N, double, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
-        case PK_P1_USER_DD: return launch_k(k_p1<N, dd, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);
+        case PK_P1_USER_F64: return launch_k(k_p1<N, double, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s, U64::TR);
+        case PK_P1_USER_DD: return launch_k(k_p1<N, dd, P1_PLAIN, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s, Cfg<N, dd, Plan<N>::N1, 3>::TR);
         case PK_P5_USER_F32: return launch_k(k_p5<N, float, P5_PLAIN, float, 1, Plan<N>::N1, 3>, u32, U32::smem_rows, a, s);
         case PK_P5_DOT_USER_F64:
             return launch_k(k_p5<N, double, P5_DOT, double, 1, Plan<N>::N1, 3>, u64, U64::smem_rows, a, s);

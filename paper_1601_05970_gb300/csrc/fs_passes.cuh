@@ -58,7 +58,8 @@ struct FsArgs {
 // one vector per component; FP64 at most 2), shared-memory budgets (KB) of
 // the row passes and of P3, and the minimum resident blocks per SM of the
 // FP32 P1 and P5 (a bound on their registers; the FP64 ones take what they
-// need: they are bound by FP64 arithmetic, not by memory). Set by timing
+// need: they are bound by FP64 arithmetic, not by memory; the double-float P1
+// with two blocks per SM 2.08 ms at 243^3, with one 3.16). Set by timing
 // variants on the 243^3 finite-strain workload (per CG iteration, FP32):
 // one voxel per lane and 40 KB of rows (R = 4) gave P1 0.66 ms (3 or 4
 // blocks per SM alike; 4 spills a little) and P5 0.34 ms with 4 blocks per
@@ -159,7 +160,7 @@ __device__ __forceinline__ void svk_tangent_apply(const T (&h)[9], T lam, T mu, 
 // [x += alpha p; p = r + beta p]; tau = K : p or tau = input; x3 R2C FFT of
 // R rows per block.
 template <int N, typename T, int MODE>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : 1) k_fs_p1(FsArgs a) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : is_dd_v<T> ? 2 : 1) k_fs_p1(FsArgs a) {
     using C = FsCfg<N, T>;
     constexpr int R = C::R, H = C::H, HP = C::HP, VW = C::VW;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;

@@ -237,6 +237,12 @@ struct Cfg {
     // single-stage plans (N2 = 1): the threads of the middle phase, one a point
     static constexpr int T3c = W3 * N >= 256 ? 256 : rup32(W3 * N) < 64 ? 64 : rup32(W3 * N);
     static constexpr int T3 = PN2 == 1 ? (T3a > T3c ? cap(T3a) : T3c) : cap(T3a > T3b ? T3a : T3b);
+    // Threads of P1: 256 in FP32 and with one-stage plans; in FP64 and
+    // double-float, where a block has few rows, one stage-A item each (128 at
+    // 243^3, where 256 left more than half of them idle in that stage:
+    // double-float 1.69 -> 1.19 ms, 16 cells of 75^3 0.57 -> 0.48 ms)
+    static constexpr int TRa = rup32(3 * R * PN2);
+    static constexpr int TR = CS == 8 || PN2 == 1 || TRa > 256 ? 256 : TRa < 128 ? 128 : TRa;
     static constexpr size_t smem_rows = (size_t)(3 * R * N + N) * CS;
     static constexpr size_t smem_p3 = (size_t)(6 * W3 * N + N) * CS;
     static constexpr size_t smem_p24 = (size_t)(S2 * W2 * N + N) * CS;
@@ -253,6 +259,15 @@ template <>
 struct PlainIn<dd> {
     using type = double;
 };
+
+// An input value in the FFT type.
+template <typename T, typename TIn>
+__device__ __forceinline__ T fft_value(TIn v) {
+    if constexpr (is_dd_v<T>)
+        return dd_split(v);
+    else
+        return T(v);
+}
 
 template <typename T>
 __device__ __forceinline__ void load_tw(cplx<T>* tw, const void* src, int n) {
@@ -301,11 +316,12 @@ struct Vec16<double> {
 // projection of an FP32 field at 243^3 takes 741 us; with the field copied
 // to and from the padded layout (96 B per voxel) it took 1169.
 template <int N, typename T, int MODE, int U = 0, int NA = Plan<N>::N1, int TV = 0>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
-    k_p1(PassArgs a) {
+__global__ void __launch_bounds__(Cfg<N, T, NA, TV>::TR, sizeof(T) == 4 ? FFTG_P1_MINB
+                                                        : (is_dd_v<T> ? FFTG_DD_MINB : 2) * kThreads /
+                                                              Cfg<N, T, NA, TV>::TR) k_p1(PassArgs a) {
     using C = Cfg<N, T, NA, TV>;
     constexpr int R = C::R, H = C::H, HP = C::HP;
-    constexpr int N1 = NA, N2 = N / NA;
+    constexpr int N1 = NA, N2 = N / NA, NT = C::TR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
     cplx<T>* z = tw + N;  // [3][R][N]
@@ -342,19 +358,21 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
         static_assert(MODE == P1_PLAIN || MODE == P1_TAN, "a caller's field is projected or multiplied");
         constexpr int UN = sizeof(TIn) == 4 ? 4 : 2;
         const long long us = a.ucs;
-        for (int j0 = tid; j0 < R * N; j0 += UN * kThreads) {
+        for (int j0 = tid; j0 < R * N; j0 += UN * NT) {
             TIn t[UN][6];
 #pragma unroll
             for (int u = 0; u < UN; ++u) {
-                const int j = j0 + u * kThreads;
+                const int j = j0 + u * NT;
 #pragma unroll
                 for (int c = 0; c < 6; ++c) t[u][c] = j < nel ? in[c * us + base + j] : TIn(0);
             }
 #pragma unroll
             for (int u = 0; u < UN; ++u) {
-                const int j = j0 + u * kThreads;
+                const int j = j0 + u * NT;
                 if (j >= R * N) continue;
-                T s[6] = {T(t[u][0]), T(t[u][1]), T(t[u][2]), T(t[u][3]), T(t[u][4]), T(t[u][5])};
+                T s[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) s[c] = fft_value<T>(t[u][c]);
                 if constexpr (MODE == P1_TAN) {
                     if (j < nel) {
                         T t7[7], pe[6] = {s[0], s[1], s[2], s[3], s[4], s[5]};
@@ -369,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
             }
         }
     }
-    for (int j = U ? R * N : tid; j < (R * N) / VW; j += kThreads) {
+    for (int j = U ? R * N : tid; j < (R * N) / VW; j += NT) {
         const int i0 = j * VW;
         T s[6][VW];
         if (i0 < nel) {
@@ -408,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
                     TIn t[VW];
                     ldv<VW, TIn>(in + c * cs + v0, t);
 #pragma unroll
-                    for (int e = 0; e < VW; ++e) p[c][e] = T(t[e]);
+                    for (int e = 0; e < VW; ++e) p[c][e] = fft_value<T>(t[e]);
                 }
             }
             if (MODE == P1_PLAIN) {
@@ -445,13 +463,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     }
     __syncthreads();
     constexpr int NP = 3 * R;
-    for (int it = tid; it < NP * N2; it += kThreads) {
+    for (int it = tid; it < NP * N2; it += NT) {
         const int pc = it % NP, t = it / NP;
         if (pc % R < nrows) fwdA<N, N1, T>(z + pc * N, 1, z + pc * N, 1, t, tw);
     }
     __syncthreads();
     if (N2 > 1) {
-        for (int it = tid; it < NP * N1; it += kThreads) {
+        for (int it = tid; it < NP * N1; it += NT) {
             const int pc = it % NP, k1 = it / NP;
             if (pc % R < nrows) fwdB<N, N1, false, T>(z + pc * N, 1, z + pc * N, 1, k1, tw);
         }
@@ -459,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P1_MINB : is_d
     }
     cplx<T>* out = (cplx<T>*)a.out + f * a.sstride;
     const long long HS = (long long)N * N * HP;
-    for (int it = tid; it < nrows * H; it += kThreads) {
+    for (int it = tid; it < nrows * H; it += NT) {
         const int row = it / H, k = it - row * H;
         const int pk = perm_pos<N, N1>(k), pn = perm_pos<N, N1>(k == 0 ? 0 : N - k);
         const long long o = (long long)(row0 + row) * HP + k;
