@@ -63,11 +63,12 @@ struct PassArgs {
 // Tuning of the elementwise phases of P1 and P5: voxels per lane (1, 2 or 4,
 // moved as one vector per component) and the minimum resident blocks per SM
 // (an upper bound on registers). Chosen by timing the variants at 243^3:
-// P1 with 4 voxels per lane and 3 blocks per SM (80 registers) took 0.355 ms
-// per CG iteration against 0.44 ms (1 block) and 0.39 ms (2 voxels, 4 blocks):
-// its 19 loads per voxel need many bytes in flight. P5 with 2 voxels per
-// lane and 4 blocks per SM took 0.223 ms against 0.245 (1 or 4 voxels) and
-// 0.31-0.38 ms with 2 blocks per SM.
+// an FP32 P1 that also updated x and p of a CG iteration (19 loads per voxel;
+// those updates are in k_x1i now) took 0.355 ms with 4 voxels per lane and 3
+// blocks per SM (80 registers) against 0.44 ms (1 block) and 0.39 ms (2
+// voxels, 4 blocks). P5 with 2 voxels per lane and 4 blocks per SM took
+// 0.223 ms against 0.245 (1 or 4 voxels) and 0.31-0.38 ms with 2 blocks per
+// SM.
 #ifndef FFTG_P1_VW
 #define FFTG_P1_VW 4
 #endif
@@ -80,10 +81,10 @@ struct PassArgs {
 #ifndef FFTG_P5_MINB
 #define FFTG_P5_MINB 4
 #endif
-// P5: rounds of spectrum loads (LDB) and of p loads (PB) issued together,
-// so that more loads are in flight per thread: at 243^3 LDB = 4, PB = 2
-// took P5 from 0.177 to 0.157 ms (PB = 4 or one voxel per lane: no further
-// gain; 3 blocks per SM instead of 4: 0.173 ms).
+// P5: rounds of spectrum loads (LDB) and of loads of its other field (PB)
+// issued together, so that more are in flight per thread: at 243^3 LDB = 4,
+// PB = 2 took the residual form of P5 from 0.177 to 0.157 ms (PB = 4 or one
+// voxel per lane: no further gain; 3 blocks per SM instead of 4: 0.173 ms).
 #ifndef FFTG_P5_LDB
 #define FFTG_P5_LDB 4
 #endif
