@@ -1878,10 +1878,8 @@ int fftg_get_field(fftg_handle* h, int which, double* out) {
     }
 }
 
-// A caller's field as the kernels can take it: device pointers are read and
-// written in place; one that is not aligned to its elements goes through the
-// handle's scratch (`tmp`, contiguous).
-static bool element_aligned(const void* p, size_t es) { return ((uintptr_t)p & (es - 1)) == 0; }
+// The operators read and write a caller's fields where they are (in_place);
+// others go through the handle's scratch (`tmp`, contiguous).
 static bool overlap(const void* a, const void* b, size_t bytes) {
     const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
     return x < y + bytes && y < x + bytes;
@@ -1896,11 +1894,11 @@ int fftg_op_project(fftg_handle* h, int precision, const void* tau, void* out) {
     // scratch: sigma and q hold no state between increments
     void* tmp = f64 ? (void*)h->sigma : h->q;
     const void* in = tau;
-    if (!element_aligned(tau, es)) {
+    if (!in_place(tau, es)) {
         CK(cudaMemcpyAsync(tmp, tau, bytes, cudaMemcpyDeviceToDevice, h->stream));
         in = tmp;
     }
-    void* dst = element_aligned(out, es) ? out : tmp;
+    void* dst = in_place(out, es) ? out : tmp;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     // P1 has read all of `in` before P5 writes, so the fields may overlap
     PassArgs a = base_args_fft(h, prec);
@@ -1926,16 +1924,16 @@ int fftg_op_constitutive(fftg_handle* h, const double dE[6], const double* eps, 
     CK(cudaMemcpyAsync(h->Edev + 6 * cell, h->h_E + 6 * cell, 48, cudaMemcpyHostToDevice, h->stream));
     const size_t bytes = 6 * (size_t)h->V * 8;
     // a voxel's strain is read before its stress is written, by one thread:
-    // the fields may be the same; where they overlap otherwise, or are not
-    // aligned, they go through the handle's
+    // the fields may be the same; where they overlap otherwise they go
+    // through the handle's
     const double* ue = eps;
     double* us = sigma;
     const bool stage = eps && sigma && (const void*)eps != (void*)sigma && overlap(eps, sigma, bytes);
-    if (eps && (stage || !element_aligned(eps, 8))) {
+    if (eps && (stage || !in_place(eps, 8))) {
         CK(cudaMemcpyAsync(h->eps_work, eps, bytes, cudaMemcpyDeviceToDevice, h->stream));
         ue = h->eps_work;
     }
-    if (sigma && !element_aligned(sigma, 8)) us = h->sigma;
+    if (sigma && !in_place(sigma, 8)) us = h->sigma;
     int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, true, false, ue, us);
     if (rc) return rc;
     if (us != sigma) CK(cudaMemcpyAsync(sigma, us, bytes, cudaMemcpyDeviceToDevice, h->stream));
@@ -1955,11 +1953,11 @@ int fftg_op_matvec(fftg_handle* h, int precision, const void* p, void* q, double
     // the fields may be the same; otherwise as in fftg_op_constitutive
     const void* up = p;
     void* uq = q;
-    if ((p != q && overlap(p, q, bytes)) || !element_aligned(p, es)) {
+    if ((p != q && overlap(p, q, bytes)) || !in_place(p, es)) {
         CK(cudaMemcpyAsync(h->p, p, bytes, cudaMemcpyDeviceToDevice, h->stream));
         up = h->p;
     }
-    if (!element_aligned(q, es)) uq = h->q;
+    if (!in_place(q, es)) uq = h->q;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     PassArgs a = base_args(h, f64);
     a.in = up;

@@ -1188,10 +1188,10 @@ int fftg_fs_op_project(fftg_fs_handle* h, int precision, const void* A_dev, void
     const bool f64 = prec != FFT_F32;  // FP64 buffers (FFTG_FP64, FFTG_DD)
     const size_t el = f64 ? 8 : 4, bytes = 9 * (size_t)h->V * el;
     if (!f64 && !h->mixed) return FFTG_EINVAL;  // FP32 transforms exist only in a mixed handle
-    // device pointers are used in place (P1 has read all of A before P5 writes);
-    // one that is not aligned to its elements goes through P (FP64) or q (FP32)
+    // the caller's fields are used in place (P1 has read all of A before P5
+    // writes), or go through P (FP64) or q (FP32)
     void* tmp = f64 ? (void*)h->P : h->q;
-    const bool in_ok = ((uintptr_t)A_dev & (el - 1)) == 0, out_ok = ((uintptr_t)out_dev & (el - 1)) == 0;
+    const bool in_ok = in_place(A_dev, el), out_ok = in_place(out_dev, el);
     if (f64 && !(in_ok && out_ok)) h->P_current = false;
     if (!in_ok) CK(cudaMemcpyAsync(tmp, A_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
     FsArgs a = fs_args(h, prec);
@@ -1220,13 +1220,13 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     if ((rc = fs_constitutive(h, h->Fstar, true, nullptr))) return rc;
     h->P_current = true;
     // p is read again for <p, q> while q is written, a voxel by one thread: the
-    // fields may be the same; where they overlap otherwise, or are not aligned
-    // to their elements, they go through the handle's
+    // fields may be the same; where they overlap otherwise they go through the
+    // handle's
     const size_t bytes = 9 * (size_t)h->V * el;
     const uintptr_t pa = (uintptr_t)p_dev, qa = (uintptr_t)q_dev;
     const void* up = p_dev;
-    void* uq = (qa & (el - 1)) ? h->q : q_dev;
-    if ((pa != qa && pa < qa + bytes && qa < pa + bytes) || (pa & (el - 1))) {
+    void* uq = in_place(q_dev, el) ? q_dev : h->q;
+    if ((pa != qa && pa < qa + bytes && qa < pa + bytes) || !in_place(p_dev, el)) {
         CK(cudaMemcpyAsync(h->p, p_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
         up = h->p;
     }

@@ -75,6 +75,26 @@ def test_project_and_matvec_fields(N, precision, fs):
     cell.close()
 
 
+@pytest.mark.parametrize("fs", [False, True])
+def test_page_locked_host_fields(fs):
+    N, nc = 15, 9 if fs else 6
+    ph, _, _ = I.random_spheres(N, 0.3, 5, r_min=1.0, r_max=2.0)
+    cell = (fftg.FsCell if fs else fftg.Cell)(N, ph, I.SVK_TWO_PHASE if fs else I.TWO_PHASE, precision="mixed")
+    if not fs:
+        cell.constitutive(DE)
+    lib, pre = fftg.load(), "fftg_fs_op_" if fs else "fftg_op_"
+    x = torch.randn(nc * N ** 3, generator=torch.Generator().manual_seed(N)).pin_memory()
+    xd = x.cuda()
+    for call in (lambda a, b: getattr(lib, pre + "project")(cell.h, fftg.FFTG_MIXED, a, b),
+                 lambda a, b: getattr(lib, pre + "matvec")(cell.h, fftg.FFTG_MIXED, a, b, None)):
+        ref, out = torch.empty_like(xd), torch.zeros_like(x).pin_memory()
+        assert call(_ptr(xd, 0), _ptr(ref, 0)) == 0
+        assert call(_ptr(x, 0), _ptr(out, 0)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref.cpu())
+    cell.close()
+
+
 @pytest.mark.parametrize("N", [3, 15, 45])
 def test_constitutive_fields(N):
     ph, _, _ = I.random_spheres(N, 0.3, 5, r_min=1.0, r_max=2.0)
