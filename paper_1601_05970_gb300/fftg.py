@@ -231,6 +231,15 @@ def workspace_size(N: int, opt: fftg_options) -> int:
     return b.value
 
 
+def _field(t, nbytes: int, call: str):
+    """Address of a tensor whose storage holds the nbytes that the operators
+    read or write from it: past its end a kernel could fault, and a copy fails
+    only where the allocation ends."""
+    if t.untyped_storage().nbytes() - t.storage_offset() * t.element_size() < nbytes:
+        check(FFTG_EINVAL, call)
+    return C.c_void_p(t.data_ptr())
+
+
 class Cell:
     """A handle of one or more periodic cells whose device memory comes from
     PyTorch.
@@ -368,8 +377,9 @@ class Cell:
             prec = FFTG_DD
         if out is None:
             out = torch.empty_like(tau)
+        nb = tau.numel() * tau.element_size()
         check(self._lib.fftg_op_project(self.h, prec, C.c_void_p(tau.data_ptr()),
-                                        C.c_void_p(out.data_ptr())), "fftg_op_project")
+                                        _field(out, nb, "fftg_op_project")), "fftg_op_project")
         return out
 
     def constitutive(self, dE=None, eps=None, sigma=None):
@@ -379,8 +389,8 @@ class Cell:
             sigma = torch.empty(6 * self.V, dtype=torch.float64, device=self.device)
         check(self._lib.fftg_op_constitutive(
             self.h, None if d is None else _dptr(d),
-            None if eps is None else C.c_void_p(eps.data_ptr()),
-            C.c_void_p(sigma.data_ptr())), "fftg_op_constitutive")
+            None if eps is None else _field(eps, 48 * self.V, "fftg_op_constitutive"),
+            _field(sigma, 48 * self.V, "fftg_op_constitutive")), "fftg_op_constitutive")
         return sigma
 
     # -- profiling ------------------------------------------------------------
@@ -409,8 +419,9 @@ class Cell:
         if q is None:
             q = torch.empty_like(p)
         pq = C.c_double(0.0)
-        check(self._lib.fftg_op_matvec(self.h, prec, C.c_void_p(p.data_ptr()),
-                                       C.c_void_p(q.data_ptr()), C.byref(pq)), "fftg_op_matvec")
+        nb = 6 * self.V * (8 if prec == FFTG_FP64 else 4)
+        check(self._lib.fftg_op_matvec(self.h, prec, _field(p, nb, "fftg_op_matvec"),
+                                       _field(q, nb, "fftg_op_matvec"), C.byref(pq)), "fftg_op_matvec")
         return q, pq.value
 
 
@@ -652,8 +663,9 @@ class FsCell:
             prec = FFTG_DD
         if out is None:
             out = torch.empty_like(A)
+        nb = A.numel() * A.element_size()
         check(self._lib.fftg_fs_op_project(self.h, prec, C.c_void_p(A.data_ptr()),
-                                           C.c_void_p(out.data_ptr())), "fftg_fs_op_project")
+                                           _field(out, nb, "fftg_fs_op_project")), "fftg_fs_op_project")
         return out
 
     def matvec(self, p, q=None):
@@ -664,8 +676,9 @@ class FsCell:
         if q is None:
             q = torch.empty_like(p)
         pq = C.c_double(0.0)
+        nb = p.numel() * p.element_size()
         check(self._lib.fftg_fs_op_matvec(self.h, prec, C.c_void_p(p.data_ptr()),
-                                          C.c_void_p(q.data_ptr()), C.byref(pq)), "fftg_fs_op_matvec")
+                                          _field(q, nb, "fftg_fs_op_matvec"), C.byref(pq)), "fftg_fs_op_matvec")
         return q, pq.value
 
     def profile(self, on=True):
