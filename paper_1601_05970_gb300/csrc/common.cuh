@@ -248,4 +248,19 @@ __device__ __forceinline__ void reduce_partials(const double* partials, int nblo
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
+// A caller's buffer that kernels can take in place: memory of the current
+// device or managed memory, aligned to its elements. All else goes through
+// cudaMemcpyAsync and a buffer of the handle: that reaches page-locked host
+// memory and peers, and refuses with an error what a kernel would fault on.
+inline bool in_place(const void* p, size_t es) {
+    if ((uintptr_t)p & (es - 1)) return false;
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+}
+
 }  // namespace fftg

@@ -1,10 +1,7 @@
 // Host-side helpers shared by the small- and finite-strain drivers.
 #pragma once
 
-#include <cuda_runtime.h>
-
 #include <cmath>
-#include <cstdint>
 
 namespace fftg {
 
@@ -42,21 +39,6 @@ constexpr int spec_pitch(int N) {
 constexpr int kCoefTile = 8;
 constexpr long long coef_elements(int N) {
     return 3LL * N * N * (((N + 1) / 2 + kCoefTile - 1) / kCoefTile * kCoefTile);
-}
-
-// A caller's buffer that kernels can take in place: memory of the current
-// device or managed memory, aligned to its elements. All else goes through
-// cudaMemcpyAsync and a buffer of the handle: that reaches page-locked host
-// memory and peers, and refuses with an error what a kernel would fault on.
-inline bool in_place(const void* p, size_t es) {
-    if ((uintptr_t)p & (es - 1)) return false;
-    cudaPointerAttributes at{};
-    int dev = -1;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
 }
 
 // w_N^j = exp(-2 pi i j / N), evaluated in long double on the host: FP64,
