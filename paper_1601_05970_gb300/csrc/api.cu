@@ -28,7 +28,7 @@
 namespace fftg {
 #define FFTG_EXTERN_N(n)                                                                  \
     extern template cudaError_t run_pass_n<n>(PassKind, const PassArgs&, int, cudaStream_t); \
-    extern template cudaError_t run_cluster_n<n>(const PassArgs&, int, int, int, int*, cudaStream_t);
+    extern template cudaError_t run_cluster_n<n>(const PassArgs&, int, int, unsigned int, int*, cudaStream_t);
 FFTG_EXTERN_N(3)
 FFTG_EXTERN_N(5)
 FFTG_EXTERN_N(9)
@@ -62,7 +62,8 @@ cudaError_t run_pass(int N, PassKind kind, const PassArgs& a, int nf, cudaStream
     }
 }
 
-static cudaError_t run_cluster(int N, const PassArgs& a, int nf, int cl, int cap, int* size, cudaStream_t s) {
+static cudaError_t run_cluster(int N, const PassArgs& a, int nf, int cl, unsigned int cap, int* size,
+                               cudaStream_t s) {
     switch (N) {
 #define FFTG_CASE(n) case n: return run_cluster_n<n>(a, nf, cl, cap, size, s);
         FFTG_CASE(3) FFTG_CASE(5) FFTG_CASE(9) FFTG_CASE(15) FFTG_CASE(25) FFTG_CASE(27)
@@ -681,8 +682,7 @@ static int build_cg_graph(fftg_handle* h, int nf, const void* tangent, long long
     if (cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) !=
         cudaSuccess)
         return FFTG_ECUDA;
-    const unsigned int cap =
-        (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
+    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 4);
     int rc = launch_cg_iteration(h, nf, tangent, tstride, CgLoop{cond, h->guard, cap});
     cudaGraph_t captured = nullptr;
     if (cudaStreamEndCapture(h->stream, &captured) != cudaSuccess || rc) return FFTG_ECUDA;
@@ -834,7 +834,7 @@ static int launch_cg_cluster(fftg_handle* h, int nf, const void* tangent, long l
     a.out = h->spec;
     a.cg = h->cg;
     a.scale = 1.0 / ((double)h->N * h->N * h->N);
-    const int cap = (h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4;
+    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 4);
     const int slot = prof_begin(h, KK_CG_CLUSTER);
     const cudaError_t e = run_cluster(h->N, a, nf, cluster_blocks(h->cluster, nf), cap, nullptr, h->stream);
     prof_end(h, slot);
@@ -877,8 +877,8 @@ static int run_cg(fftg_handle* h, int nf, const void* tangent, long long tstride
     CK(cudaMemcpyAsync(h->h_cg, h->cg, nf * sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     int chunk = 2;
-    int launched = 0;
-    const int cap = (h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 1;
+    unsigned int launched = 0;
+    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 1);
     for (;;) {
         bool all = true;
         for (int f = 0; f < nf; ++f) all = all && h->h_cg[f].done != CG_RUNNING;
@@ -1076,6 +1076,7 @@ int newton_decide(fftg_handle* h, int cell, const RoundOut& ro, double normE, do
     st.cg_iters += ro.cg_it;
     *it = i + 1;
     st.newton_iters = *it;
+    if (ro.cg_done == CG_RUNNING) return FFTG_ENOCONV_CG;  // the solve was cut off: x is not its answer
     if (ro.cg_done == CG_BREAKDOWN || !std::isfinite(rel)) return FFTG_ENAN;
     if (h->opt.fixed_newton > 0) return *it >= h->opt.fixed_newton ? 1 : 0;
     if (rel <= tol_newton || nde == 0.0) return 1;
@@ -1215,7 +1216,7 @@ IncArgs inc_args(fftg_handle* h, double tol_newton, double tol_inner) {
     a.fixed_newton = h->opt.fixed_newton;
     a.newton_guard = h->guard + 1;
     a.cg_guard = h->guard;
-    a.newton_cap = (unsigned int)((h->opt.fixed_newton > 0 ? h->opt.fixed_newton : h->opt.max_newton) + 2);
+    a.newton_cap = pass_cap(h->opt.fixed_newton, h->opt.max_newton, 2);
     CGState& c = a.cg_template;
     c.tol2 = tol_inner * tol_inner;
     c.max_it = h->opt.max_cg;
@@ -1275,8 +1276,7 @@ int capture_branch(fftg_handle* h, cudaGraph_t top, cudaStream_t s1, cudaStream_
                     cudaSuccess) {
                     rc = FFTG_ECUDA;
                 } else {
-                    const unsigned int cap =
-                        (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
+                    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 4);
                     rc = launch_cg_iteration(h, h->B, h->tangent, 7 * h->cs, CgLoop{cC, h->guard, cap});
                     cudaGraph_t g3 = nullptr;
                     if (cudaStreamEndCapture(s3, &g3) != cudaSuccess) rc = FFTG_ECUDA;
@@ -1780,6 +1780,7 @@ int fftg_tangent(fftg_handle* h, double tol_cg, double C_out[36], int* cg_iters)
     }
     int total = 0;
     for (int f = 0; f < 6; ++f) {
+        if (h->h_cg[f].done == CG_RUNNING) return FFTG_ENOCONV_CG;
         if (h->h_cg[f].done == CG_BREAKDOWN) return FFTG_ENAN;
         total += h->h_cg[f].it;
     }

@@ -98,7 +98,9 @@ __global__ void k_inc_decide(cudaGraphConditionalHandle cond, IncArgs a) {
         const double nde = sqrt(a.nd[b].de2);
         const double rel = s.normE > 0.0 ? nde / s.normE : (nde == 0.0 ? 0.0 : INFINITY);
         int verdict = 0;  // 0 iterate, 1 converged, < 0 failed
-        if (c.done == CG_BREAKDOWN || !isfinite(rel))
+        if (c.done == CG_RUNNING)
+            verdict = FFTG_ENOCONV_CG;  // the solve was cut off: x is not its answer
+        else if (c.done == CG_BREAKDOWN || !isfinite(rel))
             verdict = FFTG_ENAN;
         else if (a.fixed_newton > 0)
             verdict = s.newton >= a.fixed_newton ? 1 : 0;

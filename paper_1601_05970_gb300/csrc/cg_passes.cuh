@@ -818,7 +818,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 template <int N>
-__global__ void __launch_bounds__(ClusterCg<N>::NT, 2) k_cg_cluster(PassArgs a, int cl, int cap) {
+__global__ void __launch_bounds__(ClusterCg<N>::NT, 2) k_cg_cluster(PassArgs a, int cl, unsigned int cap) {
     using T = float;
     using S = ClusterCg<N>;
     constexpr int GT = S::GT;
@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(ClusterCg<N>::NT, 2) k_cg_cluster(PassArgs a, 
     double* part = a.partials + (size_t)f * S::partials;
     double* part_x1 = part + N;
     const double unit = (double)CoefScale<N>::value * a.scale;
-    for (int pass = 0; pass < cap && st.done == CG_RUNNING; ++pass) {
+    for (unsigned int pass = 0; pass < cap && st.done == CG_RUNNING; ++pass) {
         for (int j = group; j < X1<N>::blocks; j += groups) {
             x1i_tile<N, X1I_CG, false, GT, true>(j % X1<N>::tiles, j / X1<N>::tiles, st.it, (T)st.alpha, (T)st.beta,
                                                  st.pend != 0, r, p, x, sp, buf, tw, tid, bar);
@@ -972,7 +972,7 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
 // The solve of nf fields by clusters of cl blocks (cl = 0: the largest size,
 // 16 or 8, that the device takes, or 0, is written to *size and nothing runs).
 template <int N>
-cudaError_t run_cluster_n(const PassArgs& a, int nf, int cl, int cap, int* size, cudaStream_t s) {
+cudaError_t run_cluster_n(const PassArgs& a, int nf, int cl, unsigned int cap, int* size, cudaStream_t s) {
     if constexpr (!ClusterCg<N>::ok) {
         if (size) *size = 0;
         return cl ? cudaErrorInvalidValue : cudaSuccess;

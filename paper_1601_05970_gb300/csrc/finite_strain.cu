@@ -758,7 +758,7 @@ int fs_build_graph(fftg_fs_handle* h) {
         cudaSuccess)
         return FFTG_ECUDA;
     const long long before = h->launches;
-    const unsigned int cap = (unsigned int)((h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 4);
+    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 4);
     const int rc = fs_cg_iteration(h, FsLoop{cond, true, cap});
     h->launches = before;  // capture enqueues nothing
     cudaGraph_t captured = nullptr;
@@ -795,8 +795,9 @@ int fs_run_cg(fftg_fs_handle* h) {
     }
     CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    int chunk = 2, launched = 0;
-    const int cap = (h->opt.fixed_cg > 0 ? h->opt.fixed_cg : h->opt.max_cg) + 1;
+    int chunk = 2;
+    unsigned int launched = 0;
+    const unsigned int cap = pass_cap(h->opt.fixed_cg, h->opt.max_cg, 1);
     while (h->h_cg->done == CG_RUNNING) {
         if (launched > cap) return FFTG_ENOCONV_CG;  // defensive: should not happen
         for (int k = 0; k < chunk; ++k) {
@@ -1031,6 +1032,10 @@ int fftg_fs_step(fftg_fs_handle* h, const double dF[9], double tol_newton, doubl
         }
         st.cg_iters += c.it;
         st.newton_iters = ++it;
+        if (c.done == CG_RUNNING) {
+            status = FFTG_ENOCONV_CG;  // the solve was cut off: x is not its answer
+            break;
+        }
         if (c.done == CG_BREAKDOWN || !std::isfinite(rel)) {
             status = FFTG_ENAN;
             break;
@@ -1108,6 +1113,7 @@ int fftg_fs_tangent(fftg_fs_handle* h, double tol_cg, double C_out[81], int* cg_
         }
         if ((rc = fs_run_cg(h)) || (!f64 && (rc = fs_solution(h, false)))) return rc;
         if (!f64) u.x = h->q;
+        if (h->h_cg->done == CG_RUNNING) return FFTG_ENOCONV_CG;
         if (h->h_cg->done == CG_BREAKDOWN) return FFTG_ENAN;
         total += h->h_cg->it;
         slot = fs_prof_begin(h, FSK_TANGENT_AVERAGE);

@@ -41,6 +41,13 @@ constexpr long long coef_elements(int N) {
     return 3LL * N * N * (((N + 1) / 2 + kCoefTile - 1) / kCoefTile * kCoefTile);
 }
 
+// Passes after which a device loop over iterations stops whatever its solves
+// report: the option's cap and some slack. Unsigned: caps up to INT_MAX are
+// options ("no limit").
+constexpr unsigned int pass_cap(int fixed, int most, unsigned int slack) {
+    return (unsigned int)(fixed > 0 ? fixed : most) + slack;
+}
+
 // w_N^j = exp(-2 pi i j / N), evaluated in long double on the host: FP64,
 // FP32 and (when twdd is not null) double-float (hi, lo) pairs, 4 floats
 // per twiddle (re.hi, re.lo, im.hi, im.lo).

@@ -8,5 +8,5 @@
 
 namespace fftg {
 template cudaError_t run_pass_n<FFTG_N>(PassKind, const PassArgs&, int, cudaStream_t);
-template cudaError_t run_cluster_n<FFTG_N>(const PassArgs&, int, int, int, int*, cudaStream_t);
+template cudaError_t run_cluster_n<FFTG_N>(const PassArgs&, int, int, unsigned int, int*, cudaStream_t);
 }
