@@ -411,18 +411,20 @@ static inline double* cell_field(double* base, const fftg_handle* h, int c) {
 }
 
 // Constitutive update of `ncells` cells starting at cell0 at E (Edev, one
-// 6-vector per cell) + eps against the committed history; mask_dev (may be
-// null) skips cells.
+// 6-vector per cell, or E_host, taken by value, for all of them) + eps against
+// the committed history; mask_dev (may be null) skips cells.
 static int launch_constitutive(fftg_handle* h, const int* mask_dev, int ncells, int cell0,
                                const double* eps, double* sigma, bool write_history, CGState* cg,
                                bool write_tangent = true, bool elastic_only = false,
-                               const double* user_eps = nullptr, double* user_sigma = nullptr) {
+                               const double* user_eps = nullptr, double* user_sigma = nullptr,
+                               const double* E_host = nullptr) {
     ConstArgs a{};
     a.V = h->V;
     a.cs = h->cs;
     a.ecs = user_eps ? h->V : h->cs;
     a.scs = user_sigma ? h->V : h->cs;
-    a.Edev = h->Edev + 6 * cell0;
+    a.Edev = E_host ? nullptr : h->Edev + 6 * cell0;
+    if (E_host) std::memcpy(a.E, E_host, sizeof(a.E));
     a.eps = eps + (size_t)cell0 * 6 * h->cs;
     a.eps_p = h->eps_p + (size_t)cell0 * 6 * h->cs;
     a.epbar = h->epbar + (size_t)cell0 * h->cs;
@@ -1843,9 +1845,8 @@ int fftg_get_field(fftg_handle* h, int which, double* out) {
             // return would relax the stress again). Non-linear elastic
             // phases have no history and are evaluated as usual. The tangent
             // of the increment is left untouched.
-            std::memcpy(h->h_E + 6 * cell, h->E.data() + 6 * cell, 6 * sizeof(double));
-            CK(cudaMemcpyAsync(h->Edev + 6 * cell, h->h_E + 6 * cell, 48, cudaMemcpyHostToDevice, h->stream));
-            int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, false, true);
+            int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, false, true,
+                                         nullptr, nullptr, h->E.data() + 6 * cell);
             if (rc) return rc;
             CK(copy_field(h, out, false, cell_field(h->sigma, h, cell), true, 8, cudaMemcpyDeviceToHost));
             CK(cudaStreamSynchronize(h->stream));
@@ -1921,8 +1922,10 @@ int fftg_op_project(fftg_handle* h, int precision, const void* tau, void* out) {
 int fftg_op_constitutive(fftg_handle* h, const double dE[6], const double* eps, double* sigma) {
     if (!h) return FFTG_EINVAL;
     const int cell = h->sel;
-    for (int c = 0; c < 6; ++c) h->h_E[6 * cell + c] = h->E[6 * cell + c] + (dE ? dE[c] : 0.0);
-    CK(cudaMemcpyAsync(h->Edev + 6 * cell, h->h_E + 6 * cell, 48, cudaMemcpyHostToDevice, h->stream));
+    // E + dE goes with the launch: the call returns after enqueueing, and the
+    // next one may come before the stream gets here
+    double E[6];
+    for (int c = 0; c < 6; ++c) E[c] = h->E[6 * cell + c] + (dE ? dE[c] : 0.0);
     const size_t bytes = 6 * (size_t)h->V * 8;
     // a voxel's strain is read before its stress is written, by one thread:
     // the fields may be the same; where they overlap otherwise they go
@@ -1935,7 +1938,7 @@ int fftg_op_constitutive(fftg_handle* h, const double dE[6], const double* eps, 
         ue = h->eps_work;
     }
     if (sigma && !in_place(sigma, 8)) us = h->sigma;
-    int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, true, false, ue, us);
+    int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, true, false, ue, us, E);
     if (rc) return rc;
     if (us != sigma) CK(cudaMemcpyAsync(sigma, us, bytes, cudaMemcpyDeviceToDevice, h->stream));
     h->have_tangent[cell] = 0;
@@ -1947,9 +1950,13 @@ int fftg_op_matvec(fftg_handle* h, int precision, const void* p, void* q, double
     const bool f64 = precision == FFTG_FP64;
     if (f64 == (bool)h->mixed) return FFTG_EINVAL;  // must match the tangent's precision
     const size_t es = f64 ? 8 : 4, bytes = 6 * (size_t)h->V * es;
-    set_cg_params(h, 1, 1.0, nullptr);
-    h->h_cg[0].rr = 1.0;
-    CK(cudaMemcpyAsync(h->cg, h->h_cg, h->nf * sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
+    // a scratch solve for <p, q>, by value as the strain above
+    CGState one{};
+    one.rr = 1.0;
+    one.max_it = 1;
+    k_set_cg<<<1, 1, 0, h->stream>>>(h->cg, one);
+    CK(cudaGetLastError());
+    ++h->launches;
     // p is read again for <p, q> while q is written, a voxel by one thread:
     // the fields may be the same; otherwise as in fftg_op_constitutive
     const void* up = p;

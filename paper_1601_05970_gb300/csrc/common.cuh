@@ -89,6 +89,10 @@ __device__ __forceinline__ void cg_start(CGState* cg, double rr, double gs2) {
     }
 }
 
+// Sets a solve's state from a kernel argument: no host memory has to stay
+// unchanged until the stream gets here.
+static __global__ void k_set_cg(CGState* cg, CGState value) { *cg = value; }
+
 // After the matvec of an iteration: alpha = <r, r>/<p, q>, or the fixed
 // Richardson step.
 __device__ __forceinline__ void cg_after_dot(CGState* cg, double pq) {
