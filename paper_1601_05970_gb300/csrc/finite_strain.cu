@@ -95,7 +95,7 @@ struct FsDev {
 
 struct FsPointArgs {
     long long V, cs;
-    const double* Fbar;     // [9] on the device
+    double Fbar[9];         // constitutive: the mean of F
     const double* Fs;       // F* [9][cs]
     double* P;              // [9][cs] or null
     void* hgrad;            // H = F - I [9][cs] in the inner precision, or null
@@ -400,7 +400,7 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct FsLayout {
     size_t off_phase, off_lame, off_Fstar, off_Fwork, off_P, off_hgrad, off_x, off_r, off_p, off_q,
-        off_spec, off_tw32, off_tw64, off_twdd, off_partials, off_cg, off_dev, off_Fbar, off_guard, total;
+        off_spec, off_tw32, off_tw64, off_twdd, off_partials, off_cg, off_dev, off_guard, total;
 };
 
 FsLayout fs_layout(int N, bool mixed) {
@@ -435,7 +435,6 @@ FsLayout fs_layout(int N, bool mixed) {
     L.off_partials = take(npart * 8);
     L.off_cg = take(sizeof(CGState));
     L.off_dev = take(sizeof(FsDev));
-    L.off_Fbar = take(9 * 8);
     L.off_guard = take(64);
     L.total = o;
     return L;
@@ -475,11 +474,9 @@ struct fftg_fs_handle {
     double* partials = nullptr;
     CGState* cg = nullptr;
     FsDev* dev = nullptr;
-    double* Fbar_dev = nullptr;
     unsigned int* guard = nullptr;
     CGState* h_cg = nullptr;   // pinned mirrors
     FsDev* h_dev = nullptr;
-    double* h_Fbar = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool graph_broken = false;
@@ -567,7 +564,6 @@ FsPointArgs point_args(fftg_fs_handle* h) {
     FsPointArgs u{};
     u.V = h->V;
     u.cs = h->cs;
-    u.Fbar = h->Fbar_dev;
     u.Fs = h->Fstar;
     u.hgrad = h->hgrad;
     u.phase = h->phase;
@@ -593,9 +589,12 @@ int fs_p234(fftg_fs_handle* h, int prec, double scale, CGState* cg) {
     return FFTG_OK;
 }
 
-// P and H at Fbar_dev + F (F = Fwork or Fstar); totals in dev; CG floor.
-int fs_constitutive(fftg_fs_handle* h, const double* F, bool write_h, CGState* cg) {
+// P and H at Fbar + F (F = Fwork or Fstar); totals in dev; CG floor. Fbar goes
+// with the launch: no host memory has to stay unchanged until the stream gets
+// there.
+int fs_constitutive(fftg_fs_handle* h, const double Fbar[9], const double* F, bool write_h, CGState* cg) {
     FsPointArgs u = point_args(h);
+    std::memcpy(u.Fbar, Fbar, sizeof(u.Fbar));
     u.Fs = F;
     u.P = h->P;
     u.hgrad = write_h ? h->hgrad : nullptr;
@@ -871,12 +870,6 @@ cudaError_t fs_copy(fftg_fs_handle* h, void* dst, bool dst_padded, const void* s
     return cudaMemcpy2DAsync(dst, dp, src, sp, w, 9, kind, h->stream);
 }
 
-int fs_upload_Fbar(fftg_fs_handle* h, const double F[9]) {
-    std::memcpy(h->h_Fbar, F, 9 * sizeof(double));
-    CK(cudaMemcpyAsync(h->Fbar_dev, h->h_Fbar, 9 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    return FFTG_OK;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------- public API
@@ -902,7 +895,6 @@ void fftg_fs_destroy(fftg_fs_handle* h) {
     if (h->ws) cudaFree(h->ws);
     if (h->h_cg) cudaFreeHost(h->h_cg);
     if (h->h_dev) cudaFreeHost(h->h_dev);
-    if (h->h_Fbar) cudaFreeHost(h->h_Fbar);
     delete h;
 }
 
@@ -953,11 +945,9 @@ int fftg_fs_create(fftg_fs_handle** out, int N, const uint8_t* phase, int nphase
     h->partials = (double*)(h->ws + L.off_partials);
     h->cg = (CGState*)(h->ws + L.off_cg);
     h->dev = (FsDev*)(h->ws + L.off_dev);
-    h->Fbar_dev = (double*)(h->ws + L.off_Fbar);
     h->guard = (unsigned int*)(h->ws + L.off_guard);
     if (cudaMallocHost((void**)&h->h_cg, sizeof(CGState)) != cudaSuccess ||
-        cudaMallocHost((void**)&h->h_dev, sizeof(FsDev)) != cudaSuccess ||
-        cudaMallocHost((void**)&h->h_Fbar, 9 * sizeof(double)) != cudaSuccess) {
+        cudaMallocHost((void**)&h->h_dev, sizeof(FsDev)) != cudaSuccess) {
         cudaGetLastError();
         fftg_fs_destroy(h);
         return FFTG_ENOMEM;
@@ -969,8 +959,6 @@ int fftg_fs_create(fftg_fs_handle** out, int N, const uint8_t* phase, int nphase
         lame[2 * i] = mats[i].lambda;
         lame[2 * i + 1] = mats[i].mu;
     }
-    const double I9[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    std::memcpy(h->h_Fbar, I9, sizeof(I9));
     cudaStream_t s = h->stream;
     if (cudaMemsetAsync(h->ws, 0, L.total, s) != cudaSuccess ||
         cudaMemcpyAsync(h->phase, phase, V, cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -978,7 +966,6 @@ int fftg_fs_create(fftg_fs_handle** out, int N, const uint8_t* phase, int nphase
         cudaMemcpyAsync(h->tw64, tw64.data(), tw64.size() * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(h->tw32, tw32.data(), tw32.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(h->twdd, twdd.data(), twdd.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(h->Fbar_dev, h->h_Fbar, 9 * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         h->last_cuda = cudaGetLastError();
         fftg_fs_destroy(h);
@@ -1005,15 +992,14 @@ int fftg_fs_step(fftg_fs_handle* h, const double dF[9], double tol_newton, doubl
         nH2 += hk * hk;
     }
     const double normH = std::sqrt((double)h->V * nH2);
-    int rc = fs_upload_Fbar(h, Ft);
-    if (rc) return rc;
+    int rc = FFTG_OK;
     CK(cudaMemcpyAsync(h->Fwork, h->Fstar, 9 * h->cs * 8, cudaMemcpyDeviceToDevice, h->stream));
     h->P_current = false;
     int it = 0, status = FFTG_OK;
     for (;;) {
         fs_set_cg(h, tol_inner);
         CK(cudaMemcpyAsync(h->cg, h->h_cg, sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
-        if ((rc = fs_constitutive(h, h->Fwork, true, h->cg)) || (rc = fs_residual(h)) || (rc = fs_run_cg(h)) ||
+        if ((rc = fs_constitutive(h, Ft, h->Fwork, true, h->cg)) || (rc = fs_residual(h)) || (rc = fs_run_cg(h)) ||
             (rc = fs_newton_update(h)))
             break;
         CK(cudaMemcpyAsync(h->h_cg, h->cg, sizeof(CGState), cudaMemcpyDeviceToHost, h->stream));
@@ -1054,13 +1040,9 @@ int fftg_fs_step(fftg_fs_handle* h, const double dF[9], double tol_newton, doubl
     h->stats.status = status;
     if (newton_iters) *newton_iters = it;
     if (cg_iters) *cg_iters = h->stats.cg_iters;
-    if (status != FFTG_OK) {
-        rc = fs_upload_Fbar(h, h->Fbar);  // back to the committed Fbar
-        if (rc == FFTG_OK) cudaStreamSynchronize(h->stream);
-        return status;
-    }
+    if (status != FFTG_OK) return status;
     // stress at the converged state, homogenised; commit
-    if ((rc = fs_constitutive(h, h->Fwork, false, nullptr))) return rc;
+    if ((rc = fs_constitutive(h, Ft, h->Fwork, false, nullptr))) return rc;
     CK(cudaMemcpyAsync(h->h_dev, h->dev, sizeof(FsDev), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(h->Fstar, h->Fwork, 9 * h->cs * 8, cudaMemcpyDeviceToDevice, h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1079,9 +1061,8 @@ int fftg_fs_tangent(fftg_fs_handle* h, double tol_cg, double C_out[81], int* cg_
     const double tol_inner = h->mixed ? std::max(tol_cg, h->opt.cg_inner_floor) : tol_cg;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     // tangent data H at the committed state
-    int rc = fs_upload_Fbar(h, h->Fbar);
+    int rc = fs_constitutive(h, h->Fbar, h->Fstar, true, nullptr);
     if (rc) return rc;
-    if ((rc = fs_constitutive(h, h->Fstar, true, nullptr))) return rc;
     h->P_current = true;
     int total = 0;
     for (int unit = 0; unit < 9; ++unit) {
@@ -1148,8 +1129,7 @@ int fftg_fs_get_field(fftg_fs_handle* h, int which, double* host_out) {
     }
     if (which == FFTG_FS_FIELD_STRESS) {
         if (!h->P_current) {
-            int rc = fs_upload_Fbar(h, h->Fbar);  // the committed Fbar
-            if (rc == FFTG_OK) rc = fs_constitutive(h, h->Fstar, false, nullptr);
+            int rc = fs_constitutive(h, h->Fbar, h->Fstar, false, nullptr);
             if (rc) return rc;
             h->P_current = true;
         }
@@ -1179,8 +1159,6 @@ int fftg_fs_set_state(fftg_fs_handle* h, const void* host_buf, size_t bytes) {
     for (size_t k = 0; k < 9 + 9 * (size_t)h->V; ++k)
         if (!std::isfinite(d[k])) return FFTG_EINVAL;
     CK(fs_copy(h, h->Fstar, true, d + 9, false, 8, cudaMemcpyHostToDevice));
-    int rc = fs_upload_Fbar(h, d);
-    if (rc) return rc;
     CK(cudaStreamSynchronize(h->stream));
     std::memcpy(h->Fbar, d, 9 * sizeof(double));
     h->P_current = false;
@@ -1221,9 +1199,8 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     if (f64 == (bool)h->mixed) return FFTG_EINVAL;  // the handle's inner precision
     const size_t el = f64 ? 8 : 4;
     // tangent data H at the committed state
-    int rc = fs_upload_Fbar(h, h->Fbar);
+    int rc = fs_constitutive(h, h->Fbar, h->Fstar, true, nullptr);
     if (rc) return rc;
-    if ((rc = fs_constitutive(h, h->Fstar, true, nullptr))) return rc;
     h->P_current = true;
     // p is read again for <p, q> while q is written, a voxel by one thread: the
     // fields may be the same; where they overlap otherwise they go through the
@@ -1242,9 +1219,12 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     a.ucs = h->V;
     CK(fs_pass(h, f64 ? FK_P1_TAN_F64 : FK_P1_TAN_F32, a));
     if ((rc = fs_p234(h, prec, 1.0 / ((double)h->N * h->N * h->N), nullptr))) return rc;
-    // <p, q> through the DOT pass on a scratch CG state
-    fs_set_cg(h, 1.0);
-    CK(cudaMemcpyAsync(h->cg, h->h_cg, sizeof(CGState), cudaMemcpyHostToDevice, h->stream));
+    // <p, q> through the DOT pass on a scratch CG state, by value as Fbar
+    CGState one{};
+    one.max_it = 1;
+    k_set_cg<<<1, 1, 0, h->stream>>>(h->cg, one);
+    CK(cudaGetLastError());
+    ++h->launches;
     FsArgs b = fs_args(h, prec);
     b.in = h->spec;
     b.out = uq;

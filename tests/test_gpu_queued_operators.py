@@ -83,3 +83,32 @@ def test_small_strain(precision):
         assert np.array_equal(a, b), i
     del keep
     c.close()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_finite_strain(precision):
+    c = fftg.FsCell(N, _phase(), I.SVK_TWO_PHASE, precision=precision)
+    dF = np.array([[0.02, 0.03, 0.0], [0.01, -0.02, 0.01], [0.0, 0.02, 0.01]])
+    c.step(dF, 1e-7, 1e-8)
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    code = fftg.FFTG_FP64 if precision == "fp64" else fftg.FFTG_MIXED
+    g = torch.Generator(device="cuda").manual_seed(N)
+    p = torch.randn(9 * N ** 3, dtype=dt, device="cuda", generator=g)
+    state = c.get_state()
+
+    def run(wait):
+        q = torch.empty_like(p)
+        assert fftg.load().fftg_fs_op_matvec(c.h, code, C.c_void_p(p.data_ptr()), C.c_void_p(q.data_ptr()), None) == 0
+        if wait:
+            torch.cuda.synchronize()
+        P = c.step(dF, 1e-7, 1e-8)[0]
+        return q.cpu().numpy(), P
+
+    ref = run(True)
+    c.set_state(state)
+    torch.cuda.synchronize()
+    keep = _busy()
+    for a, b in zip(ref, run(False)):
+        assert np.array_equal(a, b)
+    del keep
+    c.close()
