@@ -248,7 +248,16 @@ void fftg_destroy(fftg_handle* h);
  * their own iteration and for parity tests. All run in the handle's stream
  * and return after enqueueing, except where a host output is written (then
  * the stream is synchronised). `precision` selects FP64 (double buffers) or
- * FP32 (float buffers) for the FFT-side operators. */
+ * FP32 (float buffers) for the FFT-side operators.
+ *
+ * A field in memory of the handle's device (or managed memory), aligned to
+ * its elements and inside one allocation, is read and written where it is: it
+ * must stay allocated, an input unchanged and an output unused, until the
+ * stream has run the call. Any other field is copied to or from a buffer of
+ * the handle in the stream, which reaches page-locked host memory and fields
+ * at odd addresses; FFTG_ECUDA where such a copy is refused (host memory that
+ * is not page-locked, a buffer that ends before its field). Inputs and outputs
+ * may be the same field or overlap. */
 
 /* out = G tau (Eq. discrete_projection) for a real field tau [6][N^3]:
  * forward DFT, Ghat of Appendix A Eq. (FT_projection) at every frequency

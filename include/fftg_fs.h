@@ -96,7 +96,8 @@ int fftg_fs_get_field(fftg_fs_handle* h, int which, double* host_out);
  * FP32 for FFTG_MIXED, which needs a mixed handle): forward DFT, Ghat above
  * at every frequency, inverse DFT; FFTG_DD runs the FFTs in double-float
  * arithmetic, as the mixed path's residual does. A and out may alias.
- * Enqueued on the handle's stream. */
+ * Enqueued on the handle's stream; fields are taken in place or copied as
+ * fftg.h says for its operators. */
 int fftg_fs_op_project(fftg_fs_handle* h, int precision, const void* A_dev, void* out_dev);
 
 /* q = G (K : p) with K = dP/dF at the committed F (St. Venant-Kirchhoff's

@@ -1896,11 +1896,11 @@ int fftg_op_project(fftg_handle* h, int precision, const void* tau, void* out) {
     // scratch: sigma and q hold no state between increments
     void* tmp = f64 ? (void*)h->sigma : h->q;
     const void* in = tau;
-    if (!in_place(tau, es)) {
+    if (!in_place(tau, bytes, es)) {
         CK(cudaMemcpyAsync(tmp, tau, bytes, cudaMemcpyDeviceToDevice, h->stream));
         in = tmp;
     }
-    void* dst = in_place(out, es) ? out : tmp;
+    void* dst = in_place(out, bytes, es) ? out : tmp;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     // P1 has read all of `in` before P5 writes, so the fields may overlap
     PassArgs a = base_args_fft(h, prec);
@@ -1933,11 +1933,11 @@ int fftg_op_constitutive(fftg_handle* h, const double dE[6], const double* eps, 
     const double* ue = eps;
     double* us = sigma;
     const bool stage = eps && sigma && (const void*)eps != (void*)sigma && overlap(eps, sigma, bytes);
-    if (eps && (stage || !in_place(eps, 8))) {
+    if (eps && (stage || !in_place(eps, bytes, 8))) {
         CK(cudaMemcpyAsync(h->eps_work, eps, bytes, cudaMemcpyDeviceToDevice, h->stream));
         ue = h->eps_work;
     }
-    if (sigma && !in_place(sigma, 8)) us = h->sigma;
+    if (sigma && !in_place(sigma, bytes, 8)) us = h->sigma;
     int rc = launch_constitutive(h, nullptr, 1, cell, h->eps_star, h->sigma, false, nullptr, true, false, ue, us, E);
     if (rc) return rc;
     if (us != sigma) CK(cudaMemcpyAsync(sigma, us, bytes, cudaMemcpyDeviceToDevice, h->stream));
@@ -1961,11 +1961,11 @@ int fftg_op_matvec(fftg_handle* h, int precision, const void* p, void* q, double
     // the fields may be the same; otherwise as in fftg_op_constitutive
     const void* up = p;
     void* uq = q;
-    if ((p != q && overlap(p, q, bytes)) || !in_place(p, es)) {
+    if ((p != q && overlap(p, q, bytes)) || !in_place(p, bytes, es)) {
         CK(cudaMemcpyAsync(h->p, p, bytes, cudaMemcpyDeviceToDevice, h->stream));
         up = h->p;
     }
-    if (!in_place(q, es)) uq = h->q;
+    if (!in_place(q, bytes, es)) uq = h->q;
     const double invN3 = 1.0 / ((double)h->N * h->N * h->N);
     PassArgs a = base_args(h, f64);
     a.in = up;

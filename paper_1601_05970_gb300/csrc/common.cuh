@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "host_common.h"
+
 namespace fftg {
 
 constexpr int kThreads = 256;
@@ -252,19 +254,37 @@ __device__ __forceinline__ void reduce_partials(const double* partials, int nblo
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
-// A caller's buffer that kernels can take in place: memory of the current
-// device or managed memory, aligned to its elements. All else goes through
-// cudaMemcpyAsync and a buffer of the handle: that reaches page-locked host
-// memory and peers, and refuses with an error what a kernel would fault on.
-inline bool in_place(const void* p, size_t es) {
-    if ((uintptr_t)p & (es - 1)) return false;
+// The allocation that a caller's buffer starts in (host_common.h), as the
+// driver reports it. The range is the driver API's to give; its entry point is
+// looked up once.
+inline BufferRange buffer_range(const void* p) {
+    using GetRange = int (*)(unsigned long long*, size_t*, unsigned long long);
+    static const GetRange get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (GetRange)f;
+    }();
+    BufferRange r;
     cudaPointerAttributes at{};
     int dev = -1;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return r;
     }
-    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+    r.here = at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+    unsigned long long base = 0;
+    if (r.here && get && get(&base, &r.size, (unsigned long long)(uintptr_t)p) == 0)
+        r.base = (uintptr_t)base;
+    else
+        r.size = 0;
+    return r;
 }
+inline bool in_place(const void* p, size_t bytes, size_t es) { return usable_in_place(buffer_range(p), p, bytes, es); }
 
 }  // namespace fftg

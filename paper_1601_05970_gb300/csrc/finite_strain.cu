@@ -1175,7 +1175,7 @@ int fftg_fs_op_project(fftg_fs_handle* h, int precision, const void* A_dev, void
     // the caller's fields are used in place (P1 has read all of A before P5
     // writes), or go through P (FP64) or q (FP32)
     void* tmp = f64 ? (void*)h->P : h->q;
-    const bool in_ok = in_place(A_dev, el), out_ok = in_place(out_dev, el);
+    const bool in_ok = in_place(A_dev, bytes, el), out_ok = in_place(out_dev, bytes, el);
     if (f64 && !(in_ok && out_ok)) h->P_current = false;
     if (!in_ok) CK(cudaMemcpyAsync(tmp, A_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
     FsArgs a = fs_args(h, prec);
@@ -1208,8 +1208,8 @@ int fftg_fs_op_matvec(fftg_fs_handle* h, int precision, const void* p_dev, void*
     const size_t bytes = 9 * (size_t)h->V * el;
     const uintptr_t pa = (uintptr_t)p_dev, qa = (uintptr_t)q_dev;
     const void* up = p_dev;
-    void* uq = in_place(q_dev, el) ? q_dev : h->q;
-    if ((pa != qa && pa < qa + bytes && qa < pa + bytes) || !in_place(p_dev, el)) {
+    void* uq = in_place(q_dev, bytes, el) ? q_dev : h->q;
+    if ((pa != qa && pa < qa + bytes && qa < pa + bytes) || !in_place(p_dev, bytes, el)) {
         CK(cudaMemcpyAsync(h->p, p_dev, bytes, cudaMemcpyDeviceToDevice, h->stream));
         up = h->p;
     }

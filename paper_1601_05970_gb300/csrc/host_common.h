@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cmath>
+#include <cstddef>
+#include <cstdint>
 
 namespace fftg {
 
@@ -46,6 +48,25 @@ constexpr long long coef_elements(int N) {
 // options ("no limit").
 constexpr unsigned int pass_cap(int fixed, int most, unsigned int slack) {
     return (unsigned int)(fixed > 0 ? fixed : most) + slack;
+}
+
+// Memory that a caller's buffer starts in: the current device's or managed
+// (here), and the allocation it belongs to (size 0: not known).
+struct BufferRange {
+    bool here = false;
+    uintptr_t base = 0;
+    size_t size = 0;
+};
+
+// Whether kernels can take a caller's field of `bytes` bytes where it is:
+// memory they reach, aligned to its elements, and an allocation that holds all
+// of the field. All else goes through cudaMemcpyAsync and a buffer of the
+// handle: that reaches page-locked host memory, peers and fields over several
+// mappings, and refuses with an error what a kernel would fault on.
+inline bool usable_in_place(const BufferRange& r, const void* p, size_t bytes, size_t es) {
+    const uintptr_t a = (uintptr_t)p;
+    if (!r.here || (a & (es - 1)) || a < r.base) return false;
+    return r.size >= a - r.base && r.size - (a - r.base) >= bytes;
 }
 
 // w_N^j = exp(-2 pi i j / N), evaluated in long double on the host: FP64,
