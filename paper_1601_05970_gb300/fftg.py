@@ -240,6 +240,12 @@ def _field(t, nbytes: int, call: str):
     return C.c_void_p(t.data_ptr())
 
 
+def _field_bytes(prec: int, values: int) -> int:
+    """Bytes of a field of so many values as the operators take it: the C call
+    knows the precision code only, not the tensor's type."""
+    return values * (4 if prec == FFTG_MIXED else 8)
+
+
 class Cell:
     """A handle of one or more periodic cells whose device memory comes from
     PyTorch.
@@ -377,8 +383,8 @@ class Cell:
             prec = FFTG_DD
         if out is None:
             out = torch.empty_like(tau)
-        nb = tau.numel() * tau.element_size()
-        check(self._lib.fftg_op_project(self.h, prec, C.c_void_p(tau.data_ptr()),
+        nb = _field_bytes(prec, 6 * self.V)
+        check(self._lib.fftg_op_project(self.h, prec, _field(tau, nb, "fftg_op_project"),
                                         _field(out, nb, "fftg_op_project")), "fftg_op_project")
         return out
 
@@ -419,7 +425,7 @@ class Cell:
         if q is None:
             q = torch.empty_like(p)
         pq = C.c_double(0.0)
-        nb = 6 * self.V * (8 if prec == FFTG_FP64 else 4)
+        nb = _field_bytes(prec, 6 * self.V)
         check(self._lib.fftg_op_matvec(self.h, prec, _field(p, nb, "fftg_op_matvec"),
                                        _field(q, nb, "fftg_op_matvec"), C.byref(pq)), "fftg_op_matvec")
         return q, pq.value
@@ -663,8 +669,8 @@ class FsCell:
             prec = FFTG_DD
         if out is None:
             out = torch.empty_like(A)
-        nb = A.numel() * A.element_size()
-        check(self._lib.fftg_fs_op_project(self.h, prec, C.c_void_p(A.data_ptr()),
+        nb = _field_bytes(prec, 9 * self.V)
+        check(self._lib.fftg_fs_op_project(self.h, prec, _field(A, nb, "fftg_fs_op_project"),
                                            _field(out, nb, "fftg_fs_op_project")), "fftg_fs_op_project")
         return out
 
@@ -676,8 +682,8 @@ class FsCell:
         if q is None:
             q = torch.empty_like(p)
         pq = C.c_double(0.0)
-        nb = p.numel() * p.element_size()
-        check(self._lib.fftg_fs_op_matvec(self.h, prec, C.c_void_p(p.data_ptr()),
+        nb = _field_bytes(prec, 9 * self.V)
+        check(self._lib.fftg_fs_op_matvec(self.h, prec, _field(p, nb, "fftg_fs_op_matvec"),
                                           _field(q, nb, "fftg_fs_op_matvec"), C.byref(pq)), "fftg_fs_op_matvec")
         return q, pq.value
 
