@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     TO* out = (TO*)a.out;
     const TO* pin = (const TO*)a.aux;  // FS_P5_DOT: p
     double* Fw = MODE == FS_P5_NEWTON ? (double*)a.aux3 : nullptr;
-    dd accx(0.0f, 0.0f);  // FS_P5_NEWTON: squares of x, exact products summed in double-float
+    double accx = 0.0;  // FS_P5_NEWTON: squares of x
     T acc0 = T(0);
     double acc1 = 0.0;
     // VO voxels per lane (at most 16 bytes of TO): p is loaded before q is
@@ -561,8 +561,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
             for (int c = 0; c < 9; ++c) {
 #pragma unroll
                 for (int e = 0; e < VO; ++e) {
-                    fv[c][e] += (double)q[c][e];
-                    if (i0 + e < nel) accx += dd_two_prod(q[c][e], q[c][e]);
+                    const double d = (double)q[c][e];
+                    fv[c][e] += d;
+                    if (i0 + e < nel) accx += d * d;
                 }
                 stv<VO, double>(Fw + c * cs + v0, fv[c]);
             }
@@ -590,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     double part[2];
     if (MODE == FS_P5_NEWTON) {
         // the block's part of ||x||^2 (k_fs_newton_norm sums the parts)
-        part[0] = block_sum((double)accx);
+        part[0] = block_sum(accx);
         if (tid == 0) a.partials[blockIdx.x] = part[0];
         return;
     }

@@ -910,7 +910,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     constexpr int PB = FFTG_P5_PB < NRE ? FFTG_P5_PB : NRE;
     const TO* pin = (const TO*)a.aux + f * a.fstride;  // P5_DOT: p
     double* eps = MODE == P5_NEWTON ? (double*)a.aux3 + f * a.fstride : nullptr;
-    dd accx(0.0f, 0.0f);  // P5_NEWTON: squares of x, exact products summed in double-float
+    // P5_NEWTON: squares of x, normal and shear components. FP64: FP32's range
+    // ends above the squares of strains below 1e-19 (at 243^3 532 us; double-float
+    // sums took 419)
+    double accx[2] = {0.0, 0.0};
 #pragma unroll
     for (int r0 = 0; r0 < NRE; r0 += PB) {
         TO pv[PB][6][VO];
@@ -951,11 +954,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
                     ldv<VO, double>(eps + c * cs + v0, ev);
 #pragma unroll
                     for (int e = 0; e < VO; ++e) {
-                        ev[e] += (double)q[c][e];
-                        if (i0 + e < nel) {
-                            const dd sq = dd_two_prod(q[c][e], q[c][e]);
-                            accx += c < 3 ? sq : dd(2.0f * sq.hi, 2.0f * sq.lo);
-                        }
+                        const double d = (double)q[c][e];
+                        ev[e] += d;
+                        if (i0 + e < nel) accx[c / 3] += d * d;
                     }
                     stv<VO, double>(eps + c * cs + v0, ev);
                 }
@@ -990,7 +991,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_d
     double part[2];
     if (MODE == P5_NEWTON) {
         // the block's part of ||x||^2 (k_newton_norm sums the parts)
-        part[0] = block_sum((double)accx);
+        part[0] = block_sum(accx[0] + 2.0 * accx[1]);
         if (tid == 0) a.partials[(size_t)f * nb + blockIdx.x] = part[0];
         return;
     }
