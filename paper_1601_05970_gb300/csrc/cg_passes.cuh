@@ -257,10 +257,17 @@ __device__ __forceinline__ double warp_total(const double* in, int n, int lane) 
 // ---------------------------------------------------------------- x1 forward
 // in = spectrum of tau, aux3 = r. X1F_CG: r -= alpha w and the block's part
 // of <r, r>; X1F_RHS: r = w with scale the sign and 1/N^3 of the right-hand
-// side, and the parts of <r, r> and of ||G tau||^2 before rounding.
+// side, and the parts of <r, r> and of ||G tau||^2.
 // FS: t_i = f1 A_i1 + B_i of the six fields that the x2 pass leaves, w = t / q.
+//
+// A thread's part of the sum over its tile: in FP32 for <r, r>, and in FP64 for
+// the norm of a right-hand side.
+struct X1fSums {
+    float rr;
+    double norm;
+};
 template <int N, int MODE, bool FS, int NT, bool GROUP>
-__device__ __forceinline__ float x1f_tile(int tile, int k2g, float step, const cplx<float>* sp, cplx<float>* r,
+__device__ __forceinline__ X1fSums x1f_tile(int tile, int k2g, float step, const cplx<float>* sp, cplx<float>* r,
                                           cplx<float>* buf, const cplx<float>* tw, int tid, int bar) {
     using T = float;
     using S = X1<N>;
@@ -286,7 +293,7 @@ __device__ __forceinline__ float x1f_tile(int tile, int k2g, float step, const c
         tile_sync<NT, GROUP>(bar);
     }
     const T f2 = (T)signed_freq(k2g, N);
-    T acc = T(0);
+    X1fSums sums{0.0f, 0.0};
     for (int j = tid; j < (W / 2) * N; j += NT) {
         const int w = 2 * (j % (W / 2)), kk = j / (W / 2), col = col0 + w;
         if (col >= H) continue;
@@ -329,12 +336,16 @@ __device__ __forceinline__ float x1f_tile(int tile, int k2g, float step, const c
                         z[1][e].y * z[1][e].y + z[2][e].x * z[2][e].x + z[2][e].y * z[2][e].y;
             // f3 > 0 stands for -f3 too; the column past an odd H is padding
             const T part = q * s + fr.x * fr.x + fr.y * fr.y;
-            if (col + e < H) acc += col + e == 0 ? part : T(2) * part;
+            if (col + e < H) {
+                const T both = col + e == 0 ? part : T(2) * part;
+                sums.rr += both;
+                if (MODE == X1F_RHS) sums.norm += (double)both;
+            }
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) st_pair(r + o + i * N * W, z[i]);
     }
-    return acc;
+    return sums;
 }
 
 template <int N, int MODE, bool FS = false>
@@ -350,17 +361,19 @@ __global__ void __launch_bounds__(X1<N>::NT, X1<N>::MINB) k_x1f(PassArgs a) {
     load_tw<T>(tw, a.tw, N);
     __syncthreads();
     const double unit = (double)CoefScale<N>::value * a.scale;
-    const T acc = x1f_tile<N, MODE, FS, X1<N>::NT, false>(
+    const X1fSums sums = x1f_tile<N, MODE, FS, X1<N>::NT, false>(
         blockIdx.x, blockIdx.y, MODE == X1F_CG ? (T)(-cg->alpha * unit) : (T)unit,
         (const cplx<T>*)a.in + f * a.sstride, (cplx<T>*)a.aux3 + f * coef_field<N>(), buf, tw, threadIdx.x, 0);
-    const double s = block_sum_any((double)acc) * (FS ? 0.5 : 1.0) * CoefScale<N>::square;
+    const double square = (FS ? 0.5 : 1.0) * CoefScale<N>::square;
+    const double s = block_sum_any((double)sums.rr) * square;
+    const double norm = MODE == X1F_RHS ? block_sum_any(sums.norm) * square : 0.0;
     if (threadIdx.x == 0) {
         const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
         if (MODE == X1F_CG) {
             a.partials[f * nb + b] = s;
         } else {
             a.partials[2 * (f * nb + b)] = s;
-            a.partials[2 * (f * nb + b) + 1] = s;
+            a.partials[2 * (f * nb + b) + 1] = norm;
         }
     }
 }
@@ -427,8 +440,10 @@ __global__ void __launch_bounds__(X1dd<N>::T3) k_x1f_dd(PassArgs a) {
     }
     const float f2 = (float)signed_freq(k2g, N);
     const dd scale((double)CoefScale<N>::value * a.scale);
-    float acc0 = 0.0f;
-    dd acc1(0.0f, 0.0f);
+    // <r0, r0> in double-float; the norm before rounding in FP64, a double-float a
+    // frequency
+    dd acc0(0.0f, 0.0f);
+    double acc1 = 0.0;
     for (int it = tid; it < W * N; it += NT) {
         const int w = it % W, pos = it / W, col = col0 + w;
         const int k1 = pos / N2, k2 = pos - k1 * N2;
@@ -474,16 +489,16 @@ __global__ void __launch_bounds__(X1dd<N>::T3) k_x1f_dd(PassArgs a) {
             ft = ft + dd_scale(t[i], fi);
         }
         if (FS) {
-            acc0 += wt * q * s0;
-            acc1 += dd_scale(dd_scale(s1, q), wt);
+            acc0 += dd(wt * q * s0, 0.0f);
+            acc1 += (double)dd_scale(dd_scale(s1, q), wt);
         } else {
-            acc0 += wt * (q * s0 + fr.x * fr.x + fr.y * fr.y);
-            acc1 += dd_scale(dd_scale(s1, q) + ft.x * ft.x + ft.y * ft.y, wt);
+            acc0 += dd(wt * (q * s0 + fr.x * fr.x + fr.y * fr.y), 0.0f);
+            acc1 += (double)dd_scale(dd_scale(s1, q) + ft.x * ft.x + ft.y * ft.y, wt);
         }
     }
     const double square = (FS ? 0.5 : 1.0) * CoefScale<N>::square;
     const double s0 = block_sum_any((double)acc0) * square;
-    const double s1 = block_sum_any((double)acc1) * square;
+    const double s1 = block_sum_any(acc1) * square;
     if (tid == 0) {
         const size_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = (size_t)gridDim.x * gridDim.y;
         a.partials[2 * (f * nb + b)] = s0;
@@ -866,9 +881,9 @@ __global__ void __launch_bounds__(ClusterCg<N>::NT, 2) k_cg_cluster(PassArgs a, 
         __syncthreads();
         if (st.done != CG_RUNNING) break;  // the same in every block
         for (int j = group; j < X1<N>::blocks; j += groups) {
-            const T acc = x1f_tile<N, X1F_CG, false, GT, true>(j % X1<N>::tiles, j / X1<N>::tiles,
-                                                               (T)(-st.alpha * unit), sp, r, buf, tw, tid, bar);
-            const double wv = warp_sum((double)acc);
+            const X1fSums sums = x1f_tile<N, X1F_CG, false, GT, true>(
+                j % X1<N>::tiles, j / X1<N>::tiles, (T)(-st.alpha * unit), sp, r, buf, tw, tid, bar);
+            const double wv = warp_sum((double)sums.rr);
             if ((tid & 31) == 0) wp[tid >> 5] = wv;
             tile_sync<GT, true>(bar);
             if (tid == 0) {
