@@ -655,9 +655,11 @@ static int launch_cg_iteration(fftg_handle* h, int nf, const void* tangent, long
     return FFTG_OK;
 }
 
-// Kernels of one iteration in a loop body.
+// Kernels of one iteration in a loop body: x1i, P4, the row pass, P2, x1f and
+// k_cg_rr_loop, or with one plane pass for the middle three; FP64: P1 to P5, the
+// update and k_cg_continue.
 static long long iteration_launches(const fftg_handle* h) {
-    return !h->mixed ? 8 : pass_blocks(h->N).planes ? 4 : 6;
+    return !h->mixed ? 7 : pass_blocks(h->N).planes ? 4 : 6;
 }
 
 // Device-resident CG: one graph whose conditional WHILE node repeats the
