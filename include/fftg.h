@@ -403,22 +403,24 @@ int fftg_profile_read(fftg_handle* h, int kind, double* total_ms, long long* lau
 long long fftg_launch_count(const fftg_handle* h);
 
 /* ---------------------------------------------------------------- schedules
- * The FP32 passes of the mixed CG iteration run one of FFTG_SCHED_VARIANTS
- * schedules per grid size and pass: the radix split of the pencil transform
- * (the default split or the other one, e.g. 27 x 9 or 9 x 27 at N = 243)
- * and the tile (rows per block of P1/P5, columns per block of P2-P4; for
- * P3 also the default tile with stage B, Ghat and the inverse stage B in one
- * phase).
+ * The FP32 passes of the mixed CG iteration and of the FP32 operators run one
+ * of FFTG_SCHED_VARIANTS schedules per grid size and pass: the radix split of
+ * the pencil transform (the default split or the other one, e.g. 27 x 9 or
+ * 9 x 27 at N = 243) and the tile (rows per block of P1/P5, columns per block
+ * of P2-P4; for P3 also the default tile with stage B, Ghat and the inverse
+ * stage B in one phase). Solves up to 45^3 run P1, P2 and P4 as one kernel
+ * that has no schedules; there P2 and P4 are those of the residual's and the
+ * solution's transforms and of the operators, and P1 is not used.
  * Every schedule computes the same transforms (results agree to FP32
  * rounding). The choice is process-wide per grid size and applies to
  * launches enqueued afterwards; a handle's CUDA graphs keep the kernels they
  * captured, so set or tune schedules before creating the handles that should
  * use them. Not part of the paper's method. */
-#define FFTG_SCHED_P1 0        /* x3 transform + C : p (CG)            */
+#define FFTG_SCHED_P1 0        /* inverse x3, C : p, x3 transform (CG)   */
 #define FFTG_SCHED_P2 1        /* x2 transform                          */
-#define FFTG_SCHED_P3 2        /* x1 transform + Ghat + inverse          */
+#define FFTG_SCHED_P3 2        /* x1 transform + Ghat + inverse (operators) */
 #define FFTG_SCHED_P4 3        /* inverse x2 transform                  */
-#define FFTG_SCHED_P5 4        /* inverse x3 transform + r update (CG)  */
+#define FFTG_SCHED_P5 4        /* inverse x3 transform (projection)      */
 #define FFTG_SCHED_KINDS 5
 #define FFTG_SCHED_VARIANTS 4
 #define FFTG_TUNE_CACHE 1      /* read and write the schedule cache file */
@@ -431,7 +433,7 @@ int fftg_schedule_get(int N, int kind);
  * per field of the launch. */
 int fftg_schedule_describe(int N, int kind, int variant, int shape[5]);
 /* Times every variant of every kind at grid N on one field of scratch
- * device memory (cudaMalloc'd for the call, about 170 B per voxel) in
+ * device memory (cudaMalloc'd for the call, about 80 B per voxel) in
  * `stream` (synchronised), and selects the fastest of each kind (a variant
  * replaces the default only when at least 2 % faster). ms (may be NULL):
  * [FFTG_SCHED_KINDS][FFTG_SCHED_VARIANTS] median milliseconds, -1 when the

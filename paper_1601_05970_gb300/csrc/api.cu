@@ -77,10 +77,10 @@ static cudaError_t run_cluster(int N, const PassArgs& a, int nf, int cl, unsigne
 // Most blocks of a row or x1 pass, over the schedules (for the partial sums).
 template <int N>
 static int row_blocks_n(bool fp64) {
-    return fp64 ? Cfg<N, double>::row_blocks
-                : std::max({Cfg<N, float>::row_blocks, Cfg<N, float, Plan<N>::N1, 1>::row_blocks,
-                            RowCfg<N, RowSplit<N>::N1, 1>::blocks, X1<N>::blocks,
-                            (X1dd<N>::H + X1dd<N>::W3 - 1) / X1dd<N>::W3 * N});
+    return fp64 ? std::max(Cfg<N, double>::row_blocks, UserRows<N, double>::row_blocks)
+                : std::max({UserRows<N, float>::row_blocks, Cfg<N, float>::row_blocks,
+                            Cfg<N, float, Plan<N>::N1, 1>::row_blocks, RowCfg<N, RowSplit<N>::N1, 1>::blocks,
+                            X1<N>::blocks, (X1dd<N>::H + X1dd<N>::W3 - 1) / X1dd<N>::W3 * N});
 }
 
 int row_blocks(int N, bool fp64) {

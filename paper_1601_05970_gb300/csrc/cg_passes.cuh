@@ -912,8 +912,8 @@ cudaError_t run_pass_n(PassKind kind, const PassArgs& a, int nf, cudaStream_t s)
     using CDD = Cfg<N, dd>;
     static_assert(CDD::row_blocks == C64::row_blocks && CDD::W2 == C64::W2 && CDD::S2 == C64::S2,
                   "double-float row and column passes share the FP64 geometry");
-    using U32 = Cfg<N, float, Plan<N>::N1, 3>;
-    using U64 = Cfg<N, double, Plan<N>::N1, 3>;
+    using U32 = UserRows<N, float>;
+    using U64 = UserRows<N, double>;
     const dim3 r32(C32::row_blocks, 1, nf), r64(C64::row_blocks, 1, nf);
     const dim3 u32(U32::row_blocks, 1, nf), u64(U64::row_blocks, 1, nf);
     const dim3 c32((C32::H + C32::W2 - 1) / C32::W2, (6 * N + C32::S2 - 1) / C32::S2, nf);

@@ -167,7 +167,7 @@ __device__ __forceinline__ void stv(T* p, const T (&v)[W]) {
 // Block shapes of the passes for the radix split N = NA * (N / NA) and the
 // tile variant TV (the autotuner's schedules; NA = Plan<N>::N1, TV = 0 are
 // the defaults): P1/P5 rows per block R (TV 1: half, 2: double, 3: for one
-// field), P3
+// field, 4 and 5: half and double of that), P3
 // columns per block W3 (TV 1: half, 2: double, within the shared memory of
 // a block), P2/P4 columns per block W2 (FP32, TV 1: 32 instead of 16).
 template <int N, typename T, int NA = Plan<N>::N1, int TV = 0>
@@ -193,11 +193,11 @@ struct Cfg {
     static constexpr int lo(int a, int b) { return a < b ? a : b; }
     // rows per block in P1/P5: a power of two >= 4, so that a block's rows
     // are a whole number of 16-byte vectors
-    static constexpr int R0 = FFTG_ROWS > 0 ? FFTG_ROWS : TV == 3 ? lo(fl2(ROW_BUDGET / (3 * N * CS)), fl2(N * N / FILL))
+    static constexpr int R0 = FFTG_ROWS > 0 ? FFTG_ROWS : TV >= 3 ? lo(fl2(ROW_BUDGET / (3 * N * CS)), fl2(N * N / FILL))
                                                            : fl2(ROW_BUDGET / (3 * N * CS));
     static constexpr int R1 = R0 < 4 ? 4 : R0;
-    static constexpr int R = TV == 1 ? (R1 / 2 < 4 ? 4 : R1 / 2)
-                             : TV == 2 && (size_t)(3 * 2 * R1 * N + N) * CS <= SMEM_MAX ? 2 * R1 : R1;
+    static constexpr int R = TV == 1 || TV == 4 ? (R1 / 2 < 4 ? 4 : R1 / 2)
+                             : (TV == 2 || TV == 5) && (size_t)(3 * 2 * R1 * N + N) * CS <= SMEM_MAX ? 2 * R1 : R1;
     // voxels per lane in P1's elementwise phase (FP64: at most 2 = 16 bytes)
     static constexpr int VW = (sizeof(T) == 8 && FFTG_P1_VW > 2) ? 2 : FFTG_P1_VW;
     static constexpr int W3a = fl2(BUDGET / (6 * N * CS)) > 32 ? 32 : fl2(BUDGET / (6 * N * CS));
@@ -249,6 +249,10 @@ struct Cfg {
     static constexpr size_t smem_p24 = (size_t)(S2 * W2 * N + N) * CS;
     static constexpr int row_blocks = (N * N + R - 1) / R;
 };
+
+// Rows of the operators on a caller's field.
+template <int N, typename T>
+using UserRows = Cfg<N, T, Plan<N>::N1, 3>;
 
 // Real type a plain P1 reads: the FFT type, except for double-float FFTs,
 // whose input is an FP64 field (split into hi + lo on load).

@@ -6,8 +6,10 @@
 //
 //   P1 (the row pass of the CG
 //   iteration: inverse x3, C : p,
-//   forward x3), P5 (x3, rows):   0 default; 1 the other radix split;
-//                                 2 half the rows per block; 3 twice the rows
+//   forward x3), P5 (inverse x3 of
+//   the FP32 projection):         0 default; 1 the other radix split;
+//                                 2 half the rows per block (at least 4);
+//                                 3 twice the rows
 //   P2, P4 (x2, columns):         0 default; 1 the other radix split;
 //                                 2 32 columns per block; 3 both
 //   P3 (x1 + Ghat, columns):      0 default (P3Default); 1 the other radix
@@ -23,6 +25,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cg_passes.cuh"
 
@@ -51,7 +54,8 @@ struct VariantOf {
     static constexpr int A = (fused || p3d) && N == 225 ? 25
                              : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A
                                                              : Plan<N>::N1;
-    static constexpr int TV = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
+    static constexpr int TV0 = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
+    static constexpr int TV = TK == TK_P5 ? 3 + TV0 : TV0;  // P5 writes a caller's field (UserRows)
 };
 
 template <int N, int TK, int V>
@@ -111,9 +115,10 @@ VariantShape shape_of() {
         constexpr int NA = V == 1 ? RowSplit<N>::ALT : RowSplit<N>::N1;
         using R = RowCfg<N, NA, VO::TV>;
         sh = VariantShape{NA, N / NA, R::R, C::W2, R::blocks};
-    } else if (TK == TK_P5)
+    } else if (TK == TK_P5) {
+        static_assert(TK != TK_P5 || V > 0 || std::is_same<C, UserRows<N, float>>::value, "the default launch");
         sh.blocks = C::row_blocks;
-    else if (TK == TK_P3)
+    } else if (TK == TK_P3)
         sh.blocks = ((C::H + C::W3 - 1) / C::W3) * N;
     else
         sh.blocks = ((C::H + C::W2 - 1) / C::W2) * ((6 * N + C::S2 - 1) / C::S2);
