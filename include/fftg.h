@@ -408,7 +408,7 @@ long long fftg_launch_count(const fftg_handle* h);
  * the pencil transform (the default split or the other one, e.g. 27 x 9 or
  * 9 x 27 at N = 243) and the tile (rows per block of P1/P5, columns per block
  * of P2-P4; for P3 also the default tile with stage B, Ghat and the inverse
- * stage B in one phase). Solves up to 45^3 run P1, P2 and P4 as one kernel
+ * stage B in one phase or in three, whichever the default is not). Solves up to 45^3 run P1, P2 and P4 as one kernel
  * that has no schedules; there P2 and P4 are those of the residual's and the
  * solution's transforms and of the operators, and P1 is not used.
  * Every schedule computes the same transforms (results agree to FP32

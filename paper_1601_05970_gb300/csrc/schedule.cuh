@@ -14,10 +14,11 @@
 //                                 2 32 columns per block; 3 both
 //   P3 (x1 + Ghat, columns):      0 default (P3Default); 1 the other radix
 //                                 split; 2 half the columns per block;
-//                                 3 a full tile with stage B, Ghat and the
-//                                   inverse stage B in one phase (k_p3f;
-//                                   splits with 1 < N2 <= 9, else the
-//                                   default)
+//                                 3 a full tile in the form that the default
+//                                   is not: stage B, Ghat and the inverse
+//                                   stage B in one phase (k_p3f; splits with
+//                                   1 < N2 <= 9, else the default) below 75,
+//                                   in three from there
 //
 // A schedule changes only how the same transforms are split into register
 // DFTs and how pencils are grouped into blocks: the results agree to FP32
@@ -49,12 +50,11 @@ struct AltSplit {
 template <int N, int TK, int V>
 struct VariantOf {
     static constexpr bool cols = TK == TK_P2 || TK == TK_P4;
-    static constexpr bool fused = TK == TK_P3 && V == 3;
-    static constexpr bool p3d = TK == TK_P3 && V == 0;  // as P3Default has it
-    static constexpr int A = (fused || p3d) && N == 225 ? 25
+    static constexpr bool fused = TK == TK_P3 && V == 3 && !P3Default<N>::fused;
+    static constexpr int A = TK == TK_P3 && V == 0 ? P3Default<N>::A
                              : (V == 1 || (V == 3 && cols)) ? AltSplit<N>::A
                                                              : Plan<N>::N1;
-    static constexpr int TV0 = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : fused ? 0 : 2;
+    static constexpr int TV0 = V == 0 ? 0 : V == 1 ? 0 : V == 2 ? 1 : cols ? 1 : TK == TK_P3 ? 0 : 2;
     static constexpr int TV = TK == TK_P5 ? 3 + TV0 : TV0;  // P5 writes a caller's field (UserRows)
 };
 
