@@ -17,7 +17,7 @@ def _lib():
     build.build()
     fftg.load()
     yield
-    for N in (75, 81, 125, 225):
+    for N in (75, 81, 125, 135, 225):
         for k in fftg.SCHED_KINDS:
             fftg.schedule_set(N, k, 0)
 
@@ -34,3 +34,29 @@ def test_both_forms_of_p3(N):
     cell.close()
     assert np.isfinite(out[3]).all() and not np.array_equal(out[3], out[0])
     assert np.linalg.norm(out[3] - out[0]) <= 1e-6 * np.linalg.norm(out[0])
+
+
+@pytest.mark.parametrize("N", [75, 125, 135])
+def test_schedules_of_the_solver_passes(N):
+    """Up to 45^3 a solve runs none of the tuned row and column passes; from
+    75^3 every schedule of them reaches the FP64 path's stress to 1e-6 (the
+    mixed path's tolerance)."""
+    ph = I.random_spheres(N, 0.3, 5, r_min=2.0, r_max=4.0)[0]
+    path = np.outer([2.2e-3, 6e-4], [0.4, -0.2, -0.2, 0.3, -0.25, 0.9])  # to just below the soft yield, through it
+
+    def stress(precision):
+        c = fftg.Cell(N, ph, I.TWO_PHASE, precision=precision, nrhs_tangent=0)
+        for dE in path:
+            sig, nn, nc = c.step(dE, 1e-6, 1e-8)
+        c.close()
+        torch.cuda.empty_cache()
+        assert nc > 0
+        return sig
+
+    ref = stress("fp64")
+    for kind in ("p1", "p2", "p4"):
+        for v in range(fftg.SCHED_VARIANTS):
+            fftg.schedule_set(N, kind, v)
+            sig = stress("mixed")
+            assert np.abs(sig - ref).max() <= 1e-6 * np.abs(ref).max(), (kind, v)
+        fftg.schedule_set(N, kind, 0)
