@@ -54,23 +54,19 @@ struct FsArgs {
     int red_n;             // (reduced by P2's first block, which sets alpha)
 };
 
-// Tuning: voxels per lane in the elementwise phases of P1 and P5 (moved as
-// one vector per component; FP64 at most 2), shared-memory budgets (KB) of
-// the row passes and of P3, and the minimum resident blocks per SM of the
-// FP32 P1 and P5 (a bound on their registers; the FP64 ones take what they
-// need: they are bound by FP64 arithmetic, not by memory; the double-float P1
-// with two blocks per SM 2.08 ms at 243^3, with one 3.16). Set by timing
-// variants on the 243^3 finite-strain workload (per CG iteration, FP32):
-// one voxel per lane and 40 KB of rows (R = 4) gave P1 0.66 ms (3 or 4
-// blocks per SM alike; 4 spills a little) and P5 0.34 ms with 4 blocks per
-// SM (0.39 ms with 3); two voxels per lane 0.73-0.91 ms for P1 (it spills
-// at 3 blocks per SM); 80 KB of rows 0.76 ms; P3 with 100 or 64 KB of
-// columns 0.44 and 0.71 ms against 0.39 ms with 150 KB. P5 with the
+// Tuning: shared-memory budgets (KB) of the row passes and of P3, and the
+// minimum resident blocks per SM of the FP32 P1 and P5 (a bound on their
+// registers; the FP64 ones take what they need: they are bound by FP64
+// arithmetic, not by memory; the double-float P1 with two blocks per SM
+// 2.08 ms at 243^3, with one 3.16). Set by timing variants at 243^3, FP32,
+// with a P1 that also did the vector updates of a CG iteration (those are in
+// k_x1i now): 40 KB of rows (R = 4) gave P1 0.66 ms (3 or 4 blocks per SM
+// alike; 4 spills a little) and P5 0.34 ms with 4 blocks per SM (0.39 ms with
+// 3); 80 KB of rows 0.76 ms; P3 with 100 or 64 KB of columns 0.44 and 0.71 ms
+// against 0.39 ms with 150 KB. One voxel per lane: a caller's components start
+// on any element (and two, on aligned fields, took P1 to 0.73-0.91 ms). P5 with the
 // spectrum loads of two rounds issued together: 0.323 against 0.336 ms
 // (with 3 blocks per SM 0.369 ms).
-#ifndef FFTG_FS_VW
-#define FFTG_FS_VW 1
-#endif
 #ifndef FFTG_FS_ROW_KB
 #define FFTG_FS_ROW_KB 40
 #endif
@@ -100,7 +96,6 @@ struct FsCfg {
     // >= 4, so a block's rows start on a 16-byte boundary of every component
     static constexpr int R0 = fl2(FFTG_FS_ROW_KB * 1024 / (kFsPairs * N * CS));
     static constexpr int R = R0 < 4 ? 4 : R0;
-    static constexpr int VW = (sizeof(T) == 8 && FFTG_FS_VW > 2) ? 2 : FFTG_FS_VW;
     // columns per block of P3: nine pencils per column
     static constexpr int W3 = fl2(FFTG_FS_P3_KB * 1024 / (kFsComp * N * CS));
     static constexpr int T3 = Plan<N>::N2 == 1 ? 256 : cap(rup32(kFsComp * W3 * Plan<N>::N2));
@@ -109,7 +104,6 @@ struct FsCfg {
     static constexpr int row_blocks = (N * N + R - 1) / R;
     static_assert(smem_rows <= 227 * 1024 && smem_p3 <= 227 * 1024, "shared memory per block");
     static_assert(T3 <= 1024 && T3 % 32 == 0, "threads per block");
-    static_assert(VW == 1, "a caller's components start on any element");
 };
 
 // tau = K(F) : d for St. Venant-Kirchhoff, from h = F - I.
@@ -162,7 +156,7 @@ __device__ __forceinline__ void svk_tangent_apply(const T (&h)[9], T lam, T mu, 
 template <int N, typename T, int MODE>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : is_dd_v<T> ? 2 : 1) k_fs_p1(FsArgs a) {
     using C = FsCfg<N, T>;
-    constexpr int R = C::R, H = C::H, HP = C::HP, VW = C::VW;
+    constexpr int R = C::R, H = C::H, HP = C::HP;
     constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cplx<T>* tw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -183,105 +177,68 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P1_MINB : i
         alpha = (T)a.cg->alpha;
         first = a.cg->it == 0;
     }
-    // Elementwise phase: VW consecutive voxels per lane, one vector per
-    // component. Every load of an item is issued before its first store
-    // (the fields could alias as far as the compiler knows, which would
-    // otherwise serialise one round trip per component). In the last block
-    // a vector that straddles the end of the grid touches only the padding
-    // of each component (cs >= N^3 + 4), and its lanes past the grid belong
-    // to rows the FFT stages skip.
-    for (int j = tid; j < (R * N) / VW; j += kThreads) {
-        const int i0 = j * VW;
-        T s[9][VW];
-        if (i0 < nel) {
-            const long long v0 = base + i0;
-            T p[9][VW], h[9][VW];
-            int ph[VW];
-            if (CGM) {
+    // Elementwise phase, one voxel per lane. Every load of a voxel is issued
+    // before its first store (the fields could alias as far as the compiler
+    // knows, which would otherwise serialise one round trip per component).
+    for (int i = tid; i < R * N; i += kThreads) {
+        T s[9];
+        if (i < nel) {
+            const long long v = base + i;
+            T p[9], h[9];
+            if constexpr (CGM) {
                 const T* r = (const T*)a.aux;
                 T* pp = (T*)a.aux2;
                 T* xx = (T*)a.aux3;
-                T po[9][VW], xo[9][VW];
+                T po[9], xo[9];
 #pragma unroll
-                for (int c = 0; c < 9; ++c) ldv<VW, T>(r + c * cs + v0, p[c]);
+                for (int c = 0; c < 9; ++c) p[c] = r[c * cs + v];
                 if (!first) {
 #pragma unroll
                     for (int c = 0; c < 9; ++c) {
-                        ldv<VW, T>(pp + c * cs + v0, po[c]);
-                        ldv<VW, T>(xx + c * cs + v0, xo[c]);
+                        po[c] = pp[c * cs + v];
+                        xo[c] = xx[c * cs + v];
                     }
                 }
                 const T* hg = (const T*)a.hgrad;
 #pragma unroll
-                for (int c = 0; c < 9; ++c) ldv<VW, T>(hg + c * cs + v0, h[c]);
-#pragma unroll
-                for (int e = 0; e < VW; ++e) ph[e] = a.phase[v0 + e];
+                for (int c = 0; c < 9; ++c) h[c] = hg[c * cs + v];
+                const int ph = a.phase[v];
                 if (!first) {
 #pragma unroll
                     for (int c = 0; c < 9; ++c) {
-#pragma unroll
-                        for (int e = 0; e < VW; ++e) {
-                            xo[c][e] += alpha * po[c][e];
-                            p[c][e] += beta * po[c][e];
-                        }
-                        stv<VW, T>(xx + c * cs + v0, xo[c]);
+                        xo[c] += alpha * po[c];
+                        p[c] += beta * po[c];
+                        xx[c * cs + v] = xo[c];
                     }
                 }
 #pragma unroll
-                for (int c = 0; c < 9; ++c) stv<VW, T>(pp + c * cs + v0, p[c]);
+                for (int c = 0; c < 9; ++c) pp[c * cs + v] = p[c];
+                const double* m = a.lame + 2 * ph;
+                svk_tangent_apply<T>(h, (T)m[0], (T)m[1], p, s);
             } else {
                 using TIn = typename PlainIn<T>::type;
                 const TIn* in = (const TIn*)a.in;
 #pragma unroll
-                for (int c = 0; c < 9; ++c) {
-                    TIn t[VW];
-                    if (MODE == FS_P1_TANRHS) {
+                for (int c = 0; c < 9; ++c)
+                    p[c] = T(MODE == FS_P1_TANRHS ? TIn(c == a.unit ? 1 : 0) : in[c * a.ucs + v]);
+                if constexpr (MODE == FS_P1_PLAIN) {
 #pragma unroll
-                        for (int e = 0; e < VW; ++e) t[e] = TIn(c == a.unit ? 1 : 0);
-                    } else {
-                        ldv<VW, TIn>(in + c * a.ucs + v0, t);
-                    }
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) p[c][e] = T(t[e]);
-                }
-                if (MODE == FS_P1_TAN || MODE == FS_P1_TANRHS) {
+                    for (int c = 0; c < 9; ++c) s[c] = p[c];
+                } else {
                     const T* hg = (const T*)a.hgrad;
 #pragma unroll
-                    for (int c = 0; c < 9; ++c) ldv<VW, T>(hg + c * cs + v0, h[c]);
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) ph[e] = a.phase[v0 + e];
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                if (MODE == FS_P1_PLAIN) {
-#pragma unroll
-                    for (int c = 0; c < 9; ++c) s[c][e] = p[c][e];
-                } else {
-                    T he[9], pe[9], se[9];
-#pragma unroll
-                    for (int c = 0; c < 9; ++c) {
-                        he[c] = h[c][e];
-                        pe[c] = p[c][e];
-                    }
-                    const double* m = a.lame + 2 * ph[e];
-                    svk_tangent_apply<T>(he, (T)m[0], (T)m[1], pe, se);
-#pragma unroll
-                    for (int c = 0; c < 9; ++c) s[c][e] = se[c];
+                    for (int c = 0; c < 9; ++c) h[c] = hg[c * cs + v];
+                    const double* m = a.lame + 2 * a.phase[v];
+                    svk_tangent_apply<T>(h, (T)m[0], (T)m[1], p, s);
                 }
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < 9; ++c)
-#pragma unroll
-                for (int e = 0; e < VW; ++e) s[c][e] = T(0);
+            for (int c = 0; c < 9; ++c) s[c] = T(0);
         }
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) z[c * R * N + i0 + e] = mk(s[2 * c][e], s[2 * c + 1][e]);
-            z[4 * R * N + i0 + e] = mk(s[8][e], T(0));
-        }
+        for (int c = 0; c < 4; ++c) z[c * R * N + i] = mk(s[2 * c], s[2 * c + 1]);
+        z[4 * R * N + i] = mk(s[8], T(0));
     }
     __syncthreads();
     constexpr int NP = kFsPairs * R;
@@ -526,63 +483,50 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_FS_P5_MINB : 1
     double accx = 0.0;  // FS_P5_NEWTON: squares of x
     T acc0 = T(0);
     double acc1 = 0.0;
-    // VO voxels per lane (at most 16 bytes of TO): p is loaded before q is
-    // stored. Lanes past the grid in the last block write only component
-    // padding and are left out of the sums.
-    constexpr int VO = (C::VW * (int)sizeof(TO) > 16) ? 16 / (int)sizeof(TO) : C::VW;
-    for (int j = tid; j < (R * N) / VO; j += kThreads) {
-        const int i0 = j * VO;
-        if (i0 >= nel) continue;
-        const long long v0 = base + i0;
-        TO pv[9][VO];
+    // One voxel per lane: p is loaded before q is stored. (Counted to R N: to nel
+    // the loop is unrolled, and FP64 at 27^3 takes 130 registers instead of 122,
+    // one block per SM instead of two.)
+    for (int i = tid; i < R * N; i += kThreads) {
+        if (i >= nel) continue;
+        const long long v = base + i;
+        TO pv[9];
         if (MODE == FS_P5_DOT) {
 #pragma unroll
-            for (int c = 0; c < 9; ++c) ldv<VO, TO>(pin + c * a.ucs + v0, pv[c]);
+            for (int c = 0; c < 9; ++c) pv[c] = pin[c * a.ucs + v];
         }
-        T qd[9][VO];
-        TO q[9][VO];
+        T qd[9];
+        TO q[9];
 #pragma unroll
-        for (int e = 0; e < VO; ++e) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const cplx<T> zz = z[c * R * N + i0 + e];
-                qd[2 * c][e] = zz.x;
-                qd[2 * c + 1][e] = zz.y;
-            }
-            qd[8][e] = z[4 * R * N + i0 + e].x;
-#pragma unroll
-            for (int c = 0; c < 9; ++c) q[c][e] = (TO)qd[c][e];
+        for (int c = 0; c < 4; ++c) {
+            const cplx<T> zz = z[c * R * N + i];
+            qd[2 * c] = zz.x;
+            qd[2 * c + 1] = zz.y;
         }
+        qd[8] = z[4 * R * N + i].x;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) q[c] = (TO)qd[c];
         if constexpr (MODE == FS_P5_NEWTON) {
-            double fv[9][VO];
+            double fv[9];
 #pragma unroll
-            for (int c = 0; c < 9; ++c) ldv<VO, double>(Fw + c * cs + v0, fv[c]);
+            for (int c = 0; c < 9; ++c) fv[c] = Fw[c * cs + v];
 #pragma unroll
             for (int c = 0; c < 9; ++c) {
-#pragma unroll
-                for (int e = 0; e < VO; ++e) {
-                    const double d = (double)q[c][e];
-                    fv[c][e] += d;
-                    if (i0 + e < nel) accx += d * d;
-                }
-                stv<VO, double>(Fw + c * cs + v0, fv[c]);
+                const double d = (double)q[c];
+                Fw[c * cs + v] = fv[c] + d;
+                accx += d * d;
             }
             continue;
         }
 #pragma unroll
-        for (int c = 0; c < 9; ++c) stv<VO, TO>(out + c * a.ucs + v0, q[c]);
+        for (int c = 0; c < 9; ++c) out[c * a.ucs + v] = q[c];
         if (MODE == FS_P5_PLAIN) continue;
 #pragma unroll
-        for (int e = 0; e < VO; ++e) {
-            if (i0 + e >= nel) continue;
-#pragma unroll
-            for (int c = 0; c < 9; ++c) {
-                if (MODE == FS_P5_DOT) {
-                    acc0 += (T)(pv[c][e] * q[c][e]);
-                } else {
-                    acc0 += (T)(q[c][e] * q[c][e]);
-                    acc1 += (double)(qd[c][e] * qd[c][e]);
-                }
+        for (int c = 0; c < 9; ++c) {
+            if (MODE == FS_P5_DOT) {
+                acc0 += (T)(pv[c] * q[c]);
+            } else {
+                acc0 += (T)(q[c] * q[c]);
+                acc1 += (double)(qd[c] * qd[c]);
             }
         }
     }
