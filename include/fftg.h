@@ -132,7 +132,11 @@ typedef struct {
                                whose conditional WHILE node loops on the device
                                (no host round trip per iteration); 0: enqueue
                                iterations in chunks from the host. Profiling
-                               (fftg_profile_enable) uses the chunked path. */
+                               (fftg_profile_enable) uses the chunked path, and
+                               so does a handle in the legacy default stream,
+                               which cannot be captured. FFTG_MIXED up to 27^3:
+                               a solve is one launch either way (one kernel in
+                               a profile). The choice changes no result. */
     double dt;              /* time step of each increment, for rate-dependent
                                phases (FFTG_MODEL_VISCO), > 0 (default 1) */
     int    solver;          /* linear solver of each Newton iteration (and of

@@ -2,10 +2,14 @@
 //
 // Every vector of the projected CG is compatible, so at each frequency f it
 // is f(x)w + w(x)f for one complex 3-vector w (the displacement coefficient,
-// up to a constant factor). r, p and x are held as w on the half spectrum,
-// [nf][3][N][N][HP] complex: half the bytes of a six-component real field,
-// no incompatible part can build up in them, and only p is ever taken to
-// real space, where C : p is formed:
+// up to a constant factor). r, p and x are held as w on the half spectrum
+// (tile by tile, below): half the bytes of a six-component real field and
+// compatible whatever they hold, and only p is ever taken to real space, where
+// C : p is formed. (On the plane f3 = 0 both f and -f are stored, and rounding
+// can leave w there a little off the symmetry of a real field's; the row pass
+// drops that part of p, <r, r> counts that of r. It is of the size of a few
+// roundings, where the inner solves stop at 1e-5.)
+//
 //
 //   x1i   p = r + beta p, x += alpha p_old; f(x)p + p(x)f; inverse x1
 //   P4    inverse x2 (the column pass of passes.cuh)
@@ -21,9 +25,10 @@
 //
 // An iteration moves 84.3 (x1i) + 2 x 48.2 (P4, P2) + 76.2 (rows) + 48.2
 // (x1f) = 305 B per voxel at 243^3; with r, p and x as real fields it moved
-// 388.8 (243^3: 1.12 -> 0.95 ms an iteration). The residual of a Newton iteration and a column's right-hand side
-// stop at w (x1f), and the solution is taken to real space once (x1i, P4,
-// P5), which makes a projection of it needless.
+// 388.8 (243^3: 1.12 -> 0.95 ms an iteration). The residual of a Newton
+// iteration and a column's right-hand side stop at w (x1f), and the solution is
+// taken to real space once (x1i, P4, P5), which makes a projection of it
+// needless.
 #pragma once
 
 #include "passes.cuh"
@@ -696,8 +701,8 @@ __global__ void __launch_bounds__(RowCfg<N, NA, TV>::NT, RowCfg<N, NA, TV>::MINB
 // -------------------------------------------------------------------- planes
 // P4, the row pass and P2 act within one x1 plane. Where a plane's six
 // components are small in shared memory one block takes it through all three:
-// 76 B per voxel from and to global memory instead of 173, and two launches
-// less an iteration. An iteration takes 39 instead of 50 us on one cell of
+// 77 B per voxel at 45^3 from and to global memory instead of 175, and two
+// launches less an iteration. An iteration takes 39 instead of 50 us on one cell of
 // 45^3 and 122 instead of 131 on sixteen. At 75^3 a plane takes 209 KB, one
 // block of 20 warps an SM: 64 instead of 65 us on one cell but 508 instead of
 // 481 on sixteen, so the line lies below it.
@@ -810,9 +815,8 @@ __global__ void __launch_bounds__(PlaneCfg<N>::NT, PlaneCfg<N>::MINB) k_plane_cg
 // and the loop's condition take most of the time. The phases are those above,
 // x1 tiles over groups of GT threads and planes over the blocks, with the
 // hardware's cluster barrier (which orders global memory within the cluster)
-// between them; every block
-// keeps the solve's scalars and takes the same steps, block 0 writes them
-// back. The blocks of a cluster are resident together by construction, so no
+// between them; every block keeps the solve's scalars and takes the same
+// steps, block 0 writes them back. The blocks of a cluster are resident together by construction, so no
 // wait depends on another launch. An iteration takes 11 instead of 37 us on one
 // cell of 15^3, 23 instead of 39 on one of 27^3 and 59 instead of 78 on
 // thirty-two of them.

@@ -823,8 +823,7 @@ struct P3Default {
 };
 
 // ----------------------------------------------------------------------- P5
-// T: FFT precision; TO: output real type (P5_RHS writes the CG residual r
-// in the inner precision).
+// T: FFT precision; TO: output real type (FP64 for double-float FFTs).
 // U = 1: `out` (and the p of P5_DOT) are a caller's fields, as in P1.
 template <int N, typename T, int MODE, typename TO, int U = 0, int NA = Plan<N>::N1, int TV = 0>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? FFTG_P5_MINB : is_dd_v<T> ? FFTG_DD_MINB : 2)
