@@ -78,13 +78,9 @@ def bytes_per_voxel(N):
         "p1_cgf_f32": 5 * 24 + 28 + s32,
         "p5_cgf_f32": s32 + 24 + 24,
         "cg_rr_f32": 0.0,                          # block partials only
-        "p1_tanrhs_f32": 28 + s32,
-        "p5_rhs_f32_to_f32": s32 + 24,
         "p1_cg_f64": 5 * 48 + 56 + s64,
         "p2_f64": 2 * s64, "p3_f64": 2 * s64, "p4_f64": 2 * s64,
         "p5_dot_f64": s64 + 48 + 48, "cg_update_f64": 3 * 48,
-        "p1_plain_f64": 48 + s64,
-        "p5_rhs_f64_to_f32": s64 + 24,
     }
 
 
@@ -575,11 +571,7 @@ def fs_bytes_per_voxel(N):
             # components pass x1; the row pass reads H and the phase
             "fs_x1i_cg_f32": 5 * v32 + 2 * v32, "fs_p4_grad_f32": 2 * v32 + s32,
             "fs_rows_cg_f32": 2 * s32 + 36 + 1, "fs_p2_grad_f32": s32 + 2 * v32,
-            "fs_x1f_cg_f32": 2 * v32 + 2 * v32,
-            # without the update pass: P1 as above (and <p, K:p>); P5 reads
-            # the spectrum and r and writes r
-            "fs_p1_cgf_f32": 5 * 36 + 36 + 1 + s32, "fs_p5_cgf_f32": s32 + 36 + 36,
-            "fs_cg_rr_f32": 0.0}
+            "fs_x1f_cg_f32": 2 * v32 + 2 * v32, "fs_cg_rr_f32": 0.0}
 
 
 def projection_line(N, steps, warmup):
@@ -657,30 +649,20 @@ def finite_strain_line(N=243, warm=1, timed=2):
     bpv = fs_bytes_per_voxel(N)
     it = nc_tot + nt_tot  # CG iterations of the Newton and of the tangent solves
     solves = nn_tot + 9 * timed
-    eff = {"fs_p1_cg_f32": it, "fs_p5_dot_f32": it, "fs_cg_update_f32": it,
-           "fs_p1_cgf_f32": it, "fs_p5_cgf_f32": it, "fs_cg_rr_f32": it,
-           "fs_p2_f32": it + solves + 9 * timed, "fs_p3_f32": it + solves + 9 * timed,
-           "fs_p4_f32": it + solves + 9 * timed,
-           "fs_x1i_cg_f32": it, "fs_rows_cg_f32": it, "fs_x1f_cg_f32": it,
+    eff = {"fs_x1i_cg_f32": it, "fs_rows_cg_f32": it, "fs_x1f_cg_f32": it, "fs_cg_rr_f32": it,
            "fs_p4_grad_f32": it + solves, "fs_p2_grad_f32": it + 9 * timed}
-    kind, (kms, kn) = max(((k, v) for k, v in prof.items() if k in bpv), key=lambda kv: kv[1][0])
+    kind, (kms, kn) = max(((k, v) for k, v in prof.items() if k in eff), key=lambda kv: kv[1][0])
     hbm, peak_kind = measured_hbm()
     alg = eff[kind] * V * bpv[kind]
     achieved = alg / (kms * 1e-3) / 1e9
-    coef = "fs_rows_cg_f32" in prof
-    fused = coef or "fs_p1_cgf_f32" in prof
-    it_kinds = (("fs_x1i_cg_f32", "fs_p4_grad_f32", "fs_rows_cg_f32", "fs_p2_grad_f32", "fs_x1f_cg_f32",
-                 "fs_cg_rr_f32") if coef else
-                ("fs_p1_cgf_f32", "fs_p2_f32", "fs_p3_f32", "fs_p4_f32", "fs_p5_cgf_f32", "fs_cg_rr_f32")
-                if fused else
-                ("fs_p1_cg_f32", "fs_p2_f32", "fs_p3_f32", "fs_p4_f32", "fs_p5_dot_f32", "fs_cg_update_f32"))
+    it_kinds = ("fs_x1i_cg_f32", "fs_p4_grad_f32", "fs_rows_cg_f32", "fs_p2_grad_f32", "fs_x1f_cg_f32",
+                "fs_cg_rr_f32")
     iteration = None
     if all(k in prof and eff[k] for k in it_kinds):
         ims = sum(prof[k][0] / eff[k] for k in it_kinds)
         ib = sum(bpv[k] for k in it_kinds)
         ig = ib * V / (ims * 1e-3) / 1e9
-        iteration = {"what": "one CG iteration, per field" + (" (on coefficients)" if coef else
-                                                             " (update fused into P1/P5)" if fused else ""),
+        iteration = {"what": "one CG iteration, per field (on coefficients)",
                      "ms_per_field_iter": round(ims, 4), "bytes_per_voxel": round(ib, 1),
                      "achieved": round(ig, 1), "peak": hbm, "unit": "GB/s", "frac": round(ig / hbm, 3)}
     return {
