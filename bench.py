@@ -148,7 +148,8 @@ def flops_per_voxel(N):
 # have the digest they had then (SHA-256 prefix of the files listed).
 KERNEL_FILES = ("common.cuh", "fft_core.cuh", "passes.cuh", "cg_passes.cuh")
 FS_KERNEL_FILES = KERNEL_FILES + ("fs_passes.cuh", "fs_cg_passes.cuh")
-TRAFFIC = {}
+TRAFFIC = {"rows_cg_f32": {"N": 243, "bytes": 1071.0e6, "digest": "964d61e29dc4a369", "files": KERNEL_FILES},
+           "fs_rows_cg_f32": {"N": 243, "bytes": 1567.9e6, "digest": "2fb668c93a99dae2", "files": FS_KERNEL_FILES}}
 
 
 def _strip_comments(src: bytes) -> bytes:

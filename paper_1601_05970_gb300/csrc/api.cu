@@ -817,10 +817,10 @@ static int launch_cg_finish(fftg_handle* h, int nf) {
 }
 
 // Blocks per cluster for nf solves: the largest that keeps all of them on the
-// chip together. us an iteration with 16 / 8 / 4 blocks: one cell of 27^3
-// 26 / 44 / 76, eight 34 / 45 / 78, sixteen 58 / 59 / 79, thirty-two 89 / 61 /
-// 80, sixty-four 164 / 120 / 111; 15^3: one 13 / 17 / 23, sixteen 29 / 20 / 24,
-// sixty-four 78 / 42 / 29.
+// chip together. us an iteration with 16 / 8 / 4 blocks (solves of 200): one
+// cell of 27^3 24 / 42 / 71, eight 32 / 42 / 73, sixteen 53 / 58 / 73,
+// thirty-two 84 / 59 / 73, sixty-four 156 / 113 / 107; 15^3: one 11 / 13 / 18,
+// eight 13 / 14 / 19, sixteen 23 / 17 / 19, sixty-four 62 / 32 / 23.
 static int cluster_blocks(int most, int nf) {
     int c = most;
     while (c > 4 && (long long)nf * c > (c == 16 ? 160 : 256)) c /= 2;

@@ -818,8 +818,8 @@ __global__ void __launch_bounds__(PlaneCfg<N>::NT, PlaneCfg<N>::MINB) k_plane_cg
 // between them; every block keeps the solve's scalars and takes the same
 // steps, block 0 writes them back. The blocks of a cluster are resident together by construction, so no
 // wait depends on another launch. An iteration takes 11 instead of 37 us on one
-// cell of 15^3, 23 instead of 39 on one of 27^3 and 59 instead of 78 on
-// thirty-two of them.
+// cell of 15^3, 24 instead of 39 on one of 27^3 and 59 instead of 78 on
+// thirty-two of them (cluster_blocks has the sizes of clusters).
 template <int N>
 struct ClusterCg {
     static constexpr bool ok = N <= 27;
